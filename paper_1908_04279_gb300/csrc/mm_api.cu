@@ -42,6 +42,7 @@ mm_status free_all(mm_handle* h) {
   tangent_free(h);
   for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
   h->graphs.clear();
+  if (h->res_xch) cudaFree(h->res_xch);
   if (h->diff_tab) cudaFree(h->diff_tab);
   if (h->local_n) cudaFree(h->local_n);
   void* anc[8] = {h->anc_off,  h->anc_cacc,  h->anc_fsc,    h->anc_flags,
@@ -232,7 +233,7 @@ mm_status configure(mm_handle* h) {
   if (gm > (h->ncells + 3) / 4) gm = (h->ncells + 3) / 4;
   h->grid_mom = (int)gm;
   h->npartial = std::max(h->grid_step * wpb, 4 * h->grid_mom);
-  return MM_OK;
+  return resident_configure(h);
 }
 
 // Read and clear the device status word; a set bit means a bounded device
@@ -248,6 +249,10 @@ mm_status check_status(mm_handle* h) {
     const unsigned int zeros[2] = {0u, 0u};
     CK(cudaMemcpy(&h->prm->status, &zero, sizeof zero, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(&h->prm->counter, zeros, sizeof zeros, cudaMemcpyHostToDevice));
+    if (h->res_xch) {  // and the arrivals that blocks which gave up never made
+      CK(cudaMemset(h->res_xch, 0, h->res_xch_bytes));
+      h->res_arrivals = 0;
+    }
     if (st & 8)
       return fail(h, MM_ERR_TIMEOUT,
                   "a bounded wait in the substep kernel gave up and so did the wait for its copies "
@@ -459,6 +464,8 @@ mm_status mm_create(const mm_grid* grid, const mm_rates* rates, mm_precision pre
   ALLOC(h->fields, 12 * nc * 8);
   ALLOC(h->staging, h->staging_n * 8);
   ALLOC(h->prm, sizeof(DevParams));
+  h->res_xch_bytes = 16 + 32 * (size_t)h->res_grid;
+  if (h->res_grid > 0) ALLOC(h->res_xch, h->res_xch_bytes);
 #undef ALLOC
   e = cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
@@ -524,6 +531,7 @@ mm_status mm_create(const mm_grid* grid, const mm_rates* rates, mm_precision pre
     if (e == cudaSuccess) e = cudaMemset(h->ucell, 0, 12 * nc * h->tsz);
     if (e == cudaSuccess) e = cudaMemset(h->mb, 0, h->mbn * h->tsz);
     if (e == cudaSuccess) e = cudaMemset(h->partial, 0, (size_t)h->npartial * 64);
+    if (e == cudaSuccess && h->res_xch) e = cudaMemset(h->res_xch, 0, h->res_xch_bytes);
     if (e != cudaSuccess) {
       cuda_fail(h, "initial state", e);
       return bail(MM_ERR_CUDA);
@@ -742,9 +750,13 @@ mm_status mm_micro_step(mm_handle* h, int n) {
 
 namespace mmh {
 
-// n substeps on the live state: one captured CUDA graph per (n, parity),
-// replayed (direct launches if graphs are off).
+// n substeps on the live state: one launch where the motor density fits the
+// chip (mm_resident.cu), else one captured CUDA graph per (n, parity), replayed
+// (direct launches if graphs are off).
 mm_status launch_substeps(mm_handle* h, int n) {
+  bool done = false;
+  const mm_status st = resident_substeps(h, n, &done);
+  if (st != MM_OK || done) return st;
   if (!h->use_graphs) {
     for (int i = 0; i < n; ++i) {
       CK(launch_one(h, h->parity, h->stream));

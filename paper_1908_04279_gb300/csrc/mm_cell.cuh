@@ -364,11 +364,6 @@ struct PsiConst {
   const T* trig;  // [4][nth]
 };
 
-// psi^{n+1} of the cell (lane = theta) by Eq. 1 in donor-cell flux form from
-// the staged columns psi5 / nb5 ([5][nth]: cell, east, west, north, south;
-// psi scaled by g on load), written to psi_out[cell]. Returns, per lane, the
-// partial sums of psi^{n+1} (cell_mass) and of psi^{n+1} n_b dtheta (the
-// coarse density of Eq. 5, acc) over the lane's orientations.
 // Trigonometric values of the orientation a lane handles when nth <= 32
 // (k = lane): cos, sin of theta_k and of the faces theta_{k +- 1/2}.
 template <typename T>
@@ -390,43 +385,67 @@ __device__ __forceinline__ LaneTrig<T> lane_trig(const T* trig, int nth, int lan
   return t;
 }
 
+// The psi and n_b values Eq. 1 reads for one (cell, theta): the cell, its
+// east, west, north and south neighbours, and psi at theta +- 1.
+template <typename T>
+struct PsiIn {
+  T pc, pe, pw, pn, ps, pp, pm;
+  T nc, ne, nw, nn, ns;
+};
+
+// psi^{n+1} of one (cell, theta) by Eq. 1 in donor-cell flux form. Every sum of
+// products is written as explicit fused operations, so that each kernel
+// inlining this function rounds it the same way.
+template <typename T>
+__device__ __forceinline__ T psi_point(const PsiConst<T>& q, const CellVel<T>& u,
+                                       const LaneTrig<T>& t, const PsiIn<T>& in) {
+  const T g = q.g;
+  const T Pc = g * in.pc, Pe = g * in.pe, Pw = g * in.pw, Pn = g * in.pn, Ps = g * in.ps;
+  const T ck = t.ck, sk = t.sk;
+  const T Vc = fma_t(q.glide, in.nc, q.vsp), Ve = fma_t(q.glide, in.ne, q.vsp);
+  const T Vw = fma_t(q.glide, in.nw, q.vsp);
+  const T Vn = fma_t(q.glide, in.nn, q.vsp);
+  const T Vs = fma_t(q.glide, in.ns, q.vsp);
+  const T axc = fma_t(-Vc, ck, u.uxc), axe = fma_t(-Ve, ck, u.uxe), axw = fma_t(-Vw, ck, u.uxw);
+  const T ayc = fma_t(-Vc, sk, u.uyc), ayn = fma_t(-Vn, sk, u.uyn), ays = fma_t(-Vs, sk, u.uys);
+  const T Ae = T(0.5) * (axc + axe), Aw = T(0.5) * (axw + axc);
+  const T An = T(0.5) * (ayc + ayn), As = T(0.5) * (ays + ayc);
+  const T cp = t.cp, sp = t.sp, cm = t.cm, sm = t.sm;
+  // Jeffery rotation p_perp . G . p at the faces k +- 1/2
+  const T wp = fma_t(-sp, fma_t(u.Gxx, cp, u.Gxy * sp), cp * fma_t(u.Gyx, cp, u.Gyy * sp));
+  const T wm = fma_t(-sm, fma_t(u.Gxx, cm, u.Gxy * sm), cm * fma_t(u.Gyx, cm, u.Gyy * sm));
+  const T Fe = donor(Ae, Pc, Pe), Fw = donor(Aw, Pw, Pc);
+  const T Fn = donor(An, Pc, Pn), Fs = donor(As, Ps, Pc);
+  const T Fp = donor(wp, Pc, g * in.pp), Fm = donor(wm, g * in.pm, Pc);
+  const T div = fma_t(Fp - Fm, q.inv_dth, fma_t(Fn - Fs, q.inv_dy, (Fe - Fw) * q.inv_dx));
+  return fma_t(-q.dt, div, Pc);
+}
+
+// The trigonometric values of orientation k from the table.
+template <typename T>
+__device__ __forceinline__ LaneTrig<T> trig_at(const T* trig, int nth, int k) {
+  const int km = k == 0 ? nth - 1 : k - 1;
+  return LaneTrig<T>{trig[k],           trig[nth + k],      trig[2 * nth + k],
+                     trig[3 * nth + k], trig[2 * nth + km], trig[3 * nth + km]};
+}
+
+// psi^{n+1} of the cell (lane = theta) by Eq. 1 in donor-cell flux form from
+// the staged columns psi5 / nb5 ([5][nth]: cell, east, west, north, south;
+// psi scaled by g on load), written to psi_out[cell]. Returns, per lane, the
+// partial sums of psi^{n+1} (cell_mass) and of psi^{n+1} n_b dtheta (the
+// coarse density of Eq. 5, acc) over the lane's orientations.
 template <typename T>
 __device__ __forceinline__ void psi_cell(const PsiConst<T>& q, const CellVel<T>& u,
                                          const T* psi5, const T* nb5, const T* s_nb, int nth,
                                          int lane, T* psi_out_cell, T& cell_mass, T& acc,
                                          const LaneTrig<T>* lt = nullptr) {
-  const T* cosk = q.trig;
-  const T* sink = q.trig + nth;
-  const T* cosf = q.trig + 2 * nth;
-  const T* sinf = q.trig + 3 * nth;
-  const T g = q.g;
   const bool cached = lt != nullptr && nth <= 32;
   for (int k = lane; k < nth; k += 32) {
-    const T Pc = g * psi5[k], Pe = g * psi5[nth + k], Pw = g * psi5[2 * nth + k];
-    const T Pn = g * psi5[3 * nth + k], Ps = g * psi5[4 * nth + k];
-    const T ck = cached ? lt->ck : cosk[k], sk = cached ? lt->sk : sink[k];
-    // (every sum of products below is written as explicit fused operations,
-    // so that each kernel inlining this function rounds it the same way)
-    const T Vc = fma_t(q.glide, nb5[k], q.vsp), Ve = fma_t(q.glide, nb5[nth + k], q.vsp);
-    const T Vw = fma_t(q.glide, nb5[2 * nth + k], q.vsp);
-    const T Vn = fma_t(q.glide, nb5[3 * nth + k], q.vsp);
-    const T Vs = fma_t(q.glide, nb5[4 * nth + k], q.vsp);
-    const T axc = fma_t(-Vc, ck, u.uxc), axe = fma_t(-Ve, ck, u.uxe), axw = fma_t(-Vw, ck, u.uxw);
-    const T ayc = fma_t(-Vc, sk, u.uyc), ayn = fma_t(-Vn, sk, u.uyn), ays = fma_t(-Vs, sk, u.uys);
-    const T Ae = T(0.5) * (axc + axe), Aw = T(0.5) * (axw + axc);
-    const T An = T(0.5) * (ayc + ayn), As = T(0.5) * (ays + ayc);
     const int kp = k + 1 == nth ? 0 : k + 1, km = k == 0 ? nth - 1 : k - 1;
-    const T cp = cached ? lt->cp : cosf[k], sp = cached ? lt->sp : sinf[k];
-    const T cm = cached ? lt->cm : cosf[km], sm = cached ? lt->sm : sinf[km];
-    // Jeffery rotation p_perp . G . p at the faces k +- 1/2
-    const T wp = fma_t(-sp, fma_t(u.Gxx, cp, u.Gxy * sp), cp * fma_t(u.Gyx, cp, u.Gyy * sp));
-    const T wm = fma_t(-sm, fma_t(u.Gxx, cm, u.Gxy * sm), cm * fma_t(u.Gyx, cm, u.Gyy * sm));
-    const T Fe = donor(Ae, Pc, Pe), Fw = donor(Aw, Pw, Pc);
-    const T Fn = donor(An, Pc, Pn), Fs = donor(As, Ps, Pc);
-    const T Fp = donor(wp, Pc, g * psi5[kp]), Fm = donor(wm, g * psi5[km], Pc);
-    const T div =
-        fma_t(Fp - Fm, q.inv_dth, fma_t(Fn - Fs, q.inv_dy, (Fe - Fw) * q.inv_dx));
-    const T pnew = fma_t(-q.dt, div, Pc);
+    const PsiIn<T> in{psi5[k],           psi5[nth + k],     psi5[2 * nth + k], psi5[3 * nth + k],
+                      psi5[4 * nth + k], psi5[kp],          psi5[km],          nb5[k],
+                      nb5[nth + k],      nb5[2 * nth + k],  nb5[3 * nth + k],  nb5[4 * nth + k]};
+    const T pnew = psi_point(q, u, cached ? *lt : trig_at(q.trig, nth, k), in);
     psi_out_cell[k] = pnew;
     cell_mass += pnew;
     acc = fma_t(pnew * s_nb[k], q.dth, acc);

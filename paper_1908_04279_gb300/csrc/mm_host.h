@@ -191,6 +191,12 @@ struct mm_handle {
   int stages = 1, chunk_rows = 1, chunks_per_cell = 1;
   bool tma = false;
   size_t smem = 0;
+  // many substeps in one launch with Mb on the chip (mm_resident.cu; grid 0: off)
+  int res_grid = 0, res_block = 0, res_NL = 0, res_own = 0, res_passes = 0;
+  size_t res_smem = 0;
+  unsigned res_epoch = 0, res_arrivals = 0;  // tags and arrivals used so far
+  size_t res_xch_bytes = 0;
+  unsigned long long* res_xch = nullptr;  // arrival counter and the psi sums the blocks exchange
   std::map<long long, cudaGraphExec_t> graphs;
   bool use_graphs = true;
   std::string err;
@@ -266,6 +272,10 @@ mm_status launch_substeps(mm_handle* h, int n);  // n substeps on the live state
 mm_status run_init(mm_handle* h);  // n_b, C, the scale-down and Mf of the live state
 mm_status run_moments(mm_handle* h);  // the 12 moment fields and the scalars of the live state
 mm_status velocity_update(mm_handle* h);  // h->u64 becomes the velocity in effect (and dt)
+
+// Defined in mm_resident.cu (many substeps per launch, Mb on the chip).
+mm_status resident_configure(mm_handle* h);
+mm_status resident_substeps(mm_handle* h, int n, bool* done);
 
 // Defined in mm_fluid.cu (thin-gap fluid solve).
 void fluid_free(mm_handle* h);

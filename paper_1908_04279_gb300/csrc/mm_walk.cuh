@@ -171,10 +171,13 @@ __device__ __forceinline__ void walk_dflux(const T (&M)[V], T (&D)[V], bool firs
 // element-wise steps (the halved differences, the fluxes) run as packed
 // two-value float32 instructions; the differences, the limiter's minima and
 // maxima and the flux differences stay scalar. Same value, bit for bit, as
-// walk_dflux<float, V>.
-template <int V>
+// walk_dflux<float, V>. With RAG the row's last node may be any node of its
+// last lane: keep[k] holds 0 at that node and 1 elsewhere and drops its slope
+// (one packed product per pair, against one select per node).
+template <int V, bool RAG = false>
 __device__ __forceinline__ void walk_dflux_x2(const float2 (&M)[V / 2], float2 (&D)[V / 2],
-                                              bool first, bool last, int seg) {
+                                              bool first, bool last, int seg,
+                                              const float2* keep = nullptr) {
   constexpr int H = V / 2;
   float ml = __shfl_up_sync(0xffffffffu, M[H - 1].y, 1, seg);
   const float mr = __shfl_down_sync(0xffffffffu, M[0].x, 1, seg);
@@ -192,17 +195,36 @@ __device__ __forceinline__ void walk_dflux_x2(const float2 (&M)[V / 2], float2 (
 #pragma unroll
   for (int k = 0; k < H; ++k) {
     const float b1 = k + 1 < H ? d[k + 1].x : dV, hb1 = k + 1 < H ? hd[k + 1].x : hdV;
-    const float r0 =
-        max3_t(min_xorsign_abs(d[k].x, hd[k].y), min_xorsign_abs(hd[k].x, d[k].y), 0.0f);
-    float r1 = max3_t(min_xorsign_abs(d[k].y, hb1), min_xorsign_abs(hd[k].y, b1), 0.0f);
-    if (k == H - 1 && last) r1 = 0.0f;  // plus end: F = M, no slope
-    F[k] = __fadd2_rn(M[k], make_float2(copysignf(r0, d[k].y), copysignf(r1, b1)));
+    float2 r;
+    r.x = max3_t(min_xorsign_abs(d[k].x, hd[k].y), min_xorsign_abs(hd[k].x, d[k].y), 0.0f);
+    r.y = max3_t(min_xorsign_abs(d[k].y, hb1), min_xorsign_abs(hd[k].y, b1), 0.0f);
+    if constexpr (RAG) {
+      r = __fmul2_rn(r, keep[k]);
+    } else {
+      if (k == H - 1 && last) r.y = 0.0f;  // plus end: F = M, no slope
+    }
+    F[k] = __fadd2_rn(M[k], make_float2(copysignf(r.x, d[k].y), copysignf(r.y, b1)));
   }
   float fl = __shfl_up_sync(0xffffffffu, F[H - 1].y, 1, seg);
   if (first) fl = 0.0f;
   D[0] = make_float2(fl - F[0].x, F[0].x - F[0].y);
 #pragma unroll
   for (int k = 1; k < H; ++k) D[k] = make_float2(F[k - 1].y - F[k].x, F[k].x - F[k].y);
+}
+
+// Sum of x over the nl lanes of a packed row (lanes sl = 0 .. nl - 1 of the
+// row are consecutive), valid in its first lane: the pairing of seg_sum for
+// a power-of-two nl, a tree with the missing lanes left out otherwise.
+template <typename T>
+__device__ __forceinline__ T packed_sum(T x, int nl, int sl) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    if (o < nl) {
+      const T y = __shfl_down_sync(0xffffffffu, x, o);
+      if (sl + o < nl) x += y;
+    }
+  }
+  return x;
 }
 
 template <typename T>

@@ -1,0 +1,97 @@
+"""Many substeps in one launch with the motor density resident on the chip
+(float32 form), against the float64 oracle (relative L2 1e-5, the float32
+tolerance of the parity tests) and against the same handle stepped one substep
+per call, which takes the streaming kernel (1e-6: the two differ in the order
+of a few float32 sums)."""
+import numpy as np
+import pytest
+
+from paper_1908_04279_gb300.inputs import Grid, Rates, SplitMix64, psi_isotropic_perturbed, random_divfree_flow
+
+pytestmark = pytest.mark.gpu
+
+KEYS = ("psi", "mb", "mf", "c")
+
+
+@pytest.fixture(scope="module")
+def mmod():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1908_04279_gb300 import build as B
+    B.build()
+    from paper_1908_04279_gb300 import mm
+    mm.load_library()
+    return mm
+
+
+def rel_l2(a, b):
+    nb = np.linalg.norm(b)
+    return np.linalg.norm(np.asarray(a, dtype=np.float64) - b) / (nb if nb > 0 else 1.0)
+
+
+def inputs(g, seed, scale):
+    rng = SplitMix64(seed)
+    mb = scale * rng.uniforms(g.micro_cells).reshape(g.ny, g.nx, g.ntheta, g.ns)
+    return psi_isotropic_perturbed(g, seed, amp=0.3), mb, random_divfree_flow(g, seed + 1, 5, 0.15)
+
+
+# (grid, substeps, scale of Mb): rows that end in every node of a lane and rows
+# of one node; passes that span cells (few orientations) and orientations
+# beyond a warp; fewer cells than SMs, several cells per warp; the most one
+# block holds (52 x 1024 values) and 4 times the SMs' cells; a scale-down
+@pytest.mark.parametrize("dims,n,scale", [
+    ((6, 5, 7, 1), 4, 0.3), ((9, 7, 5, 31), 5, 0.3), ((7, 6, 20, 25), 4, 0.3),
+    ((13, 11, 12, 10), 7, 0.3), ((5, 4, 40, 20), 4, 0.3), ((4, 3, 70, 36), 3, 0.3),
+    ((3, 2, 6, 128), 4, 0.3), ((1, 1, 8, 16), 6, 0.3), ((40, 31, 16, 16), 5, 0.3),
+    ((40, 40, 8, 9), 4, 0.3), ((45, 40, 24, 30), 4, 0.3), ((24, 20, 32, 32), 3, 0.3),
+    ((20, 17, 16, 24), 6, 3.0), ((19, 16, 10, 13), 5, 3.0)])
+def test_resident_substeps(mmod, dims, n, scale):
+    from oracle import oracle as O
+    g = Grid(*dims)
+    r = Rates(glide=0.3, v_sp=0.05)
+    psi, mb, u = inputs(g, 11, scale)
+    st = O.make_state(g, psi, mb)
+    dt = O.dt(g, r, st, u)
+    got = []
+    for each in (n, 1):
+        with mmod.Simulation(g, r, "fp32") as sim:
+            sim.set_state(psi, mb)
+            sim.set_velocity(u)
+            sim.set_dt(dt)
+            for _ in range(n // each):
+                sim.step(each)
+            got.append(sim.get_state())
+            _, sc = sim.moments()
+            assert abs(sc["N_psi"] - 1.0) < 1e-6  # the mass correction
+    O.run(g, r, st, u, dt, n)
+    if scale > 1:
+        assert st.mf.min() == 0.0  # the scale-down acts
+    for k in KEYS:
+        assert rel_l2(got[0][k], getattr(st, k)) <= 1e-5, k
+        assert rel_l2(got[0][k], got[1][k]) <= 1e-6, k
+
+
+def test_resident_on_two_streams(mmod):
+    """Two handles stepped alternately on two streams: the launches share the
+    device one after the other and each result is that of a handle alone."""
+    import torch
+    g = Grid(48, 40, 16, 16)
+    psi, mb, u = inputs(g, 3, 0.3)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    got = []
+    for alternate in (False, True):
+        sims = [mmod.Simulation(g, Rates(k_off=0.5 + i), "fp32", stream=s.cuda_stream)
+                for i, s in enumerate(streams)]
+        for sim in sims:
+            sim.set_state(psi, mb)
+            sim.set_velocity(u)
+        order = [(i, n) for n in (30, 31, 32) for i in (0, 1)]
+        for i, n in order if alternate else sorted(order):
+            sims[i].step(n)
+        got.append([sim.get_state() for sim in sims])
+        for sim in sims:
+            sim.close()
+    for a, b in zip(*got):
+        for k in KEYS:
+            assert np.array_equal(a[k], b[k]), k
