@@ -339,22 +339,16 @@ mm_status run_moments(mm_handle* h) {
   if (h->capture && (st = capture_rows(h)) != MM_OK) return st;
   const double dth = 2.0 * kPi / h->g.ntheta, ds = h->g.L / h->g.ns;
   const double dA = (1.0 / h->g.nx) * (1.0 / h->g.ny);
-  // the moments kernel reads rows with at most 4 values per lane
-  const int mV = h->V;  // the substep's vector width (float32 8 or 4, float64 2 or 1)
-  int mseg = 1;
-  while (mseg < h->g.ns / mV) mseg <<= 1;
   cudaError_t e;
   if (h->prec == MM_FP64)
     e = mm::launch_moments<double>((const double*)h->psi[h->parity], (const double*)h->mb,
-                                   (const double*)h->mf, (const double*)h->c, h->trig64, h->ncells, h->g.ntheta, h->g.ns, mV,
-                                   mseg, dth, ds,
-                                   h->g.L, dA, h->fields, h->partial, h->grid_mom, h->prm,
+                                   (const double*)h->mf, (const double*)h->c, h->trig64, h->ncells,
+                                   h->g.ntheta, h->g.ns, dth, ds, h->g.L, dA, h->fields, h->partial, h->grid_mom, h->prm,
                                    h->stream);
   else
     e = mm::launch_moments<float>((const float*)h->psi[h->parity], (const float*)h->mb,
-                                  (const float*)h->mf, (const float*)h->c, h->trig64, h->ncells, h->g.ntheta, h->g.ns, mV,
-                                  mseg, dth, ds,
-                                  h->g.L, dA, h->fields, h->partial, h->grid_mom, h->prm,
+                                  (const float*)h->mf, (const float*)h->c, h->trig64, h->ncells,
+                                  h->g.ntheta, h->g.ns, dth, ds, h->g.L, dA, h->fields, h->partial, h->grid_mom, h->prm,
                                   h->stream);
   CK(e);
   // with anchors (or a capture radius) the motor force of Eq. 10 acts in the
@@ -621,7 +615,11 @@ mm_status mm_set_state(mm_handle* h, const double* psi, const double* mb, const 
   if (h->tangent && (st = tangent_zero(h)) != MM_OK) return st;  // the tangent starts at zero
   if ((st = run_init(h)) != MM_OK) return st;
   // reference filament number for the float32 mass correction
-  if ((st = run_moments(h)) != MM_OK) return st;
+  CK(h->prec == MM_FP64
+         ? mm::launch_sum_psi<double>((const double*)h->psi[0], h->rows, h->partial, h->npartial,
+                                      h->prm, h->stream)
+         : mm::launch_sum_psi<float>((const float*)h->psi[0], h->rows, h->partial, h->npartial,
+                                     h->prm, h->stream));
   double sum_psi = 0.0;
   CK(cudaMemcpyAsync(&sum_psi, &h->prm->sum_psi, 8, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
@@ -806,33 +804,39 @@ mm_status mm_diffuse(mm_handle* h, double D_t, double D_r, double dt) {
                 "diffusion is not differentiated: end the adjoint recording or the tangent first");
   DeviceGuard dg(h->device);
   const int nx = h->g.nx, ny = h->g.ny, nth = h->g.ntheta;
-  if (!h->diff_tab) CK(cudaMalloc((void**)&h->diff_tab, (size_t)(3 * (nth + nx + ny) + 6) * 8));
   struct Dir {
     int mode, n;
     double hh, D;
-    double* tab;
   };
-  const Dir dirs[3] = {{0, nth, 2.0 * kPi / nth, D_r, h->diff_tab},
-                       {1, nx, 1.0 / nx, D_t, h->diff_tab + 3 * nth + 2},
-                       {2, ny, 1.0 / ny, D_t, h->diff_tab + 3 * (nth + nx) + 4}};
+  const Dir dirs[3] = {{0, nth, 2.0 * kPi / nth, D_r}, {1, nx, 1.0 / nx, D_t}, {2, ny, 1.0 / ny, D_t}};
   double a[3];
-  for (int d = 0; d < 3; ++d) a[d] = dirs[d].D * dt / (dirs[d].hh * dirs[d].hh);
-  CK(mm::launch_cn_factors(dirs[0].tab, nth, a[0], dirs[1].tab, nx, a[1], dirs[2].tab, ny, a[2],
-                           h->stream));
+  bool factors = false;
+  for (int d = 0; d < 3; ++d) {
+    a[d] = dirs[d].D * dt / (dirs[d].hh * dirs[d].hh);
+    factors = factors || !mm::cn_block_fits(dirs[d].n);
+  }
+  double* tab[3] = {nullptr, nullptr, nullptr};
+  if (factors) {  // a line too long for shared memory: Thomas factors
+    if (!h->diff_tab) CK(cudaMalloc((void**)&h->diff_tab, (size_t)(3 * (nth + nx + ny) + 6) * 8));
+    tab[0] = h->diff_tab;
+    tab[1] = h->diff_tab + 3 * nth + 2;
+    tab[2] = h->diff_tab + 3 * (nth + nx) + 4;
+    CK(mm::launch_cn_factors(tab[0], nth, a[0], tab[1], nx, a[1], tab[2], ny, a[2], h->stream));
+  }
   bool first = true;
   for (int d = 0; d < 3; ++d) {
-    if (!(dirs[d].D > 0.0) || dirs[d].n < 2) continue;  // a single point: L = 0
+    if (!(a[d] > 0.0) || dirs[d].n < 2) continue;  // a single point: L = 0
     // the float32 form folds the pending mass-correction factor into psi
     const double* sc = (first && h->prec == MM_FP32_MIXED) ? &h->prm->psi_scale : nullptr;
-    cudaError_t e =
-        h->prec == MM_FP64
-            ? mm::launch_cn_lines<double>((double*)h->psi[h->parity], dirs[d].mode, nx, ny, nth,
-                                          dirs[d].tab, dirs[d].n, -0.5 * a[d], 0.5 * a[d], sc,
-                                          h->stream)
-            : mm::launch_cn_lines<float>((float*)h->psi[h->parity], dirs[d].mode, nx, ny, nth,
-                                         dirs[d].tab, dirs[d].n, -0.5 * a[d], 0.5 * a[d], sc,
-                                         h->stream);
-    CK(e);
+    auto go = [&](auto* psi) -> cudaError_t {
+      using T = std::remove_pointer_t<decltype(psi)>;
+      if (mm::cn_block_fits(dirs[d].n))
+        return mm::launch_cn_block<T>(psi, dirs[d].mode, nx, ny, nth, dirs[d].n, a[d], sc,
+                                      h->stream);
+      return mm::launch_cn_lines<T>(psi, dirs[d].mode, nx, ny, nth, tab[d], dirs[d].n, -0.5 * a[d],
+                                    0.5 * a[d], sc, h->stream);
+    };
+    CK(h->prec == MM_FP64 ? go((double*)h->psi[h->parity]) : go((float*)h->psi[h->parity]));
     first = false;
   }
   if (!first && h->prec == MM_FP32_MIXED) CK(mm::launch_set_scale_one(&h->prm->psi_scale, h->stream));

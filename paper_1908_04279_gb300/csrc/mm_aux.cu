@@ -2,26 +2,12 @@
 // Alg. 2 scale-down), the maxima of the adaptive-substep rule, and the
 // macroscale moments (Alg. 1 after the inner loop; Eq. 10's force and force
 // dipole with anchors in the filament's own cell).
-#include "mm_walk.cuh"
+#include "mm_rows.cuh"
 
 namespace mm {
 
 namespace {
 
-
-// Sum over the block of one value per thread; result valid in thread 0.
-// `red` holds at least 32 doubles. Ends with a barrier so `red` can be reused.
-__device__ double block_sum(double x, double* red) {
-  x = warp_sum(x);
-  const int w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  if ((threadIdx.x & 31) == 0) red[w] = x;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int i = 0; i < nw; ++i) t += red[i];
-  __syncthreads();
-  return t;
-}
 
 // The copies of a CopySegs: 16-byte vectors where both addresses are 16-byte
 // aligned, then the remaining bytes one by one; every thread of the grid takes
@@ -54,58 +40,20 @@ __global__ void k_convert(TO* out, const TI* in, size_t n, const double* scale) 
   }
 }
 
-// Per cell: n_b of every row (sequential sum over s in float64, stored in the
-// state precision), C = sum_k psi n_b dtheta, the Alg. 2 scale-down where
-// C > M, Mf = M - C.
-template <typename T>
-__global__ void k_init_cells(T* mb, const T* psi, T* nb, T* mf, T* c, const T* mtot,
-                             long long ncells, int nth, int ns, double ds, double dth) {
-  __shared__ double red[32];
-  __shared__ double s_f;
-  for (long long cell = blockIdx.x; cell < ncells; cell += gridDim.x) {
-    double acc = 0.0;
-    for (int k = threadIdx.x; k < nth; k += blockDim.x) {
-      const T* row = mb + ((size_t)cell * nth + k) * ns;
-      double s0 = 0.0;
-      for (int j = 0; j < ns; ++j) s0 += (double)row[j] * ds;
-      nb[cell * nth + k] = (T)s0;
-      acc += (double)psi[cell * nth + k] * s0 * dth;
-    }
-    const double C = block_sum(acc, red);
-    if (threadIdx.x == 0) {
-      const double M = (double)mtot[cell];
-      double f = 1.0, Cc = C;
-      if (M < C) {
-        f = M / C;
-        Cc = M;
-      }
-      s_f = f;
-      c[cell] = (T)Cc;
-      mf[cell] = (T)(M - Cc);
-    }
-    __syncthreads();
-    const double f = s_f;
-    if (f != 1.0) {
-      for (int k = threadIdx.x; k < nth; k += blockDim.x) {
-        T* row = mb + ((size_t)cell * nth + k) * ns;
-        for (int j = 0; j < ns; ++j) row[j] = (T)((double)row[j] * f);
-        nb[cell * nth + k] = (T)((double)nb[cell * nth + k] * f);
-      }
-    }
-    __syncthreads();
-  }
-}
-
 __device__ __forceinline__ void atomic_max_nonneg(double* addr, double v) {
   // Non-negative doubles order like their bit patterns as unsigned integers.
   atomicMax(reinterpret_cast<unsigned long long*>(addr), (unsigned long long)__double_as_longlong(v));
 }
 
 // Maxima of the adaptive-substep rule: max(|ax|/dx + |ay|/dy),
-// max |omega(theta_{k+1/2})| / dtheta, and max_cell sum_k psi dtheta. One warp
-// per cell, lanes over theta, in the state precision (float64 in the float64
-// form, whose dt must agree with a float64 evaluation; float32 in the float32
-// form, whose state is float32 anyway); the maxima are exact.
+// max |omega(theta_{k+1/2})| / dtheta, and max_cell sum_k psi dtheta, in the
+// state precision (float64 in the float64 form, whose dt must agree with a
+// float64 evaluation; float32 in the float32 form, whose state is float32
+// anyway); the maxima are exact. A cell takes `seg` lanes (nth rounded up to a
+// power of two, 32 at most), so that a warp holds 32 / seg cells. Bound by
+// latency: full occupancy hides it, and a block reduces its maxima before the
+// three atomics (one set per warp kept the atomics of one address in a queue:
+// 128^2 x 32 15 us).
 template <typename T>
 __device__ __forceinline__ T warp_max_t(T x) {
 #pragma unroll
@@ -113,130 +61,231 @@ __device__ __forceinline__ T warp_max_t(T x) {
   return x;
 }
 
+constexpr int kDtBlock = 512;
+
 template <typename T>
-__global__ void k_dt_max(const T* psi, const T* nb, const T* u, const T* trig, long long ncells,
-                         int nx, int ny, int nth, double inv_dx64, double inv_dy64,
-                         double inv_dth64, double dth64, double glide64, double vsp64,
-                         DevParams* prm) {
+__global__ void __launch_bounds__(kDtBlock)
+    k_dt_max(const T* psi, const T* nb, const T* u, const T* trig, int ncells, int nx, int ny,
+             int nth, int seg, double inv_dx64, double inv_dy64, double inv_dth64, double dth64,
+             double glide64, double vsp64, DevParams* prm) {
   const int lane = threadIdx.x & 31;
-  const long long gw = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5);
-  const long long W = (long long)gridDim.x * (blockDim.x >> 5);
+  const int cps = 32 / seg, sub = lane / seg, kl = lane - sub * seg;
+  const long long gw = blockIdx.x * (long long)(kDtBlock / 32) + (threadIdx.x >> 5);
+  const long long W = (long long)gridDim.x * (kDtBlock / 32);
   const T g = (T)prm->psi_scale;
   const T inv_dx = (T)inv_dx64, inv_dy = (T)inv_dy64, inv_dth = (T)inv_dth64, dth = (T)dth64;
   const T glide = (T)glide64, vsp = (T)vsp64, h = T(0.5);
   T adv = T(0), rot = T(0), rhomax = T(0);
   const T* ux = u;
   const T* uy = u + ncells;
-  for (long long cell = gw; cell < ncells; cell += W) {
-    const int ix = (int)(cell % nx), iy = (int)(cell / nx);
-    const int xp = ix + 1 == nx ? 0 : ix + 1, xm = ix == 0 ? nx - 1 : ix - 1;
-    const int yp = iy + 1 == ny ? 0 : iy + 1, ym = iy == 0 ? ny - 1 : iy - 1;
-    const T Gxx = (ux[(long long)iy * nx + xp] - ux[(long long)iy * nx + xm]) * h * inv_dx;
-    const T Gxy = (ux[(long long)yp * nx + ix] - ux[(long long)ym * nx + ix]) * h * inv_dy;
-    const T Gyx = (uy[(long long)iy * nx + xp] - uy[(long long)iy * nx + xm]) * h * inv_dx;
-    const T Gyy = (uy[(long long)yp * nx + ix] - uy[(long long)ym * nx + ix]) * h * inv_dy;
+  for (long long c0 = gw * cps; c0 < ncells; c0 += W * cps) {
+    const bool on = c0 + sub < ncells;
+    const int cell = on ? (int)c0 + sub : 0;
+    const int iy = cell / nx, ix = cell - iy * nx;
+    const size_t ce = (size_t)iy * nx + (ix + 1 == nx ? 0 : ix + 1);
+    const size_t cw = (size_t)iy * nx + (ix == 0 ? nx - 1 : ix - 1);
+    const size_t cn = (size_t)(iy + 1 == ny ? 0 : iy + 1) * nx + ix;
+    const size_t cs = (size_t)(iy == 0 ? ny - 1 : iy - 1) * nx + ix;
+    const T Gxx = (ux[ce] - ux[cw]) * h * inv_dx, Gxy = (ux[cn] - ux[cs]) * h * inv_dy;
+    const T Gyx = (uy[ce] - uy[cw]) * h * inv_dx, Gyy = (uy[cn] - uy[cs]) * h * inv_dy;
     const T uxc = ux[cell], uyc = uy[cell];
     T rho = T(0);
-    for (int k = lane; k < nth; k += 32) {
-      const T V = vsp + glide * nb[cell * nth + k];
+    for (int k = kl; on && k < nth; k += seg) {
+      const size_t e = (size_t)cell * nth + k;
+      const T V = vsp + glide * nb[e];
       const T ax = uxc - V * trig[k], ay = uyc - V * trig[nth + k];
       adv = tmax(adv, fabs(ax) * inv_dx + fabs(ay) * inv_dy);
       const T cp = trig[2 * nth + k], sp = trig[3 * nth + k];
       const T w = -sp * (Gxx * cp + Gxy * sp) + cp * (Gyx * cp + Gyy * sp);
       rot = tmax(rot, fabs(w) * inv_dth);
-      rho += psi[cell * nth + k] * g * dth;
+      rho += psi[e] * g * dth;
     }
-    rhomax = tmax(rhomax, warp_sum_t(rho));
+    rhomax = tmax(rhomax, seg_sum(rho, seg));
   }
+  __shared__ T red[3][kDtBlock / 32];
   adv = warp_max_t(adv);
   rot = warp_max_t(rot);
+  rhomax = warp_max_t(rhomax);
   if (lane == 0) {
-    atomic_max_nonneg(&prm->dtmax[0], (double)adv);
-    atomic_max_nonneg(&prm->dtmax[1], (double)rot);
-    atomic_max_nonneg(&prm->dtmax[2], (double)rhomax);
+    red[0][threadIdx.x >> 5] = adv;
+    red[1][threadIdx.x >> 5] = rot;
+    red[2][threadIdx.x >> 5] = rhomax;
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    T m = red[threadIdx.x][0];
+    for (int q = 1; q < kDtBlock / 32; ++q) m = tmax(m, red[threadIdx.x][q]);
+    atomic_max_nonneg(&prm->dtmax[threadIdx.x], (double)m);
   }
 }
 
-// ---- s-row sums for the moments: n_b = sum_j Mb_j ds and m1 = sum_j s_j Mb_j ds
+constexpr int kMomPasses = 4;  // passes of rows in flight before they are reduced
 
-// Compensated float32 accumulator (hi + lo), error-free transformations of
-// Knuth (TwoSum) and of the fused multiply-add (TwoProduct).
-struct FF {
-  float hi, lo;
-};
-__device__ __forceinline__ void ff_add(FF& a, float x) {
-  const float s = a.hi + x;
-  const float bb = s - a.hi;
-  const float e = (a.hi - (s - bb)) + (x - bb);
-  a.hi = s;
-  a.lo += e;
-}
-__device__ __forceinline__ void ff_add_prod(FF& a, float u, float v) {
-  const float p = __fmul_rn(u, v);  // not contracted into the sum below
-  const float pe = __fmaf_rn(u, v, -p);
-  ff_add(a, p);
-  a.lo += pe;
-}
-__device__ __forceinline__ void ff_merge(FF& a, const FF& b) {
-  const float lo = a.lo + b.lo;
-  a.lo = 0.0f;
-  ff_add(a, b.hi);
-  a.lo += lo;
-}
-// a + b (TwoSum of the high parts, low parts added)
-__device__ __forceinline__ FF ff_sum(const FF& a, const FF& b) {
-  const float s = __fadd_rn(a.hi, b.hi);
-  const float bb = __fsub_rn(s, a.hi);
-  const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(b.hi, bb));
-  return FF{s, __fadd_rn(e, __fadd_rn(a.lo, b.lo))};
-}
-// p w for a float p and a float-float w (TwoProduct of the high part)
-__device__ __forceinline__ FF ff_scale(float p, const FF& w) {
-  const float h = __fmul_rn(p, w.hi);
-  return FF{h, __fmaf_rn(p, w.lo, __fmaf_rn(p, w.hi, -h))};
-}
-// a w for float-float a and w (the lo * lo term dropped)
-__device__ __forceinline__ FF ff_prod(const FF& a, const FF& w) {
-  const float h = __fmul_rn(a.hi, w.hi);
-  return FF{h, __fmaf_rn(a.hi, w.lo, __fmaf_rn(a.lo, w.hi, __fmaf_rn(a.hi, w.hi, -h)))};
-}
-
-// Row sums of the V values a lane holds, reduced over the row's `seg` lanes;
-// every lane of the segment gets (n_b / ds, m1 / ds) in float64.
-template <int V>
-__device__ __forceinline__ void row_sums(const double (&m)[V], const double (&sj)[V], int seg,
-                                         double& nb, double& m1) {
-  double a = 0.0, b = 0.0;
+// Set-up of a state, a warp per cell: n_b of every row (float-float in the
+// float32 form: exact to 2^-48 before its one rounding), C = sum_k psi n_b
+// dtheta, the Alg. 2 scale-down where C > M, Mf = M - C. Bound by HBM beyond
+// the L2: every lane loads 32 (64) consecutive bytes, four passes of rows in
+// flight per warp (a thread per row, one node per load and a float64 sum per
+// node took 90 us at 128^2 x 32^2 where the bytes need 10).
+template <typename T, int VW>
+__global__ void __launch_bounds__(128)
+    k_init_cells(T* mb, const T* psi, T* nb, T* mf, T* c, const T* mtot, int ncells, int nth,
+                 int ns, double ds, double dth, float2 dsf, float2 dthf) {
+  const int lane = threadIdx.x & 31;
+  const PackedGeom g = packed_geom(lane, ns);
+  const int gw = blockIdx.x * 4 + (threadIdx.x >> 5), W = gridDim.x * 4;
+  for (long long cl = gw; cl < ncells; cl += W) {
+    const int cell = (int)cl;
+    T* rows = mb + (size_t)cell * nth * ns + g.sl * 8;
+    const T* pc = psi + (size_t)cell * nth;
+    T* nbc = nb + (size_t)cell * nth;
+    FF accf{0.f, 0.f};
+    double acc = 0.0;
+    for (int r0 = 0; r0 < nth; r0 += kMomPasses * g.rpp) {
+      T m[kMomPasses][8];
 #pragma unroll
-  for (int v = 0; v < V; ++v) {
-    a += m[v];
-    b += sj[v] * m[v];
+      for (int u = 0; u < kMomPasses; ++u) {
+        const int k = r0 + u * g.rpp + g.rslot;
+        load_row8<T, VW>(rows + (size_t)(k < nth ? k : 0) * ns, k < nth ? g.nv : 0, m[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < kMomPasses; ++u) {
+        const int k = r0 + u * g.rpp + g.rslot;
+        const bool own = g.sl == 0 && g.rslot < g.rpp && k < nth;
+        if constexpr (sizeof(T) == 4) {
+          const FF s = packed_sum_ff<0>(row_sum8(m[u]), g.nl, g.sl);
+          if (own) {
+            const FF n = ff_prod(s, FF{dsf.x, dsf.y});
+            nbc[k] = n.hi + n.lo;
+            accf = ff_sum(accf, ff_scale(pc[k], n));
+          }
+        } else {
+          const double s =
+              packed_sum(((m[u][0] + m[u][1]) + (m[u][2] + m[u][3])) +
+                             ((m[u][4] + m[u][5]) + (m[u][6] + m[u][7])),
+                         g.nl, g.sl) *
+              ds;
+          if (own) {
+            nbc[k] = s;
+            acc = fma(pc[k], s, acc);
+          }
+        }
+      }
+    }
+    // C, and the scale-down where it exceeds the total motors
+    const T M = mtot[cell];
+    double C = 0.0;
+    bool over;
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+        accf = ff_sum(accf, FF{__shfl_xor_sync(0xffffffffu, accf.hi, o),
+                               __shfl_xor_sync(0xffffffffu, accf.lo, o)});
+      const FF Cf = ff_prod(accf, FF{dthf.x, dthf.y});
+      const FF left = ff_sum(FF{M, 0.f}, FF{-Cf.hi, -Cf.lo});  // M - C
+      const float mfc = left.hi + left.lo;
+      if (fabsf(mfc) <= 3.402823466e38f) {
+        over = mfc < 0.f;
+        C = over ? (double)Cf.hi + (double)Cf.lo : 0.0;
+        if (!over && lane == 0) {
+          c[cell] = Cf.hi + Cf.lo;
+          mf[cell] = mfc;
+        }
+      } else {
+        // sums beyond float32 (or not finite): the cell again in float64
+        for (int k = lane; k < nth; k += 32) {
+          const T* row = mb + ((size_t)cell * nth + k) * ns;
+          double s = 0.0;
+          for (int j = 0; j < ns; ++j) s += (double)row[j] * ds;
+          nbc[k] = (T)s;
+          acc += (double)pc[k] * s * dth;
+        }
+        C = warp_sum(acc);
+        over = (double)M < C;
+        if (!over && lane == 0) {
+          c[cell] = (T)C;
+          mf[cell] = (T)((double)M - C);
+        }
+        __syncwarp();
+      }
+    } else {
+      C = warp_sum(acc) * dth;
+      over = M < C;
+      if (!over && lane == 0) {
+        c[cell] = C;
+        mf[cell] = M - C;
+      }
+    }
+    if (over) {
+      const double f = (double)M / C;
+      if (lane == 0) {
+        c[cell] = M;
+        mf[cell] = T(0);
+      }
+      __syncwarp();
+      T* all = mb + (size_t)cell * nth * ns;
+      for (int e = lane; e < nth * ns; e += 32) all[e] = (T)((double)all[e] * f);
+      for (int k = lane; k < nth; k += 32) nbc[k] = (T)((double)nbc[k] * f);
+    }
   }
-  for (int o = seg >> 1; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(0xffffffffu, a, o, seg);
-    b += __shfl_xor_sync(0xffffffffu, b, o, seg);
-  }
-  nb = a;
-  m1 = b;
 }
 
-// Float32 form: the float-float row sums (n_b / ds and m1 / ds) left
-// unconverted; every lane of the segment gets them.
-template <int V>
-__device__ __forceinline__ void row_sums_ff(const float (&m)[V], const float (&sj)[V], int seg,
-                                            FF& a, FF& b) {
-  a = FF{0.f, 0.f};
-  b = FF{0.f, 0.f};
-#pragma unroll
-  for (int v = 0; v < V; ++v) {
-    ff_add(a, m[v]);
-    ff_add_prod(b, sj[v], m[v]);
+// The sum of psi over all cells and angles into prm->sum_psi (the reference of
+// the float32 form's mass correction): per thread, block and last block in a
+// fixed order, float-float in the float32 form.
+template <typename T>
+__global__ void __launch_bounds__(512) k_sum_psi(const T* psi, size_t n, double* partial,
+                                                 DevParams* prm) {
+  __shared__ double s_red[16];
+  __shared__ unsigned int s_last;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const size_t stride = (size_t)gridDim.x * blockDim.x;
+  size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if constexpr (sizeof(T) == 4) {
+    float2* red = reinterpret_cast<float2*>(s_red);
+    float2* part = reinterpret_cast<float2*>(partial);
+    float2 a = make_float2(0.f, 0.f), b = a;
+    for (; i + stride < n; i += 2 * stride) {
+      const float x = psi[i], y = psi[i + stride];
+      two_sum_acc2(a, x);
+      two_sum_acc2(b, y);
+    }
+    if (i < n) two_sum_acc2(a, psi[i]);
+    a = warp_sum_ff2(ff2_add(a, b));
+    if (lane == 0) red[w] = a;
+    __syncthreads();
+    if (w == 0) {
+      a = warp_sum_ff2(lane < 16 ? red[lane] : make_float2(0.f, 0.f));
+      if (lane == 0) part[blockIdx.x] = a;
+    }
+  } else {
+    double a = 0.0, b = 0.0;
+    for (; i + stride < n; i += 2 * stride) {
+      a += psi[i];
+      b += psi[i + stride];
+    }
+    if (i < n) a += psi[i];
+    a = warp_sum(a + b);
+    if (lane == 0) s_red[w] = a;
+    __syncthreads();
+    if (w == 0) {
+      a = warp_sum(lane < 16 ? s_red[lane] : 0.0);
+      if (lane == 0) partial[blockIdx.x] = a;
+    }
   }
-  for (int o = seg >> 1; o > 0; o >>= 1) {
-    FF ao{__shfl_xor_sync(0xffffffffu, a.hi, o, seg), __shfl_xor_sync(0xffffffffu, a.lo, o, seg)};
-    FF bo{__shfl_xor_sync(0xffffffffu, b.hi, o, seg), __shfl_xor_sync(0xffffffffu, b.lo, o, seg)};
-    ff_merge(a, ao);
-    ff_merge(b, bo);
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicInc(&prm->counter2, gridDim.x - 1) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last || w != 0) return;
+  __threadfence();
+  if constexpr (sizeof(T) == 4) {
+    const float2 t = warp_sum_ldcg_ff2(reinterpret_cast<const float2*>(partial), (int)gridDim.x, lane);
+    if (lane == 0) prm->sum_psi = (double)t.x + (double)t.y;
+  } else {
+    const double t = warp_sum_ldcg(partial, (int)gridDim.x, 1, lane);
+    if (lane == 0) prm->sum_psi = t;
   }
 }
 
@@ -280,25 +329,20 @@ __device__ __forceinline__ int scatter_field(int lane) {
   return ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
 }
 
-constexpr int kMomPasses = 4;
-
-template <typename T, int V>
-struct alignas(sizeof(T) * V) VPack {
-  T v[V];
-};
-
 // Moments, one warp per cell, no block barriers before the final sums. The s-rows of the cell are
-// read with the substep kernel's lane mapping (a row over `seg` lanes, V
-// consecutive nodes per lane, vector loads) and reduced to n_b and m1: in
-// float64 in the float64 form, compensated float32 (float-float) converted to
-// float64 per row in the float32 form -- these are the s-reductions feeding
-// the force and the force dipole. Then lanes over theta form the 12 fields.
+// read as packed rows (eight consecutive nodes per lane, vector loads) and
+// reduced to n_b and m1: in float64 in the float64 form (the float64 pipe bounds
+// it: eight nodes per lane leave 2.5 additions a node with the cross-lane sums,
+// two per lane 6: 128^2 x 32^2 343 -> 161 us), float-float in the float32 form
+// (the float32 pipe: 17 operations a node, the two sums as one pair; a node per
+// lane where ns is not a multiple of 4 had the cross-lane sums at every node: 85 x
+// 61 x 24 x 30 42 -> 24 us; 256^2 x 64^2 352 -> 315 us) -- these are the
+// s-reductions feeding the force and the force dipole. Then lanes over theta form the 12 fields.
 // Each warp keeps partial global sums, added per block at the end; the last
 // block to finish adds the block partials in a fixed order.
-template <typename T, int V>
-__global__ void k_moments(const T* psi, const T* mb, const T* mf, const T* c,
-                          const double* trig, long long ncells, int nth, int ns, int seg,
-                          double dth, double ds, double L, double dA, float hds, double* fields,
+template <typename T, int VW, int NL>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1) k_moments(const T* psi, const T* mb, const T* mf, const T* c,
+                          const double* trig, long long ncells, int nth, int ns, double dth, double ds, double L, double dA, float hds, double* fields,
                           double* partial, DevParams* prm) {
   extern __shared__ double msm[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -311,17 +355,16 @@ __global__ void k_moments(const T* psi, const T* mb, const T* mf, const T* c,
   const long long W = (long long)gridDim.x * (blockDim.x >> 5);
   const double g = prm->psi_scale;
   const double Fm = prm->force_scale, ell = prm->ell;
-  const int sl = lane & (seg - 1), rslot = lane / seg, rpp = 32 / seg;
-  const int nl = ns / V;
-  const bool lane_ok = sl < nl;
-  T sj[V];
+  const PackedGeom pg = packed_geom(lane, ns);
+  const int sl = pg.sl, rslot = pg.rslot, rpp = pg.rpp;
+  T sj[8];
 #pragma unroll
-  for (int v = 0; v < V; ++v) {
+  for (int v = 0; v < 8; ++v) {
     // s_j = (2j + 1 - ns) ds / 2; the float32 form in float32 (one rounding)
     if constexpr (sizeof(T) == 4)
-      sj[v] = (float)(2 * (sl * V + v) + 1 - ns) * hds;
+      sj[v] = (float)(2 * (sl * 8 + v) + 1 - ns) * hds;
     else
-      sj[v] = -0.5 * L + ((double)(sl * V + v) + 0.5) * ds;
+      sj[v] = -0.5 * L + ((double)(sl * 8 + v) + 0.5) * ds;
   }
   // global accumulators: N_psi, bound, free, sum psi cos, sum psi sin, sum psi, sum tr
   double gs[7] = {0, 0, 0, 0, 0, 0, 0};
@@ -342,33 +385,32 @@ __global__ void k_moments(const T* psi, const T* mb, const T* mf, const T* c,
     // kMomPasses passes of rows loaded before they are reduced (more bytes in
     // flight per warp)
     for (int r0 = 0; r0 < nth; r0 += kMomPasses * rpp) {
-      T m[kMomPasses][V];
+      T m[kMomPasses][8];
 #pragma unroll
       for (int u = 0; u < kMomPasses; ++u) {
         const int k = r0 + u * rpp + rslot;
-        if (k < nth && lane_ok) {
-          const VPack<T, V> q =
-              *reinterpret_cast<const VPack<T, V>*>(mb + ((size_t)cell * nth + k) * ns + sl * V);
-#pragma unroll
-          for (int v = 0; v < V; ++v) m[u][v] = q.v[v];
-        } else {
-#pragma unroll
-          for (int v = 0; v < V; ++v) m[u][v] = T(0);
-        }
+        load_row8<T, VW>(mb + ((size_t)cell * nth + (k < nth ? k : 0)) * ns + sl * 8,
+                         k < nth ? pg.nv : 0, m[u]);
       }
 #pragma unroll
       for (int u = 0; u < kMomPasses; ++u) {
         const int k = r0 + u * rpp + rslot;
+        const bool own = sl == 0 && rslot < rpp && k < nth;
         if constexpr (sizeof(T) == 4) {
-          FF a, b;
-          row_sums_ff<V>(m[u], sj, seg, a, b);
-          if (sl == 0 && k < nth) s_ff[k] = make_float4(a.hi, a.lo, b.hi, b.lo);
+          const FF2x a = packed_sum_ff2x<NL>(row_sums8(m[u], sj), pg.nl, sl);
+          if (own) s_ff[k] = make_float4(a.hi.x, a.lo.x, a.hi.y, a.lo.y);
         } else {
-          double nbk, m1k;
-          row_sums<V>(m[u], sj, seg, nbk, m1k);
-          if (sl == 0 && k < nth) {
-            s_nb[k] = nbk * ds;
-            s_m1[k] = m1k * ds;
+          double a = 0.0, b = 0.0;
+#pragma unroll
+          for (int v = 0; v < 8; ++v) {
+            a += m[u][v];
+            b = fma(sj[v], m[u][v], b);
+          }
+          a = packed_sum(a, pg.nl, sl);
+          b = packed_sum(b, pg.nl, sl);
+          if (own) {
+            s_nb[k] = a * ds;
+            s_m1[k] = b * ds;
           }
         }
       }
@@ -638,13 +680,40 @@ cudaError_t launch_prep_ucell(T* ucell, const double* u64, long long ncells, int
   return cudaGetLastError();
 }
 
+// Widest vector of 16 bytes at most whose values divide ns.
+template <typename T>
+int row_vector(int ns) {
+  for (int v = 16 / (int)sizeof(T); v > 1; v /= 2)
+    if (ns % v == 0) return v;
+  return 1;
+}
+float2 float_pair(double x) {
+  const float hi = (float)x;
+  return make_float2(hi, (float)(x - (double)hi));
+}
+
 template <typename T>
 cudaError_t launch_init_cells(T* mb, const T* psi, T* nb, T* mf, T* c, const T* mtot,
                               long long ncells, int nth, int ns, double ds, double dth,
                               cudaStream_t s) {
-  int block = nth >= 128 ? 128 : (nth >= 64 ? 64 : 32);
-  long long g = ncells < 152 * 16 ? ncells : 152 * 16;
-  k_init_cells<T><<<(int)g, block, 0, s>>>(mb, psi, nb, mf, c, mtot, ncells, nth, ns, ds, dth);
+  const int g = grid_for(ncells * 32, 128);
+  auto go = [&](auto kern) {
+    kern<<<g, 128, 0, s>>>(mb, psi, nb, mf, c, mtot, (int)ncells, nth, ns, ds, dth,
+                           float_pair(ds), float_pair(dth));
+    return cudaGetLastError();
+  };
+  const int vw = row_vector<T>(ns);
+  if constexpr (sizeof(T) == 4)
+    if (vw == 4) return go(k_init_cells<T, 4>);
+  return vw == 2 ? go(k_init_cells<T, 2>) : go(k_init_cells<T, 1>);
+}
+
+template <typename T>
+cudaError_t launch_sum_psi(const T* psi, size_t n, double* partial, int max_partial,
+                           DevParams* prm, cudaStream_t s) {
+  int g = grid_for((long long)((n + 7) / 8), 512);
+  if (g > max_partial) g = max_partial;
+  k_sum_psi<T><<<g, 512, 0, s>>>(psi, n, partial, prm);
   return cudaGetLastError();
 }
 
@@ -652,10 +721,12 @@ template <typename T>
 cudaError_t launch_dt_max(const T* psi, const T* nb, const T* u, const T* trig, long long ncells,
                           int nx, int ny, int nth, double inv_dx, double inv_dy, double inv_dth,
                           double dth, double glide, double vsp, DevParams* prm, cudaStream_t s) {
-  long long g = (ncells + 3) / 4;  // warp per cell, 4 warps per block
-  if (g > 152 * 8) g = 152 * 8;
-  k_dt_max<T><<<(int)g, 128, 0, s>>>(psi, nb, u, trig, ncells, nx, ny, nth, inv_dx, inv_dy,
-                                     inv_dth, dth, glide, vsp, prm);
+  int seg = 1;
+  while (seg < 32 && seg < nth) seg <<= 1;
+  int g = grid_for((ncells + 32 / seg - 1) / (32 / seg) * 32, kDtBlock);
+  if (g > 152 * 4) g = 152 * 4;
+  k_dt_max<T><<<g, kDtBlock, 0, s>>>(psi, nb, u, trig, (int)ncells, nx, ny, nth, seg, inv_dx,
+                                     inv_dy, inv_dth, dth, glide, vsp, prm);
   return cudaGetLastError();
 }
 
@@ -666,9 +737,9 @@ cudaError_t launch_dt_finalize(DevParams* prm, double ds, double L, double cfl, 
 
 template <typename T>
 cudaError_t launch_moments(const T* psi, const T* mb, const T* mf, const T* c,
-                           const double* trig, long long ncells, int nth, int ns, int V, int seg,
-                           double dth, double ds, double L, double dA, double* fields,
-                           double* partial, int nblocks, DevParams* prm, cudaStream_t s) {
+                           const double* trig, long long ncells, int nth, int ns, double dth,
+                           double ds, double L, double dA, double* fields, double* partial,
+                           int nblocks, DevParams* prm, cudaStream_t s) {
   // nblocks blocks of 4 warps; the partial buffer holds 8 doubles per warp
   const int block = 128;
   // per warp: n_b and m1 of the rows (float64), and their float-float sums
@@ -678,17 +749,24 @@ cudaError_t launch_moments(const T* psi, const T* mb, const T* mf, const T* c,
       cudaError_t e = mm::raise_smem_limit(kern, (int)smem);
       if (e != cudaSuccess) return e;
     }
-    kern<<<nblocks, block, smem, s>>>(psi, mb, mf, c, trig, ncells, nth, ns, seg, dth, ds, L, dA,
+    kern<<<nblocks, block, smem, s>>>(psi, mb, mf, c, trig, ncells, nth, ns, dth, ds, L, dA,
                                       (float)(0.5 * ds), fields, partial, prm);
     return cudaGetLastError();
   };
-  if constexpr (sizeof(T) == 4)
-    if (V == 8) return go(k_moments<T, 8>);
-  if (V == 4) return go(k_moments<T, 4>);
-  if (V == 2) return go(k_moments<T, 2>);
-  return go(k_moments<T, 1>);
+  const int vw = row_vector<T>(ns);
+  if constexpr (sizeof(T) == 4) {
+    if (ns == 64) return go(k_moments<T, 4, 8>);
+    if (ns == 32) return go(k_moments<T, 4, 4>);
+    if (ns == 16) return go(k_moments<T, 4, 2>);
+    if (vw == 4) return go(k_moments<T, 4, 0>);
+  }
+  return vw == 2 ? go(k_moments<T, 2, 0>) : go(k_moments<T, 1, 0>);
 }
 
+template cudaError_t launch_sum_psi<float>(const float*, size_t, double*, int, DevParams*,
+                                           cudaStream_t);
+template cudaError_t launch_sum_psi<double>(const double*, size_t, double*, int, DevParams*,
+                                            cudaStream_t);
 template cudaError_t launch_convert<float, double>(float*, const double*, size_t, const double*,
                                                    cudaStream_t);
 template cudaError_t launch_convert<double, float>(double*, const float*, size_t, const double*,
@@ -712,12 +790,12 @@ template cudaError_t launch_dt_max<double>(const double*, const double*, const d
                                            const double*, long long, int, int, int, double, double,
                                            double, double, double, double, DevParams*, cudaStream_t);
 template cudaError_t launch_moments<float>(const float*, const float*, const float*,
-                                           const float*, const double*, long long, int, int, int,
-                                           int, double, double, double, double, double*, double*,
-                                           int, DevParams*, cudaStream_t);
+                                           const float*, const double*, long long, int, int,
+                                           double, double, double, double, double*, double*, int,
+                                           DevParams*, cudaStream_t);
 template cudaError_t launch_moments<double>(const double*, const double*, const double*,
                                             const double*, const double*, long long, int, int,
-                                            int, int, double, double, double, double, double*,
-                                            double*, int, DevParams*, cudaStream_t);
+                                            double, double, double, double, double*, double*, int,
+                                            DevParams*, cudaStream_t);
 
 }  // namespace mm

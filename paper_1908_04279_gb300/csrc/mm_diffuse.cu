@@ -4,12 +4,24 @@
 // one direction at a time (theta, x, y). Each direction is a batch of
 // constant-coefficient periodic tridiagonal systems
 //   (I - a/2 L) psi' = (I + a/2 L) psi,  (L psi)_i = psi_{i-1} - 2 psi_i + psi_{i+1},
-// one per line, solved by one thread per line: a Thomas sweep for the
-// tridiagonal part with the periodic corners folded in by the Sherman-Morrison
-// formula (the factors are the same for every line). Arithmetic in float64,
-// storage in the state precision; the line is overwritten in place (forward
-// sweep, back substitution, correction). The factors are computed on the
-// device too, so a call needs no host round trip.
+// one per line. Arithmetic in float64, storage in the state precision, in place.
+//
+// k_cn_block solves them by two first-order cyclic recursions. With S the
+// cyclic shift, I - a/2 L = kappa (I - r S)(I - r S^-1) where
+// r = a / (1 + a + sqrt(1 + 2 a)) (0 < r < 1) and kappa = a / (2 r): solve
+// y_i = d_i + r y_{i-1}, then x_i = y_i + r x_{i+1}, both cyclic, d the right
+// side over kappa. There are no factors to compute or to read, and a
+// recursion splits: a block takes 32 lines (a lane each, so that neighbouring
+// lanes read neighbouring addresses) and cuts them into one segment per warp;
+// a segment's value at its end from a zero start is known at once, and the
+// true starts follow from the other segments' ends and powers of r. The
+// lines live in shared memory between the passes, so psi is read and written
+// once, and is rounded to the state precision once per direction.
+//
+// k_cn_lines, a thread per line with a Thomas sweep and the corners by the
+// Sherman-Morrison formula, stays for lines too long for shared memory.
+#include <cmath>
+
 #include "mm_internal.cuh"
 
 namespace mm {
@@ -105,6 +117,113 @@ __global__ void k_cn_lines(T* psi, int mode, int nx, int ny, int nth, const doub
   }
 }
 
+constexpr int kCnPitch = 33;   // shared-memory row of 32 lines, padded
+constexpr int kCnWarps = 16;   // segments of a line at most
+
+// One direction for 32 lines per block: hk = a / 2 / kappa, ck = (1 - a) /
+// kappa; rl and re: r to the segment length and to the last segment's; wrap =
+// 1 / (1 - r^n). len: points per segment.
+template <typename T>
+__global__ void __launch_bounds__(32 * kCnWarps)
+    k_cn_block(T* psi, int mode, int nx, int ny, int nth, int n, int len, double r, double hk,
+               double ck, double rl, double re, double wrap, const double* scale) {
+  extern __shared__ __align__(16) double cn_t[];  // [n][kCnPitch], then [2][warps][32]
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  double* ends = cn_t + (size_t)n * kCnPitch;
+  const long long nlines = mode == 0 ? (long long)nx * ny : mode == 1 ? (long long)ny * nth
+                                                                      : (long long)nx * nth;
+  const long long L0 = blockIdx.x * 32LL, Ln = L0 + lane;
+  const bool on = Ln < nlines;
+  const long long La = on ? Ln : nlines - 1;
+  // first value and stride of the lane's line
+  size_t base, stride;
+  if (mode == 0) {
+    base = (size_t)La * nth;
+    stride = 1;
+  } else if (mode == 1) {
+    const long long y = La / nth;
+    base = (size_t)y * nx * nth + (size_t)(La - y * nth);
+    stride = (size_t)nth;
+  } else {
+    base = (size_t)La;
+    stride = (size_t)nx * nth;
+  }
+  const double g = scale ? *scale : 1.0;
+  const double h = hk * g, c = ck * g;
+  const int i0 = w * len, i1 = min(n, i0 + len);
+  // a theta line is contiguous: the block's lines as one run, transposed
+  // through shared memory
+  if (mode == 0) {
+    const int cnt = (int)min(32LL, nlines - L0) * nth;
+    for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
+      const int l = e / nth, i = e - l * nth;
+      cn_t[i * kCnPitch + l] = (double)psi[(size_t)L0 * nth + e];
+    }
+    __syncthreads();
+  }
+  auto at = [&](int i) {
+    return mode == 0 ? cn_t[i * kCnPitch + lane] : (double)psi[base + (size_t)i * stride];
+  };
+  // d, and the segment's end of the forward recursion from a zero start
+  double acc = 0.0;
+  {
+    double prev = at(i0 == 0 ? n - 1 : i0 - 1), cur = at(i0);
+    const double beyond = at(i1 == n ? 0 : i1);
+    __syncthreads();  // every neighbour has been read
+#pragma unroll 4
+    for (int i = i0; i < i1; ++i) {
+      const double next = i + 1 < i1 ? at(i + 1) : beyond;
+      const double d = fma(h, prev + next, c * cur);
+      cn_t[i * kCnPitch + lane] = d;
+      acc = fma(r, acc, d);
+      prev = cur;
+      cur = next;
+    }
+  }
+  ends[w * 32 + lane] = acc;
+  __syncthreads();
+  // the value before the segment: one turn over all segments, closed by wrap
+  double y = 0.0;
+  for (int q = 0; q < nw; ++q) {
+    const int s = w + q < nw ? w + q : w + q - nw;
+    y = fma(s == nw - 1 ? re : rl, y, ends[s * 32 + lane]);
+  }
+  y *= wrap;
+#pragma unroll 4
+  for (int i = i0; i < i1; ++i) {
+    y = fma(r, y, cn_t[i * kCnPitch + lane]);
+    cn_t[i * kCnPitch + lane] = y;
+  }
+  // the backward recursion in the same way
+  acc = 0.0;
+#pragma unroll 4
+  for (int i = i1 - 1; i >= i0; --i) acc = fma(r, acc, cn_t[i * kCnPitch + lane]);
+  ends[(nw + w) * 32 + lane] = acc;
+  __syncthreads();
+  double x = 0.0;
+  for (int q = 0; q < nw; ++q) {
+    const int s = w - q >= 0 ? w - q : w - q + nw;
+    x = fma(s == nw - 1 ? re : rl, x, ends[(nw + s) * 32 + lane]);
+  }
+  x *= wrap;
+#pragma unroll 4
+  for (int i = i1 - 1; i >= i0; --i) {
+    x = fma(r, x, cn_t[i * kCnPitch + lane]);
+    if (mode == 0)
+      cn_t[i * kCnPitch + lane] = x;
+    else if (on)
+      psi[base + (size_t)i * stride] = (T)x;
+  }
+  if (mode == 0) {
+    __syncthreads();
+    const int cnt = (int)min(32LL, nlines - L0) * nth;
+    for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
+      const int l = e / nth, i = e - l * nth;
+      psi[(size_t)L0 * nth + e] = (T)cn_t[i * kCnPitch + l];
+    }
+  }
+}
+
 __global__ void k_set_scale_one(double* scale) {
   if (threadIdx.x == 0 && blockIdx.x == 0) *scale = 1.0;
 }
@@ -114,6 +233,35 @@ __global__ void k_set_scale_one(double* scale) {
 cudaError_t launch_cn_factors(double* tab0, int n0, double a0, double* tab1, int n1, double a1,
                               double* tab2, int n2, double a2, cudaStream_t s) {
   k_cn_factors<<<1, 32, 0, s>>>(tab0, n0, a0, tab1, n1, a1, tab2, n2, a2);
+  return cudaGetLastError();
+}
+
+// Shared memory of k_cn_block for lines of n points in `warps` segments.
+size_t cn_block_smem(int n, int warps) {
+  return ((size_t)n * kCnPitch + 2 * (size_t)warps * 32) * sizeof(double);
+}
+bool cn_block_fits(int n) { return cn_block_smem(n, kCnWarps) <= 227 * 1024; }
+
+// One direction of n >= 2 points, a = D dt / h^2 > 0, by k_cn_block.
+template <typename T>
+cudaError_t launch_cn_block(T* psi, int mode, int nx, int ny, int nth, int n, double a,
+                            const double* scale, cudaStream_t s) {
+  const long long nlines = mode == 0 ? (long long)nx * ny : mode == 1 ? (long long)ny * nth
+                                                                      : (long long)nx * nth;
+  // segments of at least 8 points
+  int warps = n / 8 < 1 ? 1 : n / 8 > kCnWarps ? kCnWarps : n / 8;
+  const int len = (n + warps - 1) / warps;
+  warps = (n + len - 1) / len;
+  const size_t smem = cn_block_smem(n, warps);
+  if (smem > 48 * 1024) {
+    const cudaError_t e = raise_smem_limit(k_cn_block<T>, smem);
+    if (e != cudaSuccess) return e;
+  }
+  const double r = a / (1.0 + a + sqrt(1.0 + 2.0 * a)), kappa = 0.5 * a / r;
+  const double rl = pow(r, len), re = pow(r, n - (warps - 1) * len);
+  const double wrap = 1.0 / (-expm1(n * log(r)));
+  k_cn_block<T><<<(unsigned)((nlines + 31) / 32), 32 * warps, smem, s>>>(
+      psi, mode, nx, ny, nth, n, len, r, 0.5 * a / kappa, (1.0 - a) / kappa, rl, re, wrap, scale);
   return cudaGetLastError();
 }
 
@@ -133,6 +281,10 @@ cudaError_t launch_set_scale_one(double* scale, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+template cudaError_t launch_cn_block<float>(float*, int, int, int, int, int, double,
+                                            const double*, cudaStream_t);
+template cudaError_t launch_cn_block<double>(double*, int, int, int, int, int, double,
+                                             const double*, cudaStream_t);
 template cudaError_t launch_cn_lines<float>(float*, int, int, int, int, const double*, int, double,
                                             double, const double*, cudaStream_t);
 template cudaError_t launch_cn_lines<double>(double*, int, int, int, int, const double*, int,

@@ -171,9 +171,13 @@ cudaError_t launch_dt_max(const T* psi, const T* nb, const T* u, const T* trig, 
 cudaError_t launch_dt_finalize(DevParams* prm, double ds, double L, double cfl, cudaStream_t s);
 template <typename T>
 cudaError_t launch_moments(const T* psi, const T* mb, const T* mf, const T* c,
-                           const double* trig, long long ncells, int nth, int ns, int V, int seg,
-                           double dth, double ds, double L, double dA, double* fields,
-                           double* partial, int nblocks, DevParams* prm, cudaStream_t s);
+                           const double* trig, long long ncells, int nth, int ns, double dth,
+                           double ds, double L, double dA, double* fields, double* partial,
+                           int nblocks, DevParams* prm, cudaStream_t s);
+// Sum of psi into prm->sum_psi (partial: max_partial values of scratch).
+template <typename T>
+cudaError_t launch_sum_psi(const T* psi, size_t n, double* partial, int max_partial,
+                           DevParams* prm, cudaStream_t s);
 
 // Adjoint kernels (mm_adjoint.cu).
 template <typename T>
@@ -201,10 +205,15 @@ template <typename T>
 cudaError_t launch_adj_psi0(const T* lpsi, const T* lmf, int units, const T* nb, double dth,
                             long long rows, int nth, double* out, cudaStream_t s);
 
-// Filament diffusion (mm_diffuse.cu): the Crank-Nicolson factors of the three
-// directions (3 n + 2 values each), then one direction (mode 0 theta, 1 x,
-// 2 y) for every line of psi; scale (device, may be NULL) multiplies psi on
-// load.
+// Filament diffusion (mm_diffuse.cu): one direction (mode 0 theta, 1 x, 2 y)
+// for every line of psi; scale (device, may be NULL) multiplies psi on load.
+// By launch_cn_block where a line fits shared memory (cn_block_fits), else by
+// launch_cn_lines with the Crank-Nicolson factors of launch_cn_factors (3 n + 2
+// values per direction).
+bool cn_block_fits(int n);
+template <typename T>
+cudaError_t launch_cn_block(T* psi, int mode, int nx, int ny, int nth, int n, double a,
+                            const double* scale, cudaStream_t s);
 cudaError_t launch_cn_factors(double* tab0, int n0, double a0, double* tab1, int n1, double a1,
                               double* tab2, int n2, double a2, cudaStream_t s);
 template <typename T>

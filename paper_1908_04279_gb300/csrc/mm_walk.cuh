@@ -280,6 +280,13 @@ __device__ __forceinline__ float2 ff2_add(float2 a, float2 b) {
   const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(b.x, bb));
   return make_float2(s, __fadd_rn(e, __fadd_rn(a.y, b.y)));
 }
+// a += x (TwoSum)
+__device__ __forceinline__ void two_sum_acc2(float2& a, float x) {
+  const float s = __fadd_rn(a.x, x);
+  const float bb = __fsub_rn(s, a.x);
+  a.y = __fadd_rn(a.y, __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(x, bb)));
+  a.x = s;
+}
 __device__ __forceinline__ float2 warp_sum_ff2(float2 v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)

@@ -1,0 +1,63 @@
+"""Edges of the state set-up and the diffusion kernels against the oracle:
+line lengths around the segments of the cyclic solve and beyond what shared
+memory holds (float64, 1e-12), and motor densities whose row sums leave
+float32 (float32, 1e-5)."""
+import numpy as np
+import pytest
+
+from paper_1908_04279_gb300.inputs import Grid, Rates, SplitMix64, psi_isotropic_perturbed
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mmod():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1908_04279_gb300 import build as B
+    B.build()
+    from paper_1908_04279_gb300 import mm
+    mm.load_library()
+    return mm
+
+
+def rel_l2(a, b):
+    return np.linalg.norm(np.asarray(a, dtype=np.float64) - b) / np.linalg.norm(b)
+
+
+# two points; one segment, a segment and a point more, 16 segments and one
+# over; a short last segment; more than 32 lines; a line of 900 points (the
+# thread-per-line solve); a stiff and a nearly vanishing step
+@pytest.mark.parametrize("dims,D,dt", [
+    ((2, 3, 4), 0.3, 1.0), ((15, 16, 8), 0.02, 1.0), ((17, 9, 31), 0.01, 1.0),
+    ((129, 5, 3), 0.002, 1.0), ((131, 7, 12), 1e-3, 0.3), ((900, 2, 4), 1e-5, 1.0),
+    ((20, 24, 16), 40.0, 1.0), ((20, 24, 16), 1e-7, 1e-3)])
+def test_cyclic_diffusion(mmod, dims, D, dt):
+    from oracle import oracle as O
+    g = Grid(*dims, 4)
+    psi = psi_isotropic_perturbed(g, 5, amp=0.5)
+    with mmod.Simulation(g, Rates(), "fp64") as sim:
+        sim.set_state(psi)
+        sim.diffuse(D, 0.7 * D, dt)
+        got = sim.get_state()["psi"]
+    assert rel_l2(got, O.diffuse(g, psi, D, 0.7 * D, dt)) <= 1e-12
+
+
+@pytest.mark.parametrize("ns", [8, 7])
+def test_set_up_beyond_float32_sums(mmod, ns):
+    """Row sums and coarse densities above the float32 range (each motor value
+    is within it): the scale-down brings the state back."""
+    from oracle import oracle as O
+    g = Grid(5, 4, 12, ns)
+    rng = SplitMix64(3)
+    psi = psi_isotropic_perturbed(g, 2)
+    mb = 2e38 * (0.5 + 0.5 * rng.uniforms(g.micro_cells).reshape(g.ny, g.nx, g.ntheta, g.ns))
+    mb[1:] = 0.2  # and cells that are not scaled
+    st = O.make_state(g, psi, mb)
+    with mmod.Simulation(g, Rates(), "fp32") as sim:
+        sim.set_state(psi, mb)
+        got = sim.get_state()
+    for k in ("mb", "c"):
+        assert rel_l2(got[k], getattr(st, k)) <= 1e-5, k
+    assert np.abs(got["mf"] - st.mf).max() <= 1e-6
