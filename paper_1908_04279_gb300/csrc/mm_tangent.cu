@@ -17,6 +17,7 @@
 #include <algorithm>
 
 #include "mm_cell.cuh"
+#include "mm_rows.cuh"
 #include "mm_host.h"
 
 namespace mm {
@@ -360,58 +361,132 @@ __global__ void __launch_bounds__(128) k_substep_tl(const TanArgs<T> t) {
   }
 }
 
-// Per cell, the sums an observable and its tangent need (float64): sum psi cos,
-// sum psi sin, sum psi, sum psi m1, and the same of the tangent (psi taken
-// with the pending correction factor g, dpsi with g as a constant), into
-// out[cell][8] (warp per cell, lanes over theta).
-template <typename T>
-__global__ void k_tan_cells(const T* psi, const T* mb, const T* dpsi, const T* dmb,
-                            const double* trig64, const DevParams* prm, long long ncells, int nth,
-                            int ns, double ds, double L, double* out) {
-  const int lane = threadIdx.x & 31;
+// The sums a built-in observable and its derivative need: sum psi cos, sum psi
+// sin, sum psi, sum psi m1, and the same of the tangent (psi taken with the
+// pending correction factor g, dpsi with g as a constant), over all cells into
+// tot[8]. A warp per cell: the rows' m1 of Mb and dMb (packed rows, eight nodes
+// per lane), then lanes over theta; float-float in the float32 form. Partial
+// sums per warp, block and last block in a fixed order. Bound by HBM beyond the
+// L2 (a thread per row with a float64 sum per node and one warp for the total
+// took 620 us at 128^2 x 32^2).
+template <typename T, int VW>
+__global__ void __launch_bounds__(128)
+    k_tan_sums(const T* psi, const T* mb, const T* dpsi, const T* dmb, const double* trig64,
+               DevParams* prm, long long ncells, int nth, int ns, double ds, double L,
+               double* partial, double* tot) {
+  extern __shared__ __align__(16) unsigned char tan_raw[];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const PackedGeom pg = packed_geom(lane, ns);
+  double2* s_d = reinterpret_cast<double2*>(tan_raw) + (size_t)wib * nth;  // m1, dm1 over their unit
+  float4* s_f = reinterpret_cast<float4*>(tan_raw) + (size_t)wib * nth;    // (float pairs)
   const double g = prm->psi_scale;
-  for (long long cell = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5);
-       cell < ncells; cell += (long long)gridDim.x * (blockDim.x >> 5)) {
-    double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  T sj[8];
+#pragma unroll
+  for (int v = 0; v < 8; ++v) {
+    if constexpr (sizeof(T) == 4)
+      sj[v] = (float)(2 * (pg.sl * 8 + v) + 1 - ns);  // 2 s_j / ds, an integer
+    else
+      sj[v] = -0.5 * L + ((double)(pg.sl * 8 + v) + 0.5) * ds;
+  }
+  double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  FF f[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) f[q] = FF{0.f, 0.f};
+  const float2* wf = reinterpret_cast<const float2*>(trig64 + 14 * (size_t)nth);
+  for (long long cell = blockIdx.x * 4LL + wib; cell < ncells; cell += (long long)gridDim.x * 4) {
+    for (int r0 = 0; r0 < nth; r0 += 2 * pg.rpp) {
+      T m[4][8];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int k = r0 + u * pg.rpp + pg.rslot;
+        const size_t off = ((size_t)cell * nth + (k < nth ? k : 0)) * ns + pg.sl * 8;
+        load_row8<T, VW>(mb + off, k < nth ? pg.nv : 0, m[2 * u]);
+        load_row8<T, VW>(dmb + off, k < nth ? pg.nv : 0, m[2 * u + 1]);
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int k = r0 + u * pg.rpp + pg.rslot;
+        const bool own = pg.sl == 0 && pg.rslot < pg.rpp && k < nth;
+        if constexpr (sizeof(T) == 4) {
+          const FF a = packed_sum_ff<0>(row_dot8(m[2 * u], sj), pg.nl, pg.sl);
+          const FF b = packed_sum_ff<0>(row_dot8(m[2 * u + 1], sj), pg.nl, pg.sl);
+          if (own) s_f[k] = make_float4(a.hi, a.lo, b.hi, b.lo);
+        } else {
+          double a = 0.0, b = 0.0;
+#pragma unroll
+          for (int v = 0; v < 8; ++v) {
+            a = fma(sj[v], m[2 * u][v], a);
+            b = fma(sj[v], m[2 * u + 1][v], b);
+          }
+          a = packed_sum(a, pg.nl, pg.sl);
+          b = packed_sum(b, pg.nl, pg.sl);
+          if (own) s_d[k] = make_double2(a, b);
+        }
+      }
+    }
+    __syncwarp();
     for (int k = lane; k < nth; k += 32) {
       const size_t r = (size_t)cell * nth + k;
-      const double p = g * (double)psi[r], dp = g * (double)dpsi[r];
-      double m1 = 0.0, dm1 = 0.0;
-      for (int j = 0; j < ns; ++j) {
-        const double sj = -0.5 * L + (j + 0.5) * ds;
-        m1 += sj * (double)mb[r * ns + j] * ds;
-        dm1 += sj * (double)dmb[r * ns + j] * ds;
+      const T p = psi[r], dp = dpsi[r];
+      if constexpr (sizeof(T) == 4) {
+        const float2 ct = wf[5 * (size_t)nth + k], st = wf[6 * (size_t)nth + k];
+        const FF c{ct.x, ct.y}, sn{st.x, st.y};
+        const float4 m = s_f[k];
+        const FF m1{m.x, m.y}, dm1{m.z, m.w};
+        f[0] = ff_sum(f[0], ff_scale(p, c));
+        f[1] = ff_sum(f[1], ff_scale(p, sn));
+        ff_add(f[2], p);
+        f[3] = ff_sum(f[3], ff_scale(p, m1));
+        f[4] = ff_sum(f[4], ff_scale(dp, c));
+        f[5] = ff_sum(f[5], ff_scale(dp, sn));
+        ff_add(f[6], dp);
+        f[7] = ff_sum(f[7], ff_sum(ff_scale(dp, m1), ff_scale(p, dm1)));
+      } else {
+        const double c = trig64[k], sn = trig64[nth + k];
+        const double2 m = s_d[k];
+        s[0] = fma(p, c, s[0]);
+        s[1] = fma(p, sn, s[1]);
+        s[2] += p;
+        s[3] = fma(p, m.x, s[3]);
+        s[4] = fma(dp, c, s[4]);
+        s[5] = fma(dp, sn, s[5]);
+        s[6] += dp;
+        s[7] += dp * m.x + p * m.y;
       }
-      const double ck = trig64[k], sk = trig64[nth + k];
-      s[0] += p * ck;
-      s[1] += p * sk;
-      s[2] += p;
-      s[3] += p * m1;
-      s[4] += dp * ck;
-      s[5] += dp * sk;
-      s[6] += dp;
-      s[7] += dp * m1 + p * dm1;
     }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) s[q] = warp_sum(s[q]);
-    if (lane < 8) {
-      double v = s[0];
-#pragma unroll
-      for (int q = 1; q < 8; ++q)
-        if (lane == q) v = s[q];
-      out[(size_t)cell * 8 + lane] = v;
-    }
+    __syncwarp();
   }
-}
-
-// One warp adds the per-cell sums in a fixed order: tot[8].
-__global__ void k_tan_total(const double* cells, long long ncells, double* tot) {
-  const int lane = threadIdx.x & 31;
+  __shared__ double s_part[4][8];
+  __shared__ unsigned int s_last;
+#pragma unroll
   for (int q = 0; q < 8; ++q) {
-    double s = 0.0;
-    for (long long c = lane; c < ncells; c += 32) s += cells[(size_t)c * 8 + q];
-    s = warp_sum(s);
-    if (lane == 0) tot[q] = s;
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+        f[q] = ff_sum(f[q], FF{__shfl_xor_sync(0xffffffffu, f[q].hi, o),
+                               __shfl_xor_sync(0xffffffffu, f[q].lo, o)});
+      s[q] = (double)f[q].hi + (double)f[q].lo;
+    } else {
+      s[q] = warp_sum(s[q]);
+    }
+    if (lane == 0) s_part[wib][q] = s[q];
+  }
+  __syncthreads();
+  if (threadIdx.x < 8) {
+    double b = s_part[0][threadIdx.x];
+    for (int w = 1; w < 4; ++w) b += s_part[w][threadIdx.x];
+    partial[(size_t)blockIdx.x * 8 + threadIdx.x] = b;
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicInc(&prm->counter2, gridDim.x - 1) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  for (int q = wib; q < 8; q += 4) {
+    const double t = warp_sum_ldcg(partial + q, (int)gridDim.x, 8, lane);
+    const double m1 = sizeof(T) == 4 ? 0.5 * ds * ds : ds;  // the row sums' unit
+    if (lane == 0) tot[q] = g * (q == 3 || q == 7 ? m1 * t : t);
   }
 }
 
@@ -597,18 +672,26 @@ mm_status mm_tangent_observable(mm_handle* h, int observable, double* value, dou
   // per-cell sums in the moments' field buffer (12 doubles per cell available)
   double* cells = h->fields;
   double* tot = h->partial;  // 8 doubles; the partial sums are free between substeps
+  const int nth = h->g.ntheta, ns = h->g.ns;
   const int grid = (int)std::max<long long>(1, std::min<long long>((nc + 3) / 4, 8LL * h->sms));
+  const size_t smem = 4 * (size_t)nth * 16;
+  auto go = [&](auto kern, auto t) -> cudaError_t {
+    using T = decltype(t);
+    if (smem > 48 * 1024) {
+      const cudaError_t e = mm::raise_smem_limit(kern, smem);
+      if (e != cudaSuccess) return e;
+    }
+    kern<<<grid, 128, smem, h->stream>>>((const T*)h->psi[h->parity], (const T*)h->mb,
+                                         (const T*)h->tan_psi[h->parity], (const T*)h->tan_mb,
+                                         h->trig64, h->prm, nc, nth, ns, ds, h->g.L, cells, tot);
+    return cudaGetLastError();
+  };
   if (h->prec == MM_FP64)
-    mm::k_tan_cells<double><<<grid, 128, 0, h->stream>>>(
-        (const double*)h->psi[h->parity], (const double*)h->mb, (const double*)h->tan_psi[h->parity],
-        (const double*)h->tan_mb, h->trig64, h->prm, nc, h->g.ntheta, h->g.ns, ds, h->g.L, cells);
+    CK(ns % 2 == 0 ? go(mm::k_tan_sums<double, 2>, 0.0) : go(mm::k_tan_sums<double, 1>, 0.0));
   else
-    mm::k_tan_cells<float><<<grid, 128, 0, h->stream>>>(
-        (const float*)h->psi[h->parity], (const float*)h->mb, (const float*)h->tan_psi[h->parity],
-        (const float*)h->tan_mb, h->trig64, h->prm, nc, h->g.ntheta, h->g.ns, ds, h->g.L, cells);
-  CK(cudaGetLastError());
-  mm::k_tan_total<<<1, 32, 0, h->stream>>>(cells, nc, tot);
-  CK(cudaGetLastError());
+    CK(ns % 4 == 0   ? go(mm::k_tan_sums<float, 4>, 0.f)
+       : ns % 2 == 0 ? go(mm::k_tan_sums<float, 2>, 0.f)
+                     : go(mm::k_tan_sums<float, 1>, 0.f));
   double s[8];
   CK(cudaMemcpyAsync(s, tot, sizeof s, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
