@@ -26,6 +26,7 @@
 #include <utility>
 
 #include "mm_async.cuh"
+#include "mm_rows.cuh"
 #include "mm_cell.cuh"
 #include "mm_host.h"
 
@@ -654,23 +655,20 @@ __global__ void __launch_bounds__(128) k_anchor_fix(const AnchorArgs<T> x, T* mb
   }
 }
 
-// Row sums and the scatter of a given state: mode 0 n_b and psi ds dth Mb into
-// the coarse accumulators (state set-up); mode 1 the motor force of Eq. 10,
-// F p psi Mb ds dth, into fx, fy (float64, [cells] each). psi is scaled by g.
+// Row sums and the scatter of a given state (state set-up): n_b, and psi ds
+// dtheta Mb into the coarse accumulators. psi is scaled by g.
 template <typename T, int V>
 __global__ void __launch_bounds__(128) k_anchor_scatter(const AnchorArgs<T> x, const T* mb,
-                                                        const T* psi, T* nb, double* fx,
-                                                        double* fy, const double* trig64,
-                                                        const DevParams* prm, int mode, int nx,
-                                                        int ny, int nth, int ns, int seg,
-                                                        double ds, double dth, long long ncells) {
+                                                        const T* psi, T* nb,
+                                                        const DevParams* prm, int nx, int ny,
+                                                        int nth, int ns, int seg, double ds,
+                                                        double dth, long long ncells) {
   const int lane = threadIdx.x & 31;
   const int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int W = gridDim.x * (blockDim.x >> 5);
   const LaneGeom lg = lane_geom(lane, seg, ns, V);
   const double g = prm->psi_scale;
-  const double Fm = prm->force_scale;
-  if (mode == 0 && blockIdx.x == 0 && threadIdx.x == 0) x.flags[x.flag] = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) x.flags[x.flag] = 0;
   for (int cell = gw; cell < (int)ncells; cell += W) {
     const int iy = cell / nx, ix = cell - iy * nx;
     for (int r0 = 0; r0 < nth; r0 += lg.rpp) {
@@ -690,18 +688,76 @@ __global__ void __launch_bounds__(128) k_anchor_scatter(const AnchorArgs<T> x, c
           Mv[v] = (double)q.v[v];
           snb += q.v[v];
         }
-        if (mode == 0) {
-          scatter_runs<double, V>(x.cacc, anc, Mv, w);
-        } else {
-          scatter_runs<double, V>(fx, anc, Mv, Fm * trig64[k] * w);
-          scatter_runs<double, V>(fy, anc, Mv, Fm * trig64[nth + k] * w);
-        }
+        scatter_runs<double, V>(x.cacc, anc, Mv, w);
       }
-      if (mode == 0) {
-        snb = seg_sum(snb, seg);
-        if (lg.first && row_ok) nb[(size_t)cell * nth + k] = snb * (T)ds;
+      snb = seg_sum(snb, seg);
+      if (lg.first && row_ok) nb[(size_t)cell * nth + k] = snb * (T)ds;
+    }
+  }
+}
+
+// The motor force of Eq. 10 in the cells under the heads, F sum p psi Mb ds
+// dtheta over the configurations anchored at the cell, as a gather: a warp per
+// anchor cell, lanes over the configurations (k, j), each read from the filament
+// cell its offset names (neighbouring nodes mostly share it, so a warp reads
+// runs of a row). Every motor value is read once, the sum has a fixed order
+// (float-float in the float32 form) and needs no atomics: two float64 atomics
+// per run of a row took 200 us at 128^2 x 32^2, l/L = 0.05.
+template <typename T>
+__global__ void __launch_bounds__(128)
+    k_anchor_force(const int2* off, const T* mb, const T* psi, const double* trig64,
+                   const DevParams* prm, int nx, int ny, int nth, int ns, double ds, double dth,
+                   long long ncells, double* fx, double* fy) {
+  const int lane = threadIdx.x & 31;
+  const float2* wf = reinterpret_cast<const float2*>(trig64 + 14 * (size_t)nth);
+  const int kq = 32 / ns, jr = 32 - kq * ns, k0 = lane / ns, j0 = lane - k0 * ns;
+  const int nconf = nth * ns;
+  for (long long cell = blockIdx.x * 4LL + (threadIdx.x >> 5); cell < ncells;
+       cell += (long long)gridDim.x * 4) {
+    const int ay = (int)cell / nx, ax = (int)cell - ay * nx;
+    FF sx{0.f, 0.f}, sy{0.f, 0.f};
+    double dx = 0.0, dy = 0.0;
+    int k = k0, j = j0;
+#pragma unroll 4
+    for (int e = lane; e < nconf; e += 32) {
+      const int2 o = off[e];
+      int fxc = ax - o.x, fyc = ay - o.y;
+      fxc += fxc < 0 ? nx : 0;
+      fyc += fyc < 0 ? ny : 0;
+      const size_t row = ((size_t)fyc * nx + fxc) * nth + k;
+      const T m = mb[row * ns + j], p = psi[row];
+      if constexpr (sizeof(T) == 4) {
+        const float2 c = wf[5 * (size_t)nth + k], s = wf[6 * (size_t)nth + k];
+        const FF pm = ff_scale(p, FF{m, 0.f});
+        sx = ff_sum(sx, ff_prod(pm, FF{c.x, c.y}));
+        sy = ff_sum(sy, ff_prod(pm, FF{s.x, s.y}));
+      } else {
+        dx = fma(p * m, trig64[k], dx);
+        dy = fma(p * m, trig64[nth + k], dy);
+      }
+      k += kq;
+      j += jr;
+      if (j >= ns) {
+        j -= ns;
+        ++k;
       }
     }
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        sx = ff_sum(sx, FF{__shfl_xor_sync(0xffffffffu, sx.hi, o),
+                           __shfl_xor_sync(0xffffffffu, sx.lo, o)});
+        sy = ff_sum(sy, FF{__shfl_xor_sync(0xffffffffu, sy.hi, o),
+                           __shfl_xor_sync(0xffffffffu, sy.lo, o)});
+      }
+      if (lane < 2) dx = lane == 0 ? (double)sx.hi + (double)sx.lo : (double)sy.hi + (double)sy.lo;
+    } else {
+      dx = warp_sum(dx);
+      dy = warp_sum(dy);
+      if (lane == 1) dx = dy;
+    }
+    if (lane < 2)
+      (lane == 0 ? fx : fy)[cell] = dx * (prm->force_scale * prm->psi_scale * ds * dth);
   }
 }
 
@@ -826,21 +882,30 @@ cudaError_t anchor_substep_t(mm_handle* h, int parity, cudaStream_t s) {
 }
 
 template <typename T, int V>
-cudaError_t anchor_scatter_t(mm_handle* h, int mode, double* fx, double* fy) {
+cudaError_t anchor_scatter_t(mm_handle* h) {
   const mm::AnchorArgs<T> x = anchor_args<T>(h, 2);
   const int grid = blocks_for(h->ncells, 4, 8 * h->sms);
   const double ds = h->g.L / h->g.ns, dth = 2.0 * kPi / h->g.ntheta;
   mm::k_anchor_scatter<T, V><<<grid, 128, 0, h->stream>>>(
-      x, (const T*)h->mb, (const T*)h->psi[h->parity], (T*)h->nb[h->parity], fx, fy, h->trig64,
-      h->prm, mode, h->g.nx, h->g.ny, h->g.ntheta, h->g.ns, h->seg, ds, dth, h->ncells);
+      x, (const T*)h->mb, (const T*)h->psi[h->parity], (T*)h->nb[h->parity], h->prm, h->g.nx,
+      h->g.ny, h->g.ntheta, h->g.ns, h->seg, ds, dth, h->ncells);
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || mode != 0) return e;
+  if (e != cudaSuccess) return e;
   mm::k_anchor_close<T><<<blocks_for(h->ncells, 256, 8 * h->sms), 256, 0, h->stream>>>(
       x, (const T*)h->mtot, (T*)h->mf, (T*)h->c, h->ncells);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   mm::k_anchor_fix<T, V><<<grid, 128, 0, h->stream>>>(x, (T*)h->mb, (T*)h->nb[h->parity],
                                                       h->g.nx, h->g.ny, h->g.ntheta, h->g.ns,
                                                       h->seg, ds, h->ncells);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t anchor_force_t(mm_handle* h, double* fx, double* fy) {
+  mm::k_anchor_force<T><<<blocks_for(h->ncells, 4, 16 * h->sms), 128, 0, h->stream>>>(
+      (const int2*)h->anc_off, (const T*)h->mb, (const T*)h->psi[h->parity], h->trig64, h->prm,
+      h->g.nx, h->g.ny, h->g.ntheta, h->g.ns, h->g.L / h->g.ns, 2.0 * kPi / h->g.ntheta,
+      h->ncells, fx, fy);
   return cudaGetLastError();
 }
 
@@ -863,9 +928,7 @@ struct PrepareF {
 };
 template <typename T, int V>
 struct ScatterF {
-  static cudaError_t run(mm_handle* h, int mode, double* fx, double* fy) {
-    return anchor_scatter_t<T, V>(h, mode, fx, fy);
-  }
+  static cudaError_t run(mm_handle* h) { return anchor_scatter_t<T, V>(h); }
 };
 
 }  // namespace
@@ -1048,15 +1111,14 @@ cudaError_t launch_anchor_substep(mm_handle* h, int parity, cudaStream_t s) {
 // State set-up with anchors: n_b, C at the anchors, the scale-down, Mf.
 mm_status run_init_anchor(mm_handle* h) {
   CK(cudaMemsetAsync(h->anc_cacc, 0, (size_t)h->ncells * 8, h->stream));
-  CK(by_width<ScatterF>(h, 0, (double*)nullptr, (double*)nullptr));
+  CK(by_width<ScatterF>(h));
   return MM_OK;
 }
 
 // The motor force of Eq. 10 at the anchors into fields 7 and 8.
 mm_status anchor_force(mm_handle* h) {
-  const size_t nc = (size_t)h->ncells;
-  CK(cudaMemsetAsync(h->fields + 7 * nc, 0, 2 * nc * 8, h->stream));
-  CK(by_width<ScatterF>(h, 1, h->fields + 7 * nc, h->fields + 8 * nc));
+  double *fx = h->fields + 7 * (size_t)h->ncells, *fy = fx + h->ncells;
+  CK(h->prec == MM_FP64 ? anchor_force_t<double>(h, fx, fy) : anchor_force_t<float>(h, fx, fy));
   return MM_OK;
 }
 
