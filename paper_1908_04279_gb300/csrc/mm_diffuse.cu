@@ -6,17 +6,21 @@
 //   (I - a/2 L) psi' = (I + a/2 L) psi,  (L psi)_i = psi_{i-1} - 2 psi_i + psi_{i+1},
 // one per line. Arithmetic in float64, storage in the state precision, in place.
 //
-// k_cn_block solves them by two first-order cyclic recursions. With S the
-// cyclic shift, I - a/2 L = kappa (I - r S)(I - r S^-1) where
-// r = a / (1 + a + sqrt(1 + 2 a)) (0 < r < 1) and kappa = a / (2 r): solve
-// y_i = d_i + r y_{i-1}, then x_i = y_i + r x_{i+1}, both cyclic, d the right
-// side over kappa. There are no factors to compute or to read, and a
-// recursion splits: a block takes 32 lines (a lane each, so that neighbouring
-// lanes read neighbouring addresses) and cuts them into one segment per warp;
-// a segment's value at its end from a zero start is known at once, and the
-// true starts follow from the other segments' ends and powers of r. The
-// lines live in shared memory between the passes, so psi is read and written
-// once, and is rounded to the state precision once per direction.
+// k_cn_block uses I + a/2 L = 2 I - (I - a/2 L): psi' = 2 q - psi with
+// (I - a/2 L) q = psi, which keeps the right side positive (with L psi formed
+// first, a stiff step, a = 16000, lost a digit more), and solves for q by two
+// first-order cyclic recursions. With S the cyclic shift, I - a/2 L = kappa (I -
+// r S)(I - r S^-1) where r = a / (1 + a + sqrt(1 + 2 a)) (0 < r < 1) and kappa =
+// a / (2 r): solve y_i = d_i + r y_{i-1}, then q_i = y_i + r q_{i+1}, both cyclic,
+// d = psi / kappa. There are no factors to compute or to read, and a recursion
+// splits: a block takes 32 lines (a lane each, so that neighbouring lanes read
+// neighbouring addresses) and cuts them into one segment per warp; a segment's
+// value at its end from a zero start is known at once, and the true starts
+// follow from the other segments' ends and powers of r. The lines live in shared
+// memory between the passes, and psi is rounded to the state precision once per
+// direction. Bound by the float64 pipe (8 operations a value) and latency: 128^2 x
+// 32, three directions, 321 (a thread per line, and the factors on one thread)
+// -> 51 us.
 //
 // k_cn_lines, a thread per line with a Thomas sweep and the corners by the
 // Sherman-Morrison formula, stays for lines too long for shared memory.
@@ -120,13 +124,13 @@ __global__ void k_cn_lines(T* psi, int mode, int nx, int ny, int nth, const doub
 constexpr int kCnPitch = 33;   // shared-memory row of 32 lines, padded
 constexpr int kCnWarps = 16;   // segments of a line at most
 
-// One direction for 32 lines per block: hk = a / 2 / kappa, ck = (1 - a) /
-// kappa; rl and re: r to the segment length and to the last segment's; wrap =
-// 1 / (1 - r^n). len: points per segment.
+// One direction for 32 lines per block: ik = 1 / kappa; rl and re: r to the
+// segment length and to the last segment's; wrap = 1 / (1 - r^n). len: points
+// per segment.
 template <typename T>
 __global__ void __launch_bounds__(32 * kCnWarps)
-    k_cn_block(T* psi, int mode, int nx, int ny, int nth, int n, int len, double r, double hk,
-               double ck, double rl, double re, double wrap, const double* scale) {
+    k_cn_block(T* psi, int mode, int nx, int ny, int nth, int n, int len, double r, double ik,
+               double rl, double re, double wrap, const double* scale) {
   extern __shared__ __align__(16) double cn_t[];  // [n][kCnPitch], then [2][warps][32]
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   double* ends = cn_t + (size_t)n * kCnPitch;
@@ -149,7 +153,7 @@ __global__ void __launch_bounds__(32 * kCnWarps)
     stride = (size_t)nx * nth;
   }
   const double g = scale ? *scale : 1.0;
-  const double h = hk * g, c = ck * g;
+  const double gk = ik * g;
   const int i0 = w * len, i1 = min(n, i0 + len);
   // a theta line is contiguous: the block's lines as one run, transposed
   // through shared memory
@@ -161,24 +165,14 @@ __global__ void __launch_bounds__(32 * kCnWarps)
     }
     __syncthreads();
   }
-  auto at = [&](int i) {
-    return mode == 0 ? cn_t[i * kCnPitch + lane] : (double)psi[base + (size_t)i * stride];
-  };
   // d, and the segment's end of the forward recursion from a zero start
   double acc = 0.0;
-  {
-    double prev = at(i0 == 0 ? n - 1 : i0 - 1), cur = at(i0);
-    const double beyond = at(i1 == n ? 0 : i1);
-    __syncthreads();  // every neighbour has been read
 #pragma unroll 4
-    for (int i = i0; i < i1; ++i) {
-      const double next = i + 1 < i1 ? at(i + 1) : beyond;
-      const double d = fma(h, prev + next, c * cur);
-      cn_t[i * kCnPitch + lane] = d;
-      acc = fma(r, acc, d);
-      prev = cur;
-      cur = next;
-    }
+  for (int i = i0; i < i1; ++i) {
+    const double d =
+        gk * (mode == 0 ? cn_t[i * kCnPitch + lane] : (double)psi[base + (size_t)i * stride]);
+    cn_t[i * kCnPitch + lane] = d;
+    acc = fma(r, acc, d);
   }
   ends[w * 32 + lane] = acc;
   __syncthreads();
@@ -211,15 +205,18 @@ __global__ void __launch_bounds__(32 * kCnWarps)
     x = fma(r, x, cn_t[i * kCnPitch + lane]);
     if (mode == 0)
       cn_t[i * kCnPitch + lane] = x;
-    else if (on)
-      psi[base + (size_t)i * stride] = (T)x;
+    else if (on) {
+      T* p = psi + base + (size_t)i * stride;
+      *p = (T)fma(2.0, x, -g * (double)*p);
+    }
   }
   if (mode == 0) {
     __syncthreads();
     const int cnt = (int)min(32LL, nlines - L0) * nth;
     for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
       const int l = e / nth, i = e - l * nth;
-      psi[(size_t)L0 * nth + e] = (T)cn_t[i * kCnPitch + l];
+      T* p = psi + (size_t)L0 * nth + e;
+      *p = (T)fma(2.0, cn_t[i * kCnPitch + l], -g * (double)*p);
     }
   }
 }
@@ -261,7 +258,7 @@ cudaError_t launch_cn_block(T* psi, int mode, int nx, int ny, int nth, int n, do
   const double rl = pow(r, len), re = pow(r, n - (warps - 1) * len);
   const double wrap = 1.0 / (-expm1(n * log(r)));
   k_cn_block<T><<<(unsigned)((nlines + 31) / 32), 32 * warps, smem, s>>>(
-      psi, mode, nx, ny, nth, n, len, r, 0.5 * a / kappa, (1.0 - a) / kappa, rl, re, wrap, scale);
+      psi, mode, nx, ny, nth, n, len, r, 1.0 / kappa, rl, re, wrap, scale);
   return cudaGetLastError();
 }
 
