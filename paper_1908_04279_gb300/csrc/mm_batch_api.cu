@@ -21,19 +21,27 @@ using namespace mmh;
 
 namespace mmh {
 
+// Tiles and launch shape of the batched kernel over a set of members.
+struct TilePlan {
+  int S = 2, stage_elems = 0, nth_max = 0, block = 128, grid = 1, ntiles = 0;
+  size_t smem = 0;
+  mm::BatchTile* d_tiles = nullptr;
+  double* tile_mass = nullptr;
+  std::map<int, cudaGraphExec_t> graphs;
+};
+
 struct BatchPlan {
   std::vector<mm_handle*> members;
+  std::vector<ResidentGroup> groups;  // members that resident launches take
+  std::vector<char> resident;         // [members] whether one does
+  bool any_rest = false;              // whether any member is in no group
   int V = 1;                  // values per lane, common to all members
   int tile_work = 8192;       // target motor values (rows x ns) per tile
   int chunk_bytes = kChunkBytes;
   int pairs = 1;              // members that can go two cells to a warp do
-  int S = 2, stage_elems = 0, nth_max = 0, block = 128, grid = 1, ntiles = 0;
-  size_t smem = 0;
+  TilePlan all, rest;         // every member; the members of no group (when there are both)
   void* d_args = nullptr;     // [2][n] StepArgs: members at their parities, and flipped
-  mm::BatchTile* d_tiles = nullptr;
-  double* tile_mass = nullptr;
   std::vector<int> args_par;  // member parities the argument tables were built for
-  std::map<int, cudaGraphExec_t> graphs;
   int tuned = 0;
 };
 
@@ -56,9 +64,16 @@ std::string batch_signature(const mm_handle* h) {
   return sig;
 }
 
-void clear_graphs(BatchPlan* B) {
-  for (auto& kv : B->graphs) cudaGraphExecDestroy(kv.second);
-  B->graphs.clear();
+void clear_graphs(TilePlan& P) {
+  for (auto& kv : P.graphs) cudaGraphExecDestroy(kv.second);
+  P.graphs.clear();
+}
+void free_tiles(TilePlan& P) {
+  clear_graphs(P);
+  if (P.d_tiles) cudaFree(P.d_tiles);
+  if (P.tile_mass) cudaFree(P.tile_mass);
+  P.d_tiles = nullptr;
+  P.tile_mass = nullptr;
 }
 
 // Rows per chunk of a member under the chunk limit (the largest divisor of
@@ -97,14 +112,16 @@ cudaError_t prepare(int V, int block, size_t smem, int* bps) {
   }
 }
 
-// Tiles, shared-memory plan and grid for (tile_work, chunk_bytes).
-mm_status make_plan(mm_handle* h, int tile_work, int chunk_bytes) {
+// Tiles, shared-memory plan and grid for (tile_work, chunk_bytes), over every
+// member or (rest_only) over those of no group.
+mm_status make_tiles(mm_handle* h, TilePlan& P, bool rest_only, int tile_work, int chunk_bytes) {
   BatchPlan* B = h->batch;
   const int n = (int)B->members.size();
   std::vector<mm::BatchTile> tiles;
   int max_chunk_elems = 1, nth_max = 1;
   for (int i = 0; i < n; ++i) {
     const mm_handle* m = B->members[i];
+    if (rest_only && B->resident[i]) continue;
     // units of 1 cell (rows in ch chunks of rc) or of 2 cells (one chunk of
     // both cells' rows); tiles of about tile_work motor values, whole units
     const int cpu = B->pairs && member_pairs(m, B->V) ? 2 : 1;
@@ -159,25 +176,27 @@ mm_status make_plan(mm_handle* h, int tile_work, int chunk_bytes) {
   grid = std::min(grid, need);
 
   // device tables
-  if (B->d_tiles) cudaFree(B->d_tiles);
-  if (B->tile_mass) cudaFree(B->tile_mass);
-  B->d_tiles = nullptr;
-  B->tile_mass = nullptr;
-  CK(cudaMalloc((void**)&B->d_tiles, tiles.size() * sizeof(mm::BatchTile)));
-  CK(cudaMalloc((void**)&B->tile_mass, tiles.size() * sizeof(double)));
-  CK(cudaMemcpy(B->d_tiles, tiles.data(), tiles.size() * sizeof(mm::BatchTile),
+  free_tiles(P);
+  CK(cudaMalloc((void**)&P.d_tiles, tiles.size() * sizeof(mm::BatchTile)));
+  CK(cudaMalloc((void**)&P.tile_mass, tiles.size() * sizeof(double)));
+  CK(cudaMemcpy(P.d_tiles, tiles.data(), tiles.size() * sizeof(mm::BatchTile),
                 cudaMemcpyHostToDevice));
+  P.S = S;
+  P.stage_elems = max_chunk_elems;
+  P.nth_max = nth_max;
+  P.block = block;
+  P.smem = smem;
+  P.grid = (int)grid;
+  P.ntiles = (int)tiles.size();
+  return MM_OK;
+}
+mm_status make_plan(mm_handle* h, int tile_work, int chunk_bytes) {
+  BatchPlan* B = h->batch;
   B->tile_work = tile_work;
   B->chunk_bytes = chunk_bytes;
-  B->S = S;
-  B->stage_elems = max_chunk_elems;
-  B->nth_max = nth_max;
-  B->block = block;
-  B->smem = smem;
-  B->grid = (int)grid;
-  B->ntiles = (int)tiles.size();
-  clear_graphs(B);
-  return MM_OK;
+  const mm_status st = make_tiles(h, B->all, false, tile_work, chunk_bytes);
+  if (st != MM_OK || B->groups.empty() || !B->any_rest) return st;
+  return make_tiles(h, B->rest, true, tile_work, chunk_bytes);
 }
 
 // Kernel-argument tables for the members' current parities (table 0) and the
@@ -216,23 +235,47 @@ mm_status upload_args(mm_handle* h) {
 }
 
 // One batched substep with argument table `table` (0: current parities).
-cudaError_t launch_batch(mm_handle* h, int table, cudaStream_t s) {
+cudaError_t launch_batch(mm_handle* h, const TilePlan& P, int table, cudaStream_t s) {
   BatchPlan* B = h->batch;
   const int n = (int)B->members.size();
   if (h->prec == MM_FP64) {
     const StepArgs<double>* a = (const StepArgs<double>*)B->d_args + (size_t)table * n;
-    return mm::launch_substep_batch<double, 2>(a, B->d_tiles, B->ntiles, B->tile_mass, B->S,
-                                               B->stage_elems, B->nth_max, false, B->grid,
-                                               B->block, B->smem, s);
+    return mm::launch_substep_batch<double, 2>(a, P.d_tiles, P.ntiles, P.tile_mass, P.S,
+                                               P.stage_elems, P.nth_max, false, P.grid, P.block,
+                                               P.smem, s);
   }
   const StepArgs<float>* a = (const StepArgs<float>*)B->d_args + (size_t)table * n;
   if (B->V == 8)
-    return mm::launch_substep_batch<float, 8>(a, B->d_tiles, B->ntiles, B->tile_mass, B->S,
-                                              B->stage_elems, B->nth_max, true, B->grid, B->block,
-                                              B->smem, s);
-  return mm::launch_substep_batch<float, 4>(a, B->d_tiles, B->ntiles, B->tile_mass, B->S,
-                                            B->stage_elems, B->nth_max, true, B->grid, B->block,
-                                            B->smem, s);
+    return mm::launch_substep_batch<float, 8>(a, P.d_tiles, P.ntiles, P.tile_mass, P.S,
+                                              P.stage_elems, P.nth_max, true, P.grid, P.block,
+                                              P.smem, s);
+  return mm::launch_substep_batch<float, 4>(a, P.d_tiles, P.ntiles, P.tile_mass, P.S,
+                                            P.stage_elems, P.nth_max, true, P.grid, P.block,
+                                            P.smem, s);
+}
+
+// n substeps of a plan's members as one captured graph; the caller advances
+// their parities.
+mm_status graph_steps(mm_handle* h, TilePlan& P, int n) {
+  mm_status st;
+  if ((st = upload_args(h)) != MM_OK) return st;
+  auto it = P.graphs.find(n);
+  if (it == P.graphs.end()) {
+    cudaGraph_t graph;
+    CK(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
+    cudaError_t le = cudaSuccess;
+    for (int i = 0; i < n && le == cudaSuccess; ++i) le = launch_batch(h, P, i & 1, h->cap);
+    cudaError_t ce = cudaStreamEndCapture(h->cap, &graph);
+    if (le != cudaSuccess) return cuda_fail(h, "batched substep launch during capture", le);
+    CK(ce);
+    cudaGraphExec_t exec;
+    cudaError_t ie = cudaGraphInstantiate(&exec, graph, 0);
+    cudaGraphDestroy(graph);
+    CK(ie);
+    it = P.graphs.emplace(n, exec).first;
+  }
+  CK(cudaGraphLaunch(it->second, h->stream));
+  return MM_OK;
 }
 
 // Device snapshot of every member's evolving state (for the autotuner).
@@ -288,7 +331,6 @@ mm_status batch_micro_step(mm_handle* h, int n) {
   }
   DeviceGuard dg(h->device);
   mm_status st;
-  if ((st = upload_args(h)) != MM_OK) return st;
   bool recording = false;
   for (mm_handle* m : B->members) {
     recording = recording || m->rec.active;
@@ -296,6 +338,7 @@ mm_status batch_micro_step(mm_handle* h, int n) {
       return fail(h, MM_ERR_STATE, "a member's recording: more substeps than reserved");
   }
   if (recording || !h->use_graphs) {
+    if ((st = upload_args(h)) != MM_OK) return st;
     // direct launches; recording members take their checkpoints between them
     for (int i = 0; i < n; ++i) {
       for (mm_handle* m : B->members)
@@ -303,28 +346,23 @@ mm_status batch_micro_step(mm_handle* h, int n) {
           h->err = m->err;
           return st;
         }
-      CK(launch_batch(h, i & 1, h->stream));
+      CK(launch_batch(h, B->all, i & 1, h->stream));
       for (mm_handle* m : B->members) m->parity ^= 1;
     }
     return MM_OK;
   }
-  auto it = B->graphs.find(n);
-  if (it == B->graphs.end()) {
-    cudaGraph_t graph;
-    CK(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
-    cudaError_t le = cudaSuccess;
-    for (int i = 0; i < n && le == cudaSuccess; ++i) le = launch_batch(h, i & 1, h->cap);
-    cudaError_t ce = cudaStreamEndCapture(h->cap, &graph);
-    if (le != cudaSuccess) return cuda_fail(h, "batched substep launch during capture", le);
-    CK(ce);
-    cudaGraphExec_t exec;
-    cudaError_t ie = cudaGraphInstantiate(&exec, graph, 0);
-    cudaGraphDestroy(graph);
-    CK(ie);
-    it = B->graphs.emplace(n, exec).first;
+  if (B->groups.empty() || !resident_group_applies(h, n)) {
+    if ((st = graph_steps(h, B->all, n)) != MM_OK) return st;
+    for (mm_handle* m : B->members) m->parity ^= (n & 1);
+    return MM_OK;
   }
-  CK(cudaGraphLaunch(it->second, h->stream));
-  for (mm_handle* m : B->members) m->parity ^= (n & 1);
+  if (B->any_rest) {
+    if ((st = graph_steps(h, B->rest, n)) != MM_OK) return st;
+    for (size_t i = 0; i < B->members.size(); ++i)
+      if (!B->resident[i]) B->members[i]->parity ^= (n & 1);
+  }
+  for (ResidentGroup& G : B->groups)
+    if ((st = resident_group_step(h, B->members, G, n)) != MM_OK) return st;
   return MM_OK;
 }
 
@@ -350,8 +388,9 @@ const std::vector<mm_handle*>& batch_members(mm_handle* h) { return h->batch->me
 // chunk (values), tiles, V, tile_work, chunk_bytes, tuned, two cells per warp
 mm_status batch_launch_info(mm_handle* h, int* info, int n) {
   const BatchPlan* B = h->batch;
-  const int v[12] = {B->grid,    B->block, (int)B->smem,   1,         B->S,     B->stage_elems,
-                     B->ntiles,  B->V,     B->tile_work,   B->chunk_bytes, B->tuned, B->pairs};
+  const TilePlan& P = B->all;
+  const int v[12] = {P.grid,   P.block, (int)P.smem,  1,              P.S,      P.stage_elems,
+                     P.ntiles, B->V,    B->tile_work, B->chunk_bytes, B->tuned, B->pairs};
   for (int i = 0; i < n && i < 12; ++i) info[i] = v[i];
   return MM_OK;
 }
@@ -359,14 +398,14 @@ mm_status batch_launch_info(mm_handle* h, int* info, int n) {
 void batch_free(mm_handle* h) {
   BatchPlan* B = h->batch;
   if (!B) return;
-  clear_graphs(B);
+  resident_group_free(&B->groups);
+  free_tiles(B->all);
+  free_tiles(B->rest);
   for (mm_handle* m : B->members) {
     m->owner = nullptr;
     mm_destroy(m);
   }
   if (B->d_args) cudaFree(B->d_args);
-  if (B->d_tiles) cudaFree(B->d_tiles);
-  if (B->tile_mass) cudaFree(B->tile_mass);
   delete B;
   h->batch = nullptr;
 }
@@ -442,7 +481,10 @@ mm_status mm_create_batch(int n, const mm_grid* grids, const mm_rates* rates, mm
     h->batch->pairs = c->second.pairs;
     h->batch->tuned = 1;
   }
-  mm_status st = make_plan(h, tw, cb);
+  BatchPlan* B = h->batch;
+  mm_status st = resident_group_plan(h, B->members, &B->groups, &B->resident);
+  for (char in : B->resident) B->any_rest = B->any_rest || !in;
+  if (st == MM_OK) st = make_plan(h, tw, cb);
   if (st != MM_OK) return bail(st);
   *out = h;
   return MM_OK;
@@ -486,9 +528,9 @@ mm_status mm_batch_autotune(mm_handle* h, int substeps, mm_batch_tune* results, 
       B->args_par.clear();
       if ((st = upload_args(h)) != MM_OK) break;
       // one warm-up substep, then the timed ones, all from the saved state
-      CK(launch_batch(h, 0, h->stream));
+      CK(launch_batch(h, B->all, 0, h->stream));
       CK(cudaEventRecord(e0, h->stream));
-      for (int i = 0; i < substeps; ++i) CK(launch_batch(h, (i + 1) & 1, h->stream));
+      for (int i = 0; i < substeps; ++i) CK(launch_batch(h, B->all, (i + 1) & 1, h->stream));
       CK(cudaEventRecord(e1, h->stream));
       CK(cudaEventSynchronize(e1));
       float ms = 0.f;

@@ -192,8 +192,7 @@ struct mm_handle {
   bool tma = false;
   size_t smem = 0;
   // many substeps in one launch with Mb on the chip (mm_resident.cu; grid 0: off)
-  int res_grid = 0, res_block = 0, res_NL = 0, res_own = 0, res_passes = 0;
-  size_t res_smem = 0;
+  int res_grid = 0, res_NL = 0;
   unsigned res_epoch = 0, res_arrivals = 0;  // tags and arrivals used so far
   size_t res_xch_bytes = 0;
   unsigned long long* res_xch = nullptr;  // arrival counter and the psi sums the blocks exchange
@@ -276,6 +275,20 @@ mm_status velocity_update(mm_handle* h);  // h->u64 becomes the velocity in effe
 // Defined in mm_resident.cu (many substeps per launch, Mb on the chip).
 mm_status resident_configure(mm_handle* h);
 mm_status resident_substeps(mm_handle* h, int n, bool* done);
+// Members of a batch that one resident launch advances together: blocks[k] SMs
+// for member[k].
+struct ResidentGroup {
+  std::vector<int> member, blocks;
+  int grid = 0, block = 0;
+  size_t smem = 0;
+  void *map = nullptr, *tab = nullptr;  // device: block -> (entry, its block); kernel arguments
+};
+mm_status resident_group_plan(mm_handle* h, const std::vector<mm_handle*>& members,
+                              std::vector<ResidentGroup>* groups, std::vector<char>* in);
+void resident_group_free(std::vector<ResidentGroup>* groups);
+mm_status resident_group_step(mm_handle* h, const std::vector<mm_handle*>& members,
+                              ResidentGroup& G, int n);
+bool resident_group_applies(mm_handle* h, int n);
 
 // Defined in mm_fluid.cu (thin-gap fluid solve).
 void fluid_free(mm_handle* h);

@@ -39,11 +39,24 @@
 // takes one lane per orientation, 32 / seg cells at once where nth <= 16 (seg:
 // nth rounded up to a power of two).
 //
-// Bound by instruction issue at the larger sizes (27 cells of 32 x 32 values per
-// SM) and by the chain rows -> close -> arrival -> neighbours' psi at the
-// smallest. Measured on a GB300, us per substep against k_substep in a CUDA
-// graph: 32^2 x 16^2 8.0 -> 4.5, 64^2 x 32^2 13.2 -> 6.6, 85 x 61 x 24 x 30
-// 57 -> 7.9, 128^2 x 16^2 (108 cells per SM) 24 -> 10.2.
+// Where Mb is larger than the shared memory of all SMs, a worker keeps the first
+// `tiles` passes of its rows and reads and writes the others every substep, each
+// lane copying its own values to its own slots two passes ahead (cp.async) and
+// storing the new ones straight back; they stay in the L2 up to about twice its
+// size (resident_pays says where k_substep takes over).
+//
+// A batch's members are independent, so several go into one launch
+// (k_substep_resident_group), each over its own share of the SMs with its own
+// exchange.
+//
+// Bound by instruction issue at the larger sizes (about 58 % of the slots; the
+// rest goes to fixed latencies, psi loads and the half-rate minima) and by the
+// chain rows -> close -> arrival -> neighbours' psi at the smallest. 15 workers of
+// 128 registers: 19 of 96 are within 3 %, 11 or 23 slower. Measured on a GB300,
+// us per substep against k_substep in a CUDA graph: 32^2 x 16^2 7.2 -> 4.1, 64^2 x
+// 32^2 13.4 -> 6.4, 128^2 x 16^2 23 -> 9.8, 128^2 x 32^2 35.2 -> 25.3, 256^2 x 16^2
+// 77 -> 35, 85 x 61 x 24 x 30 57 -> 8.0, 200 x 150 x 24 x 30 231 -> 43; the 64-member
+// ensemble 594 (tuned) -> 427.
 #include <map>
 #include <mutex>
 
@@ -54,6 +67,7 @@
 namespace mm {
 
 constexpr int kResXch = 5;        // published sums a lane of the exchange warp reads: 160 blocks
+constexpr int kResRing = 2;       // ring stages of a worker
 constexpr int kResMaxWarps = 15;  // workers of a block, beside the exchange warp
 
 struct ResidentArgs {
@@ -62,7 +76,12 @@ struct ResidentArgs {
   int nl, rpp;              // lanes per row, rows per pass
   int vl;                   // nodes of a row's last lane
   int own;                  // most cells of a worker
-  int passes;               // passes of a worker's rows at most
+  int tiles;                // passes of a worker kept in shared memory at most
+  int ring;                 // stages of a worker for the passes read every substep (0: none)
+  int vw;                   // values of a vector that divides ns: 4, 2 or 1
+  int workers;              // worker warps of a block
+  int grid;                 // blocks of the instance
+  int NL;                   // lanes per row when ns = 8 NL fills them (2, 4 or 8), else 0
   int seg;                  // lanes per cell of the psi phase
   unsigned epoch;           // tags of this launch: epoch + 1 .. epoch + n
   unsigned arrivals;        // the arrival counter at this launch's start
@@ -72,19 +91,20 @@ struct ResidentArgs {
 struct ResidentSmem {
   size_t mass, cell, nb, tiles, total;
 };
-constexpr int kResCell = 20;  // 32-bit words per cell: u[10], Mf, M, five cell indices, spare
-__host__ __device__ inline ResidentSmem resident_smem(int workers, int own, int nth, int passes) {
+constexpr int kResCell = 20;  // 32-bit words per cell: u[10], Mf, M, offsets of the five
+                              // cells' columns, whether its west neighbour is the cell before
+__host__ __device__ inline ResidentSmem resident_smem(int workers, int own, int nth, int tiles) {
   ResidentSmem L;
   size_t off = 64;  // three mbarriers, the factor and the abort flag
   L.mass = off;
-  off += 128;  // one float pair per worker
+  off += 256;  // one float pair per worker
   L.cell = off;
   off += (size_t)workers * own * kResCell * 4;
   L.nb = off;
   off += (size_t)workers * own * nth * 4;
   off = (off + 15) & ~(size_t)15;
   L.tiles = off;
-  off += (size_t)workers * passes * 1024;
+  off += (size_t)workers * tiles * 1024;  // kept passes, then ring stages
   L.total = off;
   return L;
 }
@@ -101,8 +121,9 @@ __device__ __forceinline__ unsigned long long tagged(float v, unsigned tag) {
 // The exchange warp: per substep, the block's psi sum out, all blocks' sums in.
 // Returns early (abort flag set, workers released) when a wait gives up.
 __device__ void exchange(const ResidentArgs& a, uint64_t* bars, const float2* s_mass,
-                         volatile float* s_scale, volatile int* s_abort, int workers, int lane) {
-  const unsigned G = gridDim.x;
+                         volatile float* s_scale, volatile int* s_abort, int block, int lane) {
+  const unsigned G = (unsigned)a.grid;
+  const int workers = a.workers;
   DevParams* P = a.s.prm;
   const uint32_t limit = P->wait_limit;
   const bool never = (P->debug_flags & 1u) != 0;  // test knob: every wait runs out
@@ -116,13 +137,13 @@ __device__ void exchange(const ResidentArgs& a, uint64_t* bars, const float2* s_
     if (lane == 0) {
       __threadfence();
       asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(
-                       words + 2 * (size_t)blockIdx.x),
+                       words + 2 * (size_t)block),
                    "l"(tagged(own.x, tag)), "l"(tagged(own.y, tag))
                    : "memory");
       asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(a.xch) : "memory");
     }
     const bool done = t + 1 == a.n;
-    if (done && blockIdx.x != 0) break;  // block 0 stores the final sum
+    if (done && block != 0) break;  // block 0 stores the final sum
     if (lane == 0 && ok) {
       const unsigned target = a.arrivals + (unsigned)(t + 1) * G;
       for (uint32_t i = 0;; ++i) {
@@ -188,16 +209,52 @@ __device__ void exchange(const ResidentArgs& a, uint64_t* bars, const float2* s_
   }
 }
 
+// A lane's nv values of a row from global memory (src) into its slots of a
+// ring stage, in vectors of vw values.
+template <bool RAG>
+__device__ __forceinline__ void stage_row8(float* slot, const float* src, int nv, int vw) {
+  if (!RAG || vw == 4) {
+    cp_async16(slot, src);
+    if (!RAG || nv > 4) cp_async16(slot + 128, src + 4);
+  } else if (vw == 2) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (2 * q < nv) cp_async8(slot + (q & 1) * 2 + (q >> 1) * 128, src + 2 * q);
+  } else {
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (q < nv) cp_async_t(slot + (q & 3) + (q >> 2) * 128, src + q);
+  }
+}
+template <bool RAG>
+__device__ __forceinline__ void store_row8(float* dst, const float2 (&M)[4], int nv, int vw) {
+  if (!RAG || vw == 4) {
+    reinterpret_cast<float4*>(dst)[0] = make_float4(M[0].x, M[0].y, M[1].x, M[1].y);
+    if (!RAG || nv > 4)
+      reinterpret_cast<float4*>(dst)[1] = make_float4(M[2].x, M[2].y, M[3].x, M[3].y);
+  } else if (vw == 2) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (2 * q < nv) reinterpret_cast<float2*>(dst)[q] = M[q];
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (2 * q < nv) dst[2 * q] = M[q].x;
+      if (2 * q + 1 < nv) dst[2 * q + 1] = M[q].y;
+    }
+  }
+}
+
+// The whole of one block: block `block` of the a.grid blocks of an instance.
 // NL: lanes per row when ns = 8 NL fills its lanes (2, 4 or 8); 0: any row.
 template <int NL>
-__global__ void __launch_bounds__(32 * (kResMaxWarps + 1), 1)
-    k_substep_resident(const ResidentArgs a) {
+__device__ __forceinline__ void resident_block(const ResidentArgs& a, int block) {
   constexpr bool RAG = NL == 0;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int nth = a.s.nth, ns = a.s.ns, nx = a.s.nx, ny = a.s.ny;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int NW = (int)(blockDim.x >> 5) - 1;
-  const ResidentSmem L = resident_smem(NW, a.own, nth, a.passes);
+  const int NW = a.workers;
+  const ResidentSmem L = resident_smem(NW, a.own, nth, a.tiles + a.ring);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem_raw);  // written, readable, factor
   volatile float* s_scale = reinterpret_cast<float*>(smem_raw + 24);
   volatile int* s_abort = reinterpret_cast<int*>(smem_raw + 28);
@@ -210,15 +267,13 @@ __global__ void __launch_bounds__(32 * (kResMaxWarps + 1), 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  if (w == NW) {
-    exchange(a, bars, s_mass, s_scale, s_abort, NW, lane);
-    return;
-  }
+  if (w == NW) exchange(a, bars, s_mass, s_scale, s_abort, block, lane);
+  if (w >= NW) return;
 
   // this warp's cells cw .. cw + ncw - 1 of the block's run
   const long long nc = a.s.ncells;
-  const int c0 = (int)(nc * blockIdx.x / gridDim.x);
-  const int ncl = (int)(nc * (blockIdx.x + 1) / gridDim.x) - c0;
+  const int c0 = (int)(nc * block / a.grid);
+  const int ncl = (int)(nc * (block + 1) / a.grid) - c0;
   const int cw = c0 + w * a.own;
   const int ncw = max(0, min(a.own, ncl - w * a.own));
   const int nrows = ncw * nth;
@@ -240,31 +295,26 @@ __global__ void __launch_bounds__(32 * (kResMaxWarps + 1), 1)
   }
   float* s_cell = reinterpret_cast<float*>(smem_raw + L.cell) + (size_t)w * a.own * kResCell;
   float* s_nb = reinterpret_cast<float*>(smem_raw + L.nb) + (size_t)w * a.own * nth;
-  float4* tile = reinterpret_cast<float4*>(smem_raw + L.tiles) + (size_t)w * a.passes * 64 + lane;
+  float4* tile =
+      reinterpret_cast<float4*>(smem_raw + L.tiles) + (size_t)w * (a.tiles + a.ring) * 64 + lane;
+  float4* ring = tile + a.tiles * 64;
+  const int kept = min(passes, a.tiles), streamed = passes - kept;
+  // the lane's slot of pass p: row R = p rpp + rslot of the run, which is row
+  // cw nth + R of Mb
+  float* rows = a.s.mb_out + ((size_t)cw * nth + rslot) * ns + sl * 8;
+  const size_t pass_vals = (size_t)rpp * ns;
 
-  // load: the rows (row R of the warp's run is row cw nth + R of Mb), the
-  // per-cell scalars and the neighbour indices
-  for (int p = 0; p < passes; ++p) {
-    const int R = p * rpp + rslot;
-    float v[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = 0.f;
-    if (lane_ok && R < nrows) {
-      const float* src = a.s.mb_in + ((size_t)cw * nth + R) * ns + sl * 8;
-      if constexpr (RAG) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (q < nv) v[q] = src[q];
-      } else {
-        const float4 x = reinterpret_cast<const float4*>(src)[0];
-        const float4 y = reinterpret_cast<const float4*>(src)[1];
-        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-        v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
-      }
-    }
-    tile[p * 64] = make_float4(v[0], v[1], v[2], v[3]);
-    tile[p * 64 + 32] = make_float4(v[4], v[5], v[6], v[7]);
+  // load: the kept rows, the per-cell scalars and the neighbour indices
+  for (int p = 0; p < kept + a.ring; ++p) {
+    tile[p * 64] = make_float4(0.f, 0.f, 0.f, 0.f);
+    tile[p * 64 + 32] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
+  __syncwarp();
+  for (int p = 0; p < kept; ++p)
+    if (lane_ok && p * rpp + rslot < nrows)
+      stage_row8<RAG>(reinterpret_cast<float*>(tile + p * 64), rows + p * pass_vals, nv, a.vw);
+  cp_async_commit();
+  cp_async_wait<0>();
   for (int j = 0; j < ncw; ++j) {
     const int cell = cw + j;
     float* sc = s_cell + j * kResCell;
@@ -273,12 +323,13 @@ __global__ void __launch_bounds__(32 * (kResMaxWarps + 1), 1)
     if (lane == 11) sc[11] = a.s.mtot[cell];
     if (lane == 12) {
       const int iy = cell / nx, ix = cell - iy * nx;
-      int* id = reinterpret_cast<int*>(sc + 12);
-      id[0] = cell;
-      id[1] = iy * nx + (ix + 1 == nx ? 0 : ix + 1);
-      id[2] = iy * nx + (ix == 0 ? nx - 1 : ix - 1);
-      id[3] = (iy + 1 == ny ? 0 : iy + 1) * nx + ix;
-      id[4] = (iy == 0 ? ny - 1 : iy - 1) * nx + ix;
+      unsigned* id = reinterpret_cast<unsigned*>(sc + 12);
+      id[0] = (unsigned)cell * nth;
+      id[1] = (unsigned)(iy * nx + (ix + 1 == nx ? 0 : ix + 1)) * nth;
+      id[2] = (unsigned)(iy * nx + (ix == 0 ? nx - 1 : ix - 1)) * nth;
+      id[3] = (unsigned)((iy + 1 == ny ? 0 : iy + 1) * nx + ix) * nth;
+      id[4] = (unsigned)((iy == 0 ? ny - 1 : iy - 1) * nx + ix) * nth;
+      id[5] = ix != 0;
     }
   }
   __syncwarp();
@@ -292,12 +343,15 @@ __global__ void __launch_bounds__(32 * (kResMaxWarps + 1), 1)
   const float2 e1_ = make_float2(e1, e1), e2_ = make_float2(e2, e2);
   PsiConst<float> pq{sc.dt,     sc.g,       sc.glide, sc.vsp, sc.inv_dx,
                      sc.inv_dy, sc.inv_dth, sc.dth,   a.s.trig};
-  // psi phase: lane (sub, kl) takes orientations kl, kl + seg, ... of every
-  // cps-th cell of the warp from its sub-th on
+  // psi phase: lane (sub, kl) takes orientations kl, kl + seg, ... of the cells
+  // of the sub-th part of the warp's run, `half` cells
   const int seg = a.seg, cps = 32 / seg;
   const int sub = lane / seg, kl = lane - sub * seg;
+  const int half = (ncw + cps - 1) / cps;
   const int nk = (nth + seg - 1) / seg;  // 1 unless nth > 32
   const LaneTrig<float> lt = lane_trig(a.s.trig, nth, kl);
+  const int up = sub * seg + (kl + 1 >= nth ? 0 : kl + 1);    // lanes of theta + 1 and
+  const int down = sub * seg + (kl == 0 ? nth - 1 : kl - 1);  // theta - 1 (nth <= 32)
   float* pbuf[2] = {const_cast<float*>(a.s.psi_in), a.s.psi_out};
   float* nbuf[2] = {const_cast<float*>(a.s.nb_in), a.s.nb_out};
   const int jq = rpp / nth, jr = rpp - jq * nth;  // rows of a pass in cells and rows
@@ -308,14 +362,15 @@ __global__ void __launch_bounds__(32 * (kResMaxWarps + 1), 1)
     // ---- the motor rows of this warp's cells by Eq. 4
     {
       int j = j0, r = r0;  // cell and orientation of the lane's row
-#pragma unroll kStepUnroll
-      for (int p = 0; p < passes; ++p) {
+      auto rk2 = [&](const float4* t, int p, float2 (&M)[4]) {
         const float mf = s_cell[min(j, ncw - 1) * kResCell + 10];
         const float c3 = hk * mf, e3 = fk * mf;
         const float2 c3_ = make_float2(c3, c3), e3_ = make_float2(e3, e3);
-        const float4 x = tile[p * 64], y = tile[p * 64 + 32];
-        float2 M[4] = {make_float2(x.x, x.y), make_float2(x.z, x.w), make_float2(y.x, y.y),
-                       make_float2(y.z, y.w)};
+        const float4 x = t[0], y = t[32];
+        M[0] = make_float2(x.x, x.y);
+        M[1] = make_float2(x.z, x.w);
+        M[2] = make_float2(y.x, y.y);
+        M[3] = make_float2(y.z, y.w);
         float2 D[4], Ms[4];
         walk_dflux_x2<8, RAG>(M, D, first, last, 32, keep);
 #pragma unroll
@@ -328,8 +383,6 @@ __global__ void __launch_bounds__(32 * (kResMaxWarps + 1), 1)
 #pragma unroll
           for (int h = 0; h < 4; ++h) M[h] = __fmul2_rn(M[h], valid[h]);
         }
-        tile[p * 64] = make_float4(M[0].x, M[0].y, M[1].x, M[1].y);
-        tile[p * 64 + 32] = make_float4(M[2].x, M[2].y, M[3].x, M[3].y);
         float2 acc = M[0];
 #pragma unroll
         for (int h = 1; h < 4; ++h) acc = __fadd2_rn(acc, M[h]);
@@ -342,6 +395,37 @@ __global__ void __launch_bounds__(32 * (kResMaxWarps + 1), 1)
           r -= nth;
           ++j;
         }
+      };
+      // streamed passes: a lane copies its own values to its own slots `ring`
+      // passes ahead (the first of them under the kept passes) and stores the
+      // new ones straight back
+      auto issue = [&](int q) {
+        const int p = kept + q;
+        if (q < streamed && lane_ok && p * rpp + rslot < nrows)
+          stage_row8<RAG>(reinterpret_cast<float*>(ring + (q % kResRing) * 64),
+                          rows + p * pass_vals, nv, a.vw);
+        cp_async_commit();
+      };
+      if (streamed > 0) {
+        __threadfence_block();  // after this lane's stores of the substep before
+        for (int q = 0; q < kResRing; ++q) issue(q);
+      }
+#pragma unroll 1
+      for (int p = 0; p < kept; ++p) {
+        float2 M[4];
+        rk2(tile + p * 64, p, M);
+        tile[p * 64] = make_float4(M[0].x, M[0].y, M[1].x, M[1].y);
+        tile[p * 64 + 32] = make_float4(M[2].x, M[2].y, M[3].x, M[3].y);
+      }
+#pragma unroll 1
+      for (int q = 0; q < streamed; ++q) {
+        cp_async_wait<kResRing - 1>();
+        const int p = kept + q;
+        float2 M[4];
+        rk2(ring + (q % kResRing) * 64, p, M);
+        if (lane_ok && p * rpp + rslot < nrows)
+          store_row8<RAG>(rows + p * pass_vals, M, nv, a.vw);
+        issue(q + kResRing);
       }
     }
     __syncwarp();
@@ -358,66 +442,14 @@ __global__ void __launch_bounds__(32 * (kResMaxWarps + 1), 1)
     const float* nb_in = nbuf[t & 1];
     float* psi_out = pbuf[(t & 1) ^ 1];
     float* nb_out = nbuf[(t & 1) ^ 1];
-    // (cell, theta) values are read through L2: other SMs wrote them
-    auto load = [&](int j, int kk) {
-      PsiIn<float> in{};
-      const int k = kk * seg + kl;
-      if (j < ncw && k < nth) {
-        const int* id = reinterpret_cast<const int*>(s_cell + j * kResCell + 12);
-        const int kp = k + 1 == nth ? 0 : k + 1, km = k == 0 ? nth - 1 : k - 1;
-        const size_t o0 = (size_t)id[0] * nth, o1 = (size_t)id[1] * nth, o2 = (size_t)id[2] * nth;
-        const size_t o3 = (size_t)id[3] * nth, o4 = (size_t)id[4] * nth;
-        in.pc = __ldcg(psi_in + o0 + k);
-        in.pe = __ldcg(psi_in + o1 + k);
-        in.pw = __ldcg(psi_in + o2 + k);
-        in.pn = __ldcg(psi_in + o3 + k);
-        in.ps = __ldcg(psi_in + o4 + k);
-        in.pp = __ldcg(psi_in + o0 + kp);
-        in.pm = __ldcg(psi_in + o0 + km);
-        in.nc = __ldcg(nb_in + o0 + k);
-        in.ne = __ldcg(nb_in + o1 + k);
-        in.nw = __ldcg(nb_in + o2 + k);
-        in.nn = __ldcg(nb_in + o3 + k);
-        in.ns = __ldcg(nb_in + o4 + k);
-      }
-      return in;
-    };
-    PsiIn<float> next = load(sub, 0);
-    if (t > 0) {
-      const bool ok = mbar_wait(&bars[2], (uint32_t)((t - 1) & 1), kDrainLimit);
-      if (!__all_sync(0xffffffffu, ok) || *s_abort) {
-        aborted = true;
-        break;
-      }
-      pq.g = *s_scale;
-    }
-
-    // ---- Eq. 1 for psi, then Eq. 5, Alg. 2 and Eq. 6 (the next cells' values
-    // loaded while one set is computed)
     float mass_hi = 0.f, mass_lo = 0.f;
-    for (int jb = 0; jb < ncw; jb += cps) {
-      const int j = jb + sub;
-      const bool on = j < ncw;
-      float* scl = s_cell + (on ? j : 0) * kResCell;
-      const CellVel<float> uv{scl[0], scl[1], scl[2], scl[3], scl[4],
-                              scl[5], scl[6], scl[7], scl[8], scl[9]};
-      const float* nbc = s_nb + (on ? j : 0) * nth;
-      const size_t cbase = (size_t)(cw + j) * nth;
-      float acc = 0.f, cell_mass = 0.f;
-      for (int kk = 0; kk < nk; ++kk) {
-        const PsiIn<float> in = next;
-        next = kk + 1 < nk ? load(j, kk + 1) : load(j + cps, 0);
-        const int k = kk * seg + kl;
-        if (on && k < nth) {
-          const float pnew = psi_point(pq, uv, nk == 1 ? lt : trig_at(a.s.trig, nth, k), in);
-          __stcg(psi_out + cbase + k, pnew);
-          cell_mass += pnew;
-          acc = fma_t(pnew * nbc[k], pq.dth, acc);
-        }
-      }
+    // Eq. 5, Alg. 2 and Eq. 6 of cell j (of each sub's cell at once), from the
+    // lanes' parts of the coarse density
+    auto close = [&](int it, int j, bool on, float cell_mass, float acc, float mtot) {
+      float* scl = s_cell + j * kResCell;
+      const float* nbc = s_nb + j * nth;
       two_sum_acc(mass_hi, mass_lo, cell_mass);
       const float Cpre = seg_sum(acc, seg);
-      const float mtot = scl[11];
       float f = 1.f, C = Cpre;
       if (on && mtot < Cpre) {
         f = mtot / Cpre;
@@ -426,21 +458,25 @@ __global__ void __launch_bounds__(32 * (kResMaxWarps + 1), 1)
       if (__any_sync(0xffffffffu, f != 1.f)) {  // Alg. 2 scale-down (rare): the cells' rows
         for (int q = 0; q < cps; ++q) {
           const float fq = __shfl_sync(0xffffffffu, f, q * seg);
-          const int lo = (jb + q) * nth, hi = lo + nth;
+          const int lo = (q * half + it) * nth, hi = lo + nth;
           if (fq != 1.f)
             for (int p = lo / rpp; p <= (hi - 1) / rpp; ++p) {
               const int R = p * rpp + rslot;
-              if (R >= lo && R < hi)
+              if (!lane_ok || R < lo || R >= hi) continue;
+              if (p < kept) {
                 for (int g = 0; g < 64; g += 32) {
                   float4 x = tile[p * 64 + g];
                   x.x *= fq; x.y *= fq; x.z *= fq; x.w *= fq;
                   tile[p * 64 + g] = x;
                 }
+              } else {
+                for (int v = 0; v < nv; ++v) rows[p * pass_vals + v] *= fq;
+              }
             }
         }
       }
-      for (int k = kl; on && k < nth; k += seg)
-        __stcg(nb_out + cbase + k, f != 1.f ? nbc[k] * f : nbc[k]);
+      float* nbo = nb_out + (size_t)(cw + j) * nth;
+      for (int k = kl; on && k < nth; k += seg) __stcg(nbo + k, f != 1.f ? nbc[k] * f : nbc[k]);
       __syncwarp();
       if (on && kl == 0) {
         scl[10] = mtot - C;
@@ -448,6 +484,146 @@ __global__ void __launch_bounds__(32 * (kResMaxWarps + 1), 1)
           a.s.c[cw + j] = C;
           a.s.mf_out[cw + j] = mtot - C;
         }
+      }
+    };
+    auto factor = [&]() {  // the pending correction factor; false: a wait gave up
+      if (t > 0) {
+        const bool ok = mbar_wait(&bars[2], (uint32_t)((t - 1) & 1), kDrainLimit);
+        if (!__all_sync(0xffffffffu, ok) || *s_abort) return false;
+        pq.g = *s_scale;
+      }
+      return true;
+    };
+
+    // ---- Eq. 1 for psi, then Eq. 5, Alg. 2 and Eq. 6, a cell (one per sub) at a
+    // time with the next one's values loaded ahead; psi and n_b are read
+    // through L2, other SMs wrote them
+    if (nk == 1) {
+      // The cells of a run follow one another in x: the cell before is the west
+      // neighbour, and its east face, its own centre and its east neighbour are
+      // this cell's west face, west neighbour and centre, the same bits. The
+      // theta neighbours come by shuffle, as does the flux of the face theta - 1/2.
+      struct In {
+        float pe, pn, ps, ne, nn, ns, pc, pw, nc, nw;
+      };
+      const float* pk = psi_in + kl;
+      const float* nbk = nb_in + kl;
+      const bool kon = kl < nth;
+      auto load = [&](int it) {
+        In in{};
+        const int j = sub * half + it;
+        if (kon && it < half && j < ncw) {
+          const uint4 o = *reinterpret_cast<const uint4*>(s_cell + j * kResCell + 12);
+          const uint2 o2 = *reinterpret_cast<const uint2*>(s_cell + j * kResCell + 16);
+          in.pe = __ldcg(pk + o.y);
+          in.pn = __ldcg(pk + o.w);
+          in.ps = __ldcg(pk + o2.x);
+          in.ne = __ldcg(nbk + o.y);
+          in.nn = __ldcg(nbk + o.w);
+          in.ns = __ldcg(nbk + o2.x);
+          if (it == 0 || !o2.y) {
+            in.pc = __ldcg(pk + o.x);
+            in.pw = __ldcg(pk + o.z);
+            in.nc = __ldcg(nbk + o.x);
+            in.nw = __ldcg(nbk + o.z);
+          }
+        }
+        return in;
+      };
+      In next = load(0);
+      if (!factor()) {
+        aborted = true;
+        break;
+      }
+      const float g = pq.g;
+      const float ck = lt.ck, sk = lt.sk, cp = lt.cp, sp = lt.sp;
+      float Pe = 0.f, Ve = 0.f, axe = 0.f, Fe = 0.f;  // the cell before's
+      for (int it = 0; it < half; ++it) {
+        const In in = next;
+        next = load(it + 1);
+        const bool on = sub * half + it < ncw;
+        const int j = on ? sub * half + it : 0;
+        const float4* q4 = reinterpret_cast<const float4*>(s_cell + j * kResCell);
+        const float4 ua = q4[0], ub = q4[1], uc = q4[2];  // u at c, e, w (x) and n, s (y); grad u
+        float Pc = Pe, Vc = Ve, axc = axe, Fw = Fe;
+        if (it == 0 || !reinterpret_cast<const unsigned*>(q4)[17]) {
+          const float Pw = g * in.pw, Vw = fma_t(pq.glide, in.nw, pq.vsp);
+          Pc = g * in.pc;
+          Vc = fma_t(pq.glide, in.nc, pq.vsp);
+          axc = fma_t(-Vc, ck, ua.x);
+          const float axw = fma_t(-Vw, ck, ua.w);
+          Fw = donor(0.5f * (axw + axc), Pw, Pc);
+        }
+        Pe = g * in.pe;
+        const float Pn = g * in.pn, Ps = g * in.ps;
+        Ve = fma_t(pq.glide, in.ne, pq.vsp);
+        const float Vn = fma_t(pq.glide, in.nn, pq.vsp), Vs = fma_t(pq.glide, in.ns, pq.vsp);
+        axe = fma_t(-Ve, ck, ua.z);
+        const float ayc = fma_t(-Vc, sk, ua.y);
+        const float ayn = fma_t(-Vn, sk, ub.x), ays = fma_t(-Vs, sk, ub.y);
+        const float wp = fma_t(-sp, fma_t(ub.z, cp, ub.w * sp), cp * fma_t(uc.x, cp, uc.y * sp));
+        Fe = donor(0.5f * (axc + axe), Pc, Pe);
+        const float Fn = donor(0.5f * (ayc + ayn), Pc, Pn);
+        const float Fs = donor(0.5f * (ays + ayc), Ps, Pc);
+        const float Fp = donor(wp, Pc, __shfl_sync(0xffffffffu, Pc, up));
+        const float Fm = __shfl_sync(0xffffffffu, Fp, down);
+        const float div =
+            fma_t(Fp - Fm, pq.inv_dth, fma_t(Fn - Fs, pq.inv_dy, (Fe - Fw) * pq.inv_dx));
+        const float pnew = fma_t(-pq.dt, div, Pc);
+        float acc = 0.f;
+        if (on && kon) {
+          __stcg(psi_out + (size_t)(cw + j) * nth + kl, pnew);
+          acc = fma_t(pnew * s_nb[j * nth + kl], pq.dth, 0.f);
+        }
+        close(it, j, on, on && kon ? pnew : 0.f, acc, uc.w);
+      }
+    } else {
+      // more than 32 orientations: a lane takes several of every cell
+      auto load = [&](int j, int kk) {
+        PsiIn<float> in{};
+        const int k = kk * 32 + lane;
+        if (j < ncw && k < nth) {
+          const unsigned* id = reinterpret_cast<const unsigned*>(s_cell + j * kResCell + 12);
+          const int kp = k + 1 == nth ? 0 : k + 1, km = k == 0 ? nth - 1 : k - 1;
+          const float *p0 = psi_in + id[0], *n0 = nb_in + k;
+          in.pc = __ldcg(p0 + k);
+          in.pp = __ldcg(p0 + kp);
+          in.pm = __ldcg(p0 + km);
+          in.pe = __ldcg(psi_in + id[1] + k);
+          in.pw = __ldcg(psi_in + id[2] + k);
+          in.pn = __ldcg(psi_in + id[3] + k);
+          in.ps = __ldcg(psi_in + id[4] + k);
+          in.nc = __ldcg(n0 + id[0]);
+          in.ne = __ldcg(n0 + id[1]);
+          in.nw = __ldcg(n0 + id[2]);
+          in.nn = __ldcg(n0 + id[3]);
+          in.ns = __ldcg(n0 + id[4]);
+        }
+        return in;
+      };
+      PsiIn<float> next = load(0, 0);
+      if (!factor()) {
+        aborted = true;
+        break;
+      }
+      for (int j = 0; j < ncw; ++j) {
+        const float* scl = s_cell + j * kResCell;
+        const CellVel<float> uv{scl[0], scl[1], scl[2], scl[3], scl[4],
+                                scl[5], scl[6], scl[7], scl[8], scl[9]};
+        const float* nbc = s_nb + j * nth;
+        float acc = 0.f, cell_mass = 0.f;
+        for (int kk = 0; kk < nk; ++kk) {
+          const PsiIn<float> in = next;
+          next = kk + 1 < nk ? load(j, kk + 1) : load(j + 1, 0);
+          const int k = kk * 32 + lane;
+          if (k < nth) {
+            const float pnew = psi_point(pq, uv, trig_at(a.s.trig, nth, k), in);
+            __stcg(psi_out + (size_t)(cw + j) * nth + k, pnew);
+            cell_mass += pnew;
+            acc = fma_t(pnew * nbc[k], pq.dth, acc);
+          }
+        }
+        close(j, j, true, cell_mass, acc, scl[11]);
       }
     }
     const float2 wsum = warp_sum_ff2(make_float2(mass_hi, mass_lo));
@@ -457,21 +633,44 @@ __global__ void __launch_bounds__(32 * (kResMaxWarps + 1), 1)
   }
   if (aborted) return;
 
-  // store the rows
-  for (int p = 0; p < passes; ++p) {
-    const int R = p * rpp + rslot;
-    if (!(lane_ok && R < nrows)) continue;
+  // store the kept rows
+  for (int p = 0; p < kept; ++p) {
+    if (!(lane_ok && p * rpp + rslot < nrows)) continue;
     const float4 x = tile[p * 64], y = tile[p * 64 + 32];
-    float* dst = a.s.mb_out + ((size_t)cw * nth + R) * ns + sl * 8;
-    if constexpr (RAG) {
-      const float v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (q < nv) dst[q] = v[q];
-    } else {
-      reinterpret_cast<float4*>(dst)[0] = x;
-      reinterpret_cast<float4*>(dst)[1] = y;
-    }
+    const float2 M[4] = {make_float2(x.x, x.y), make_float2(x.z, x.w), make_float2(y.x, y.y),
+                         make_float2(y.z, y.w)};
+    store_row8<RAG>(rows + p * pass_vals, M, nv, a.vw);
+  }
+}
+
+template <int NL>
+__global__ void __launch_bounds__(32 * (kResMaxWarps + 1), 1)
+    k_substep_resident(const ResidentArgs a) {
+  resident_block<NL>(a, blockIdx.x);
+}
+
+// (its own function per row form: the register allocation of one is not that of
+// all four together)
+template <int NL>
+__device__ __noinline__ void resident_block_of_group(const ResidentArgs& a, int block) {
+  resident_block<NL>(a, block);
+}
+
+// Several independent instances in one launch: map[blockIdx.x] = (entry of tab,
+// block of that instance). Each instance has its own exchange.
+__global__ void __launch_bounds__(32 * (kResMaxWarps + 1), 1)
+    k_substep_resident_group(const ResidentArgs* __restrict__ tab, const int2* __restrict__ map) {
+  __shared__ ResidentArgs s_a;
+  const int2 m = map[blockIdx.x];
+  static_assert(sizeof(ResidentArgs) % 4 == 0, "copied by words");
+  for (unsigned i = threadIdx.x; i < sizeof(ResidentArgs) / 4; i += blockDim.x)
+    reinterpret_cast<unsigned*>(&s_a)[i] = reinterpret_cast<const unsigned*>(tab + m.x)[i];
+  __syncthreads();
+  switch (s_a.NL) {
+    case 2: resident_block_of_group<2>(s_a, m.y); break;
+    case 4: resident_block_of_group<4>(s_a, m.y); break;
+    case 8: resident_block_of_group<8>(s_a, m.y); break;
+    default: resident_block_of_group<0>(s_a, m.y); break;
   }
 }
 
@@ -481,13 +680,78 @@ namespace mmh {
 
 namespace {
 
-constexpr size_t kResidentBudget = 227 * 1024;  // shared memory a block may have
+constexpr size_t kResidentBudget = 226 * 1024;  // dynamic shared memory of a block
 
 const void* resident_kernel(int NL) {
   return NL == 2   ? (const void*)mm::k_substep_resident<2>
          : NL == 4 ? (const void*)mm::k_substep_resident<4>
          : NL == 8 ? (const void*)mm::k_substep_resident<8>
                    : (const void*)mm::k_substep_resident<0>;
+}
+
+// How an instance goes over `grid` blocks of one SM each: ceil(cells / grid) cells
+// to a block, the same number `own` to each worker, `tiles` passes of a worker's
+// rows kept in shared memory and, where that is not all of them, a ring for the
+// others, which are read and written every substep. False where it does not
+// fit, or where keeping too little of Mb on the chip gains nothing over
+// k_substep.
+struct ResidentPlan {
+  int own, workers, tiles, ring;
+  size_t smem;
+};
+bool resident_plan(const mm_handle* h, int grid, ResidentPlan* p) {
+  const int nth = h->g.ntheta, nl = (h->g.ns + 7) / 8, rpp = 32 / nl;
+  const long long cells = (h->ncells + grid - 1) / grid;
+  if (cells > 1 << 16 || h->rows > 0x7fffffffULL) return false;  // (column offsets are 32-bit)
+  p->own = (int)((cells + mm::kResMaxWarps - 1) / mm::kResMaxWarps);
+  p->workers = (int)((cells + p->own - 1) / p->own);
+  const long long passes = ((long long)p->own * nth + rpp - 1) / rpp;
+  const size_t fixed = mm::resident_smem(p->workers, p->own, nth, 0).total;
+  if (fixed >= kResidentBudget) return false;
+  const long long room = (long long)((kResidentBudget - fixed) / ((size_t)p->workers * 1024));
+  p->ring = passes <= room ? 0 : mm::kResRing;
+  p->tiles = (int)(passes <= room ? passes : room - p->ring);
+  if (p->tiles < 0) return false;
+  p->smem = mm::resident_smem(p->workers, p->own, nth, p->tiles + p->ring).total;
+  return true;
+}
+
+// Whether the resident kernel is the faster one for an instance it can hold.
+// Its arithmetic runs at about 650 G motor updates per second (25 us a substep
+// at 128^2 x 32^2, where k_substep takes 35), k_substep's at HBM speed where a
+// row fills its lanes: from about 250 MB of Mb on, twice the L2, HBM bounds both
+// and the bulk-copy rings of k_substep keep more of it in flight (256^2 x 32^2,
+// 268 MB: 127 against 131 us; 160^2 x 64^2, 420 MB: 189 against 155). Rows that
+// are no multiple of 4 nodes have one node to a lane in k_substep: 200 x 150 x
+// 24 x 30 44 against 231 us, whatever the size.
+bool resident_pays(const mm_handle* h) {
+  return h->g.ns % 4 != 0 || h->mbn * h->tsz <= (size_t)250 << 20;
+}
+
+// Kernel arguments of n substeps of h's live state; the exchange's tags and
+// arrivals of those substeps are taken.
+mm::ResidentArgs resident_args(mm_handle* h, int grid, const ResidentPlan& p, int n) {
+  mm::ResidentArgs a{};
+  a.s = step_args<float>(h, h->parity);
+  a.n = n;
+  a.nl = (h->g.ns + 7) / 8;
+  a.rpp = 32 / a.nl;
+  a.vl = h->g.ns - 8 * (a.nl - 1);
+  a.vw = h->g.ns % 4 == 0 ? 4 : h->g.ns % 2 == 0 ? 2 : 1;
+  a.own = p.own;
+  a.tiles = p.tiles;
+  a.ring = p.ring;
+  a.workers = p.workers;
+  a.grid = grid;
+  a.NL = h->res_NL;
+  a.seg = 1;
+  while (a.seg < 32 && a.seg < h->g.ntheta) a.seg <<= 1;
+  a.epoch = h->res_epoch;
+  a.arrivals = h->res_arrivals;
+  a.xch = h->res_xch;
+  h->res_epoch += (unsigned)n;
+  h->res_arrivals += (unsigned)n * (unsigned)grid;
+  return a;
 }
 
 // Resident launches of one device run one after the other, on whatever
@@ -505,64 +769,10 @@ DeviceOrder& device_order() {
 
 }  // namespace
 
-// Plan: one block per SM with ceil(cells / SMs) cells, as many workers as give
-// every warp the same number of cells. Off (h->res_grid = 0) in float64 and
-// where a block's rows do not fit its shared memory.
-mm_status resident_configure(mm_handle* h) {
-  h->res_grid = 0;
-  if (h->prec != MM_FP32_MIXED) return MM_OK;
-  int coop = 0;
-  CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device));
-  if (!coop) return MM_OK;
-  const int ns = h->g.ns, nth = h->g.ntheta;
-  const int nl = (ns + 7) / 8;
-  h->res_NL = ns % 8 == 0 && (nl == 2 || nl == 4 || nl == 8) ? nl : 0;
-  const long long grid = std::min<long long>({h->sms, h->ncells, 32 * mm::kResXch});
-  const long long cells = (h->ncells + grid - 1) / grid;
-  if (cells * nth * nl * 32 > (long long)kResidentBudget) return MM_OK;
-  h->res_own = (int)((cells + mm::kResMaxWarps - 1) / mm::kResMaxWarps);
-  const int workers = (int)((cells + h->res_own - 1) / h->res_own);
-  const int rpp = 32 / nl;
-  h->res_passes = (h->res_own * nth + rpp - 1) / rpp;
-  const size_t smem = mm::resident_smem(workers, h->res_own, nth, h->res_passes).total;
-  if (smem > kResidentBudget) return MM_OK;
-  const void* f = resident_kernel(h->res_NL);
-  CK(mm::raise_smem_limit(f, smem));
-  int bps = 0;
-  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, f, 32 * (workers + 1), smem));
-  if (bps < 1) return MM_OK;
-  h->res_block = 32 * (workers + 1);
-  h->res_smem = smem;
-  h->res_grid = (int)grid;
-  return MM_OK;
-}
+namespace {
 
-// n substeps on the live state in one launch; *done = false (and nothing
-// launched) where the resident kernel does not apply: no plan, a single
-// substep, another substep kernel in effect, or a stream being captured (the
-// ordering event belongs to no capture).
-mm_status resident_substeps(mm_handle* h, int n, bool* done) {
-  *done = false;
-  if (h->res_grid == 0 || n < 2 || h->anchors || h->capture || h->tangent) return MM_OK;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  CK(cudaStreamIsCapturing(h->stream, &cs));
-  if (cs != cudaStreamCaptureStatusNone) return MM_OK;
-  mm::ResidentArgs a{};
-  a.s = step_args<float>(h, h->parity);
-  a.n = n;
-  a.nl = (h->g.ns + 7) / 8;
-  a.rpp = 32 / a.nl;
-  a.vl = h->g.ns - 8 * (a.nl - 1);
-  a.own = h->res_own;
-  a.passes = h->res_passes;
-  a.seg = 1;
-  while (a.seg < 32 && a.seg < h->g.ntheta) a.seg <<= 1;
-  a.epoch = h->res_epoch;
-  a.arrivals = h->res_arrivals;
-  a.xch = h->res_xch;
-  h->res_epoch += (unsigned)n;
-  h->res_arrivals += (unsigned)n * (unsigned)h->res_grid;
-  void* args[1] = {&a};
+mm_status launch_ordered(mm_handle* h, const void* f, int grid, int block, size_t smem,
+                         void** args) {
   DeviceOrder& o = device_order();
   std::lock_guard<std::mutex> lock(o.m);
   cudaEvent_t& ev = o.last[h->device];
@@ -570,12 +780,196 @@ mm_status resident_substeps(mm_handle* h, int n, bool* done) {
     CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
   else
     CK(cudaStreamWaitEvent(h->stream, ev, 0));
-  CK(cudaLaunchCooperativeKernel(resident_kernel(h->res_NL), dim3((unsigned)h->res_grid),
-                                 dim3((unsigned)h->res_block), args, h->res_smem, h->stream));
+  CK(cudaLaunchCooperativeKernel(f, dim3((unsigned)grid), dim3((unsigned)block), args, smem,
+                                 h->stream));
   CK(cudaEventRecord(ev, h->stream));
+  return MM_OK;
+}
+
+}  // namespace
+
+// Off (h->res_grid = 0) in float64 and where no plan fits.
+mm_status resident_configure(mm_handle* h) {
+  h->res_grid = 0;
+  if (h->prec != MM_FP32_MIXED) return MM_OK;
+  int coop = 0;
+  CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device));
+  if (!coop) return MM_OK;
+  const int ns = h->g.ns, nl = (ns + 7) / 8;
+  h->res_NL = ns % 8 == 0 && (nl == 2 || nl == 4 || nl == 8) ? nl : 0;
+  const int grid = (int)std::min<long long>({h->sms, h->ncells, 32 * mm::kResXch});
+  ResidentPlan p;
+  if (!resident_pays(h) || !resident_plan(h, grid, &p)) return MM_OK;
+  const void* f = resident_kernel(h->res_NL);
+  CK(mm::raise_smem_limit(f, kResidentBudget));
+  int bps = 0;
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, f, 32 * (p.workers + 1), p.smem));
+  if (bps < 1) return MM_OK;
+  h->res_grid = grid;
+  return MM_OK;
+}
+
+// Whether n substeps of h go through the resident kernel: not without a plan
+// that pays, for a single substep, with another substep kernel in effect, or on
+// a stream being captured (the ordering event belongs to no capture).
+static bool resident_applies(mm_handle* h, int n) {
+  if (h->res_grid == 0 || n < 2 || h->anchors || h->capture || h->tangent) return false;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(h->stream, &cs) == cudaSuccess &&
+         cs == cudaStreamCaptureStatusNone;
+}
+
+// n substeps on the live state in one launch; *done = false (and nothing
+// launched) where the resident kernel does not apply.
+mm_status resident_substeps(mm_handle* h, int n, bool* done) {
+  *done = false;
+  if (!resident_applies(h, n)) return MM_OK;
+  ResidentPlan p;
+  if (!resident_plan(h, h->res_grid, &p)) return MM_OK;
+  mm::ResidentArgs a = resident_args(h, h->res_grid, p, n);
+  void* args[1] = {&a};
+  const mm_status st = launch_ordered(h, resident_kernel(h->res_NL), h->res_grid,
+                                      32 * (p.workers + 1), p.smem, args);
+  if (st != MM_OK) return st;
   h->parity ^= n & 1;
   *done = true;
   return MM_OK;
+}
+
+// ---- groups of batch members
+
+namespace {
+
+// Relative work of one cell in a substep: a pass of rows and, for psi and the
+// close, about 0.8 of one (half where two cells share a warp).
+double cell_work(const mm_handle* h) {
+  const int nth = h->g.ntheta, nl = (h->g.ns + 7) / 8;
+  int seg = 1;
+  while (seg < 32 && seg < nth) seg <<= 1;
+  return nth * nl / 32.0 + 0.8 * (seg / 32.0) * ((nth + seg - 1) / seg);
+}
+double block_work(const mm_handle* h, int grid) {
+  ResidentPlan p;
+  if (!resident_plan(h, grid, &p)) return 1e30;
+  return p.workers * p.own * cell_work(h);
+}
+
+}  // namespace
+
+// Splits the members that the resident kernel holds into groups that run one
+// after the other, each over all SMs: as many members as shared memory takes
+// and as the L2 holds what is not kept there (about 110 MB of Mb), the largest
+// first; within a group every member gets the fewest SMs it fits on and the
+// others go to whichever has the most work per SM. in[i] = 1 for the members
+// taken.
+mm_status resident_group_plan(mm_handle* h, const std::vector<mm_handle*>& members,
+                              std::vector<ResidentGroup>* groups, std::vector<char>* in) {
+  constexpr size_t kGroupBytes = (size_t)110 << 20;
+  groups->clear();
+  in->assign(members.size(), 0);
+  if (h->prec != MM_FP32_MIXED) return MM_OK;
+  std::vector<int> order;
+  for (size_t i = 0; i < members.size(); ++i)
+    if (members[i]->res_grid > 0) order.push_back((int)i);
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int a, int b) { return members[a]->mbn > members[b]->mbn; });
+  struct Load {
+    int sms = 0;
+    size_t bytes = 0;
+  };
+  std::vector<Load> loads;
+  for (int i : order) {
+    const mm_handle* m = members[i];
+    ResidentPlan p;
+    int g = 1;
+    while (g < m->res_grid && !resident_plan(m, g, &p)) ++g;
+    if (!resident_plan(m, g, &p)) continue;
+    const size_t bytes = m->mbn * m->tsz;
+    size_t q = 0;
+    while (q < groups->size() && (loads[q].sms + g > h->sms ||
+                                  (loads[q].bytes > 0 && loads[q].bytes + bytes > kGroupBytes)))
+      ++q;
+    if (q == groups->size()) {
+      groups->push_back({});
+      loads.push_back({});
+    }
+    (*groups)[q].member.push_back(i);
+    (*groups)[q].blocks.push_back(g);
+    loads[q].sms += g;
+    loads[q].bytes += bytes;
+    (*in)[i] = 1;
+  }
+  for (size_t q = 0; q < groups->size(); ++q) {
+    ResidentGroup& G = (*groups)[q];
+    std::vector<double> work;
+    for (size_t k = 0; k < G.member.size(); ++k)
+      work.push_back(block_work(members[G.member[k]], G.blocks[k]));
+    for (int left = h->sms - loads[q].sms; left > 0; --left) {
+      int best = -1;
+      for (size_t k = 0; k < work.size(); ++k)
+        if (G.blocks[k] < members[G.member[k]]->res_grid && (best < 0 || work[k] > work[best]))
+          best = (int)k;
+      if (best < 0) break;
+      ++G.blocks[best];
+      work[best] = block_work(members[G.member[best]], G.blocks[best]);
+    }
+    G.grid = G.block = 0;
+    G.smem = 0;
+    std::vector<int2> map;
+    for (size_t k = 0; k < G.member.size(); ++k) {
+      ResidentPlan p;
+      resident_plan(members[G.member[k]], G.blocks[k], &p);
+      G.block = std::max(G.block, 32 * (p.workers + 1));
+      G.smem = std::max(G.smem, p.smem);
+      for (int b = 0; b < G.blocks[k]; ++b) map.push_back(make_int2((int)k, b));
+    }
+    G.grid = (int)map.size();
+    CK(cudaMalloc(&G.map, map.size() * sizeof(int2)));
+    CK(cudaMemcpy(G.map, map.data(), map.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    CK(cudaMalloc(&G.tab, G.member.size() * sizeof(mm::ResidentArgs)));
+  }
+  if (!groups->empty())
+    CK(mm::raise_smem_limit((const void*)mm::k_substep_resident_group, kResidentBudget));
+  return MM_OK;
+}
+
+void resident_group_free(std::vector<ResidentGroup>* groups) {
+  for (ResidentGroup& G : *groups) {
+    if (G.map) cudaFree(G.map);
+    if (G.tab) cudaFree(G.tab);
+  }
+  groups->clear();
+}
+
+// n substeps of a group's members; their parities advance.
+mm_status resident_group_step(mm_handle* h, const std::vector<mm_handle*>& members,
+                              ResidentGroup& G, int n) {
+  std::vector<mm::ResidentArgs> tab;
+  for (size_t k = 0; k < G.member.size(); ++k) {
+    mm_handle* m = members[G.member[k]];
+    ResidentPlan p;
+    resident_plan(m, G.blocks[k], &p);
+    tab.push_back(resident_args(m, G.blocks[k], p, n));
+  }
+  // stream-ordered after the launch that read the table before; the pageable
+  // source is staged before the call returns
+  CK(cudaMemcpyAsync(G.tab, tab.data(), tab.size() * sizeof(mm::ResidentArgs),
+                     cudaMemcpyHostToDevice, h->stream));
+  const mm::ResidentArgs* dt = (const mm::ResidentArgs*)G.tab;
+  const int2* dm = (const int2*)G.map;
+  void* args[2] = {&dt, &dm};
+  const mm_status st = launch_ordered(h, (const void*)mm::k_substep_resident_group, G.grid,
+                                      G.block, G.smem, args);
+  if (st != MM_OK) return st;
+  for (int i : G.member) members[i]->parity ^= n & 1;
+  return MM_OK;
+}
+
+// Whether n substeps of a batch may go through its groups.
+bool resident_group_applies(mm_handle* h, int n) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  return n >= 2 && cudaStreamIsCapturing(h->stream, &cs) == cudaSuccess &&
+         cs == cudaStreamCaptureStatusNone;
 }
 
 }  // namespace mmh

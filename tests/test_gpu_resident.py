@@ -97,3 +97,73 @@ def test_resident_on_two_streams(mmod):
     for a, b in zip(*got):
         for k in KEYS:
             assert np.array_equal(a[k], b[k]), k
+
+
+# rows kept in part: whole vectors, halves and single values of 16-byte copies,
+# a grid a block of which holds cells of several rows
+@pytest.mark.parametrize("dims", [(130, 96, 40, 24), (128, 128, 32, 32), (150, 120, 24, 30),
+                                  (141, 130, 23, 29), (120, 110, 48, 36)])
+def test_partly_kept_rows(mmod, dims):
+    """Instances beyond the chip: the substeps of one call against one substep
+    per call, and the conserved sums."""
+    g = Grid(*dims)
+    psi, mb, u = inputs(g, 7, 0.3)
+    got = []
+    for each in (5, 1):
+        with mmod.Simulation(g, Rates(glide=0.3), "fp32") as sim:
+            sim.set_state(psi, mb)
+            sim.set_velocity(u)
+            for _ in range(5 // each):
+                sim.step(each)
+            got.append(sim.get_state())
+            _, sc = sim.moments()
+            assert abs(sc["N_psi"] - 1.0) < 1e-6 and abs(sc["motors"] - 1.0) < 1e-5
+    for k in KEYS:
+        assert rel_l2(got[0][k], got[1][k]) <= 1e-6, k
+
+
+def test_partly_kept_rows_scale_down(mmod):
+    """The scale-down on rows that are not kept, against the oracle."""
+    from oracle import oracle as O
+    g = Grid(120, 110, 32, 24)
+    r = Rates(k_on=400.0)
+    psi, mb, u = inputs(g, 5, 0.3)
+    st = O.make_state(g, psi, mb)
+    dt = O.dt(g, Rates(), st, u)
+    with mmod.Simulation(g, r, "fp32") as sim:
+        sim.set_state(psi, mb)
+        sim.set_velocity(u)
+        sim.set_dt(dt)
+        sim.step(3)
+        got = sim.get_state()
+    O.run(g, r, st, u, dt, 3)
+    for k in ("psi", "mb", "c"):
+        assert rel_l2(got[k], getattr(st, k)) <= 1e-5, k
+
+
+def test_batch_groups(mmod):
+    """A batch whose members are too many for one group (their Mb together is
+    above a group's share of the L2) with one that no resident launch holds:
+    every member equals itself stepped alone by single substeps."""
+    grids = [Grid(96, 96, 32, 32), Grid(16, 16, 16, 16), Grid(80, 72, 32, 32), Grid(33, 20, 8, 12),
+             Grid(128, 128, 32, 32), Grid(64, 48, 16, 20), Grid(96, 64, 64, 64), Grid(192, 128, 64, 48)]
+    rates = [Rates(k_off=0.3 + 0.2 * i, glide=0.2) for i in range(len(grids))]
+    states = [inputs(g, 20 + i, 0.3) for i, g in enumerate(grids)]
+    with mmod.Batch(grids, rates, "fp32") as b:
+        for sim, (psi, mb, u) in zip(b.members, states):
+            sim.set_state(psi, mb)
+            sim.set_velocity(u)
+        b.step(3)
+        b.members[2].step(2)  # one member alone in between
+        b.step(2)
+        b.sync()
+        got = [sim.get_state() for sim in b.members]
+    for i, (g, r, (psi, mb, u)) in enumerate(zip(grids, rates, states)):
+        with mmod.Simulation(g, r, "fp32") as sim:
+            sim.set_state(psi, mb)
+            sim.set_velocity(u)
+            for _ in range(7 if i == 2 else 5):
+                sim.step(1)
+            ref = sim.get_state()
+        for k in KEYS:
+            assert rel_l2(got[i][k], ref[k]) <= 1e-6, (i, k)
