@@ -122,26 +122,28 @@ StepArgs<T> step_args(mm_handle* h, int parity) {
 template StepArgs<float> step_args<float>(mm_handle*, int);
 template StepArgs<double> step_args<double>(mm_handle*, int);
 
+// The substep kernel of h's plan on given arguments.
+template <typename T>
+cudaError_t launch_step(const mm_handle* h, const StepArgs<T>& a, cudaStream_t s, bool overlap) {
+  return mm::launch_substep<T>(a, h->grid_step, h->block, h->smem, h->tma, s, overlap);
+}
+cudaError_t launch_plain(mm_handle* h, int parity, cudaStream_t s) {
+  return h->prec == MM_FP64 ? launch_step(h, step_args<double>(h, parity), s, false)
+                            : launch_step(h, step_args<float>(h, parity), s, false);
+}
+
 cudaError_t launch_one(mm_handle* h, int parity, cudaStream_t s) {
   if (h->anchors) return launch_anchor_substep(h, parity, s);
   if (h->capture) return launch_capture_substep(h, parity, s);
   if (h->tangent) return launch_tangent_substep(h, parity, s);
-  if (h->prec == MM_FP64) {
-    StepArgs<double> a = step_args<double>(h, parity);
-    return h->V == 2 ? mm::launch_substep<double, 2>(a, h->grid_step, h->block, h->smem, h->tma, s)
-                     : mm::launch_substep<double, 1>(a, h->grid_step, h->block, h->smem, h->tma, s);
-  }
-  StepArgs<float> a = step_args<float>(h, parity);
-  if (h->V == 8) return mm::launch_substep<float, 8>(a, h->grid_step, h->block, h->smem, h->tma, s);
-  return h->V == 4 ? mm::launch_substep<float, 4>(a, h->grid_step, h->block, h->smem, h->tma, s)
-                   : mm::launch_substep<float, 1>(a, h->grid_step, h->block, h->smem, h->tma, s);
+  return launch_plain(h, parity, s);
 }
 
 // Launch plan of the substep kernel: one warp per cell, the cell's rows
 // streamed in chunks of chunk_rows rows (at most kChunkBytes) through a ring of
-// `stages` shared-memory stages per warp filled by bulk copies (TMA) when an
-// s-row is a whole number of 16-byte vectors; otherwise rows are read from
-// global memory directly.
+// `stages` shared-memory stages per warp filled by bulk copies (TMA) when a
+// chunk and a cell are whole numbers of 16-byte vectors; otherwise the warp
+// copies each chunk into its one stage itself.
 
 // One substep with explicit state buffers (recomputing a recorded segment).
 struct StepPtrs {
@@ -167,23 +169,15 @@ StepArgs<T> step_args_ptrs(mm_handle* h, const StepPtrs& p) {
 // (direct launches of the recording and the reverse sweep: overlapped with
 // the previous kernel of the stream)
 cudaError_t launch_ptrs(mm_handle* h, const StepPtrs& p, cudaStream_t s) {
-  const int g = h->grid_step, b = h->block;
-  const size_t sm = h->smem;
-  if (h->prec == MM_FP64) {
-    StepArgs<double> a = step_args_ptrs<double>(h, p);
-    return h->V == 2 ? mm::launch_substep_overlapped<double, 2>(a, g, b, sm, h->tma, s)
-                     : mm::launch_substep_overlapped<double, 1>(a, g, b, sm, h->tma, s);
-  }
-  StepArgs<float> a = step_args_ptrs<float>(h, p);
-  if (h->V == 8) return mm::launch_substep_overlapped<float, 8>(a, g, b, sm, h->tma, s);
-  return h->V == 4 ? mm::launch_substep_overlapped<float, 4>(a, g, b, sm, h->tma, s)
-                   : mm::launch_substep_overlapped<float, 1>(a, g, b, sm, h->tma, s);
+  return h->prec == MM_FP64 ? launch_step(h, step_args_ptrs<double>(h, p), s, true)
+                            : launch_step(h, step_args_ptrs<float>(h, p), s, true);
 }
 
 mm_status configure(mm_handle* h) {
   const int ns = h->g.ns, nth = h->g.ntheta;
-  // values per lane: the widest instantiated vector that divides ns -- float64
-  // {2, 1}, float32 {8, 4, 1} (two 16-byte vectors, one, or scalar lanes)
+  // values per lane of the kernels beside the substep's own: the widest
+  // instantiated vector that divides ns -- float64 {2, 1}, float32 {8, 4, 1} (two
+  // 16-byte vectors, one, or scalar lanes)
   h->V = 1;
   if (h->prec == MM_FP64) {
     if (ns % 2 == 0) h->V = 2;
@@ -198,18 +192,24 @@ mm_status configure(mm_handle* h) {
   int seg = 1;
   while (seg < nl) seg <<= 1;
   h->seg = seg;
-  h->tma = ((size_t)h->V * h->tsz) % 16 == 0;
   const size_t row_bytes = (size_t)ns * h->tsz;
-  int ch = 1;
-  while (ch < nth && (nth % ch != 0 || (size_t)(nth / ch) * row_bytes > kChunkBytes)) ++ch;
+  // the fewest chunks of at most kChunkBytes, of whole 16-byte vectors where
+  // that can be had
+  int ch = 0;
+  for (int c = 1; c <= nth; ++c) {
+    if (nth % c != 0 || (c < nth && (size_t)(nth / c) * row_bytes > kChunkBytes)) continue;
+    const bool vec = (size_t)(nth / c) * row_bytes % 16 == 0;
+    if (ch == 0 || vec) ch = c;
+    if (vec) break;
+  }
   h->chunks_per_cell = ch;
   h->chunk_rows = nth / ch;
   const size_t chunk_bytes = (size_t)h->chunk_rows * row_bytes;
+  h->tma = chunk_bytes % 16 == 0;
   int S = (int)(kWarpInflightBytes / std::max<size_t>(chunk_bytes, 1));
   S = std::max(2, std::min(8, S));
   h->stages = h->tma ? S : 1;
-  const size_t per_warp =
-      mm::step_smem_per_warp(h->stages, h->tma ? h->chunk_rows * ns : 0, nth, (int)h->tsz);
+  const size_t per_warp = mm::step_smem_per_warp(h->stages, h->chunk_rows * ns, nth, (int)h->tsz);
   const int wpb = (int)std::min<size_t>(kMaxWarpsPerBlock, kSmemBudget / per_warp);
   if (wpb < 1) return fail(h, MM_ERR_UNSUPPORTED, "ntheta too large for the shared-memory plan");
   h->block = 32 * wpb;
@@ -217,12 +217,9 @@ mm_status configure(mm_handle* h) {
   int bps = 0;
   cudaError_t e;
   if (h->prec == MM_FP64)
-    e = h->V == 2 ? mm::substep_prepare<double, 2>(h->block, h->smem, h->tma, &bps)
-                  : mm::substep_prepare<double, 1>(h->block, h->smem, h->tma, &bps);
+    e = mm::substep_prepare<double>(ns, h->block, h->smem, h->tma, &bps);
   else
-    e = h->V == 8 ? mm::substep_prepare<float, 8>(h->block, h->smem, h->tma, &bps)
-        : h->V == 4 ? mm::substep_prepare<float, 4>(h->block, h->smem, h->tma, &bps)
-                    : mm::substep_prepare<float, 1>(h->block, h->smem, h->tma, &bps);
+    e = mm::substep_prepare<float>(ns, h->block, h->smem, h->tma, &bps);
   CK(e);
   if (bps < 1) return fail(h, MM_ERR_UNSUPPORTED, "substep kernel cannot be resident");
   long long g = (long long)bps * h->sms;

@@ -25,7 +25,7 @@ namespace mm {
 #endif
 template <typename T>
 constexpr int batch_min_blocks() {
-  return sizeof(T) == 8 ? 3 : MM_BATCH_MIN_BLOCKS;
+  return sizeof(T) == 8 ? 2 : MM_BATCH_MIN_BLOCKS;
 }
 
 // The psi and n_b columns of two cells of one row (x0 and x0 + 1, y0; nx is
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(128, batch_min_blocks<T>())
         ds = sc.ds;
         rk = RkConst<T>{hdt * sc.cw, T(1) - hdt * sc.koff, T(0), dt * sc.cw, -dt * sc.koff, T(0),
                         T(0), T(0), nth};
-        lg = lane_geom(lane, seg, ns, V);
+        lg = sizeof(T) == 8 ? packed_lanes(lane, ns) : lane_geom(lane, seg, ns, V);
         iy = ct.cell0 / nx;
         ix = ct.cell0 - iy * nx;
       } else if ((ix += ct.cpu) >= nx) {  // consecutive units of the tile
@@ -293,8 +293,12 @@ __global__ void __launch_bounds__(128, batch_min_blocks<T>())
     // (rows from the unit's row nth on -- the second cell of a unit of 2 --
     // bind to that cell's Mf; a chunk may hold rows of either or both)
     rk.rsplit = nth - part * ct.rc;
-    rows_chunk<T, V, true>(stages + (size_t)s * stage_elems, A->mb_out + chunk_off, ct.rc, ns, seg,
-                           lg, rk, ds, s_nb + part * ct.rc);
+    if constexpr (sizeof(T) == 8)  // (an even ns: whole 16-byte vectors)
+      rows_packed<T, 2, true>(stages + (size_t)s * stage_elems, A->mb_out + chunk_off, ct.rc, ns, lg,
+                              rk, ds, s_nb + part * ct.rc);
+    else
+      rows_chunk<T, V, true>(stages + (size_t)s * stage_elems, A->mb_out + chunk_off, ct.rc, ns,
+                             seg, lg, rk, ds, s_nb + part * ct.rc);
     __syncwarp();
     if (lane == 0 && issued < nchunks) issue_next();
     if (++s == S) { s = 0; par ^= 1u; }

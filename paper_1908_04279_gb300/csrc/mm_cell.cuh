@@ -183,11 +183,25 @@ __device__ __forceinline__ double warp_sum_ff(double hi, double lo) {
 // ------------------------------------------------------------- s-row chunk
 
 // Where a lane sits in the s-rows of a pass: `seg` lanes per row (V nodes
-// each), rpp = 32 / seg rows per pass.
+// each), rpp = 32 / seg rows per pass. Packed rows (packed_lanes): nl = ceil(ns
+// / 8) lanes of eight nodes, floor(32 / nl) rows per pass; nv nodes in this lane.
 struct LaneGeom {
   int sl, rslot, rpp;
   bool first, last, lane_ok;
+  int nl, nv;
 };
+__device__ __forceinline__ LaneGeom packed_lanes(int lane, int ns) {
+  LaneGeom g;
+  g.nl = (ns + 7) / 8;
+  g.rpp = 32 / g.nl;
+  g.rslot = lane / g.nl;
+  g.sl = lane - g.rslot * g.nl;
+  g.first = g.sl == 0;
+  g.last = g.sl == g.nl - 1;
+  g.lane_ok = g.rslot < g.rpp;
+  g.nv = g.last ? ns - 8 * (g.nl - 1) : 8;
+  return g;
+}
 __device__ __forceinline__ LaneGeom lane_geom(int lane, int seg, int ns, int V) {
   LaneGeom g;
   g.sl = lane & (seg - 1);
@@ -319,6 +333,98 @@ __device__ __forceinline__ void rows_chunk(const T* src_rows, T* dst, int RC, in
   }
 }
 
+// A lane's nv values of a packed row at p, in vectors of VW values (VW divides
+// ns, hence nv).
+template <typename T, int VW>
+__device__ __forceinline__ void load_packed(const T* p, int nv, T (&m)[8]) {
+#pragma unroll
+  for (int q = 0; q < 8 / VW; ++q) {
+    Pack<T, VW> x{};
+    if (VW * q < nv) x = reinterpret_cast<const Pack<T, VW>*>(p)[q];
+#pragma unroll
+    for (int v = 0; v < VW; ++v) m[VW * q + v] = x.v[v];
+  }
+}
+template <typename T, int VW>
+__device__ __forceinline__ void store_packed(T* p, int nv, const T (&m)[8]) {
+#pragma unroll
+  for (int q = 0; q < 8 / VW; ++q) {
+    Pack<T, VW> x;
+#pragma unroll
+    for (int v = 0; v < VW; ++v) x.v[v] = m[VW * q + v];
+    if (VW * q < nv) reinterpret_cast<Pack<T, VW>*>(p)[q] = x;
+  }
+}
+
+// One chunk of RC packed s-rows: as rows_chunk, with eight nodes per lane for any
+// ns, in float64 (where the float64 pipe is what bounds the substep: eight
+// nodes per lane leave 12.3 float64 operations a node against 18 with two) and
+// in float32 where a row is not a power of two of full lanes. Rows of whole
+// 16-byte vectors (VW values) go straight to dst; others are written back into
+// the stage, from where the caller copies the chunk coalesced. Per substep on a
+// GB300: float64 128^2 x 32^2 850 (two nodes per lane) -> 585 us, 64^2 x 32 x 31
+// 297 (one) -> 160; float32 480 x 400 x 24 x 30 1630 (one) -> 388, 512^2 x 24 x 20
+// 513 (four) -> 502.
+template <typename T, int VW, bool SPLIT = false>
+__device__ __forceinline__ void rows_packed(T* stage, T* dst, int RC, int ns, const LaneGeom& lg,
+                                            const RkConst<T>& k, T ds, T* s_nb_chunk) {
+  constexpr bool direct = VW * sizeof(T) == 16;
+  const int passes = (RC + lg.rpp - 1) / lg.rpp;
+  [[maybe_unused]] float2 keep[4];
+  if constexpr (sizeof(T) == 4) {
+#pragma unroll
+    for (int h = 0; h < 4; ++h)
+      keep[h] = make_float2(lg.last && 2 * h == lg.nv - 1 ? 0.f : 1.f,
+                            lg.last && 2 * h + 1 == lg.nv - 1 ? 0.f : 1.f);
+  }
+  constexpr int kUnroll = sizeof(T) == 4 ? kStepUnroll : 1;
+#pragma unroll kUnroll
+  for (int p = 0; p < passes; ++p) {
+    const int r = p * lg.rpp + lg.rslot;  // row within the chunk
+    const bool hi = SPLIT && r >= k.rsplit;
+    const T c3 = hi ? k.c3b : k.c3, e3 = hi ? k.e3b : k.e3;
+    const bool act = r < RC && lg.lane_ok;
+    const int off = (act ? r : 0) * ns + lg.sl * 8;
+    T M[8];
+    load_packed<T, VW>(stage + off, act ? lg.nv : 0, M);
+    if constexpr (sizeof(T) == 4) {
+      float2 m[4], D[4], Ms[4];
+      const float2 c1 = make_float2(k.c1, k.c1), c2 = make_float2(k.c2, k.c2);
+      const float2 e1 = make_float2(k.e1, k.e1), e2 = make_float2(k.e2, k.e2);
+      const float2 c3_ = make_float2(c3, c3), e3_ = make_float2(e3, e3);
+#pragma unroll
+      for (int h = 0; h < 4; ++h) m[h] = make_float2(M[2 * h], M[2 * h + 1]);
+      walk_dflux_x2<8, true>(m, D, lg.first, lg.last, 32, keep);
+#pragma unroll
+      for (int h = 0; h < 4; ++h) Ms[h] = __ffma2_rn(c1, D[h], __ffma2_rn(c2, m[h], c3_));
+      walk_dflux_x2<8, true>(Ms, D, lg.first, lg.last, 32, keep);
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        m[h] = __ffma2_rn(e1, D[h], __ffma2_rn(e2, Ms[h], __fadd2_rn(m[h], e3_)));
+        M[2 * h] = m[h].x;
+        M[2 * h + 1] = m[h].y;
+      }
+    } else {
+      T D[8], Ms[8];
+      walk64<8, true>(M, D, lg.first, lg.last, lg.nv);
+#pragma unroll
+      for (int v = 0; v < 8; ++v) Ms[v] = fma_t(k.c1, D[v], fma_t(k.c2, M[v], c3));
+      walk64<8, true>(Ms, D, lg.first, lg.last, lg.nv);
+#pragma unroll
+      for (int v = 0; v < 8; ++v)
+        M[v] = fma_t(k.e1, D[v], fma_t(k.e2, Ms[v], add_rn(M[v], e3)));
+    }
+    // (pairs first, as walk_dflux_x2's rows: node 2h and 2h + 1 in two sums)
+    T a[8];
+#pragma unroll
+    for (int v = 0; v < 8; ++v) a[v] = v < lg.nv ? M[v] : T(0);
+    const T lo = ((a[0] + a[2]) + a[4]) + a[6], up = ((a[1] + a[3]) + a[5]) + a[7];
+    const T snb = packed_sum(lo + up, lg.nl, lg.sl);
+    if (act) store_packed<T, VW>((direct ? dst : stage) + off, lg.nv, M);
+    if (lg.first && act) s_nb_chunk[r] = snb * ds;
+  }
+}
+
 // The psi and n_b columns of a cell and its east, west, north and south
 // neighbours into psi5 / nb5 ([5][nth]), completing on `nbar`: lane 0 posts
 // the expected bytes, then lanes 0-9 each issue one of the 10 bulk copies.
@@ -408,8 +514,8 @@ __device__ __forceinline__ T psi_point(const PsiConst<T>& q, const CellVel<T>& u
   const T Vs = fma_t(q.glide, in.ns, q.vsp);
   const T axc = fma_t(-Vc, ck, u.uxc), axe = fma_t(-Ve, ck, u.uxe), axw = fma_t(-Vw, ck, u.uxw);
   const T ayc = fma_t(-Vc, sk, u.uyc), ayn = fma_t(-Vn, sk, u.uyn), ays = fma_t(-Vs, sk, u.uys);
-  const T Ae = T(0.5) * (axc + axe), Aw = T(0.5) * (axw + axc);
-  const T An = T(0.5) * (ayc + ayn), As = T(0.5) * (ays + ayc);
+  const T Ae = half_t(axc + axe), Aw = half_t(axw + axc);
+  const T An = half_t(ayc + ayn), As = half_t(ays + ayc);
   const T cp = t.cp, sp = t.sp, cm = t.cm, sm = t.sm;
   // Jeffery rotation p_perp . G . p at the faces k +- 1/2
   const T wp = fma_t(-sp, fma_t(u.Gxx, cp, u.Gxy * sp), cp * fma_t(u.Gyx, cp, u.Gyy * sp));

@@ -137,13 +137,14 @@ struct BatchTile {
                    // cells' rows; a half-warp each takes psi and the close)
 };
 
-// Kernel launchers (defined in mm_step.cu); V = values per lane.
-template <typename T, int V>
+// Kernel launchers (defined in mm_step.cu); overlap: launched overlapped with the
+// previous kernel of the stream (direct launches only).
+template <typename T>
 cudaError_t launch_substep(const StepArgs<T>& a, int grid, int block, size_t smem, bool tma,
-                           cudaStream_t s);
+                           cudaStream_t s, bool overlap);
 size_t step_smem_per_warp(int S, int chunk_elems, int nth, int tsz);
-template <typename T, int V>
-cudaError_t substep_prepare(int block, size_t smem, bool tma, int* blocks_per_sm);
+template <typename T>
+cudaError_t substep_prepare(int ns, int block, size_t smem, bool tma, int* blocks_per_sm);
 
 // Batched-ensemble launchers (mm_batch.cu): every instance's arguments in a
 // device table, tiles in a device table, per-tile float64 sums of psi.

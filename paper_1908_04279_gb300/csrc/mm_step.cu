@@ -37,16 +37,29 @@ size_t step_smem_per_warp(int S, int chunk_elems, int nth, int tsz) {
   return warp_smem_layout(S, chunk_elems, nth, tsz).total;
 }
 
-template <typename T, int V, bool TMA, bool MASSCORR>
-__global__ void __launch_bounds__(128, MM_STEP_MIN_BLOCKS) k_substep(const StepArgs<T> a) {
+// VW: rows eight nodes to a lane whatever ns is, moved in vectors of VW values
+// (rows_packed: float64, and float32 rows of no multiple of 8 nodes); 0: float32
+// rows of a multiple of 8 (rows_chunk). Without TMA (a chunk or a cell is no
+// multiple of 16 bytes; packed only) the warp copies each chunk to its one stage
+// itself. float64 takes 3 blocks per SM: its 168 registers hold both stages of
+// eight nodes, and 12 warps keep the float64 pipe busy.
+template <typename T>
+constexpr int step_min_blocks() {
+  return sizeof(T) == 8 ? 3 : MM_STEP_MIN_BLOCKS;
+}
+
+template <typename T, int VW, bool TMA>
+__global__ void __launch_bounds__(128, step_min_blocks<T>()) k_substep(const StepArgs<T> a) {
+  constexpr bool MASSCORR = sizeof(T) == 4, PACKED = VW > 0;
+  // rows of whole 16-byte vectors are stored straight to global memory
+  constexpr bool direct = VW == 0 || VW * sizeof(T) == 16;
   griddep_wait();  // launched overlapped outside graphs (recording, replays)
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int nth = a.nth, ns = a.ns, seg = a.seg;
   const int S = a.stages, RC = a.chunk_rows, CH = a.chunks_per_cell;
   const int chunk_elems = RC * ns;
   const uint32_t chunk_bytes = (uint32_t)(chunk_elems * sizeof(T));
-  // the ring exists only with bulk copies (the host sizes shared memory alike)
-  const WarpSmem L = warp_smem_layout(S, TMA ? chunk_elems : 0, nth, (int)sizeof(T));
+  const WarpSmem L = warp_smem_layout(S, chunk_elems, nth, (int)sizeof(T));
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   unsigned char* wbase = smem_raw + (size_t)wib * L.total;
   uint64_t* bars = reinterpret_cast<uint64_t*>(wbase + L.bars);
@@ -67,7 +80,7 @@ __global__ void __launch_bounds__(128, MM_STEP_MIN_BLOCKS) k_substep(const StepA
   const int my_cells = gw < nc ? (nc - 1 - gw) / W + 1 : 0;
   const int nchunks = my_cells * CH;
 
-  const LaneGeom lg = lane_geom(lane, seg, ns, V);
+  const LaneGeom lg = PACKED ? packed_lanes(lane, ns) : lane_geom(lane, seg, ns, 8);
 
   const DevParams* P = a.prm;
   const StepScalars<T> sc = step_scalars<T, MASSCORR>(P, a, lane);
@@ -158,8 +171,11 @@ __global__ void __launch_bounds__(128, MM_STEP_MIN_BLOCKS) k_substep(const StepA
 
     // ---- motor rows of this chunk
     const size_t chunk_off = ((size_t)cell * nth + (size_t)part * RC) * ns;
-    const T* src_rows = TMA ? stages + (size_t)s * chunk_elems : a.mb_in + chunk_off;
-    if (TMA) {
+    T* stage = stages + (size_t)s * chunk_elems;
+    if (!TMA) {
+      for (int e = lane; e < chunk_elems; e += 32) stage[e] = a.mb_in[chunk_off + e];
+      __syncwarp();
+    } else {
       const bool ok = __all_sync(0xffffffffu, wait_never ? mbar_wait(never, 0u, wait_limit)
                                                          : mbar_wait(&bars[s], par, wait_limit));
       if (!ok) {
@@ -172,7 +188,24 @@ __global__ void __launch_bounds__(128, MM_STEP_MIN_BLOCKS) k_substep(const StepA
         break;
       }
     }
-    rows_chunk<T, V>(src_rows, a.mb_out + chunk_off, RC, ns, seg, lg, rk, ds, s_nb + part * RC);
+    if constexpr (PACKED) {
+      T* out = a.mb_out + chunk_off;
+      rows_packed<T, VW>(stage, out, RC, ns, lg, rk, ds, s_nb + part * RC);
+      if constexpr (!direct) {  // the chunk as it lies, coalesced
+        __syncwarp();
+        if (TMA) {
+          constexpr int kv = 16 / sizeof(T);
+          for (int e = lane; e < chunk_elems / kv; e += 32)
+            reinterpret_cast<float4*>(out)[e] = reinterpret_cast<const float4*>(stage)[e];
+          // the rows written into the stage, before the next bulk copy into it
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        } else {
+          for (int e = lane; e < chunk_elems; e += 32) out[e] = stage[e];
+        }
+      }
+    } else {
+      rows_chunk<T, 8>(stage, a.mb_out + chunk_off, RC, ns, seg, lg, rk, ds, s_nb + part * RC);
+    }
     __syncwarp();
     // the stage is consumed: refill it with the chunk S ahead
     if (TMA && lane == 0 && issued < nchunks) issue_next();
@@ -280,68 +313,39 @@ __global__ void __launch_bounds__(128, MM_STEP_MIN_BLOCKS) k_substep(const StepA
   }
 }
 
-template <typename T, int V>
-cudaError_t launch_substep_impl(const StepArgs<T>& a, int grid, int block, size_t smem, bool tma,
-                                cudaStream_t s, bool overlap) {
-  void (*k)(StepArgs<T>) = tma ? (a.mass_correct ? k_substep<T, V, true, true>
-                                                 : k_substep<T, V, true, false>)
-                               : (a.mass_correct ? k_substep<T, V, false, true>
-                                                 : k_substep<T, V, false, false>);
+// The instance of the kernel for rows of ns nodes.
+template <typename T>
+auto step_kernel(int ns, bool tma) -> void (*)(StepArgs<T>) {
+  if constexpr (sizeof(T) == 4) {
+    if (ns % 8 == 0) return k_substep<T, 0, true>;
+    if (ns % 4 == 0) return k_substep<T, 4, true>;
+  }
+  if (ns % 2 == 0) return tma ? k_substep<T, 2, true> : k_substep<T, 2, false>;
+  return tma ? k_substep<T, 1, true> : k_substep<T, 1, false>;
+}
+
+template <typename T>
+cudaError_t launch_substep(const StepArgs<T>& a, int grid, int block, size_t smem, bool tma,
+                           cudaStream_t s, bool overlap) {
+  void (*k)(StepArgs<T>) = step_kernel<T>(a.ns, tma);
   if (overlap) return launch_overlapped(k, grid, block, smem, s, a);
   k<<<grid, block, smem, s>>>(a);
   return cudaGetLastError();
 }
-template <typename T, int V>
-cudaError_t launch_substep(const StepArgs<T>& a, int grid, int block, size_t smem, bool tma,
-                           cudaStream_t s) {
-  return launch_substep_impl<T, V>(a, grid, block, smem, tma, s, false);
-}
-// The same launched overlapped with the previous kernel of the stream (direct
-// launches: the recording's last segment, the replays of the reverse sweep).
-template <typename T, int V>
-cudaError_t launch_substep_overlapped(const StepArgs<T>& a, int grid, int block, size_t smem,
-                                      bool tma, cudaStream_t s) {
-  return launch_substep_impl<T, V>(a, grid, block, smem, tma, s, true);
+
+template <typename T>
+cudaError_t substep_prepare(int ns, int block, size_t smem, bool tma, int* blocks_per_sm) {
+  void (*k)(StepArgs<T>) = step_kernel<T>(ns, tma);
+  const cudaError_t e = mm::raise_smem_limit(k, smem);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, block, smem);
 }
 
-template <typename T, int V>
-cudaError_t substep_prepare(int block, size_t smem, bool tma, int* blocks_per_sm) {
-  const void* fns[4] = {(const void*)k_substep<T, V, true, true>,
-                        (const void*)k_substep<T, V, true, false>,
-                        (const void*)k_substep<T, V, false, true>,
-                        (const void*)k_substep<T, V, false, false>};
-  for (const void* f : fns) {
-    cudaError_t e = mm::raise_smem_limit(f, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      blocks_per_sm, tma ? k_substep<T, V, true, true> : k_substep<T, V, false, true>, block, smem);
-}
-
-template cudaError_t launch_substep<float, 8>(const StepArgs<float>&, int, int, size_t, bool,
-                                              cudaStream_t);
-template cudaError_t launch_substep<float, 4>(const StepArgs<float>&, int, int, size_t, bool,
-                                              cudaStream_t);
-template cudaError_t launch_substep<float, 1>(const StepArgs<float>&, int, int, size_t, bool,
-                                              cudaStream_t);
-template cudaError_t launch_substep<double, 2>(const StepArgs<double>&, int, int, size_t, bool,
-                                               cudaStream_t);
-template cudaError_t launch_substep<double, 1>(const StepArgs<double>&, int, int, size_t, bool,
-                                               cudaStream_t);
-template cudaError_t launch_substep_overlapped<float, 8>(const StepArgs<float>&, int, int, size_t,
-                                                         bool, cudaStream_t);
-template cudaError_t substep_prepare<float, 8>(int, size_t, bool, int*);
-template cudaError_t launch_substep_overlapped<float, 4>(const StepArgs<float>&, int, int, size_t,
-                                                         bool, cudaStream_t);
-template cudaError_t substep_prepare<float, 4>(int, size_t, bool, int*);
-template cudaError_t launch_substep_overlapped<float, 1>(const StepArgs<float>&, int, int, size_t,
-                                                         bool, cudaStream_t);
-template cudaError_t substep_prepare<float, 1>(int, size_t, bool, int*);
-template cudaError_t launch_substep_overlapped<double, 2>(const StepArgs<double>&, int, int, size_t,
-                                                          bool, cudaStream_t);
-template cudaError_t substep_prepare<double, 2>(int, size_t, bool, int*);
-template cudaError_t launch_substep_overlapped<double, 1>(const StepArgs<double>&, int, int, size_t,
-                                                          bool, cudaStream_t);
-template cudaError_t substep_prepare<double, 1>(int, size_t, bool, int*);
+#define MM_STEP_INST(T)                                                              \
+  template cudaError_t launch_substep<T>(const StepArgs<T>&, int, int, size_t, bool, \
+                                         cudaStream_t, bool);                        \
+  template cudaError_t substep_prepare<T>(int, int, size_t, bool, int*);
+MM_STEP_INST(float)
+MM_STEP_INST(double)
 
 }  // namespace mm

@@ -78,6 +78,35 @@ __device__ __forceinline__ Lim64 superbee64(double a, double ha, double b, doubl
   return q;
 }
 
+// The float64 donor-cell flux with the upwind state picked by the sign bit of
+// the velocity (integer pipe): one product instead of two comparisons, a product
+// and an fma on the float64 pipe, the same value; a NaN velocity gives no flux, as
+// with the maximum and minimum.
+__device__ __forceinline__ double donor(double A, double pl, double pr) {
+  const int hi = __double2hiint(A);
+  const double F = A * (hi < 0 ? pr : pl);
+  const unsigned mag = (unsigned)(hi & 0x7fffffff) + (__double2loint(A) != 0);
+  return mag > 0x7ff00000u ? 0.0 : F;
+}
+
+// d / 2 on the integer pipe (a product left in a branch is hoisted out of it):
+// one subtraction in the exponent of a normal value whose half is normal; the
+// magnitude shifted, ties to even, where the half is subnormal or zero;
+// infinities and NaN as they are.
+__device__ __forceinline__ double half64(double d) {
+  const int hi = __double2hiint(d), lo = __double2loint(d);
+  const unsigned mag = (unsigned)hi & 0x7fffffffu;
+  const unsigned slo = __funnelshift_r((unsigned)lo, mag, 1);
+  const unsigned long long sub =
+      (((unsigned long long)(mag >> 1) << 32) | slo) + ((lo & 3) == 3 ? 1u : 0u);
+  const bool normal = mag - 0x00200000u < 0x7fd00000u;  // exponents 2 .. 2046
+  const bool small = mag < 0x00200000u;
+  const int h = normal ? hi - 0x00100000 : small ? (int)(sub >> 32) | (hi & (int)0x80000000) : hi;
+  return __hiloint2double(h, small ? (int)(unsigned)sub : lo);
+}
+__device__ __forceinline__ float half_t(float x) { return 0.5f * x; }
+__device__ __forceinline__ double half_t(double x) { return half64(x); }
+
 // min(|a|, |b|) carrying the sign sign(a) xor sign(b): positive where a and b
 // agree in sign, negative where they disagree (one instruction).
 __device__ __forceinline__ float min_xorsign_abs(float a, float b) {
@@ -210,6 +239,36 @@ __device__ __forceinline__ void walk_dflux_x2(const float2 (&M)[V / 2], float2 (
   D[0] = make_float2(fl - F[0].x, F[0].x - F[0].y);
 #pragma unroll
   for (int k = 1; k < H; ++k) D[k] = make_float2(F[k - 1].y - F[k].x, F[k].x - F[k].y);
+}
+
+// walk_dflux in float64 for packed rows of V nodes per lane (nv of them in the
+// row's last lane): the difference across the right edge comes from the next
+// lane instead of being formed twice, and the halves are taken on the exponent,
+// so that a node costs three float64 operations (difference, flux, flux
+// difference), the limiter running on the integer pipe.
+template <int V, bool RAG>
+__device__ __forceinline__ void walk64(const double (&M)[V], double (&D)[V], bool first, bool last,
+                                       int nv) {
+  double ml = __shfl_up_sync(0xffffffffu, M[V - 1], 1);
+  if (first) ml = 0.0;
+  double d[V + 1];
+  d[0] = M[0] - ml;
+#pragma unroll
+  for (int v = 1; v < V; ++v) d[v] = M[v] - M[v - 1];
+  d[V] = __shfl_down_sync(0xffffffffu, d[0], 1);  // (not used by the row's last node)
+  double F[V], h = half64(d[0]);
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    const double hn = half64(d[v + 1]);
+    const bool end = last && (RAG ? v == nv - 1 : v == V - 1);
+    F[v] = superbee64(d[v], h, d[v + 1], hn, end, M[v]).F;
+    h = hn;
+  }
+  double fl = __shfl_up_sync(0xffffffffu, F[V - 1], 1);
+  if (first) fl = 0.0;
+  D[0] = fl - F[0];
+#pragma unroll
+  for (int v = 1; v < V; ++v) D[v] = F[v - 1] - F[v];
 }
 
 // Sum of x over the nl lanes of a packed row (lanes sl = 0 .. nl - 1 of the

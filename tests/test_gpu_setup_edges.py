@@ -61,3 +61,29 @@ def test_set_up_beyond_float32_sums(mmod, ns):
     for k in ("mb", "c"):
         assert rel_l2(got[k], getattr(st, k)) <= 1e-5, k
     assert np.abs(got["mf"] - st.mf).max() <= 1e-6
+
+
+@pytest.mark.parametrize("dims", [(7, 6, 12, 16), (6, 5, 10, 13)])
+def test_subnormal_motor_densities(mmod, dims):
+    """The float64 limiter halves differences on their bit patterns: motor
+    densities from zero through the subnormal range against the oracle."""
+    from oracle import oracle as O
+    g = Grid(*dims)
+    r = Rates(k_on=0.0)
+    rng = SplitMix64(9)
+    x = rng.uniforms(2 * g.micro_cells).reshape(2, g.ny, g.nx, g.ntheta, g.ns)
+    mb = np.where(x[1] < 0.2, 0.0, 8e-308 * x[0] ** 3)
+    psi = psi_isotropic_perturbed(g, 4)
+    u = np.zeros((2, g.ny, g.nx))
+    st = O.make_state(g, psi, mb)
+    dt = O.dt(g, r, st, u)
+    with mmod.Simulation(g, r, "fp64") as sim:
+        sim.set_state(psi, mb)
+        sim.set_velocity(u)
+        sim.set_dt(dt)
+        sim.step(3)
+        got = sim.get_state()
+    O.run(g, r, st, u, dt, 3)
+    scale = 1e308  # out of the subnormal range for the norms
+    assert rel_l2(got["mb"] * scale, st.mb * scale) <= 1e-12
+    assert rel_l2(got["psi"], st.psi) <= 1e-12
