@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(256, 2) k_motor_local(const LocalArgs<T> a) {
   }
   __syncthreads();
 
-  const LaneGeom lg = lane_geom(lane, seg, ns, V);
+  const LaneGeom lg = sizeof(T) == 8 ? packed_lanes(lane, ns) : lane_geom(lane, seg, ns, V);
   const int r0 = w * a.rows_per_warp;
   const int cnt = max(0, min(a.rows_per_warp, nth - r0));
   const T ds = (T)a.ds, dth = (T)a.dth;
@@ -208,9 +208,22 @@ __global__ void __launch_bounds__(256, 2) k_motor_local(const LocalArgs<T> a) {
       const bool last = step == n - 1;
       T* nbs = nbcol + (step & 1) * nth;
       T* dst = last ? gdst : rows;
-      if (cnt > 0)
+      if constexpr (sizeof(T) == 8) {
+        // eight nodes to a lane (the float64 pipe bounds this kernel too); rows of
+        // odd length are updated in place and copied out at the end
+        if (cnt > 0) {
+          rows_packed<T, V>(rows + (size_t)r0 * ns, dst + (size_t)r0 * ns, cnt, ns, lg, rk, ds,
+                            nbs + r0);
+          if (V == 1 && last) {
+            __syncwarp();
+            for (int e = lane; e < cnt * ns; e += 32)
+              dst[(size_t)r0 * ns + e] = rows[(size_t)r0 * ns + e];
+          }
+        }
+      } else if (cnt > 0) {
         rows_chunk<T, V>(rows + (size_t)r0 * ns, dst + (size_t)r0 * ns, cnt, ns, seg, lg, rk, ds,
                          nbs + r0);
+      }
       __syncthreads();
       // Eq. 5 with the frozen psi: every warp forms the same sum
       T acc = T(0);
@@ -410,7 +423,7 @@ struct LocalPlan {
 template <typename T, int V>
 mm_status local_plan(mm_handle* h, LocalPlan* p) {
   const int nth = h->g.ntheta, ns = h->g.ns;
-  const int rpp = 32 / h->seg;
+  const int rpp = sizeof(T) == 8 ? 32 / ((ns + 7) / 8) : 32 / h->seg;
   const int groups = (nth + rpp - 1) / rpp;
   const int passes = (groups + 7) / 8;
   const int nw = (groups + passes - 1) / passes;
