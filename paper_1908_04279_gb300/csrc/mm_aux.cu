@@ -28,16 +28,51 @@ __global__ void k_copy_multi(const CopySegs c) {
   }
 }
 
+// float32 to float64 on the integer and float32 pipes (exact; the conversion
+// instruction runs on the narrow float64 pipe, which held the exports at 4.7 TB/s
+// of the 6.8 a copy reaches): the exponent rebiased, subnormal values brought
+// into the normal range first.
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u0 = __float_as_uint(x), mag = u0 & 0x7fffffffu;
+  const bool sub = mag < 0x00800000u;
+  const unsigned u = __float_as_uint(x * (sub ? 16777216.0f : 1.0f));
+  const unsigned bias = sub ? 0x36800000u : mag < 0x7f800000u ? 0x38000000u : 0x70000000u;
+  const unsigned hi = mag == 0u ? 0u : ((u & 0x7fffffffu) >> 3) + bias;
+  return __hiloint2double((int)(hi | (u0 & 0x80000000u)), (int)(u << 29));
+}
+template <typename TO, typename TI>
+__device__ __forceinline__ TO converted(TI x) {
+  if constexpr (sizeof(TO) == 8 && sizeof(TI) == 4)
+    return widen(x);
+  else
+    return (TO)x;
+}
+
+// out = in (times *scale); without a scale in pairs, 8 bytes on one side and 16 on
+// the other, where the addresses allow it (512^2 x 64^2 exports 0.69 -> 0.52 ms
+// per 268 M values).
 template <typename TO, typename TI>
 __global__ void k_convert(TO* out, const TI* in, size_t n, const double* scale) {
-  const double sc = scale ? *scale : 1.0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x) {
-    if (scale)
-      out[i] = (TO)((double)in[i] * sc);
-    else
-      out[i] = (TO)in[i];
+  const size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  const size_t stride = (size_t)gridDim.x * blockDim.x;
+  if (scale) {
+    const double sc = *scale;
+    for (size_t i = tid; i < n; i += stride) out[i] = (TO)((double)in[i] * sc);
+    return;
   }
+  struct alignas(2 * sizeof(TI)) In {
+    TI a, b;
+  };
+  struct alignas(2 * sizeof(TO)) Out {
+    TO a, b;
+  };
+  const bool vec = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
+  const size_t nv = vec ? n / 2 : 0;
+  for (size_t i = tid; i < nv; i += stride) {
+    const In v = reinterpret_cast<const In*>(in)[i];
+    reinterpret_cast<Out*>(out)[i] = Out{converted<TO, TI>(v.a), converted<TO, TI>(v.b)};
+  }
+  for (size_t i = 2 * nv + tid; i < n; i += stride) out[i] = converted<TO, TI>(in[i]);
 }
 
 __device__ __forceinline__ void atomic_max_nonneg(double* addr, double v) {
@@ -669,7 +704,7 @@ cudaError_t launch_copy_multi(const CopySegs& c, cudaStream_t s) {
 template <typename TO, typename TI>
 cudaError_t launch_convert(TO* out, const TI* in, size_t n, const double* scale, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  k_convert<TO, TI><<<grid_for((long long)n, 256), 256, 0, s>>>(out, in, n, scale);
+  k_convert<TO, TI><<<grid_for((long long)((n + 1) / 2), 256), 256, 0, s>>>(out, in, n, scale);
   return cudaGetLastError();
 }
 
