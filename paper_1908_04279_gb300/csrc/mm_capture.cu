@@ -20,15 +20,15 @@
 // within a line. One substep is three launches:
 //   k_rc_psi    warp per cell: psi by Eq. 1 (velocities from n_b and u), the
 //               float32 form's mass sums;
-//   k_rc_motor  warp per anchor r0 (Alg. 2's loop over r0): the anchor's
-//               configurations in chunks of whole lines, positions across the
-//               lanes (p = 32 v + lane, coalesced loads), the walking stencil
-//               by shuffles with per-position line-start / line-end flags; the
-//               line sums of Mb ds (kept per (r0, line) for n_b), the coarse
-//               density C(r0) with psi^{n+1} of each line's filament cell, the
-//               scale-down and Mf(r0) -- all local to the warp, no atomics;
-//   k_rc_nb     thread per (x, theta): n_b = the line sums of its lines over
-//               the anchors, in template order (deterministic).
+//   k_rc_motor  block per anchor r0 (Alg. 2's loop over r0): the anchor's
+//               configurations in chunks of whole lines, dealt to the block's four
+//               warps, the walking stencil by shuffles with per-position line-start
+//               / line-end flags; the line sums of Mb ds (kept per (r0, line) for
+//               n_b), the coarse density C(r0) with psi^{n+1} of each line's
+//               filament cell, the scale-down and Mf(r0) -- all local to the
+//               block, no atomics;
+//   k_rc_nb     lane per (x, theta): n_b = the line sums of its lines over the
+//               anchors, in template order (deterministic).
 #include <algorithm>
 #include <vector>
 
@@ -44,7 +44,7 @@ struct RcArgs {
   int nx, ny, nth, ns, nconf, nlines, nchunks;
   long long ncells;
   T* mb;                       // [cells][nconf] motor density, anchor-major
-  T* ls;                       // [cells][nlines] sum of Mb ds of every line
+  T* ls;                       // [nlines][cells] sum of Mb ds of every line
   const int4* line;            // [nlines] {dx, dy, k, len}: filament cell = r0 - (dx, dy)
   const int* loff;             // [nlines] first entry of the line in mb[r0][]
   const int4* chunk;           // [nchunks] {first entry, entries, first line, lines}
@@ -110,7 +110,7 @@ __device__ __forceinline__ void rc_walk(const T (&M)[kRcV], unsigned mask, T (&D
     const T left = ((mask >> v) & 1u) ? T(0) : (v > 0 ? M[v - 1] : ml);
     const T right = v + 1 < kRcV ? M[v + 1] : mr;
     const T a = M[v] - left, b = right - M[v];
-    const T ha = T(0.5) * a, hb = T(0.5) * b;
+    const T ha = half_t(a), hb = half_t(b);
     const bool last = ((mask >> (8 + v)) & 1u) != 0;
     if constexpr (sizeof(T) == 4) {
       float r = max3_t(min_xorsign_abs(a, hb), min_xorsign_abs(ha, b), 0.0f);
@@ -128,27 +128,33 @@ __device__ __forceinline__ void rc_walk(const T (&M)[kRcV], unsigned mask, T (&D
   }
 }
 
-// Alg. 2 per anchor r0 (warp per anchor, grid-strided): the RK2 of Eq. 4 on
+// Alg. 2 per anchor r0 (block per anchor, grid-strided): the RK2 of Eq. 4 on
 // every configuration of B_rc(r0) (Mf(r0) frozen over both stages, binding
 // k_on Mf(r0) w), the line sums of Mb ds, C(r0) = sum over lines of
 // psi(filament cell, k) (line sum) dtheta with psi = psi_c (psi^{n+1}), the
-// scale-down where C exceeds M (the warp rescales the entries and line sums it
+// scale-down where C exceeds M (the block rescales the entries and line sums it
 // wrote) and Mf = M - C. init = 1: dt = 0 (the set-up: C, the scale-down, Mf
 // and the line sums of a loaded state).
-// The warp's (anchor, chunk) items stream through a ring of S shared-memory
+// A block rather than a warp takes an anchor so that the last wave is short: at
+// 64^2 x 32^2 the 4096 anchors are 4.5 to a block, six blocks to an SM, but were one
+// to a warp, 27 of an SM's 32 warps each 62 chunks deep. Six blocks per SM leave 80
+// registers (eight leave 64). Bound by instruction issue and the latency of the
+// tables and of psi: 222 -> 180 us at 64^2 x 32^2, r_c = 1.5 cells. Factors in place
+// of the flags' selects (packed products) and table entries loaded a chunk ahead
+// cost more in registers than they saved.
+// A warp's (anchor, chunk) items stream through a ring of S shared-memory
 // stages filled by asynchronous copies S items ahead (coalesced 4/8-byte
 // copies: a chunk may start anywhere); lane l computes the chunk's entries
 // 8 l .. 8 l + 7, and the new values go back through the stage so that the
 // global stores are coalesced too.
 #ifndef MM_RC_MIN_BLOCKS
-#define MM_RC_MIN_BLOCKS 8
+#define MM_RC_MIN_BLOCKS 6
 #endif
 template <typename T, int S>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? MM_RC_MIN_BLOCKS : 1)
     k_rc_motor(const RcArgs<T> x, const T* psi_c, int init) {
   extern __shared__ __align__(16) unsigned char rc_ring_raw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const long long gw = blockIdx.x * 4LL + wib, W = (long long)gridDim.x * 4;
   T* ring = reinterpret_cast<T*>(rc_ring_raw) + (size_t)wib * S * kRcChunk;
   const double dt64 = init ? 0.0 : x.prm->dt;
   const T dt = (T)dt64, hdt = (T)(0.5 * dt64);
@@ -157,154 +163,168 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? MM_RC_MIN_BLOCKS : 1)
   const T hk = hdt * kon, fk = dt * kon;
   const T ds = (T)x.ds, dth = (T)x.dth;
   const int nx = x.nx, ny = x.ny, nth = x.nth, nch = x.nchunks;
-  const long long na = gw < x.ncells ? (x.ncells - gw + W - 1) / W : 0;
-  const long long nitems = na * nch;
-  auto issue = [&](long long q) {
-    if (q < nitems) {
-      const long long a = gw + (q / nch) * W;
-      const int4 cd = x.chunk[(int)(q % nch)];
-      T* st = ring + (size_t)(q % S) * kRcChunk;
-      const T* src = x.mb + (size_t)a * x.nconf + cd.x;
+  const long long G = gridDim.x;
+  // this warp's items: chunks wib, wib + 4, ... of the block's anchors in turn;
+  // the cursor of the next one to copy runs S items ahead
+  long long ia = wib < nch ? blockIdx.x : x.ncells;
+  int ich = wib, istage = 0;
+  auto issue = [&]() {
+    if (ia < x.ncells) {
+      const int4 cd = x.chunk[ich];
+      T* st = ring + (size_t)istage * kRcChunk;
+      const T* src = x.mb + (size_t)ia * x.nconf + cd.x;
 #pragma unroll
       for (int v = 0; v < kRcV; ++v) {
         const int p = 32 * v + lane;
         if (p < cd.y) cp_async_t(st + p, src + p);
       }
+      if ((ich += 4) >= nch) {
+        ich = wib;
+        ia += G;
+      }
+      if (++istage == S) istage = 0;
     }
     cp_async_commit();  // one group per item, empty past the end
   };
 #pragma unroll
-  for (int q = 0; q < S; ++q) issue(q);
-  T cacc = T(0), mfa = T(0);
-  for (long long q = 0; q < nitems; ++q) {
-    const int ch = (int)(q % nch);
-    const long long a = gw + (q / nch) * W;
-    if (ch == 0) {
-      mfa = x.mf[a];
-      cacc = T(0);
-    }
-    const int4 cd = x.chunk[ch];
-    const unsigned mask = x.cmask[ch * 32 + lane];
-    T wv[kRcV];
-    lds8(x.cw + (size_t)ch * kRcChunk + 8 * lane, wv);  // 16-byte vector loads (global)
-    cp_async_wait<S - 1>();
-    __syncwarp();
-    T* st = ring + (size_t)(q % S) * kRcChunk;
-    T M[kRcV], D[kRcV], Ms[kRcV];
-    lds8(st + 8 * lane, M);
-#pragma unroll
-    for (int v = 0; v < kRcV; ++v)
-      if (!((mask >> (16 + v)) & 1u)) M[v] = T(0);
-    rc_walk<T>(M, mask, D);
-    if constexpr (sizeof(T) == 4) {
-      // the element-wise stage updates as packed two-value float32 operations
-      const float2 c1_ = make_float2(c1, c1), c2_ = make_float2(c2, c2);
-      const float2 e1_ = make_float2(e1, e1), e2_ = make_float2(e2, e2);
-      const float2 hm = make_float2(hk * mfa, hk * mfa), fm = make_float2(fk * mfa, fk * mfa);
-      float2 bh[kRcV / 2], bf[kRcV / 2];
-#pragma unroll
-      for (int h = 0; h < kRcV / 2; ++h) {
-        const float2 w2 = make_float2(wv[2 * h], wv[2 * h + 1]);
-        bh[h] = __fmul2_rn(hm, w2);
-        bf[h] = __fmul2_rn(fm, w2);
-        const float2 r = __ffma2_rn(c1_, make_float2(D[2 * h], D[2 * h + 1]),
-                                    __ffma2_rn(c2_, make_float2(M[2 * h], M[2 * h + 1]), bh[h]));
-        Ms[2 * h] = r.x;
-        Ms[2 * h + 1] = r.y;
-      }
-      rc_walk<T>(Ms, mask, D);
-#pragma unroll
-      for (int h = 0; h < kRcV / 2; ++h) {
-        const float2 r = __ffma2_rn(
-            e1_, make_float2(D[2 * h], D[2 * h + 1]),
-            __ffma2_rn(e2_, make_float2(Ms[2 * h], Ms[2 * h + 1]),
-                       __fadd2_rn(make_float2(M[2 * h], M[2 * h + 1]), bf[h])));
-        M[2 * h] = r.x;
-        M[2 * h + 1] = r.y;
-      }
-    } else {
-#pragma unroll
-      for (int v = 0; v < kRcV; ++v) Ms[v] = fma_t(c1, D[v], fma_t(c2, M[v], hk * (mfa * wv[v])));
-      rc_walk<T>(Ms, mask, D);
+  for (int q = 0; q < S; ++q) issue();
+  __shared__ T s_c[2][4];
+  int stage = 0, par = 0;
+  for (long long a = blockIdx.x; a < x.ncells; a += G, par ^= 1) {
+    const T mfa = x.mf[a];
+    const int ay = (int)a / nx, ax = (int)a - ay * nx;
+    T* La = x.ls + a;  // (line l at l ncells)
+    T cacc = T(0);
+    for (int ch = wib; ch < nch; ch += 4) {
+      const int4 cd = x.chunk[ch];
+      const unsigned mask = x.cmask[ch * 32 + lane];
+      T wv[kRcV];
+      lds8(x.cw + (size_t)ch * kRcChunk + 8 * lane, wv);  // 16-byte vector loads (global)
+      cp_async_wait<S - 1>();
+      __syncwarp();
+      T* st = ring + (size_t)stage * kRcChunk;
+      if (++stage == S) stage = 0;
+      T M[kRcV], D[kRcV], Ms[kRcV];
+      lds8(st + 8 * lane, M);
 #pragma unroll
       for (int v = 0; v < kRcV; ++v)
-        M[v] = fma_t(e1, D[v], fma_t(e2, Ms[v], M[v] + fk * (mfa * wv[v])));
-    }
-    __syncwarp();
-    sts8(st + 8 * lane, M);
-    __syncwarp();
-    T* Ma = x.mb + (size_t)a * x.nconf + cd.x;
-    if (!init) {
+        if (!((mask >> (16 + v)) & 1u)) M[v] = T(0);
+      rc_walk<T>(M, mask, D);
+      if constexpr (sizeof(T) == 4) {
+        // the element-wise stage updates as packed two-value float32 operations
+        const float2 c1_ = make_float2(c1, c1), c2_ = make_float2(c2, c2);
+        const float2 e1_ = make_float2(e1, e1), e2_ = make_float2(e2, e2);
+        const float2 hm = make_float2(hk * mfa, hk * mfa), fm = make_float2(fk * mfa, fk * mfa);
+        float2 bh[kRcV / 2], bf[kRcV / 2];
 #pragma unroll
-      for (int v = 0; v < kRcV; ++v) {
-        const int p = 32 * v + lane;
-        if (p < cd.y) Ma[p] = st[p];
-      }
-    }
-    // each lane's running sums of the new values, restarted at every line
-    // start, into the stage (entry 8 lane + v): a line's sum is then its last
-    // entry's running sum plus the lane-end sums of the lanes it leaves
-    {
-      T r = T(0);
+        for (int h = 0; h < kRcV / 2; ++h) {
+          const float2 w2 = make_float2(wv[2 * h], wv[2 * h + 1]);
+          bh[h] = __fmul2_rn(hm, w2);
+          bf[h] = __fmul2_rn(fm, w2);
+          const float2 r = __ffma2_rn(c1_, make_float2(D[2 * h], D[2 * h + 1]),
+                                      __ffma2_rn(c2_, make_float2(M[2 * h], M[2 * h + 1]), bh[h]));
+          Ms[2 * h] = r.x;
+          Ms[2 * h + 1] = r.y;
+        }
+        rc_walk<T>(Ms, mask, D);
 #pragma unroll
-      for (int v = 0; v < kRcV; ++v) {
-        r = ((mask >> v) & 1u) ? M[v] : r + M[v];
-        M[v] = r;
+        for (int h = 0; h < kRcV / 2; ++h) {
+          const float2 r = __ffma2_rn(
+              e1_, make_float2(D[2 * h], D[2 * h + 1]),
+              __ffma2_rn(e2_, make_float2(Ms[2 * h], Ms[2 * h + 1]),
+                         __fadd2_rn(make_float2(M[2 * h], M[2 * h + 1]), bf[h])));
+          M[2 * h] = r.x;
+          M[2 * h + 1] = r.y;
+        }
+      } else {
+#pragma unroll
+        for (int v = 0; v < kRcV; ++v) Ms[v] = fma_t(c1, D[v], fma_t(c2, M[v], hk * (mfa * wv[v])));
+        rc_walk<T>(Ms, mask, D);
+#pragma unroll
+        for (int v = 0; v < kRcV; ++v)
+          M[v] = fma_t(e1, D[v], fma_t(e2, Ms[v], M[v] + fk * (mfa * wv[v])));
       }
-      __syncwarp();  // every lane has read the stage for the stores above
+      __syncwarp();
       sts8(st + 8 * lane, M);
       __syncwarp();
-    }
-    // lanes over the chunk's lines: the line sum of Mb ds, and the line's
-    // part of the coarse density
-    const int ay = (int)(a / nx), ax = (int)(a - (long long)ay * nx);
-    T* La = x.ls + (size_t)a * x.nlines;
-    for (int li = lane; li < cd.w; li += 32) {
-      const int l = cd.z + li;
-      const int4 ln = x.line[l];
-      int fx = ax - ln.x, fy = ay - ln.y;
-      fx += fx < 0 ? nx : (fx >= nx ? -nx : 0);
-      fy += fy < 0 ? ny : (fy >= ny ? -ny : 0);
-      const T pf = psi_c[((size_t)fy * nx + fx) * nth + ln.z];
-      const int b0 = x.loff[l] - cd.x, e = b0 + ln.w - 1;
-      T s0 = T(0);
-      for (int q2 = (b0 >> 3) * 8 + 7; q2 < e; q2 += 8) s0 += st[q2];
-      const T s = (s0 + st[e]) * ds;
-      La[l] = s;
-      cacc = fma_t(pf * s, dth, cacc);
-    }
-    __syncwarp();
-    issue(q + S);
-    if (ch == nch - 1) {
-      const T C = warp_sum_t(cacc);
-      const T Mt = x.mtot[a];
-      T Cc = C;
-      if (Mt < C) {  // Alg. 2 scale-down at r0 (rare): the warp rescales what it wrote
-        const T f = Mt / C;
-        T* Mall = x.mb + (size_t)a * x.nconf;
-        for (int e = lane; e < x.nconf; e += 32) Mall[e] = __ldcg(Mall + e) * f;
-        for (int l = lane; l < x.nlines; l += 32) La[l] = __ldcg(La + l) * f;
-        Cc = Mt;
+      T* Ma = x.mb + (size_t)a * x.nconf + cd.x;
+      if (!init) {
+#pragma unroll
+        for (int v = 0; v < kRcV; ++v) {
+          const int p = 32 * v + lane;
+          if (p < cd.y) Ma[p] = st[p];
+        }
       }
-      if (lane == 0) {
-        x.c[a] = Cc;
-        x.mf[a] = Mt - Cc;
+      // each lane's running sums of the new values, restarted at every line
+      // start, into the stage (entry 8 lane + v): a line's sum is then its last
+      // entry's running sum plus the lane-end sums of the lanes it leaves
+      {
+        T r = T(0);
+#pragma unroll
+        for (int v = 0; v < kRcV; ++v) {
+          r = ((mask >> v) & 1u) ? M[v] : r + M[v];
+          M[v] = r;
+        }
+        __syncwarp();  // every lane has read the stage for the stores above
+        sts8(st + 8 * lane, M);
+        __syncwarp();
       }
+      // lanes over the chunk's lines: the line sum of Mb ds, and the line's
+      // part of the coarse density
+      for (int li = lane; li < cd.w; li += 32) {
+        const int l = cd.z + li;
+        const int4 ln = x.line[l];
+        int fx = ax - ln.x, fy = ay - ln.y;
+        fx += fx < 0 ? nx : (fx >= nx ? -nx : 0);
+        fy += fy < 0 ? ny : (fy >= ny ? -ny : 0);
+        const T pf = psi_c[((size_t)fy * nx + fx) * nth + ln.z];
+        const int b0 = x.loff[l] - cd.x, e = b0 + ln.w - 1;
+        T s0 = T(0);
+        for (int q2 = (b0 >> 3) * 8 + 7; q2 < e; q2 += 8) s0 += st[q2];
+        const T s = (s0 + st[e]) * ds;
+        La[(size_t)l * x.ncells] = s;
+        cacc = fma_t(pf * s, dth, cacc);
+      }
+      __syncwarp();
+      issue();
+    }
+    // the anchor's coarse density over the block's warps, in order
+    cacc = warp_sum_t(cacc);
+    if (lane == 0) s_c[par][wib] = cacc;
+    __syncthreads();
+    const T C = ((s_c[par][0] + s_c[par][1]) + s_c[par][2]) + s_c[par][3];
+    const T Mt = x.mtot[a];
+    if (Mt < C) {  // Alg. 2 scale-down at r0 (rare): the block rescales what it wrote
+      const T f = Mt / C;
+      T* Mall = x.mb + (size_t)a * x.nconf;
+      for (int e = threadIdx.x; e < x.nconf; e += blockDim.x) Mall[e] = __ldcg(Mall + e) * f;
+      for (int l = threadIdx.x; l < x.nlines; l += blockDim.x)
+        La[(size_t)l * x.ncells] = __ldcg(La + (size_t)l * x.ncells) * f;
+    }
+    if (threadIdx.x == 0) {
+      const T Cc = Mt < C ? Mt : C;
+      x.c[a] = Cc;
+      x.mf[a] = Mt - Cc;
     }
   }
   cp_async_wait<0>();
 }
 
 // n_b(x, k) = sum over the lines of orientation k, in template order, of the
-// line sum at the anchor r0 = x + (dx, dy) (thread per (x, k)).
+// line sum at the anchor r0 = x + (dx, dy). A warp takes one orientation of 32
+// consecutive cells, so that the sums of a line, kept cell after cell, are read
+// coalesced (kept line after line, every read of a thread was a sector of its
+// own: 21 us at 64^2 x 32^2, 5.5 M line sums).
 template <typename T>
 __global__ void k_rc_nb(const RcArgs<T> x, T* nb) {
-  const long long n = x.ncells * x.nth;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long cell = t / x.nth;
-    const int k = (int)(t - cell * x.nth);
-    const int fy = (int)(cell / x.nx), fx = (int)(cell - (long long)fy * x.nx);
+  const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+  const int nc = (int)x.ncells, tiles = (nc + 31) / 32;
+  const long long units = (long long)tiles * x.nth;
+  for (long long u = blockIdx.x * (long long)wpb + (threadIdx.x >> 5); u < units;
+       u += (long long)gridDim.x * wpb) {
+    const int k = (int)(u % x.nth), cell = (int)(u / x.nth) * 32 + lane;
+    if (cell >= nc) continue;
+    const int fy = cell / x.nx, fx = cell - fy * x.nx;
     // four loads in flight, added in template order
     T s = T(0);
     const int l1 = x.krange[k + 1];
@@ -314,7 +334,7 @@ __global__ void k_rc_nb(const RcArgs<T> x, T* nb) {
       int ax = fx + ln.x, ay = fy + ln.y;
       ax += ax < 0 ? x.nx : (ax >= x.nx ? -x.nx : 0);
       ay += ay < 0 ? x.ny : (ay >= x.ny ? -x.ny : 0);
-      return __ldcg(x.ls + ((size_t)ay * x.nx + ax) * x.nlines + li);
+      return __ldcg(x.ls + (size_t)li * x.ncells + (size_t)ay * x.nx + ax);
     };
     for (; l + 3 < l1; l += 4) {
       const T v0 = at(l), v1 = at(l + 1), v2 = at(l + 2), v3 = at(l + 3);
@@ -324,7 +344,7 @@ __global__ void k_rc_nb(const RcArgs<T> x, T* nb) {
       s += v3;
     }
     for (; l < l1; ++l) s += at(l);
-    nb[t] = s;
+    nb[(size_t)cell * x.nth + k] = s;
   }
 }
 
@@ -814,7 +834,7 @@ mm_status mm_set_capture(mm_handle* h, double rc) {
          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
                &per_sm, mm::k_rc_motor<float, kRcStages>, 128, rc_ring_bytes<float>()));
   h->rc_motor_grid = (int)std::max<long long>(
-      1, std::min<long long>((h->ncells + 3) / 4, (long long)std::max(per_sm, 1) * h->sms));
+      1, std::min<long long>(h->ncells, (long long)std::max(per_sm, 1) * h->sms));
   h->capture = true;
   // a new layout: the motors are discarded (Mb = 0, Mf = M); psi is kept
   if (h->have_state) return run_init_capture(h);
