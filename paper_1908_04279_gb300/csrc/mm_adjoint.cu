@@ -407,19 +407,7 @@ struct MotorAcc {
 // stay scalar. The same values as the scalar form (the accumulations over a
 // lane's nodes run in two interleaved sums).
 
-// One node of the COEF walk: the Superbee value r (sigma/2 = sgn r) and the
-// branch coefficients, with the comparisons of walk_dflux<..., true>.
-__device__ __forceinline__ void coef_node(float A, float hA, float hB, float B, float& r,
-                                          float& ga, float& gb) {
-  const float t1 = fminf(A, hB), t2 = fminf(hA, B);
-  r = max3_t(t1, t2, 0.0f);
-  const bool pos = r > 0.0f, p1 = t1 > t2, x1a = A < hB, x2a = hA < B;
-  const float a1 = x1a ? 1.0f : 0.0f, b1 = x1a ? 0.0f : 0.5f;
-  const float a2 = x2a ? 0.5f : 0.0f, b2 = x2a ? 0.0f : 1.0f;
-  ga = pos ? (p1 ? a1 : a2) : 0.0f;
-  gb = pos ? (p1 ? b1 : b2) : 0.0f;
-}
-
+// The COEF walk on register pairs.
 template <int V>
 __device__ __forceinline__ void walk_coef_x2(const float2 (&M)[V / 2], float2 (&D)[V / 2],
                                              float2 (&ga)[V / 2], float2 (&gb)[V / 2], bool first,
@@ -444,8 +432,8 @@ __device__ __forceinline__ void walk_coef_x2(const float2 (&M)[V / 2], float2 (&
     if (k == H - 1 && last) sg.y = 0.0f;  // plus end: F = M, no slope
     const float2 A = __fmul2_rn(d[k], sg), hA = __fmul2_rn(hd[k], sg);
     float2 r;
-    coef_node(A.x, hA.x, fabsf(hd[k].y), fabsf(d[k].y), r.x, ga[k].x, gb[k].x);
-    coef_node(A.y, hA.y, fabsf(hb1), fabsf(b1), r.y, ga[k].y, gb[k].y);
+    branch_x2(A, hA, make_float2(fabsf(hd[k].y), fabsf(hb1)), make_float2(fabsf(d[k].y), fabsf(b1)),
+              r, ga[k], gb[k]);
     F[k] = __ffma2_rn(r, sg, M[k]);
   }
   float fl = __shfl_up_sync(0xffffffffu, F[H - 1].y, 1, seg);

@@ -115,6 +115,38 @@ __device__ __forceinline__ float min_xorsign_abs(float a, float b) {
   return r;
 }
 
+// 1 where a < b, else 0, as a value (one instruction; a NaN gives 0).
+__device__ __forceinline__ float less(float a, float b) {
+  float r;
+  asm("set.lt.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
+// Two nodes' Superbee values r (sigma/2 = sgn r) and the derivatives
+// (ga, gb) of sigma/2 = ga a + gb b on the branch the forward takes, from
+// A = sgn a, hA = A/2, hB = |b|/2 and B = |b|. On the magnitudes the branches
+// follow one another, so that three comparisons tell them apart:
+//   A < hB: (1, 0);  else hA < hB: (0, 1/2);  else hA < B: (1/2, 0);  else (0, 1),
+// and (0, 0) where r = 0. Each coefficient is a sum of the comparisons'
+// values, exact in float32: the same bits as selects along the maxima and
+// minima (compared over all orderings, ties and subnormals), with half of
+// their instructions on the half-rate pipe that minima, comparisons and
+// selects share, the rest as packed multiply-adds. Comparisons and selects
+// held that pipe busiest in the kernels that need the branch.
+__device__ __forceinline__ void branch_x2(float2 A, float2 hA, float2 hB, float2 B, float2& r,
+                                          float2& ga, float2& gb) {
+  r = make_float2(max3_t(fminf(A.x, hB.x), fminf(hA.x, B.x), 0.0f),
+                  max3_t(fminf(A.y, hB.y), fminf(hA.y, B.y), 0.0f));
+  const float2 s0 = make_float2(less(0.0f, r.x), less(0.0f, r.y));
+  const float2 s1 = make_float2(less(A.x, hB.x), less(A.y, hB.y));
+  const float2 s2 = make_float2(less(hA.x, hB.x), less(hA.y, hB.y));
+  const float2 s3 = make_float2(less(hA.x, B.x), less(hA.y, B.y));
+  const float2 m1 = make_float2(-1.0f, -1.0f), h = make_float2(0.5f, 0.5f);
+  const float2 one = make_float2(1.0f, 1.0f);
+  ga = __fmul2_rn(s0, __ffma2_rn(h, __ffma2_rn(s2, m1, s3), s1));
+  gb = __fmul2_rn(s0, __ffma2_rn(h, __ffma2_rn(s1, m1, s2), __ffma2_rn(s3, m1, one)));
+}
+
 // Walking-flux differences of the V nodes a lane holds (the d_s term of
 // Eq. 4 divided by v/ds): D_v = F_{j-1} - F_j with F_j = M_j + sigma_j/2 the
 // flux / v through the right face of node j = lane*V + v, F_{-1} = 0 (nothing
