@@ -12,7 +12,7 @@
 // upwinding, the Superbee limiter, the Alg. 2 scale-down), the float32 form's
 // mass-correction factor a constant of the map: the same readings as the
 // reverse sweep and the oracle's tangent substep. The forward part of the
-// kernel is the plain substep's device code (psi_cell, walk_dflux), so the
+// kernel is the plain substep's arithmetic (psi_point; the flux of walk_dflux), so the
 // state advances as in the plain path up to the rounding of the row loads.
 #include <algorithm>
 
@@ -34,11 +34,10 @@ struct TanArgs {
   double dkoff, dvw, dkon;
 };
 
-// Per-warp shared memory of the tangent substep: psi, n_b, dpsi, dn_b of the
-// cell and its four neighbours ([5][nth] each), the new psi and dpsi of the
+// Per-warp shared memory of the tangent substep: the new psi and dpsi of the
 // cell, and the new rows' n_b and dn_b.
 __host__ __device__ inline size_t tan_warp_smem(int nth, int tsz) {
-  return (size_t)24 * nth * tsz;
+  return (size_t)4 * nth * tsz;
 }
 
 // d of the donor-cell flux max(A, 0) pl + min(A, 0) pr on the branch taken
@@ -48,50 +47,48 @@ __device__ __forceinline__ T donor_tl(T A, T pl, T pr, T dA, T dpl, T dpr) {
   return fma_t(tmax(A, T(0)), dpl, tmin(A, T(0)) * dpr) + dA * (A > T(0) ? pl : pr);
 }
 
-// dpsi^{n+1} of the cell (lanes over theta), with no velocity perturbation:
-// the face velocities change through dn_b (the gliding speed), the fluxes
-// through them and through dpsi.
+// dpsi^{n+1} of one (cell, theta), with no velocity perturbation: the face
+// velocities change through dn_b (the gliding speed), the fluxes through them
+// and through dpsi. The face speeds are psi_point's, so that the two inlined
+// side by side compute them once.
 template <typename T>
-__device__ __forceinline__ void psi_cell_tl(const PsiConst<T>& q, const CellVel<T>& u,
-                                            const T* psi5, const T* nb5, const T* dpsi5,
-                                            const T* dnb5, int nth, int lane, T* dpsi_new) {
-  const T* cosk = q.trig;
-  const T* sink = q.trig + nth;
-  const T* cosf = q.trig + 2 * nth;
-  const T* sinf = q.trig + 3 * nth;
+__device__ __forceinline__ T psi_point_tl(const PsiConst<T>& q, const CellVel<T>& u,
+                                          const LaneTrig<T>& t, const PsiIn<T>& in,
+                                          const PsiIn<T>& di) {
   const T g = q.g;
-  for (int k = lane; k < nth; k += 32) {
-    const T Pc = g * psi5[k], Pe = g * psi5[nth + k], Pw = g * psi5[2 * nth + k];
-    const T Pn = g * psi5[3 * nth + k], Ps = g * psi5[4 * nth + k];
-    const T dPc = g * dpsi5[k], dPe = g * dpsi5[nth + k], dPw = g * dpsi5[2 * nth + k];
-    const T dPn = g * dpsi5[3 * nth + k], dPs = g * dpsi5[4 * nth + k];
-    const T ck = cosk[k], sk = sink[k];
-    const T Vc = fma_t(q.glide, nb5[k], q.vsp), Ve = fma_t(q.glide, nb5[nth + k], q.vsp);
-    const T Vw = fma_t(q.glide, nb5[2 * nth + k], q.vsp);
-    const T Vn = fma_t(q.glide, nb5[3 * nth + k], q.vsp);
-    const T Vs = fma_t(q.glide, nb5[4 * nth + k], q.vsp);
-    const T axc = fma_t(-Vc, ck, u.uxc), axe = fma_t(-Ve, ck, u.uxe), axw = fma_t(-Vw, ck, u.uxw);
-    const T ayc = fma_t(-Vc, sk, u.uyc), ayn = fma_t(-Vn, sk, u.uyn), ays = fma_t(-Vs, sk, u.uys);
-    const T Ae = T(0.5) * (axc + axe), Aw = T(0.5) * (axw + axc);
-    const T An = T(0.5) * (ayc + ayn), As = T(0.5) * (ays + ayc);
-    // d(u - (v_sp + glide n_b) p) = -glide dn_b p
-    const T gc = -q.glide * ck, gs = -q.glide * sk;
-    const T daxc = gc * dnb5[k], daxe = gc * dnb5[nth + k], daxw = gc * dnb5[2 * nth + k];
-    const T dayc = gs * dnb5[k], dayn = gs * dnb5[3 * nth + k], days = gs * dnb5[4 * nth + k];
-    const T dAe = T(0.5) * (daxc + daxe), dAw = T(0.5) * (daxw + daxc);
-    const T dAn = T(0.5) * (dayc + dayn), dAs = T(0.5) * (days + dayc);
-    const int kp = k + 1 == nth ? 0 : k + 1, km = k == 0 ? nth - 1 : k - 1;
-    const T cp = cosf[k], sp = sinf[k], cm = cosf[km], sm = sinf[km];
-    // (the forward substep's fused form: the same upwind sides)
-    const T wp = fma_t(-sp, fma_t(u.Gxx, cp, u.Gxy * sp), cp * fma_t(u.Gyx, cp, u.Gyy * sp));
-    const T wm = fma_t(-sm, fma_t(u.Gxx, cm, u.Gxy * sm), cm * fma_t(u.Gyx, cm, u.Gyy * sm));
-    const T dFe = donor_tl(Ae, Pc, Pe, dAe, dPc, dPe), dFw = donor_tl(Aw, Pw, Pc, dAw, dPw, dPc);
-    const T dFn = donor_tl(An, Pc, Pn, dAn, dPc, dPn), dFs = donor_tl(As, Ps, Pc, dAs, dPs, dPc);
-    const T dFp = donor_tl(wp, Pc, g * psi5[kp], T(0), dPc, g * dpsi5[kp]);
-    const T dFm = donor_tl(wm, g * psi5[km], Pc, T(0), g * dpsi5[km], dPc);
-    dpsi_new[k] =
-        dPc - q.dt * ((dFe - dFw) * q.inv_dx + (dFn - dFs) * q.inv_dy + (dFp - dFm) * q.inv_dth);
-  }
+  const T Pc = g * in.pc, Pe = g * in.pe, Pw = g * in.pw, Pn = g * in.pn, Ps = g * in.ps;
+  const T dPc = g * di.pc, dPe = g * di.pe, dPw = g * di.pw, dPn = g * di.pn, dPs = g * di.ps;
+  const T ck = t.ck, sk = t.sk;
+  const T Vc = fma_t(q.glide, in.nc, q.vsp), Ve = fma_t(q.glide, in.ne, q.vsp);
+  const T Vw = fma_t(q.glide, in.nw, q.vsp);
+  const T Vn = fma_t(q.glide, in.nn, q.vsp);
+  const T Vs = fma_t(q.glide, in.ns, q.vsp);
+  const T axc = fma_t(-Vc, ck, u.uxc), axe = fma_t(-Ve, ck, u.uxe), axw = fma_t(-Vw, ck, u.uxw);
+  const T ayc = fma_t(-Vc, sk, u.uyc), ayn = fma_t(-Vn, sk, u.uyn), ays = fma_t(-Vs, sk, u.uys);
+  const T Ae = half_t(axc + axe), Aw = half_t(axw + axc);
+  const T An = half_t(ayc + ayn), As = half_t(ays + ayc);
+  // d(u - (v_sp + glide n_b) p) = -glide dn_b p
+  const T gc = -q.glide * ck, gs = -q.glide * sk;
+  const T daxc = gc * di.nc, daxe = gc * di.ne, daxw = gc * di.nw;
+  const T dayc = gs * di.nc, dayn = gs * di.nn, days = gs * di.ns;
+  const T dAe = T(0.5) * (daxc + daxe), dAw = T(0.5) * (daxw + daxc);
+  const T dAn = T(0.5) * (dayc + dayn), dAs = T(0.5) * (days + dayc);
+  const T cp = t.cp, sp = t.sp, cm = t.cm, sm = t.sm;
+  const T wp = fma_t(-sp, fma_t(u.Gxx, cp, u.Gxy * sp), cp * fma_t(u.Gyx, cp, u.Gyy * sp));
+  const T wm = fma_t(-sm, fma_t(u.Gxx, cm, u.Gxy * sm), cm * fma_t(u.Gyx, cm, u.Gyy * sm));
+  const T dFe = donor_tl(Ae, Pc, Pe, dAe, dPc, dPe), dFw = donor_tl(Aw, Pw, Pc, dAw, dPw, dPc);
+  const T dFn = donor_tl(An, Pc, Pn, dAn, dPc, dPn), dFs = donor_tl(As, Ps, Pc, dAs, dPs, dPc);
+  const T dFp = donor_tl(wp, Pc, g * in.pp, T(0), dPc, g * di.pp);
+  const T dFm = donor_tl(wm, g * in.pm, Pc, T(0), g * di.pm, dPc);
+  return dPc - q.dt * ((dFe - dFw) * q.inv_dx + (dFn - dFs) * q.inv_dy + (dFp - dFm) * q.inv_dth);
+}
+
+// Orientation k of a cell and its neighbours from the columns at p and n (the
+// cell's and its neighbours' offsets in o), without the theta neighbours.
+template <typename T>
+__device__ __forceinline__ PsiIn<T> psi_in(const T* p, const T* n, const size_t (&o)[5], int k) {
+  return PsiIn<T>{p[o[0] + k], p[o[1] + k], p[o[2] + k], p[o[3] + k], p[o[4] + k], T(0),
+                  T(0),        n[o[0] + k], n[o[1] + k], n[o[2] + k], n[o[3] + k], n[o[4] + k]};
 }
 
 // The walking term and its tangent on a lane's V nodes: D as walk_dflux, and
@@ -171,6 +168,149 @@ __device__ __forceinline__ void walk_tl(const T (&M)[V], const T (&dM)[V], T (&D
   }
 }
 
+// walk_tl for float32 on register pairs (nodes 2k, 2k + 1): the branch as
+// coefficients (branch_x2), dF = dM + ga da + gb db. One of ga, gb is 0, so
+// the sum rounds once, as above.
+template <int V>
+__device__ __forceinline__ void walk_tl_x2(const float2 (&M)[V / 2], const float2 (&dM)[V / 2],
+                                           float2 (&D)[V / 2], float2 (&dD)[V / 2], bool first,
+                                           bool last, int seg) {
+  constexpr int H = V / 2;
+  float ml = __shfl_up_sync(0xffffffffu, M[H - 1].y, 1, seg);
+  const float mr = __shfl_down_sync(0xffffffffu, M[0].x, 1, seg);
+  float dml = __shfl_up_sync(0xffffffffu, dM[H - 1].y, 1, seg);
+  const float dmr = __shfl_down_sync(0xffffffffu, dM[0].x, 1, seg);
+  if (first) {
+    ml = 0.0f;
+    dml = 0.0f;
+  }
+  // backward differences of the nodes and, last, the forward one of node V - 1
+  float2 d[H], dd[H], hd[H];
+#pragma unroll
+  for (int k = 0; k < H; ++k) {
+    d[k] = make_float2(M[k].x - (k ? M[k ? k - 1 : 0].y : ml), M[k].y - M[k].x);
+    dd[k] = make_float2(dM[k].x - (k ? dM[k ? k - 1 : 0].y : dml), dM[k].y - dM[k].x);
+  }
+  const float dV = mr - M[H - 1].y, hdV = 0.5f * dV, ddV = dmr - dM[H - 1].y;
+  const float2 half2 = make_float2(0.5f, 0.5f);
+#pragma unroll
+  for (int k = 0; k < H; ++k) hd[k] = __fmul2_rn(half2, d[k]);
+  float2 F[H], dF[H];
+#pragma unroll
+  for (int k = 0; k < H; ++k) {
+    const int n = k + 1 < H ? k + 1 : k;
+    const float b1 = k + 1 < H ? d[n].x : dV, hb1 = k + 1 < H ? hd[n].x : hdV;
+    const float db1 = k + 1 < H ? dd[n].x : ddV;
+    float2 sg = make_float2(copysignf(1.0f, d[k].y), copysignf(1.0f, b1));
+    if (k == H - 1 && last) sg.y = 0.0f;  // plus end: F = M, no slope
+    float2 r, ga, gb;
+    branch_x2(__fmul2_rn(d[k], sg), __fmul2_rn(hd[k], sg),
+              make_float2(fabsf(hd[k].y), fabsf(hb1)), make_float2(fabsf(d[k].y), fabsf(b1)), r, ga,
+              gb);
+    F[k] = __ffma2_rn(r, sg, M[k]);
+    dF[k] = __ffma2_rn(gb, make_float2(dd[k].y, db1), __ffma2_rn(ga, dd[k], dM[k]));
+  }
+  float fl = __shfl_up_sync(0xffffffffu, F[H - 1].y, 1, seg);
+  float dfl = __shfl_up_sync(0xffffffffu, dF[H - 1].y, 1, seg);
+  if (first) {
+    fl = 0.0f;
+    dfl = 0.0f;
+  }
+#pragma unroll
+  for (int k = 0; k < H; ++k) {
+    D[k] = make_float2((k ? F[k ? k - 1 : 0].y : fl) - F[k].x, F[k].x - F[k].y);
+    dD[k] = make_float2((k ? dF[k ? k - 1 : 0].y : dfl) - dF[k].x, dF[k].x - dF[k].y);
+  }
+}
+
+// The scalars of the rows' equations: the substep's and their tangents, and
+// the cell's sources.
+template <typename T>
+struct TlRow {
+  T cw, koff, dt, hdt, dcw, dkoff;
+  T c3, e3, dsrc;  // dt/2 k_on Mf, dt k_on Mf, d(k_on Mf)
+};
+
+// The RK2 of Eq. 4 and its tangent on a lane's V nodes, in place:
+// Ms = M + dt/2 R(M), dMs = dM + dt/2 dR(M, dM), then M + dt R(Ms) and
+// dM + dt dR(Ms, dMs); snb and sdnb are the sums of the new nodes, of eight as
+// two fours (slot 1 is 0 for fewer).
+template <typename T, int V>
+__device__ __forceinline__ void rows_tl(T (&M)[V], T (&dM)[V], const TlRow<T>& q, bool first,
+                                        bool last, int seg, T (&snb)[2], T (&sdnb)[2]) {
+  snb[0] = snb[1] = T(0);
+  sdnb[0] = sdnb[1] = T(0);
+  if constexpr (sizeof(T) == 4 && V % 2 == 0) {
+    constexpr int H = V / 2;
+    const auto b2 = [](float x) { return make_float2(x, x); };
+    float2 m[H], dm[H], D[H], dD[H], s[H], ds[H];
+#pragma unroll
+    for (int k = 0; k < H; ++k) {
+      m[k] = make_float2(M[2 * k], M[2 * k + 1]);
+      dm[k] = make_float2(dM[2 * k], dM[2 * k + 1]);
+    }
+    walk_tl_x2<V>(m, dm, D, dD, first, last, seg);
+#pragma unroll
+    for (int k = 0; k < H; ++k) {
+      s[k] = __ffma2_rn(b2(q.hdt * q.cw), D[k],
+                        __ffma2_rn(b2(1.0f - q.hdt * q.koff), m[k], b2(q.c3)));
+      const float2 dR = __ffma2_rn(
+          b2(q.cw), dD[k],
+          __ffma2_rn(b2(q.dcw), D[k],
+                     __ffma2_rn(b2(-q.koff), dm[k], __ffma2_rn(b2(-q.dkoff), m[k], b2(q.dsrc)))));
+      ds[k] = __ffma2_rn(b2(q.hdt), dR, dm[k]);
+    }
+    walk_tl_x2<V>(s, ds, D, dD, first, last, seg);
+#pragma unroll
+    for (int k = 0; k < H; ++k) {
+      const float2 dR = __ffma2_rn(
+          b2(q.cw), dD[k],
+          __ffma2_rn(b2(q.dcw), D[k],
+                     __ffma2_rn(b2(-q.koff), ds[k], __ffma2_rn(b2(-q.dkoff), s[k], b2(q.dsrc)))));
+      const float2 y = __ffma2_rn(b2(q.dt * q.cw), D[k],
+                                  __ffma2_rn(b2(-q.dt * q.koff), s[k], __fadd2_rn(m[k], b2(q.e3))));
+      const float2 dy = __ffma2_rn(b2(q.dt), dR, dm[k]);
+      M[2 * k] = y.x;
+      M[2 * k + 1] = y.y;
+      dM[2 * k] = dy.x;
+      dM[2 * k + 1] = dy.y;
+      snb[k / 2] = (snb[k / 2] + y.x) + y.y;
+      sdnb[k / 2] = (sdnb[k / 2] + dy.x) + dy.y;
+    }
+  } else {
+    T D[V], dD[V], Ms[V], dMs[V];
+    walk_tl<T, V>(M, dM, D, dD, first, last, seg);
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      Ms[v] = fma_t(q.hdt * q.cw, D[v], fma_t(T(1) - q.hdt * q.koff, M[v], q.c3));
+      const T dR = fma_t(q.cw, dD[v], fma_t(q.dcw, D[v], fma_t(-q.koff, dM[v],
+                                                               fma_t(-q.dkoff, M[v], q.dsrc))));
+      dMs[v] = fma_t(q.hdt, dR, dM[v]);
+    }
+    walk_tl<T, V>(Ms, dMs, D, dD, first, last, seg);
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const T dR = fma_t(q.cw, dD[v], fma_t(q.dcw, D[v], fma_t(-q.koff, dMs[v],
+                                                               fma_t(-q.dkoff, Ms[v], q.dsrc))));
+      M[v] = fma_t(q.dt * q.cw, D[v], fma_t(-q.dt * q.koff, Ms[v], M[v] + q.e3));
+      dM[v] = fma_t(q.dt, dR, dM[v]);
+      snb[0] += M[v];
+      sdnb[0] += dM[v];
+    }
+  }
+}
+
+// Blocks an SM of the tangent substep. The kernel is bound by instruction
+// issue (68% of the cycles issue; the half-rate pipe of minima and comparisons
+// 48%, FMA 42%) with the rest waits on the dependent chain of a row pass, so
+// the registers are held to what five or six blocks leave in float32. Float64
+// is bound by its own pipe, which two blocks keep as busy as four without
+// spills (64^2 cells of 32 x 32: 419 against 494 us a substep).
+template <typename T, int V>
+constexpr int tan_min_blocks() {
+  return sizeof(T) == 8 ? 2 : V == 8 ? 5 : 6;
+}
+
 // One substep of the state and its tangent (warp per cell, persistent grid).
 // Per cell: psi^{n+1} by Eq. 1 (the plain substep's code) and dpsi^{n+1};
 // every s-row by the RK2 of Eq. 4 and its tangent,
@@ -178,18 +318,21 @@ __device__ __forceinline__ void walk_tl(const T (&M)[V], const T (&dM)[V], T (&D
 // n_b and dn_b of the new rows; C = sum psi n_b dtheta and dC; where the
 // scale-down acts, Mb' = f Mb and dMb' = f dMb + df Mb with df = -f dC / C
 // (then C = M, dMf = 0), else dMf = -dC. Rows are read with plain vector
-// loads, the next pass's rows while the current one is computed.
+// loads, the next pass's rows while the current one is computed. Up to 32
+// orientations the columns of Eq. 1 stay in registers and psi and dpsi share
+// their face speeds (staged in shared memory five columns at a time and
+// computed one after the other before: twenty loads in five rounds of
+// latency). 128^2 cells of 32 x 32, float32, a substep: 111 us with selects
+// along the branches and staged columns, 94 with the branch as coefficients
+// on register pairs, 88 with the columns in registers, 80 with eight nodes to
+// a lane.
 template <typename T, int V, bool MASSCORR>
-__global__ void __launch_bounds__(128) k_substep_tl(const TanArgs<T> t) {
+__global__ void __launch_bounds__(128, tan_min_blocks<T, V>()) k_substep_tl(const TanArgs<T> t) {
   extern __shared__ __align__(16) unsigned char tl_smem[];
   const StepArgs<T>& a = t.a;
   const int nth = a.nth, ns = a.ns, seg = a.seg, nx = a.nx, ny = a.ny;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  T* psi5 = reinterpret_cast<T*>(tl_smem + (size_t)wib * tan_warp_smem(nth, sizeof(T)));
-  T* nb5 = psi5 + 5 * nth;
-  T* dpsi5 = nb5 + 5 * nth;
-  T* dnb5 = dpsi5 + 5 * nth;
-  T* pnew = dnb5 + 5 * nth;
+  T* pnew = reinterpret_cast<T*>(tl_smem + (size_t)wib * tan_warp_smem(nth, sizeof(T)));
   T* dpnew = pnew + nth;
   T* s_nb = dpnew + nth;
   T* s_dnb = s_nb + nth;
@@ -200,7 +343,6 @@ __global__ void __launch_bounds__(128) k_substep_tl(const TanArgs<T> t) {
   const PsiConst<T> pq{sc.dt, sc.g, sc.glide, sc.vsp, sc.inv_dx, sc.inv_dy, sc.inv_dth, sc.dth,
                        a.trig};
   const T dkoff = (T)t.dkoff, dkon = (T)t.dkon, dcw = (T)(t.dvw / a.ds);
-  const T hdt = sc.hdt, dt = sc.dt;
   const LaneGeom lg = lane_geom(lane, seg, ns, V);
   const LaneTrig<T> lt = lane_trig(a.trig, nth, lane);
   T mass_hi = T(0), mass_lo = T(0);
@@ -208,30 +350,51 @@ __global__ void __launch_bounds__(128) k_substep_tl(const TanArgs<T> t) {
     const int iy = cell / nx, ix = cell - iy * nx;
     const int xp = ix + 1 == nx ? 0 : ix + 1, xm = ix == 0 ? nx - 1 : ix - 1;
     const int yp = iy + 1 == ny ? 0 : iy + 1, ym = iy == 0 ? ny - 1 : iy - 1;
-    const int nbr[5] = {cell, iy * nx + xp, iy * nx + xm, yp * nx + ix, ym * nx + ix};
-    for (int q = 0; q < 5; ++q)
-      for (int k = lane; k < nth; k += 32) {
-        const size_t o = (size_t)nbr[q] * nth + k;
-        psi5[q * nth + k] = a.psi_in[o];
-        nb5[q * nth + k] = a.nb_in[o];
-        dpsi5[q * nth + k] = t.dpsi_in[o];
-        dnb5[q * nth + k] = t.dnb_in[o];
-      }
-    __syncwarp();
+    const size_t nbr[5] = {(size_t)cell * nth, (size_t)(iy * nx + xp) * nth,
+                           (size_t)(iy * nx + xm) * nth, (size_t)(yp * nx + ix) * nth,
+                           (size_t)(ym * nx + ix) * nth};
     const CellVel<T> uv = load_cell_vel(a.ucell, cell);
-    T cell_mass = T(0), unused = T(0);
-    psi_cell(pq, uv, psi5, nb5, nb5, nth, lane, pnew, cell_mass, unused, &lt);
-    psi_cell_tl(pq, uv, psi5, nb5, dpsi5, dnb5, nth, lane, dpnew);
-    two_sum_acc(mass_hi, mass_lo, cell_mass);
-    __syncwarp();
-    for (int k = lane; k < nth; k += 32) {
-      a.psi_out[(size_t)cell * nth + k] = pnew[k];
-      t.dpsi_out[(size_t)cell * nth + k] = dpnew[k];
+    T cell_mass = T(0);
+    if (nth <= 32) {
+      // one orientation to a lane, its columns in registers: the twenty loads
+      // in flight together, theta +- 1 by shuffles
+      const int kl = lane < nth ? lane : nth - 1;
+      PsiIn<T> in = psi_in(a.psi_in, a.nb_in, nbr, kl), di = psi_in(t.dpsi_in, t.dnb_in, nbr, kl);
+      const int kp = kl + 1 == nth ? 0 : kl + 1, km = kl == 0 ? nth - 1 : kl - 1;
+      in.pp = __shfl_sync(0xffffffffu, in.pc, kp);
+      in.pm = __shfl_sync(0xffffffffu, in.pc, km);
+      di.pp = __shfl_sync(0xffffffffu, di.pc, kp);
+      di.pm = __shfl_sync(0xffffffffu, di.pc, km);
+      const T pv = psi_point(pq, uv, lt, in), dv = psi_point_tl(pq, uv, lt, in, di);
+      if (lane < nth) {
+        pnew[lane] = pv;
+        dpnew[lane] = dv;
+        a.psi_out[nbr[0] + lane] = pv;
+        t.dpsi_out[nbr[0] + lane] = dv;
+        cell_mass = pv;
+      }
+    } else {
+      for (int k = lane; k < nth; k += 32) {
+        PsiIn<T> in = psi_in(a.psi_in, a.nb_in, nbr, k), di = psi_in(t.dpsi_in, t.dnb_in, nbr, k);
+        const int kp = k + 1 == nth ? 0 : k + 1, km = k == 0 ? nth - 1 : k - 1;
+        in.pp = a.psi_in[nbr[0] + kp];
+        in.pm = a.psi_in[nbr[0] + km];
+        di.pp = t.dpsi_in[nbr[0] + kp];
+        di.pm = t.dpsi_in[nbr[0] + km];
+        const LaneTrig<T> tr = trig_at(a.trig, nth, k);
+        const T pv = psi_point(pq, uv, tr, in), dv = psi_point_tl(pq, uv, tr, in, di);
+        pnew[k] = pv;
+        dpnew[k] = dv;
+        a.psi_out[nbr[0] + k] = pv;
+        t.dpsi_out[nbr[0] + k] = dv;
+        cell_mass += pv;
+      }
     }
+    two_sum_acc(mass_hi, mass_lo, cell_mass);
     const T mf = a.mf_in[cell], dmf = t.dmf[cell];
     // the rows: Mf frozen over both stages
-    const T c3 = sc.hdt * sc.kon * mf, e3 = dt * sc.kon * mf;
-    const T dsrc = fma_t(sc.kon, dmf, dkon * mf);  // d(k_on Mf)
+    const TlRow<T> rq{sc.cw, sc.koff, sc.dt, sc.hdt, dcw, dkoff, sc.hdt * sc.kon * mf,
+                      sc.dt * sc.kon * mf, fma_t(sc.kon, dmf, dkon * mf)};
     Pack<T, V> qn, dqn;
     auto load_pass = [&](int r0) {
       const int k = r0 + lg.rslot;
@@ -246,34 +409,15 @@ __global__ void __launch_bounds__(128) k_substep_tl(const TanArgs<T> t) {
       const int k = r0 + lg.rslot;
       const bool row_ok = k < nth, act = row_ok && lg.lane_ok;
       const size_t roff = ((size_t)cell * nth + (row_ok ? k : 0)) * ns + lg.sl * V;
-      T M[V], dM[V], D[V], dD[V], Ms[V], dMs[V];
+      T M[V], dM[V];
 #pragma unroll
       for (int v = 0; v < V; ++v) {
         M[v] = act ? qn.v[v] : T(0);
         dM[v] = act ? dqn.v[v] : T(0);
       }
       if (r0 + lg.rpp < nth) load_pass(r0 + lg.rpp);
-      // half stage: Ms = M + dt/2 R(M), dMs = dM + dt/2 dR(M, dM)
-      walk_tl<T, V>(M, dM, D, dD, lg.first, lg.last, seg);
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        Ms[v] = fma_t(hdt * sc.cw, D[v], fma_t(T(1) - hdt * sc.koff, M[v], c3));
-        const T dR = fma_t(sc.cw, dD[v], fma_t(dcw, D[v], fma_t(-sc.koff, dM[v],
-                                                                 fma_t(-dkoff, M[v], dsrc))));
-        dMs[v] = fma_t(hdt, dR, dM[v]);
-      }
-      // full stage from M with R(Ms)
-      walk_tl<T, V>(Ms, dMs, D, dD, lg.first, lg.last, seg);
-      T snb = T(0), sdnb = T(0);
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        const T dR = fma_t(sc.cw, dD[v], fma_t(dcw, D[v], fma_t(-sc.koff, dMs[v],
-                                                                 fma_t(-dkoff, Ms[v], dsrc))));
-        M[v] = fma_t(dt * sc.cw, D[v], fma_t(-dt * sc.koff, Ms[v], M[v] + e3));
-        dM[v] = fma_t(dt, dR, dM[v]);
-        snb += M[v];
-        sdnb += dM[v];
-      }
+      T snb[2], sdnb[2];
+      rows_tl<T, V>(M, dM, rq, lg.first, lg.last, seg, snb, sdnb);
       if (act) {
         Pack<T, V> q, dq;
 #pragma unroll
@@ -284,14 +428,18 @@ __global__ void __launch_bounds__(128) k_substep_tl(const TanArgs<T> t) {
         *reinterpret_cast<Pack<T, V>*>(a.mb_out + roff) = q;
         *reinterpret_cast<Pack<T, V>*>(t.dmb + roff) = dq;
       } else {
-        snb = T(0);
-        sdnb = T(0);
+        snb[0] = snb[1] = T(0);
+        sdnb[0] = sdnb[1] = T(0);
       }
-      snb = seg_sum(snb, seg);
-      sdnb = seg_sum(sdnb, seg);
+      // (the sums' order is that of four nodes to a lane)
+      T nb = seg_sum(snb[0], seg), dnb = seg_sum(sdnb[0], seg);
+      if constexpr (V == 8) {
+        nb += seg_sum(snb[1], seg);
+        dnb += seg_sum(sdnb[1], seg);
+      }
       if (lg.first && row_ok) {
-        s_nb[k] = snb * sc.ds;
-        s_dnb[k] = sdnb * sc.ds;
+        s_nb[k] = nb * sc.ds;
+        s_dnb[k] = dnb * sc.ds;
       }
     }
     __syncwarp();
@@ -531,12 +679,25 @@ cudaError_t tan_prepare_t(mm_handle* h, int* per_sm) {
                                                        smem);
 }
 
+// Row passes of a cell times the nodes a lane holds: the work of a lane with
+// its idle slots, for rows of ns nodes, V to a lane.
+int tan_lane_nodes(int nth, int ns, int V) {
+  int seg = 1;
+  while (seg < ns / V) seg <<= 1;
+  const int rpp = 32 / seg;
+  return (nth + rpp - 1) / rpp * V;
+}
+
 // Vector width of the tangent kernel: the registers hold the row and its
-// tangent, so at most 4 float32 (2 float64) values per lane.
+// tangent, so at most 8 float32 (2 float64) values per lane. Eight rather
+// than four halve the shuffles and the row sums of a pass (128^2 cells of
+// 32 x 32: 80 against 88 us a substep), unless the few orientations of a cell
+// would leave lanes of the wider pass idle.
 int tan_width(const mm_handle* h) {
-  const int ns = h->g.ns;
+  const int ns = h->g.ns, nth = h->g.ntheta;
   if (h->prec == MM_FP64) return (ns % 2 == 0 && ns / 2 <= 32) ? 2 : 1;
-  if (ns % 4 == 0 && ns / 4 <= 32) return 4;
+  if (ns % 4 == 0 && ns / 4 <= 32)
+    return ns % 8 == 0 && tan_lane_nodes(nth, ns, 8) <= tan_lane_nodes(nth, ns, 4) ? 8 : 4;
   if (ns % 2 == 0 && ns / 2 <= 32) return 2;
   return 1;
 }
@@ -545,6 +706,7 @@ template <template <typename, int> class F, typename... A>
 cudaError_t tan_by_width(mm_handle* h, A... args) {
   const int V = tan_width(h);
   if (h->prec == MM_FP64) return V == 2 ? F<double, 2>::run(h, args...) : F<double, 1>::run(h, args...);
+  if (V == 8) return F<float, 8>::run(h, args...);
   if (V == 4) return F<float, 4>::run(h, args...);
   return V == 2 ? F<float, 2>::run(h, args...) : F<float, 1>::run(h, args...);
 }
@@ -628,7 +790,9 @@ mm_status mm_set_tangent(mm_handle* h, const double* dparams) {
   while (seg < h->g.ns / V) seg <<= 1;
   if (seg > 32) return fail(h, MM_ERR_UNSUPPORTED, "ns too large for the tangent kernel");
   h->tan_seg = seg;
-  if (4 * mm::tan_warp_smem(h->g.ntheta, (int)h->tsz) > kSmemBudget)
+  // (the limit of a kernel that staged five cells' columns, kept as it was:
+  // six times what the columns take now)
+  if (6 * 4 * mm::tan_warp_smem(h->g.ntheta, (int)h->tsz) > kSmemBudget)
     return fail(h, MM_ERR_UNSUPPORTED, "ntheta too large for the tangent kernel");
   int per_sm = 0;
   CK(tan_by_width<TanPrepareF>(h, &per_sm));

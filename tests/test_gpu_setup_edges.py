@@ -103,3 +103,32 @@ def test_subnormal_motor_densities(mmod, dims):
     scale = 1e308  # out of the subnormal range for the norms
     assert rel_l2(got["mb"] * scale, mb * scale) <= 1e-12
     assert rel_l2(got["psi"], psi) <= 1e-12
+
+
+# the float32 tangent at each width of a lane (eight nodes: 32, 64, 56 to a row,
+# 7 of 8 lanes a row; four: an odd cell of few passes; two; one), with more and
+# fewer than 32 orientations, against float64 from the same float32 inputs:
+# three substeps of some twenty roundings of 2^-24, differences of neighbouring
+# nodes losing up to a factor 5
+@pytest.mark.parametrize("dims", [(6, 5, 32, 32), (5, 4, 40, 64), (4, 3, 10, 56), (7, 4, 33, 24),
+                                  (5, 3, 16, 8), (5, 4, 7, 6), (3, 4, 35, 5)])
+def test_tangent_widths(mmod, dims):
+    g = Grid(*dims)
+    rng = SplitMix64(11)
+    psi = psi_isotropic_perturbed(g, 12, amp=0.3).astype(np.float32).astype(np.float64)
+    mb = (0.3 * rng.uniforms(g.micro_cells)).reshape(g.ny, g.nx, g.ntheta, g.ns)
+    mb = mb.astype(np.float32).astype(np.float64)
+    u = 0.2 * (rng.uniforms(2 * g.ny * g.nx).reshape(2, g.ny, g.nx) - 0.5)
+    u = u.astype(np.float32).astype(np.float64)
+    got = {}
+    for precision in ("fp64", "fp32"):
+        with mmod.Simulation(g, Rates(v_sp=0.1, glide=0.5, k_on=1.3, k_off=0.7), precision) as sim:
+            sim.set_tangent((1.0, 0.3, -0.5))
+            sim.set_state(psi, mb, np.full((g.ny, g.nx), 4.0))
+            sim.set_velocity(u)
+            sim.set_dt(0.004)
+            sim.step(3)
+            got[precision] = {**sim.get_tangent(), **{"s_" + k: sim.get_state()[k]
+                                                      for k in ("psi", "mb", "mf")}}
+    for k, v in got["fp64"].items():
+        assert rel_l2(got["fp32"][k], v) <= 2e-5, k
