@@ -55,6 +55,8 @@ CSRC = os.path.join(ROOT, "paper_1908_04279_gb300", "csrc")
 # sources of each kernel a committed profile summary may describe
 KERNEL_SRCS = {
     "k_substep": ("mm_step.cu", "mm_async.cuh", "mm_cell.cuh", "mm_walk.cuh", "mm_internal.cuh"),
+    "k_substep_resident": ("mm_resident.cu", "mm_async.cuh", "mm_cell.cuh", "mm_walk.cuh",
+                           "mm_internal.cuh"),
     "k_substep_batch": ("mm_batch.cu", "mm_cell.cuh", "mm_walk.cuh", "mm_internal.cuh"),
     "k_adjoint": ("mm_adjoint.cu", "mm_async.cuh", "mm_cell.cuh", "mm_walk.cuh",
                   "mm_internal.cuh"),
@@ -130,7 +132,8 @@ def read_peaks():
 # the n_b sum. The local-step kernel runs them on the float32 pipe. The float64
 # substep runs 13 of them on the float64 pipe (difference, half, flux, flux
 # difference, two stage fmas; the n_b add) and the sign transfers, minima and
-# maximum (10) on the integer pipe, on the values' bit patterns; its per-(cell,
+# maximum (10) on the integer pipe, on the values' bit patterns (the halves, counted
+# among the 13, too); its per-(cell,
 # theta) transport work, about 40 operations per row, adds under 1 per motor
 # value at 64 nodes and is left out.
 LOCAL_OPS = 23
@@ -660,8 +663,9 @@ def run_ours(args):
     def ensemble_run(steps):
         """ensemble64: 64 members with uneven grids (N in {32..128}, Ntheta and
         Ns in {16, 32}), k_off log-uniform in [0.05, 5], v_walk in [0.5, 2];
-        after mm_batch_autotune, a step is one graph of 500 batched substeps
-        (one launch per substep over all members)."""
+        after mm_batch_autotune, a step is 500 batched substeps (the members in
+        groups, each group one resident launch; kernel_ms_per_launch is the
+        time of one substep of all members)."""
         from paper_1908_04279_gb300.inputs import ensemble_members, member_inputs
         ms_ = ensemble_members()
         b = mm.Batch([m.grid for m in ms_], [m.rates for m in ms_], "fp32",
@@ -691,8 +695,7 @@ def run_ours(args):
         ms_step = sum(times) / len(times)
         launch = ms_step / ne
         best = min(tune, key=lambda x: x["ms_per_substep"])
-        return {"workload": "ensemble64 (64 members, 500 substeps per step in one CUDA graph, "
-                            "float32)",
+        return {"workload": "ensemble64 (64 members, 500 substeps per step, float32)",
                 "value": world * cells * ne / (ms_step * 1e-3), "unit": UNIT, "steps": steps,
                 "ms_per_step": ms_step, "kernel_ms_per_launch": launch,
                 "motor_cells_per_substep": cells, "algorithmic_bytes_per_launch": algo_e,
@@ -751,7 +754,7 @@ def run_ours(args):
         v["roofline"] = {"bound": "alu", "achieved": ops, "peak": packed_tops,
                          "unit": "Tops/s", "frac": ops / packed_tops,
                          "peak_source": "measured (mm_alu_peak, packed float32 fma)",
-                         "kernel": "k_motor_local (float32)",
+                         "kernel": "k_motor_local_reg (float32)",
                          "traffic": read_profile_traffic("k_motor_local", wname_of(v), "fp32")}
 
     total_ms, kern_ms, fp64_ms, fp64_kern, e2e_s, o_ms, o_kern = reduce_max(
@@ -763,15 +766,17 @@ def run_ours(args):
     achieved = algo / (launch_ms * 1e-3) / 1e9
     # the large case's capture is taken at a quarter of its cells (256x256 x
     # 64 x 64) and scaled to a full launch by the motor cells
-    traffic = (read_profile_traffic("k_substep", "large512", "fp32") if name == "large512"
-               else read_profile_traffic("k_substep", name, "fp32"))
+    # (workloads up to about the size of L2 run a macro step in one resident launch)
+    kernel, o_kernel = ("k_substep" if w_ == "large512" else "k_substep_resident"
+                        for w_ in (name, other))
+    traffic = read_profile_traffic(kernel, name, "fp32")
     fp64_value = whole_job_value(world, units_per_step * fp64_steps, fp64_ms * 1e-3)
     fp64_launch_ms = fp64_kern / (fp64_steps * nsub)
-    fp64_ops = g.micro_cells * SUBSTEP_OPS / (fp64_launch_ms * 1e-3) / 1e12
+    fp64_ops = g.micro_cells * SUBSTEP_FP64_PIPE_OPS / (fp64_launch_ms * 1e-3) / 1e12
     fp64_peak = alu["fp64"]["fma_per_s"] / 1e12
     o_launch = o_kern / (o_steps * nso)
     o_algo = algorithmic_bytes_per_launch(go, 4)
-    o_traffic = read_profile_traffic("k_substep", other, "fp32")
+    o_traffic = read_profile_traffic(o_kernel, other, "fp32")
     o_leg = {"workload": f"{other} ({go.nx}x{go.ny} x {go.ntheta} x {go.ns}, {nso} substeps per "
                          f"macro step, float32)",
              "value": whole_job_value(world, go.micro_cells * nso * o_steps, o_ms * 1e-3),
@@ -780,14 +785,16 @@ def run_ours(args):
              "roofline": {"bound": "hbm", "peak": peak, "unit": "GB/s",
                           "achieved": o_algo / (o_launch * 1e-3) / 1e9,
                           "frac": o_algo / (o_launch * 1e-3) / 1e9 / peak,
-                          "kernel": "k_substep (float32)", "peak_source": peak_src,
+                          "kernel": f"{o_kernel} (float32)", "peak_source": peak_src,
                           "traffic": o_traffic,
                           "dram_frac": (None if o_traffic is None
                                         else o_traffic / (o_launch * 1e-3) / 1e9 / peak)}}
     if other == "precision128":
-        o_leg["note"] = ("L2-resident: the 67 MB motor density stays in the 129 MB L2 within a "
-                         "macro step, so frac compares an L2-fed kernel with the HBM copy peak; "
-                         "dram_frac is its measured DRAM traffic over the same time")
+        o_leg["note"] = ("on-chip: a macro step is one launch that keeps about half of the 67 MB "
+                         "motor density in shared memory and reads the rest from the 129 MB L2, "
+                         "so frac compares it with the HBM copy peak at the bytes of a launch per "
+                         "substep; kernel_ms_per_launch is the time of one substep, dram_frac the "
+                         "measured DRAM traffic of one substep over it")
     if rank == 0:
         cpu = time_oracle_sample(name)
         ens_frac = ens["achieved_gbs"] / peak
@@ -805,7 +812,7 @@ def run_ours(args):
                        "parallelism": f"{world} independent instance(s), one per GPU"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
-                         "kernel": "k_substep (float32)", "peak_source": peak_src,
+                         "kernel": f"{kernel} (float32)", "peak_source": peak_src,
                          "kernel_ms_per_launch": launch_ms,
                          "algorithmic_bytes_per_launch": algo},
             "cpu_baseline": cpu,
@@ -816,11 +823,9 @@ def run_ours(args):
                      "roofline": {"bound": "alu", "achieved": fp64_ops, "peak": fp64_peak,
                                   "unit": "Tops/s", "frac": fp64_ops / fp64_peak,
                                   "kernel": "k_substep (float64)",
-                                  "ops_per_cell_update": SUBSTEP_OPS,
-                                  "peak_source": "measured (mm_alu_peak, float64 fma)",
-                                  "fp64_pipe_ops_per_cell_update": SUBSTEP_FP64_PIPE_OPS,
-                                  "fp64_pipe_frac": fp64_ops * SUBSTEP_FP64_PIPE_OPS
-                                  / SUBSTEP_OPS / fp64_peak}},
+                                  "ops_per_cell_update": SUBSTEP_FP64_PIPE_OPS,
+                                  "scheme_ops_per_cell_update": SUBSTEP_OPS,
+                                  "peak_source": "measured (mm_alu_peak, float64 fma)"}},
             other: o_leg,
             "alu_peaks": {k: {"fma_per_s": v["fma_per_s"], "ms_per_launch": v["ms_per_launch"]}
                           for k, v in alu.items()},
@@ -834,13 +839,14 @@ def run_ours(args):
             "capture": capture,
             "ensemble": dict(ens, roofline={"bound": "hbm", "peak": peak, "unit": "GB/s",
                                             "achieved": ens["achieved_gbs"], "frac": ens_frac,
-                                            "kernel": "k_substep_batch (float32)",
+                                            "kernel": "k_substep_resident_group (float32)",
                                             "peak_source": peak_src,
                                             "traffic": read_profile_traffic(
-                                                "k_substep_batch", "ensemble64", "fp32")}),
+                                                "k_substep_resident", "ensemble64", "fp32")}),
             # per macro step: set_velocity (precision conversion, per-cell velocity
-            # block, the two substep-rule kernels), nsub substeps, moments
-            "gpu_launches": args.steps * (nsub + 5),
+            # block, the two substep-rule kernels), nsub substeps (one launch
+            # each, or one resident launch for all), moments
+            "gpu_launches": args.steps * ((nsub if big else 1) + 5),
             "clocks": clk,
             # flat summaries of every leg (fractions of the measured peaks)
             "hbm_frac": achieved / peak,

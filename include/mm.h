@@ -155,7 +155,11 @@ mm_status mm_set_dt(mm_handle* h, double dt);
  *      stage);
  *   3. n_b, the coarse density (Eq. 5) with psi at the new time, the
  *      scale-down of Alg. 2, and Mf = M - C (Eq. 6).
- * Asynchronous on the handle's stream; launched as a captured CUDA graph. */
+ * Asynchronous on the handle's stream. MM_FP32_MIXED instances of up to about
+ * the size of L2 run all of a call's substeps (two or more) in one cooperative
+ * launch with the motor density resident on the chip; other calls run one
+ * launch per substep as a captured CUDA graph. A call on a capturing stream
+ * always runs one launch per substep. */
 mm_status mm_micro_step(mm_handle* h, int n_substeps);
 
 /* Macroscale moments (Alg. 1 after the inner loop), all float64.
@@ -433,7 +437,8 @@ mm_status mm_fluid_response(mm_handle* h, double* out, int on_device);
  * together: mm_micro_step on the batch handle runs each substep as ONE launch
  * over all instances (a table of tiles, each a run of cells of one instance
  * holding about the same number of motor values), and the n_substeps of one
- * call as one captured CUDA graph. No counterpart in the paper, which runs one
+ * call as one captured CUDA graph; float32 instances whose motor density the
+ * chip can hold go several to one cooperative launch of all n_substeps instead. No counterpart in the paper, which runs one
  * instance at a time.
  *
  * mm_create_batch(n, grids, rates, prec, stream, &batch): grids[i], rates[i]

@@ -1,10 +1,12 @@
 // Many substeps in one launch with the motor density resident on the chip
-// (float32 form): the substeps of k_substep for instances whose Mb fits the
-// shared memory of all SMs together (up to about 30 MB).
+// (float32 form): the substeps of k_substep for instances up to about the size
+// of L2. Mb is kept in the shared memory of all SMs together (about 33 MB),
+// whole or in part; the row passes that do not fit are read and written every
+// substep through each worker's ring.
 //
 // One block per SM owns a run of consecutive cells for the whole call and
-// keeps their s-rows in shared memory: Mb crosses HBM once per call instead
-// of once per substep, and the launch, the ring set-up, the scalar loads and
+// keeps their s-rows in shared memory: what is kept crosses HBM once per call
+// instead of once per substep, and the launch, the ring set-up, the scalar loads and
 // the last-block sum that every k_substep launch pays are paid once. Between
 // two substeps the blocks exchange only psi and n_b (through L2) and the
 // filament number that fixes the float32 mass-correction factor, and no block
@@ -55,7 +57,8 @@
 // 128 registers: 19 of 96 are within 3 %, 11 or 23 slower. Measured on a GB300,
 // us per substep against k_substep in a CUDA graph: 32^2 x 16^2 7.2 -> 4.1, 64^2 x
 // 32^2 13.4 -> 6.4, 128^2 x 16^2 23 -> 9.8, 128^2 x 32^2 35.2 -> 25.3, 256^2 x 16^2
-// 77 -> 35, 85 x 61 x 24 x 30 57 -> 8.0, 200 x 150 x 24 x 30 231 -> 43; the 64-member
+// 77 -> 35, 85 x 61 x 24 x 30 57 -> 8.0, 200 x 150 x 24 x 30 65 -> 43
+// (231 before k_substep's rows were packed; the 57 is from then too); the 64-member
 // ensemble 594 (tuned) -> 427.
 #include <map>
 #include <mutex>
@@ -721,9 +724,11 @@ bool resident_plan(const mm_handle* h, int grid, ResidentPlan* p) {
 // at 128^2 x 32^2, where k_substep takes 35), k_substep's at HBM speed where a
 // row fills its lanes: from about 250 MB of Mb on, twice the L2, HBM bounds both
 // and the bulk-copy rings of k_substep keep more of it in flight (256^2 x 32^2,
-// 268 MB: 127 against 131 us; 160^2 x 64^2, 420 MB: 189 against 155). Rows that
-// are no multiple of 4 nodes have one node to a lane in k_substep: 200 x 150 x
-// 24 x 30 44 against 231 us, whatever the size.
+// 268 MB: 127 against 131 us; 160^2 x 64^2, 420 MB: 189 against 155). Where a row
+// is no multiple of 4 nodes k_substep's warps copy their chunks themselves, and
+// the resident kernel is the faster one up to the most cells it takes (2^16):
+// 200 x 150 x 24 x 30, 86 MB, 43 against 65 us; 256^2 x 24 x 30, 189 MB, 93 against
+// 137; 256^2 x 32 x 31, 260 MB, 146 against 165.
 bool resident_pays(const mm_handle* h) {
   return h->g.ns % 4 != 0 || h->mbn * h->tsz <= (size_t)250 << 20;
 }

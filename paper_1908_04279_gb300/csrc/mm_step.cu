@@ -7,10 +7,10 @@
 //      full stage). The cell's rows stream through a ring of shared-memory
 //      stages filled by bulk asynchronous copies (cp.async.bulk, the Tensor
 //      Memory Accelerator) that complete on mbarriers; lane 0 keeps up to S
-//      chunks in flight ahead of the warp. A row is spread over `seg` lanes
-//      with V consecutive s-nodes per lane; the Superbee stencil reaches across
-//      lanes with warp shuffles; the new row goes straight back to global
-//      memory in place (16-byte vector stores);
+//      chunks in flight ahead of the warp. A row takes ceil(ns / 8) lanes of
+//      eight consecutive s-nodes each (rows_chunk pads them to a power of two);
+//      the Superbee stencil reaches across lanes with warp shuffles; the new
+//      row goes straight back to global memory in place;
 //   2. n_b of every row by a shuffle reduction over s (the force and force
 //      dipole are reduced in float64 by the moments kernel instead);
 //   3. psi^{n+1}(cell, :) by Eq. 1 in donor-cell flux form (lane = theta), from

@@ -322,10 +322,10 @@ constexpr int tan_min_blocks() {
 // orientations the columns of Eq. 1 stay in registers and psi and dpsi share
 // their face speeds (staged in shared memory five columns at a time and
 // computed one after the other before: twenty loads in five rounds of
-// latency). 128^2 cells of 32 x 32, float32, a substep: 111 us with selects
-// along the branches and staged columns, 94 with the branch as coefficients
-// on register pairs, 88 with the columns in registers, 80 with eight nodes to
-// a lane.
+// latency). 128^2 cells of 32 x 32, float32, a substep of a pass of 50: 97 us
+// with selects along the branches and staged columns, 94 with the branch as
+// coefficients on register pairs, 88 with the columns in registers, 80 with
+// eight nodes to a lane.
 template <typename T, int V, bool MASSCORR>
 __global__ void __launch_bounds__(128, tan_min_blocks<T, V>()) k_substep_tl(const TanArgs<T> t) {
   extern __shared__ __align__(16) unsigned char tl_smem[];
