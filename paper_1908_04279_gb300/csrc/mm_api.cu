@@ -42,7 +42,6 @@ mm_status free_all(mm_handle* h) {
   tangent_free(h);
   for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
   h->graphs.clear();
-  if (h->res_xch) cudaFree(h->res_xch);
   if (h->diff_tab) cudaFree(h->diff_tab);
   if (h->local_n) cudaFree(h->local_n);
   void* anc[8] = {h->anc_off,  h->anc_cacc,  h->anc_fsc,    h->anc_flags,
@@ -451,12 +450,15 @@ mm_status mm_create(const mm_grid* grid, const mm_rates* rates, mm_precision pre
   ALLOC(h->u64, 2 * nc * 8);
   ALLOC(h->trig, 4 * (size_t)grid->ntheta * h->tsz);
   ALLOC(h->trig64, 24 * (size_t)grid->ntheta * 8);
-  ALLOC(h->partial, (size_t)h->npartial * 8 * 8);
+  // the block sums and, behind them, what the blocks of a resident launch
+  // exchange (an allocation of its own took 0.1 ms of a handle's creation)
+  const size_t part_bytes = ((size_t)h->npartial * 64 + 255) & ~(size_t)255;
+  h->res_xch_bytes = h->res_grid > 0 ? 16 + 32 * (size_t)h->res_grid : 0;
+  ALLOC(h->partial, part_bytes + h->res_xch_bytes);
+  if (h->res_grid > 0) h->res_xch = reinterpret_cast<unsigned long long*>(h->partial + part_bytes / 8);
   ALLOC(h->fields, 12 * nc * 8);
   ALLOC(h->staging, h->staging_n * 8);
   ALLOC(h->prm, sizeof(DevParams));
-  h->res_xch_bytes = 16 + 32 * (size_t)h->res_grid;
-  if (h->res_grid > 0) ALLOC(h->res_xch, h->res_xch_bytes);
 #undef ALLOC
   e = cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
@@ -521,8 +523,7 @@ mm_status mm_create(const mm_grid* grid, const mm_rates* rates, mm_precision pre
     if (e == cudaSuccess) e = cudaMemset(h->u, 0, 2 * nc * h->tsz);
     if (e == cudaSuccess) e = cudaMemset(h->ucell, 0, 12 * nc * h->tsz);
     if (e == cudaSuccess) e = cudaMemset(h->mb, 0, h->mbn * h->tsz);
-    if (e == cudaSuccess) e = cudaMemset(h->partial, 0, (size_t)h->npartial * 64);
-    if (e == cudaSuccess && h->res_xch) e = cudaMemset(h->res_xch, 0, h->res_xch_bytes);
+    if (e == cudaSuccess) e = cudaMemset(h->partial, 0, part_bytes + h->res_xch_bytes);
     if (e != cudaSuccess) {
       cuda_fail(h, "initial state", e);
       return bail(MM_ERR_CUDA);
