@@ -414,12 +414,18 @@ __device__ __forceinline__ void rows_packed(T* stage, T* dst, int RC, int ns, co
       for (int v = 0; v < 8; ++v)
         M[v] = fma_t(k.e1, D[v], fma_t(k.e2, Ms[v], add_rn(M[v], e3)));
     }
-    // (pairs first, as walk_dflux_x2's rows: node 2h and 2h + 1 in two sums)
-    T a[8];
+    T a[8], snb;
 #pragma unroll
     for (int v = 0; v < 8; ++v) a[v] = v < lg.nv ? M[v] : T(0);
-    const T lo = ((a[0] + a[2]) + a[4]) + a[6], up = ((a[1] + a[3]) + a[5]) + a[7];
-    const T snb = packed_sum(lo + up, lg.nl, lg.sl);
+    if constexpr (sizeof(T) == 4) {
+      const float2 x[4] = {make_float2(a[0], a[1]), make_float2(a[2], a[3]),
+                           make_float2(a[4], a[5]), make_float2(a[6], a[7])};
+      snb = row_sum_x2(x, ns - 8 * (lg.nl - 1), lg.nl, lg.sl);
+    } else {
+      // (the even nodes and the odd ones, then the two)
+      const T lo = ((a[0] + a[2]) + a[4]) + a[6], up = ((a[1] + a[3]) + a[5]) + a[7];
+      snb = packed_sum(lo + up, lg.nl, lg.sl);
+    }
     if (act) store_packed<T, VW>((direct ? dst : stage) + off, lg.nv, M);
     if (lg.first && act) s_nb_chunk[r] = snb * ds;
   }

@@ -386,10 +386,7 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& a, int block)
 #pragma unroll
           for (int h = 0; h < 4; ++h) M[h] = __fmul2_rn(M[h], valid[h]);
         }
-        float2 acc = M[0];
-#pragma unroll
-        for (int h = 1; h < 4; ++h) acc = __fadd2_rn(acc, M[h]);
-        const float snb = packed_sum(acc.x + acc.y, nl, sl);
+        const float snb = row_sum_x2(M, RAG ? a.vl : 8, nl, sl);
         const int R = p * rpp + rslot;
         if (first && lane_ok && R < nrows) s_nb[R] = snb * ds;
         j += jq;

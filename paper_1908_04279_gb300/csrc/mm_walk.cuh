@@ -318,6 +318,42 @@ __device__ __forceinline__ T packed_sum(T x, int nl, int sl) {
   return x;
 }
 
+// Sum of a float32 row held eight nodes to a lane (M: the lane's nodes, zero
+// past the row's end; vl: nodes of its last lane), valid in its first lane. The
+// additions are those of the kernels that hold a row V nodes to a lane, V the
+// widest of 8, 4 and 1 that divides ns -- a lane's even and odd nodes, then the
+// two, then the lanes in halving strides -- so that n_b has the same bits
+// wherever a row is summed. Gradients need that: which Superbee branch nearly tied
+// differences take follows the last bits of n_b through the substeps, and
+// derivatives in k_off and v_walk, small differences of large terms, then move
+// by up to 2e-4 (41 x 37 x 52 x 14 over 60 substeps). V = 4: the two halves of a
+// lane as a lane each, the last stride between them. V = 1: the strides of 16
+// and 8 nodes across lanes for each node of a lane, then 4, 2 and 1 within it.
+__device__ __forceinline__ float row_sum_x2(const float2 (&M)[4], int vl, int nl, int sl) {
+  if (vl == 8) {
+    const float2 a = __fadd2_rn(__fadd2_rn(__fadd2_rn(M[0], M[1]), M[2]), M[3]);
+    return packed_sum(a.x + a.y, nl, sl);
+  }
+  if (vl == 4) {
+    const float2 a = __fadd2_rn(M[0], M[1]), b = __fadd2_rn(M[2], M[3]);
+    return packed_sum(a.x + a.y, nl, sl) + packed_sum(b.x + b.y, nl, sl);
+  }
+  float2 s[4] = {M[0], M[1], M[2], M[3]};
+#pragma unroll
+  for (int o = 2; o > 0; o >>= 1) {  // (ns <= 32 here: four lanes at most)
+    if (o < nl) {
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const float2 y = make_float2(__shfl_down_sync(0xffffffffu, s[h].x, o),
+                                     __shfl_down_sync(0xffffffffu, s[h].y, o));
+        if (sl + o < nl) s[h] = __fadd2_rn(s[h], y);
+      }
+    }
+  }
+  const float2 a = __fadd2_rn(__fadd2_rn(s[0], s[2]), __fadd2_rn(s[1], s[3]));
+  return a.x + a.y;
+}
+
 template <typename T>
 __device__ __forceinline__ T seg_sum(T x, int seg) {
   for (int o = seg >> 1; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o, seg);
