@@ -697,67 +697,46 @@ __global__ void __launch_bounds__(128) k_anchor_scatter(const AnchorArgs<T> x, c
 }
 
 // The motor force of Eq. 10 in the cells under the heads, F sum p psi Mb ds
-// dtheta over the configurations anchored at the cell, as a gather: a warp per
-// anchor cell, lanes over the configurations (k, j), each read from the filament
-// cell its offset names (neighbouring nodes mostly share it, so a warp reads
-// runs of a row). Every motor value is read once, the sum has a fixed order
-// (float-float in the float32 form) and needs no atomics: two float64 atomics
-// per run of a row took 200 us at 128^2 x 32^2, l/L = 0.05.
+// dtheta over the configurations anchored at the cell, as a gather in float64:
+// every motor value is read once, the sum has a fixed order and needs no atomics
+// (two float64 atomics per run of a row took 200 us at 128^2 x 32^2, l/L = 0.05). A
+// warp takes an anchor cell, `seg` lanes an orientation: lane sl its nodes sl, sl +
+// seg, ..., each read from the filament cell its offset names (neighbouring nodes
+// mostly share it, so that a warp reads runs of a row). Bound by the float64
+// pipe: a lane sums psi Mb over its nodes of an orientation before the two
+// components of p come in, one operation a configuration and two for the four
+// or more of a lane (float-float sums ran on the float32 pipe, with errors of 2^-48
+// in place of 2^-53).
 template <typename T>
 __global__ void __launch_bounds__(128)
     k_anchor_force(const int2* off, const T* mb, const T* psi, const double* trig64,
-                   const DevParams* prm, int nx, int ny, int nth, int ns, double ds, double dth,
-                   long long ncells, double* fx, double* fy) {
+                   const DevParams* prm, int nx, int ny, int nth, int ns, int seg, double ds,
+                   double dth, long long ncells, double* fx, double* fy) {
   const int lane = threadIdx.x & 31;
-  const float2* wf = reinterpret_cast<const float2*>(trig64 + 14 * (size_t)nth);
-  const int kq = 32 / ns, jr = 32 - kq * ns, k0 = lane / ns, j0 = lane - k0 * ns;
-  const int nconf = nth * ns;
+  const int sl = lane & (seg - 1), rslot = lane / seg, rpp = 32 / seg;
   for (long long cell = blockIdx.x * 4LL + (threadIdx.x >> 5); cell < ncells;
        cell += (long long)gridDim.x * 4) {
     const int ay = (int)cell / nx, ax = (int)cell - ay * nx;
-    FF sx{0.f, 0.f}, sy{0.f, 0.f};
     double dx = 0.0, dy = 0.0;
-    int k = k0, j = j0;
+    for (int k = rslot; k < nth; k += rpp) {
+      double q = 0.0;
 #pragma unroll 4
-    for (int e = lane; e < nconf; e += 32) {
-      const int2 o = off[e];
-      int fxc = ax - o.x, fyc = ay - o.y;
-      fxc += fxc < 0 ? nx : 0;
-      fyc += fyc < 0 ? ny : 0;
-      const size_t row = ((size_t)fyc * nx + fxc) * nth + k;
-      const T m = mb[row * ns + j], p = psi[row];
-      if constexpr (sizeof(T) == 4) {
-        const float2 c = wf[5 * (size_t)nth + k], s = wf[6 * (size_t)nth + k];
-        const FF pm = ff_scale(p, FF{m, 0.f});
-        sx = ff_sum(sx, ff_prod(pm, FF{c.x, c.y}));
-        sy = ff_sum(sy, ff_prod(pm, FF{s.x, s.y}));
-      } else {
-        dx = fma(p * m, trig64[k], dx);
-        dy = fma(p * m, trig64[nth + k], dy);
+      for (int j = sl; j < ns; j += seg) {
+        const int2 o = off[k * ns + j];
+        int fxc = ax - o.x, fyc = ay - o.y;
+        fxc += fxc < 0 ? nx : 0;
+        fyc += fyc < 0 ? ny : 0;
+        const size_t row = ((size_t)fyc * nx + fxc) * nth + k;
+        q = fma(widen(psi[row]), widen(mb[row * ns + j]), q);
       }
-      k += kq;
-      j += jr;
-      if (j >= ns) {
-        j -= ns;
-        ++k;
-      }
+      dx = fma(q, trig64[k], dx);
+      dy = fma(q, trig64[nth + k], dy);
     }
-    if constexpr (sizeof(T) == 4) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        sx = ff_sum(sx, FF{__shfl_xor_sync(0xffffffffu, sx.hi, o),
-                           __shfl_xor_sync(0xffffffffu, sx.lo, o)});
-        sy = ff_sum(sy, FF{__shfl_xor_sync(0xffffffffu, sy.hi, o),
-                           __shfl_xor_sync(0xffffffffu, sy.lo, o)});
-      }
-      if (lane < 2) dx = lane == 0 ? (double)sx.hi + (double)sx.lo : (double)sy.hi + (double)sy.lo;
-    } else {
-      dx = warp_sum(dx);
-      dy = warp_sum(dy);
-      if (lane == 1) dx = dy;
-    }
+    dx = warp_sum(dx);
+    dy = warp_sum(dy);
     if (lane < 2)
-      (lane == 0 ? fx : fy)[cell] = dx * (prm->force_scale * prm->psi_scale * ds * dth);
+      (lane == 0 ? fx : fy)[cell] =
+          (lane == 0 ? dx : dy) * (prm->force_scale * prm->psi_scale * ds * dth);
   }
 }
 
@@ -902,9 +881,11 @@ cudaError_t anchor_scatter_t(mm_handle* h) {
 
 template <typename T>
 cudaError_t anchor_force_t(mm_handle* h, double* fx, double* fy) {
+  int seg = 1;  // at least four nodes to a lane where a row has them
+  while (seg < 8 && 8 * seg <= h->g.ns) seg <<= 1;
   mm::k_anchor_force<T><<<blocks_for(h->ncells, 4, 16 * h->sms), 128, 0, h->stream>>>(
       (const int2*)h->anc_off, (const T*)h->mb, (const T*)h->psi[h->parity], h->trig64, h->prm,
-      h->g.nx, h->g.ny, h->g.ntheta, h->g.ns, h->g.L / h->g.ns, 2.0 * kPi / h->g.ntheta,
+      h->g.nx, h->g.ny, h->g.ntheta, h->g.ns, seg, h->g.L / h->g.ns, 2.0 * kPi / h->g.ntheta,
       h->ncells, fx, fy);
   return cudaGetLastError();
 }

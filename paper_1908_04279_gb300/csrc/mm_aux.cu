@@ -28,18 +28,6 @@ __global__ void k_copy_multi(const CopySegs c) {
   }
 }
 
-// float32 to float64 on the integer and float32 pipes (exact; the conversion
-// instruction runs on the narrow float64 pipe, which held the exports at 4.7 TB/s
-// of the 6.8 a copy reaches): the exponent rebiased, subnormal values brought
-// into the normal range first.
-__device__ __forceinline__ double widen(float x) {
-  const unsigned u0 = __float_as_uint(x), mag = u0 & 0x7fffffffu;
-  const bool sub = mag < 0x00800000u;
-  const unsigned u = __float_as_uint(x * (sub ? 16777216.0f : 1.0f));
-  const unsigned bias = sub ? 0x36800000u : mag < 0x7f800000u ? 0x38000000u : 0x70000000u;
-  const unsigned hi = mag == 0u ? 0u : ((u & 0x7fffffffu) >> 3) + bias;
-  return __hiloint2double((int)(hi | (u0 & 0x80000000u)), (int)(u << 29));
-}
 template <typename TO, typename TI>
 __device__ __forceinline__ TO converted(TI x) {
   if constexpr (sizeof(TO) == 8 && sizeof(TI) == 4)
@@ -156,16 +144,16 @@ __global__ void __launch_bounds__(kDtBlock)
 
 constexpr int kMomPasses = 4;  // passes of rows in flight before they are reduced
 
-// Set-up of a state, a warp per cell: n_b of every row (float-float in the
-// float32 form: exact to 2^-48 before its one rounding), C = sum_k psi n_b
-// dtheta, the Alg. 2 scale-down where C > M, Mf = M - C. Bound by HBM beyond
-// the L2: every lane loads 32 (64) consecutive bytes, four passes of rows in
-// flight per warp (a thread per row, one node per load and a float64 sum per
-// node took 90 us at 128^2 x 32^2 where the bytes need 10).
+// Set-up of a state, a warp per cell, in float64 for either state precision: n_b
+// of every row, C = sum_k psi n_b dtheta, the Alg. 2 scale-down where C > M, Mf =
+// M - C (which may cancel: float-float sums left 2^-47 of C in it). Bound by the
+// float64 pipe, one operation a node: every lane loads 32 (64) consecutive
+// bytes, four passes of rows in flight per warp (a thread per row, one node per
+// load and a serial sum took 90 us at 128^2 x 32^2 where the bytes need 10).
 template <typename T, int VW>
 __global__ void __launch_bounds__(128)
     k_init_cells(T* mb, const T* psi, T* nb, T* mf, T* c, const T* mtot, int ncells, int nth,
-                 int ns, double ds, double dth, float2 dsf, float2 dthf) {
+                 int ns, double ds, double dth) {
   const int lane = threadIdx.x & 31;
   const PackedGeom g = packed_geom(lane, ns);
   const int gw = blockIdx.x * 4 + (threadIdx.x >> 5), W = gridDim.x * 4;
@@ -174,7 +162,6 @@ __global__ void __launch_bounds__(128)
     T* rows = mb + (size_t)cell * nth * ns + g.sl * 8;
     const T* pc = psi + (size_t)cell * nth;
     T* nbc = nb + (size_t)cell * nth;
-    FF accf{0.f, 0.f};
     double acc = 0.0;
     for (int r0 = 0; r0 < nth; r0 += kMomPasses * g.rpp) {
       T m[kMomPasses][8];
@@ -185,78 +172,30 @@ __global__ void __launch_bounds__(128)
       }
 #pragma unroll
       for (int u = 0; u < kMomPasses; ++u) {
+        if (r0 + u * g.rpp >= nth) break;  // (every lane)
         const int k = r0 + u * g.rpp + g.rslot;
-        const bool own = g.sl == 0 && g.rslot < g.rpp && k < nth;
-        if constexpr (sizeof(T) == 4) {
-          const FF s = packed_sum_ff<0>(row_sum8(m[u]), g.nl, g.sl);
-          if (own) {
-            const FF n = ff_prod(s, FF{dsf.x, dsf.y});
-            nbc[k] = n.hi + n.lo;
-            accf = ff_sum(accf, ff_scale(pc[k], n));
-          }
-        } else {
-          const double s =
-              packed_sum(((m[u][0] + m[u][1]) + (m[u][2] + m[u][3])) +
-                             ((m[u][4] + m[u][5]) + (m[u][6] + m[u][7])),
-                         g.nl, g.sl) *
-              ds;
-          if (own) {
-            nbc[k] = s;
-            acc = fma(pc[k], s, acc);
-          }
+        double x[8];
+#pragma unroll
+        for (int v = 0; v < 8; ++v) x[v] = widen(m[u][v]);
+        const double s = packed_sum(((x[0] + x[1]) + (x[2] + x[3])) +
+                                        ((x[4] + x[5]) + (x[6] + x[7])),
+                                    g.nl, g.sl) *
+                         ds;
+        if (g.sl == 0 && g.rslot < g.rpp && k < nth) {
+          nbc[k] = (T)s;
+          acc = fma(widen(pc[k]), s, acc);
         }
       }
     }
     // C, and the scale-down where it exceeds the total motors
-    const T M = mtot[cell];
-    double C = 0.0;
-    bool over;
-    if constexpr (sizeof(T) == 4) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
-        accf = ff_sum(accf, FF{__shfl_xor_sync(0xffffffffu, accf.hi, o),
-                               __shfl_xor_sync(0xffffffffu, accf.lo, o)});
-      const FF Cf = ff_prod(accf, FF{dthf.x, dthf.y});
-      const FF left = ff_sum(FF{M, 0.f}, FF{-Cf.hi, -Cf.lo});  // M - C
-      const float mfc = left.hi + left.lo;
-      if (fabsf(mfc) <= 3.402823466e38f) {
-        over = mfc < 0.f;
-        C = over ? (double)Cf.hi + (double)Cf.lo : 0.0;
-        if (!over && lane == 0) {
-          c[cell] = Cf.hi + Cf.lo;
-          mf[cell] = mfc;
-        }
-      } else {
-        // sums beyond float32 (or not finite): the cell again in float64
-        for (int k = lane; k < nth; k += 32) {
-          const T* row = mb + ((size_t)cell * nth + k) * ns;
-          double s = 0.0;
-          for (int j = 0; j < ns; ++j) s += (double)row[j] * ds;
-          nbc[k] = (T)s;
-          acc += (double)pc[k] * s * dth;
-        }
-        C = warp_sum(acc);
-        over = (double)M < C;
-        if (!over && lane == 0) {
-          c[cell] = (T)C;
-          mf[cell] = (T)((double)M - C);
-        }
-        __syncwarp();
-      }
-    } else {
-      C = warp_sum(acc) * dth;
-      over = M < C;
-      if (!over && lane == 0) {
-        c[cell] = C;
-        mf[cell] = M - C;
-      }
+    const double M = widen(mtot[cell]), C = warp_sum(acc) * dth;
+    const bool over = M < C;
+    if (lane == 0) {
+      c[cell] = (T)(over ? M : C);
+      mf[cell] = (T)(over ? 0.0 : M - C);
     }
     if (over) {
-      const double f = (double)M / C;
-      if (lane == 0) {
-        c[cell] = M;
-        mf[cell] = T(0);
-      }
+      const double f = M / C;
       __syncwarp();
       T* all = mb + (size_t)cell * nth * ns;
       for (int e = lane; e < nth * ns; e += 32) all[e] = (T)((double)all[e] * f);
@@ -722,10 +661,6 @@ int row_vector(int ns) {
     if (ns % v == 0) return v;
   return 1;
 }
-float2 float_pair(double x) {
-  const float hi = (float)x;
-  return make_float2(hi, (float)(x - (double)hi));
-}
 
 template <typename T>
 cudaError_t launch_init_cells(T* mb, const T* psi, T* nb, T* mf, T* c, const T* mtot,
@@ -733,8 +668,7 @@ cudaError_t launch_init_cells(T* mb, const T* psi, T* nb, T* mf, T* c, const T* 
                               cudaStream_t s) {
   const int g = grid_for(ncells * 32, 128);
   auto go = [&](auto kern) {
-    kern<<<g, 128, 0, s>>>(mb, psi, nb, mf, c, mtot, (int)ncells, nth, ns, ds, dth,
-                           float_pair(ds), float_pair(dth));
+    kern<<<g, 128, 0, s>>>(mb, psi, nb, mf, c, mtot, (int)ncells, nth, ns, ds, dth);
     return cudaGetLastError();
   };
   const int vw = row_vector<T>(ns);

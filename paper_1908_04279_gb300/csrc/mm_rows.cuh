@@ -7,6 +7,20 @@
 
 namespace mm {
 
+// float32 to float64 on the integer and float32 pipes (exact; the conversion
+// instruction runs on the narrow float64 pipe, which held the exports at 4.7 TB/s
+// of the 6.8 a copy reaches, and which bounds the float64 sums): the exponent
+// rebiased, subnormal values brought into the normal range first.
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u0 = __float_as_uint(x), mag = u0 & 0x7fffffffu;
+  const bool sub = mag < 0x00800000u;
+  const unsigned u = __float_as_uint(x * (sub ? 16777216.0f : 1.0f));
+  const unsigned bias = sub ? 0x36800000u : mag < 0x7f800000u ? 0x38000000u : 0x70000000u;
+  const unsigned hi = mag == 0u ? 0u : ((u & 0x7fffffffu) >> 3) + bias;
+  return __hiloint2double((int)(hi | (u0 & 0x80000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 // Compensated float32 accumulator (hi + lo), error-free transformations of
 // Knuth (TwoSum) and of the fused multiply-add (TwoProduct).
 struct FF {
@@ -87,24 +101,9 @@ __device__ __forceinline__ void ff2x_add(FF2x& a, float2 x) {
   a.lo = __fadd2_rn(a.lo, __fadd2_rn(e1, e2));
   a.hi = s;
 }
-__device__ __forceinline__ FF ff2x_fold(const FF2x& a) {
-  return ff_sum(FF{a.hi.x, a.lo.x}, FF{a.hi.y, a.lo.y});
-}
-// Sum over the nl lanes of a packed row, valid in its first lane. NL: nl where
+// Sums over the nl lanes of a packed row, valid in its first lane. NL: nl where
 // it is a power of two known at compile time (what the other lanes pick up
 // from the next row is not used), else 0.
-template <int NL>
-__device__ __forceinline__ FF packed_sum_ff(FF x, int nl, int sl) {
-#pragma unroll
-  for (int o = NL ? NL / 2 : 16; o > 0; o >>= 1) {
-    if (NL || o < nl) {
-      const FF y{__shfl_down_sync(0xffffffffu, x.hi, o), __shfl_down_sync(0xffffffffu, x.lo, o)};
-      if (NL || sl + o < nl) x = ff_sum(x, y);
-    }
-  }
-  return x;
-}
-// The same of two sums at once.
 template <int NL>
 __device__ __forceinline__ FF2x packed_sum_ff2x(FF2x x, int nl, int sl) {
   const float2 m1 = make_float2(-1.f, -1.f);
@@ -127,27 +126,6 @@ __device__ __forceinline__ FF2x packed_sum_ff2x(FF2x x, int nl, int sl) {
   x.lo = __ffma2_rn(__ffma2_rn(x.hi, m1, s), m1, x.lo);
   x.hi = s;
   return x;
-}
-
-// m1 / ds and n_b / ds of a lane's nodes, the nodes even and odd apart.
-__device__ __forceinline__ FF row_dot8(const float (&m)[8], const float (&sj)[8]) {
-  FF2x t{{0.f, 0.f}, {0.f, 0.f}};
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    const float2 x = make_float2(m[2 * v], m[2 * v + 1]);
-    const float2 w = make_float2(sj[2 * v], sj[2 * v + 1]);
-    const float2 p = __fmul2_rn(x, w);
-    const float2 pe = __ffma2_rn(x, w, make_float2(-p.x, -p.y));
-    ff2x_add(t, p);
-    t.lo = __fadd2_rn(t.lo, pe);
-  }
-  return ff2x_fold(t);
-}
-__device__ __forceinline__ FF row_sum8(const float (&m)[8]) {
-  FF2x s{{0.f, 0.f}, {0.f, 0.f}};
-#pragma unroll
-  for (int v = 0; v < 4; ++v) ff2x_add(s, make_float2(m[2 * v], m[2 * v + 1]));
-  return ff2x_fold(s);
 }
 
 // n_b / ds (first) and m1 / ds (second) of a lane's nodes, one pair of

@@ -512,35 +512,26 @@ __global__ void __launch_bounds__(128, tan_min_blocks<T, V>()) k_substep_tl(cons
 // The sums a built-in observable and its derivative need: sum psi cos, sum psi
 // sin, sum psi, sum psi m1, and the same of the tangent (psi taken with the
 // pending correction factor g, dpsi with g as a constant), over all cells into
-// tot[8]. A warp per cell: the rows' m1 of Mb and dMb (packed rows, eight nodes
-// per lane), then lanes over theta; float-float in the float32 form. Partial
-// sums per warp, block and last block in a fixed order. Bound by HBM beyond the
-// L2 (a thread per row with a float64 sum per node and one warp for the total
-// took 620 us at 128^2 x 32^2).
+// tot[8], in float64 for either state precision. A warp per cell: the rows' m1
+// of Mb and dMb (packed rows, eight nodes per lane), then lanes over theta.
+// Partial sums per warp, block and last block in a fixed order. Bound by the
+// float64 pipe, two operations a node (a thread per row and one warp for the
+// total took 620 us at 128^2 x 32^2, float-float sums on the float32 pipe 70,
+// with errors of 2^-48 in place of 2^-53).
 template <typename T, int VW>
 __global__ void __launch_bounds__(128)
     k_tan_sums(const T* psi, const T* mb, const T* dpsi, const T* dmb, const double* trig64,
-               DevParams* prm, long long ncells, int nth, int ns, double ds, double L,
-               double* partial, double* tot) {
+               DevParams* prm, long long ncells, int nth, int ns, double ds, double* partial,
+               double* tot) {
   extern __shared__ __align__(16) unsigned char tan_raw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const PackedGeom pg = packed_geom(lane, ns);
-  double2* s_d = reinterpret_cast<double2*>(tan_raw) + (size_t)wib * nth;  // m1, dm1 over their unit
-  float4* s_f = reinterpret_cast<float4*>(tan_raw) + (size_t)wib * nth;    // (float pairs)
+  double2* s_d = reinterpret_cast<double2*>(tan_raw) + (size_t)wib * nth;  // 2 m1 / ds^2, of Mb and dMb
   const double g = prm->psi_scale;
-  T sj[8];
+  double sj[8];
 #pragma unroll
-  for (int v = 0; v < 8; ++v) {
-    if constexpr (sizeof(T) == 4)
-      sj[v] = (float)(2 * (pg.sl * 8 + v) + 1 - ns);  // 2 s_j / ds, an integer
-    else
-      sj[v] = -0.5 * L + ((double)(pg.sl * 8 + v) + 0.5) * ds;
-  }
+  for (int v = 0; v < 8; ++v) sj[v] = (double)(2 * (pg.sl * 8 + v) + 1 - ns);  // 2 s_j / ds
   double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  FF f[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) f[q] = FF{0.f, 0.f};
-  const float2* wf = reinterpret_cast<const float2*>(trig64 + 14 * (size_t)nth);
   for (long long cell = blockIdx.x * 4LL + wib; cell < ncells; cell += (long long)gridDim.x * 4) {
     for (int r0 = 0; r0 < nth; r0 += 2 * pg.rpp) {
       T m[4][8];
@@ -553,54 +544,33 @@ __global__ void __launch_bounds__(128)
       }
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
+        if (r0 + u * pg.rpp >= nth) break;  // (every lane)
         const int k = r0 + u * pg.rpp + pg.rslot;
-        const bool own = pg.sl == 0 && pg.rslot < pg.rpp && k < nth;
-        if constexpr (sizeof(T) == 4) {
-          const FF a = packed_sum_ff<0>(row_dot8(m[2 * u], sj), pg.nl, pg.sl);
-          const FF b = packed_sum_ff<0>(row_dot8(m[2 * u + 1], sj), pg.nl, pg.sl);
-          if (own) s_f[k] = make_float4(a.hi, a.lo, b.hi, b.lo);
-        } else {
-          double a = 0.0, b = 0.0;
+        double a = 0.0, b = 0.0;
 #pragma unroll
-          for (int v = 0; v < 8; ++v) {
-            a = fma(sj[v], m[2 * u][v], a);
-            b = fma(sj[v], m[2 * u + 1][v], b);
-          }
-          a = packed_sum(a, pg.nl, pg.sl);
-          b = packed_sum(b, pg.nl, pg.sl);
-          if (own) s_d[k] = make_double2(a, b);
+        for (int v = 0; v < 8; ++v) {
+          a = fma(sj[v], widen(m[2 * u][v]), a);
+          b = fma(sj[v], widen(m[2 * u + 1][v]), b);
         }
+        a = packed_sum(a, pg.nl, pg.sl);
+        b = packed_sum(b, pg.nl, pg.sl);
+        if (pg.sl == 0 && pg.rslot < pg.rpp && k < nth) s_d[k] = make_double2(a, b);
       }
     }
     __syncwarp();
     for (int k = lane; k < nth; k += 32) {
       const size_t r = (size_t)cell * nth + k;
-      const T p = psi[r], dp = dpsi[r];
-      if constexpr (sizeof(T) == 4) {
-        const float2 ct = wf[5 * (size_t)nth + k], st = wf[6 * (size_t)nth + k];
-        const FF c{ct.x, ct.y}, sn{st.x, st.y};
-        const float4 m = s_f[k];
-        const FF m1{m.x, m.y}, dm1{m.z, m.w};
-        f[0] = ff_sum(f[0], ff_scale(p, c));
-        f[1] = ff_sum(f[1], ff_scale(p, sn));
-        ff_add(f[2], p);
-        f[3] = ff_sum(f[3], ff_scale(p, m1));
-        f[4] = ff_sum(f[4], ff_scale(dp, c));
-        f[5] = ff_sum(f[5], ff_scale(dp, sn));
-        ff_add(f[6], dp);
-        f[7] = ff_sum(f[7], ff_sum(ff_scale(dp, m1), ff_scale(p, dm1)));
-      } else {
-        const double c = trig64[k], sn = trig64[nth + k];
-        const double2 m = s_d[k];
-        s[0] = fma(p, c, s[0]);
-        s[1] = fma(p, sn, s[1]);
-        s[2] += p;
-        s[3] = fma(p, m.x, s[3]);
-        s[4] = fma(dp, c, s[4]);
-        s[5] = fma(dp, sn, s[5]);
-        s[6] += dp;
-        s[7] += dp * m.x + p * m.y;
-      }
+      const double p = widen(psi[r]), dp = widen(dpsi[r]);
+      const double c = trig64[k], sn = trig64[nth + k];
+      const double2 m = s_d[k];
+      s[0] = fma(p, c, s[0]);
+      s[1] = fma(p, sn, s[1]);
+      s[2] += p;
+      s[3] = fma(p, m.x, s[3]);
+      s[4] = fma(dp, c, s[4]);
+      s[5] = fma(dp, sn, s[5]);
+      s[6] += dp;
+      s[7] = fma(p, m.y, fma(dp, m.x, s[7]));
     }
     __syncwarp();
   }
@@ -608,15 +578,7 @@ __global__ void __launch_bounds__(128)
   __shared__ unsigned int s_last;
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    if constexpr (sizeof(T) == 4) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
-        f[q] = ff_sum(f[q], FF{__shfl_xor_sync(0xffffffffu, f[q].hi, o),
-                               __shfl_xor_sync(0xffffffffu, f[q].lo, o)});
-      s[q] = (double)f[q].hi + (double)f[q].lo;
-    } else {
-      s[q] = warp_sum(s[q]);
-    }
+    s[q] = warp_sum(s[q]);
     if (lane == 0) s_part[wib][q] = s[q];
   }
   __syncthreads();
@@ -633,8 +595,7 @@ __global__ void __launch_bounds__(128)
   __threadfence();
   for (int q = wib; q < 8; q += 4) {
     const double t = warp_sum_ldcg(partial + q, (int)gridDim.x, 8, lane);
-    const double m1 = sizeof(T) == 4 ? 0.5 * ds * ds : ds;  // the row sums' unit
-    if (lane == 0) tot[q] = g * (q == 3 || q == 7 ? m1 * t : t);
+    if (lane == 0) tot[q] = g * (q == 3 || q == 7 ? 0.5 * ds * ds * t : t);
   }
 }
 
@@ -847,7 +808,7 @@ mm_status mm_tangent_observable(mm_handle* h, int observable, double* value, dou
     }
     kern<<<grid, 128, smem, h->stream>>>((const T*)h->psi[h->parity], (const T*)h->mb,
                                          (const T*)h->tan_psi[h->parity], (const T*)h->tan_mb,
-                                         h->trig64, h->prm, nc, nth, ns, ds, h->g.L, cells, tot);
+                                         h->trig64, h->prm, nc, nth, ns, ds, cells, tot);
     return cudaGetLastError();
   };
   if (h->prec == MM_FP64)

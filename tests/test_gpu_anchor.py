@@ -329,3 +329,27 @@ def test_anchor_large512_conservation_and_sampled_anchors(mmod, oracle_mod):
         got = float(c[int(ay), int(ax)])
         assert abs(got - want) <= 1e-5 * abs(want), (int(ay), int(ax), got, want)
         assert abs(float(mf[int(ay), int(ax)]) + got - 1.0) <= 1e-6
+
+
+@pytest.mark.parametrize("nth,ns", [(8, 6), (5, 32), (40, 24)])
+def test_force_of_a_float32_state_is_a_float64_sum(mmod, nth, ns):
+    """One bound motor value per filament cell, one orientation each: the force at
+    its anchor is a product of six factors, at most eight roundings of 2^-53 off
+    (the heads stay in the filament's own cell: l/L = 0)."""
+    g = Grid(16, 12, nth, ns)
+    r = Rates(force_scale=1.7, ell=0.0)
+    rng = SplitMix64(71)
+    k, j = ((rng.uniforms(g.ncells) * n).astype(int) for n in (nth, ns))
+    p, m = ((0.2 + rng.uniforms(g.ncells)).astype(np.float32).astype(float) for _ in range(2))
+    psi, mb = np.zeros((g.ncells, nth)), np.zeros((g.ncells, nth, ns))
+    at = np.arange(g.ncells)
+    psi[at, k], mb[at, k, j] = p, m
+    with mmod.Simulation(g, r, "fp32") as sim:
+        sim.set_anchors(True)
+        sim.set_state(psi.reshape(g.ny, g.nx, -1), mb.reshape(g.ny, g.nx, nth, ns))
+        f, _ = sim.moments()
+    th = k * (2 * np.pi / nth)
+    for name, w in (("Fx", np.cos(th)), ("Fy", np.sin(th))):
+        want = (p.astype(np.longdouble) * m * w * r.force_scale * (g.L / ns) * (2 * np.pi / nth))
+        off = np.abs(f[name].reshape(-1) - want)
+        assert np.all(off <= 8 * 2.0 ** -53 * np.abs(want)), float(np.max(off / np.abs(want)))

@@ -132,3 +132,26 @@ def test_tangent_widths(mmod, dims):
                                                       for k in ("psi", "mb", "mf")}}
     for k, v in got["fp64"].items():
         assert rel_l2(got["fp32"][k], v) <= 2e-5, k
+
+
+@pytest.mark.parametrize("nth,ns", [(8, 6), (40, 32), (5, 30)])
+def test_free_motors_of_a_float32_state_under_cancellation(mmod, nth, ns):
+    """Mf = M - C of a loaded float32 state is formed in float64: with one motor
+    value and one filament density per cell C is a product of four factors (four
+    roundings of 2^-53), M the next float32 above it, and Mf is rounded once."""
+    g = Grid(64, 48, nth, ns)
+    rng = SplitMix64(83)
+    k, j = ((rng.uniforms(g.ncells) * n).astype(int) for n in (nth, ns))
+    p, m = ((0.2 + rng.uniforms(g.ncells)).astype(np.float32).astype(float) for _ in range(2))
+    psi, mb = np.zeros((g.ncells, nth)), np.zeros((g.ncells, nth, ns))
+    at = np.arange(g.ncells)
+    psi[at, k], mb[at, k, j] = p, m
+    C = p.astype(np.longdouble) * m * (g.L / ns) * (2 * np.pi / nth)
+    M = np.nextafter(C.astype(np.float32), np.float32(np.inf)).astype(float)
+    with mmod.Simulation(g, Rates(), "fp32") as sim:
+        sim.set_state(psi.reshape(g.ny, g.nx, -1), mb.reshape(g.ny, g.nx, nth, ns),
+                      M.reshape(g.ny, g.nx))
+        got = sim.get_state()["mf"].reshape(-1)
+    want = M - C
+    off = np.abs(got - want) - 2.0 ** -24 * np.abs(want) - 4 * 2.0 ** -53 * C
+    assert np.all(off <= 0), float(np.max(off / C) * 2.0 ** 53)

@@ -204,3 +204,28 @@ def test_tangent_refusals(mmod):
         sim.set_capture(0.1)
         with pytest.raises(mmod.MMError):
             sim.set_tangent(DP)
+
+
+def test_observable_sums_are_float64(mmod):
+    """The built-in observables of a float32 state are summed in float64: with one
+    motor value and one filament density that are not zero the mean stress is a
+    product of seven factors, at most eight roundings of 2^-53 off."""
+    g = Grid(3, 2, 8, 24)
+    r = Rates(force_scale=1.7, ell=0.3)
+    rng = SplitMix64(61)
+    worst = 0.0
+    for _ in range(24):
+        cell, k, j = (int(rng.uniform() * n) for n in (g.ncells, g.ntheta, g.ns))
+        p, m = (float(np.float32(0.2 + rng.uniform())) for _ in range(2))
+        psi, mb = np.zeros((g.ncells, g.ntheta)), np.zeros((g.ncells, g.ntheta, g.ns))
+        psi[cell, k], mb[cell, k, j] = p, m
+        with mmod.Simulation(g, r, "fp32") as sim:
+            sim.set_tangent(DP)
+            sim.set_state(psi.reshape(g.ny, g.nx, -1), mb.reshape(g.ny, g.nx, g.ntheta, -1))
+            got, _ = sim.tangent_observable("mean_stress")
+        ld = np.longdouble
+        s = (2 * j + 1 - g.ns) * ld(g.L / g.ns) / 2
+        want = ld(r.force_scale) * ld(r.ell) * ld(2 * np.pi / g.ntheta) / g.ncells * (
+            ld(p) * s * ld(m) * ld(g.L / g.ns))
+        worst = max(worst, abs(float((ld(got) - want) / want)))
+    assert worst <= 8 * 2.0 ** -53, worst
