@@ -368,6 +368,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1) k_moments(const T
       }
 #pragma unroll
       for (int u = 0; u < kMomPasses; ++u) {
+        if (r0 + u * rpp >= nth) break;  // (every lane)
         const int k = r0 + u * rpp + rslot;
         const bool own = sl == 0 && rslot < rpp && k < nth;
         if constexpr (sizeof(T) == 4) {
@@ -724,9 +725,15 @@ cudaError_t launch_moments(const T* psi, const T* mb, const T* mf, const T* c,
   };
   const int vw = row_vector<T>(ns);
   if constexpr (sizeof(T) == 4) {
-    if (ns == 64) return go(k_moments<T, 4, 8>);
-    if (ns == 32) return go(k_moments<T, 4, 4>);
-    if (ns == 16) return go(k_moments<T, 4, 2>);
+    // rows of a power of two of full lanes: the cross-lane sums unrolled
+    switch (ns % 8 == 0 ? ns / 8 : 0) {
+      case 1: return go(k_moments<T, 4, 1>);
+      case 2: return go(k_moments<T, 4, 2>);
+      case 4: return go(k_moments<T, 4, 4>);
+      case 8: return go(k_moments<T, 4, 8>);
+      case 16: return go(k_moments<T, 4, 16>);
+      case 32: return go(k_moments<T, 4, 32>);
+    }
     if (vw == 4) return go(k_moments<T, 4, 0>);
   }
   return vw == 2 ? go(k_moments<T, 2, 0>) : go(k_moments<T, 1, 0>);

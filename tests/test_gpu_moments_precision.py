@@ -58,3 +58,9 @@ def test_float_float_moments_of_the_gpu_state(mmod, oracle_mod, dims, exact_s):
     for k in osc:
         tol = 1e-7 if (k == "mean_stress" and not exact_s) else 1e-11
         assert abs(gsc[k] - osc[k]) <= tol * max(abs(osc[k]), 1e-300), (k, gsc[k], osc[k])
+
+
+# rows of one, 16 and 32 lanes, cells of less than one pass of rows and of several
+@pytest.mark.parametrize("dims", [(7, 6, 5, 8), (6, 5, 70, 8), (5, 4, 9, 128), (3, 4, 6, 256)])
+def test_moments_at_each_lane_count(mmod, oracle_mod, dims):
+    test_float_float_moments_of_the_gpu_state(mmod, oracle_mod, dims, True)
