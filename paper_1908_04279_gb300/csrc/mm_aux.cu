@@ -77,10 +77,17 @@ __device__ __forceinline__ void atomic_max_nonneg(double* addr, double v) {
 // latency: full occupancy hides it, and a block reduces its maxima before the
 // three atomics (one set per warp kept the atomics of one address in a queue:
 // 128^2 x 32 15 us).
+// The greater of two non-negative values, none of them NaN (float64: on the bit
+// patterns, off the narrow float64 pipe).
+__device__ __forceinline__ float max_nonneg(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double max_nonneg(double a, double b) {
+  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+  return __longlong_as_double(x > y ? x : y);
+}
 template <typename T>
-__device__ __forceinline__ T warp_max_t(T x) {
+__device__ __forceinline__ T warp_max_nonneg(T x) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x = tmax(x, __shfl_xor_sync(0xffffffffu, x, o));
+  for (int o = 16; o > 0; o >>= 1) x = max_nonneg(x, __shfl_xor_sync(0xffffffffu, x, o));
   return x;
 }
 
@@ -126,9 +133,9 @@ __global__ void __launch_bounds__(kDtBlock)
     rhomax = tmax(rhomax, seg_sum(rho, seg));
   }
   __shared__ T red[3][kDtBlock / 32];
-  adv = warp_max_t(adv);
-  rot = warp_max_t(rot);
-  rhomax = warp_max_t(rhomax);
+  adv = warp_max_nonneg(adv);
+  rot = warp_max_nonneg(rot);
+  rhomax = warp_max_nonneg(rhomax);
   if (lane == 0) {
     red[0][threadIdx.x >> 5] = adv;
     red[1][threadIdx.x >> 5] = rot;
@@ -137,7 +144,7 @@ __global__ void __launch_bounds__(kDtBlock)
   __syncthreads();
   if (threadIdx.x < 3) {
     T m = red[threadIdx.x][0];
-    for (int q = 1; q < kDtBlock / 32; ++q) m = tmax(m, red[threadIdx.x][q]);
+    for (int q = 1; q < kDtBlock / 32; ++q) m = max_nonneg(m, red[threadIdx.x][q]);
     atomic_max_nonneg(&prm->dtmax[threadIdx.x], (double)m);
   }
 }
@@ -694,7 +701,12 @@ cudaError_t launch_dt_max(const T* psi, const T* nb, const T* u, const T* trig, 
   int seg = 1;
   while (seg < 32 && seg < nth) seg <<= 1;
   int g = grid_for((ncells + 32 / seg - 1) / (32 / seg) * 32, kDtBlock);
-  if (g > 152 * 4) g = 152 * 4;
+  // at most the blocks that run at once, in float64 half of them: a block's end
+  // costs more than a shorter share of the cells saves (mm_set_velocity in us at one,
+  // two and four blocks an SM: float64 88^2 x 32 orientations 45, 49, 54, float32
+  // 528^2 x 8 60, 53, 53)
+  const int most = 152 * (sizeof(T) == 8 ? 1 : 2);
+  if (g > most) g = most;
   k_dt_max<T><<<g, kDtBlock, 0, s>>>(psi, nb, u, trig, (int)ncells, nx, ny, nth, seg, inv_dx,
                                      inv_dy, inv_dth, dth, glide, vsp, prm);
   return cudaGetLastError();
