@@ -124,7 +124,7 @@ template StepArgs<double> step_args<double>(mm_handle*, int);
 // The substep kernel of h's plan on given arguments.
 template <typename T>
 cudaError_t launch_step(const mm_handle* h, const StepArgs<T>& a, cudaStream_t s, bool overlap) {
-  return mm::launch_substep<T>(a, h->grid_step, h->block, h->smem, h->tma, s, overlap);
+  return mm::launch_substep<T>(a, h->grid_step, h->block, h->smem, h->tma, h->packed, s, overlap);
 }
 cudaError_t launch_plain(mm_handle* h, int parity, cudaStream_t s) {
   return h->prec == MM_FP64 ? launch_step(h, step_args<double>(h, parity), s, false)
@@ -174,13 +174,13 @@ cudaError_t launch_ptrs(mm_handle* h, const StepPtrs& p, cudaStream_t s) {
 
 mm_status configure(mm_handle* h) {
   const int ns = h->g.ns, nth = h->g.ntheta;
-  // values per lane of the kernels beside the substep's own: the widest
-  // instantiated vector that divides ns -- float64 {2, 1}, float32 {8, 4, 1} (two
-  // 16-byte vectors, one, or scalar lanes)
+  // values per lane where rows are not packed: the widest instantiated vector
+  // that divides ns -- float64 {2, 1}, float32 {8, 4, 1} (two 16-byte vectors, one,
+  // or scalar lanes)
   h->V = 1;
   if (h->prec == MM_FP64) {
     if (ns % 2 == 0) h->V = 2;
-  } else if (MM_FP32_VMAX >= 8 && ns % 8 == 0) {
+  } else if (ns % 8 == 0) {
     h->V = 8;
   } else if (ns % 4 == 0) {
     h->V = 4;
@@ -191,20 +191,12 @@ mm_status configure(mm_handle* h) {
   int seg = 1;
   while (seg < nl) seg <<= 1;
   h->seg = seg;
-  const size_t row_bytes = (size_t)ns * h->tsz;
-  // the fewest chunks of at most kChunkBytes, of whole 16-byte vectors where
-  // that can be had
-  int ch = 0;
-  for (int c = 1; c <= nth; ++c) {
-    if (nth % c != 0 || (c < nth && (size_t)(nth / c) * row_bytes > kChunkBytes)) continue;
-    const bool vec = (size_t)(nth / c) * row_bytes % 16 == 0;
-    if (ch == 0 || vec) ch = c;
-    if (vec) break;
-  }
-  h->chunks_per_cell = ch;
-  h->chunk_rows = nth / ch;
-  const size_t chunk_bytes = (size_t)h->chunk_rows * row_bytes;
-  h->tma = chunk_bytes % 16 == 0;
+  const RowPlan rows = row_plan(nth, ns, h->V, (int)h->tsz, kChunkBytes);
+  h->packed = rows.packed;
+  h->chunks_per_cell = rows.chunks;
+  h->chunk_rows = rows.rows;
+  const size_t row_bytes = (size_t)ns * h->tsz, chunk_bytes = rows.rows * row_bytes;
+  h->tma = chunk_bytes % 16 == 0 && nth * row_bytes % 16 == 0;
   int S = (int)(kWarpInflightBytes / std::max<size_t>(chunk_bytes, 1));
   S = std::max(2, std::min(8, S));
   h->stages = h->tma ? S : 1;
@@ -216,9 +208,9 @@ mm_status configure(mm_handle* h) {
   int bps = 0;
   cudaError_t e;
   if (h->prec == MM_FP64)
-    e = mm::substep_prepare<double>(ns, h->block, h->smem, h->tma, &bps);
+    e = mm::substep_prepare<double>(ns, h->block, h->smem, h->tma, h->packed, &bps);
   else
-    e = mm::substep_prepare<float>(ns, h->block, h->smem, h->tma, &bps);
+    e = mm::substep_prepare<float>(ns, h->block, h->smem, h->tma, h->packed, &bps);
   CK(e);
   if (bps < 1) return fail(h, MM_ERR_UNSUPPORTED, "substep kernel cannot be resident");
   long long g = (long long)bps * h->sms;

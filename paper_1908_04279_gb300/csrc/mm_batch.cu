@@ -23,9 +23,9 @@ namespace mm {
 #ifndef MM_BATCH_MIN_BLOCKS
 #define MM_BATCH_MIN_BLOCKS MM_STEP_MIN_BLOCKS
 #endif
-template <typename T>
+template <typename T, bool PACKED>
 constexpr int batch_min_blocks() {
-  return sizeof(T) == 8 ? 2 : MM_BATCH_MIN_BLOCKS;
+  return sizeof(T) == 4 ? MM_BATCH_MIN_BLOCKS : PACKED ? 2 : 3;
 }
 
 // The psi and n_b columns of two cells of one row (x0 and x0 + 1, y0; nx is
@@ -92,10 +92,13 @@ __device__ __forceinline__ void pair_motor_close(T acc, T mtot, const T* s_nb, i
   }
 }
 
-template <typename T, int V, bool MASSCORR>
-__global__ void __launch_bounds__(128, batch_min_blocks<T>())
+// PACKED: rows packed (float64, an even ns: whole 16-byte vectors), else V nodes
+// to a lane.
+template <typename T, int V, bool PACKED>
+__global__ void __launch_bounds__(128, batch_min_blocks<T, PACKED>())
     k_substep_batch(const StepArgs<T>* __restrict__ insts, const BatchTile* __restrict__ tiles,
                     int ntiles, double* tile_mass, int S, int stage_elems, int nth_max) {
+  constexpr bool MASSCORR = sizeof(T) == 4;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const WarpSmem L = warp_smem_layout(S, stage_elems, nth_max, (int)sizeof(T));
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -125,7 +128,8 @@ __global__ void __launch_bounds__(128, batch_min_blocks<T>())
     pns = insts[pt.inst].ns;
   };
   auto issue_next = [&]() {
-    const uint32_t bytes = (uint32_t)(pt.rc * pns * sizeof(T));
+    const uint32_t bytes =
+        (uint32_t)(min(pt.rc, pnth * pt.cpu - ppart * pt.rc) * pns * sizeof(T));
     mbar_expect_tx(&bars[istage], bytes);
     bulk_g2s(stages + (size_t)istage * stage_elems,
              pmb + ((size_t)(pt.cell0 + pcell * pt.cpu) * pnth + (size_t)ppart * pt.rc) * pns, bytes,
@@ -238,7 +242,7 @@ __global__ void __launch_bounds__(128, batch_min_blocks<T>())
         ds = sc.ds;
         rk = RkConst<T>{hdt * sc.cw, T(1) - hdt * sc.koff, T(0), dt * sc.cw, -dt * sc.koff, T(0),
                         T(0), T(0), nth};
-        lg = sizeof(T) == 8 ? packed_lanes(lane, ns) : lane_geom(lane, seg, ns, V);
+        lg = PACKED ? packed_lanes(lane, ns) : lane_geom(lane, seg, ns, V);
         iy = ct.cell0 / nx;
         ix = ct.cell0 - iy * nx;
       } else if ((ix += ct.cpu) >= nx) {  // consecutive units of the tile
@@ -293,12 +297,13 @@ __global__ void __launch_bounds__(128, batch_min_blocks<T>())
     // (rows from the unit's row nth on -- the second cell of a unit of 2 --
     // bind to that cell's Mf; a chunk may hold rows of either or both)
     rk.rsplit = nth - part * ct.rc;
-    if constexpr (sizeof(T) == 8)  // (an even ns: whole 16-byte vectors)
-      rows_packed<T, 2, true>(stages + (size_t)s * stage_elems, A->mb_out + chunk_off, ct.rc, ns, lg,
+    const int rc = min(ct.rc, nth * ct.cpu - part * ct.rc);  // (the last may be shorter)
+    if constexpr (PACKED)
+      rows_packed<T, 2, true>(stages + (size_t)s * stage_elems, A->mb_out + chunk_off, rc, ns, lg,
                               rk, ds, s_nb + part * ct.rc);
     else
-      rows_chunk<T, V, true>(stages + (size_t)s * stage_elems, A->mb_out + chunk_off, ct.rc, ns,
-                             seg, lg, rk, ds, s_nb + part * ct.rc);
+      rows_chunk<T, V, true>(stages + (size_t)s * stage_elems, A->mb_out + chunk_off, rc, ns, seg,
+                             lg, rk, ds, s_nb + part * ct.rc);
     __syncwarp();
     if (lane == 0 && issued < nchunks) issue_next();
     if (++s == S) { s = 0; par ^= 1u; }
@@ -381,35 +386,34 @@ __global__ void __launch_bounds__(128, batch_min_blocks<T>())
 }
 
 template <typename T, int V>
+auto batch_kernel(bool packed) -> decltype(&k_substep_batch<T, V, false>) {
+  if constexpr (sizeof(T) == 8)
+    if (packed) return k_substep_batch<T, V, true>;
+  return k_substep_batch<T, V, false>;
+}
+
+template <typename T, int V>
 cudaError_t launch_substep_batch(const StepArgs<T>* insts, const BatchTile* tiles, int ntiles,
                                  double* tile_mass, int S, int stage_elems, int nth_max,
-                                 bool masscorr, int grid, int block, size_t smem, cudaStream_t s) {
-  if (masscorr)
-    k_substep_batch<T, V, true><<<grid, block, smem, s>>>(insts, tiles, ntiles, tile_mass, S,
-                                                          stage_elems, nth_max);
-  else
-    k_substep_batch<T, V, false><<<grid, block, smem, s>>>(insts, tiles, ntiles, tile_mass, S,
-                                                           stage_elems, nth_max);
+                                 bool packed, int grid, int block, size_t smem, cudaStream_t s) {
+  batch_kernel<T, V>(packed)<<<grid, block, smem, s>>>(insts, tiles, ntiles, tile_mass, S,
+                                                       stage_elems, nth_max);
   return cudaGetLastError();
 }
 
 template <typename T, int V>
-cudaError_t substep_batch_prepare(int block, size_t smem, int* blocks_per_sm) {
-  const void* fns[2] = {(const void*)k_substep_batch<T, V, true>,
-                        (const void*)k_substep_batch<T, V, false>};
-  for (const void* f : fns) {
-    cudaError_t e = mm::raise_smem_limit(f, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_substep_batch<T, V, true>,
-                                                       block, smem);
+cudaError_t substep_batch_prepare(int block, size_t smem, bool packed, int* blocks_per_sm) {
+  auto k = batch_kernel<T, V>(packed);
+  const cudaError_t e = mm::raise_smem_limit((const void*)k, smem);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, block, smem);
 }
 
 #define MM_BATCH_INST(T, V)                                                                    \
   template cudaError_t launch_substep_batch<T, V>(const StepArgs<T>*, const BatchTile*, int,   \
                                                   double*, int, int, int, bool, int, int,      \
                                                   size_t, cudaStream_t);                       \
-  template cudaError_t substep_batch_prepare<T, V>(int, size_t, int*);
+  template cudaError_t substep_batch_prepare<T, V>(int, size_t, bool, int*);
 MM_BATCH_INST(float, 8)
 MM_BATCH_INST(float, 4)
 MM_BATCH_INST(double, 2)

@@ -24,6 +24,7 @@ namespace mmh {
 // Tiles and launch shape of the batched kernel over a set of members.
 struct TilePlan {
   int S = 2, stage_elems = 0, nth_max = 0, block = 128, grid = 1, ntiles = 0;
+  bool packed = false;  // form of the rows (mm_plan.h)
   size_t smem = 0;
   mm::BatchTile* d_tiles = nullptr;
   double* tile_mass = nullptr;
@@ -76,17 +77,6 @@ void free_tiles(TilePlan& P) {
   P.tile_mass = nullptr;
 }
 
-// Rows per chunk of a member under the chunk limit (the largest divisor of
-// nth whose rows fit), as for the single-instance plan.
-void member_chunks(const mm_handle* m, int chunk_bytes, int* rc, int* ch) {
-  const size_t row_bytes = (size_t)m->g.ns * m->tsz;
-  const int nth = m->g.ntheta;
-  int c = 1;
-  while (c < nth && (nth % c != 0 || (size_t)(nth / c) * row_bytes > (size_t)chunk_bytes)) ++c;
-  *ch = c;
-  *rc = nth / c;
-}
-
 // Whether a member's cells go two to a warp: at most 16 orientations (one
 // half-warp per cell for psi and the close) or at most 32 (the warp takes the
 // two cells' psi and close in turn), with one cell's rows in at most 4 KB (a
@@ -101,15 +91,18 @@ bool member_pairs(const mm_handle* m, int V) {
   return fits && nth % (32 / seg) == 0 && m->g.nx % 2 == 0 && ((size_t)nth * m->tsz) % 16 == 0;
 }
 
-template <typename T>
-cudaError_t prepare(int V, int block, size_t smem, int* bps) {
-  if constexpr (sizeof(T) == 8) {
-    (void)V;
-    return mm::substep_batch_prepare<double, 2>(block, smem, bps);
-  } else {
-    return V == 8 ? mm::substep_batch_prepare<float, 8>(block, smem, bps)
-                  : mm::substep_batch_prepare<float, 4>(block, smem, bps);
-  }
+cudaError_t prepare(bool fp64, int V, int block, size_t smem, bool packed, int* bps) {
+  return fp64     ? mm::substep_batch_prepare<double, 2>(block, smem, packed, bps)
+         : V == 8 ? mm::substep_batch_prepare<float, 8>(block, smem, packed, bps)
+                  : mm::substep_batch_prepare<float, 4>(block, smem, packed, bps);
+}
+
+// The rows of a member's unit (of one cell or two) in chunks; units of two in at
+// most 4 KB whatever the limit is.
+RowPlan unit_plan(const mm_handle* m, int V, int cpu, bool packed, int chunk_bytes) {
+  const int ns = m->g.ns;
+  return chunk_plan(packed, cpu * m->g.ntheta, (size_t)ns * m->tsz,
+                    packed ? packed_rpp(ns) : lane_rpp(ns, V), cpu == 2 ? 4096 : chunk_bytes);
 }
 
 // Tiles, shared-memory plan and grid for (tile_work, chunk_bytes), over every
@@ -119,24 +112,25 @@ mm_status make_tiles(mm_handle* h, TilePlan& P, bool rest_only, int tile_work, i
   const int n = (int)B->members.size();
   std::vector<mm::BatchTile> tiles;
   int max_chunk_elems = 1, nth_max = 1;
+  // float64: the form of the rows that costs less over all members (mm_plan.h)
+  P.packed = false;
+  if (h->prec == MM_FP64) {
+    double cost[2] = {0.0, 0.0};
+    for (const mm_handle* m : B->members)
+      for (int f = 0; f < 2; ++f) {
+        const int cpu = B->pairs && member_pairs(m, B->V) ? 2 : 1;
+        cost[f] += (double)(m->ncells / cpu) * pass_cost(f, B->V, 8) *
+                   unit_plan(m, B->V, cpu, f, chunk_bytes).passes;
+      }
+    P.packed = cost[1] <= cost[0];
+  }
   for (int i = 0; i < n; ++i) {
     const mm_handle* m = B->members[i];
     if (rest_only && B->resident[i]) continue;
-    // units of 1 cell (rows in ch chunks of rc) or of 2 cells (one chunk of
-    // both cells' rows); tiles of about tile_work motor values, whole units
+    // units of 1 cell or of 2 cells; tiles of about tile_work motor values, whole units
     const int cpu = B->pairs && member_pairs(m, B->V) ? 2 : 1;
-    int rc, ch;
-    if (cpu == 2) {
-      // the unit's 2 ntheta rows in chunks of at most 4 KB (a divisor of the
-      // unit's rows: one chunk, or one cell's rows per chunk)
-      const int rows = 2 * m->g.ntheta;
-      const size_t row_bytes = (size_t)m->g.ns * m->tsz;
-      ch = 1;
-      while (ch < rows && (rows % ch != 0 || (size_t)(rows / ch) * row_bytes > 4096)) ++ch;
-      rc = rows / ch;
-    } else {
-      member_chunks(m, chunk_bytes, &rc, &ch);
-    }
+    const RowPlan rows = unit_plan(m, B->V, cpu, P.packed, chunk_bytes);
+    const int rc = rows.rows, ch = rows.chunks;
     max_chunk_elems = std::max(max_chunk_elems, rc * m->g.ns);
     nth_max = std::max(nth_max, cpu * m->g.ntheta);  // a pair stages two neighbourhoods
     const long long nu = m->ncells / cpu;             // nx even for pairs: ncells is too
@@ -167,9 +161,7 @@ mm_status make_tiles(mm_handle* h, TilePlan& P, bool rest_only, int tile_work, i
   const int block = 32 * wpb;
   const size_t smem = (size_t)wpb * per_warp;
   int bps = 0;
-  cudaError_t e = h->prec == MM_FP64 ? prepare<double>(B->V, block, smem, &bps)
-                                     : prepare<float>(B->V, block, smem, &bps);
-  CK(e);
+  CK(prepare(h->prec == MM_FP64, B->V, block, smem, P.packed, &bps));
   if (bps < 1) return fail(h, MM_ERR_UNSUPPORTED, "batch: the substep kernel cannot be resident");
   long long grid = (long long)bps * h->sms;
   const long long need = ((long long)tiles.size() + wpb - 1) / wpb;
@@ -241,16 +233,16 @@ cudaError_t launch_batch(mm_handle* h, const TilePlan& P, int table, cudaStream_
   if (h->prec == MM_FP64) {
     const StepArgs<double>* a = (const StepArgs<double>*)B->d_args + (size_t)table * n;
     return mm::launch_substep_batch<double, 2>(a, P.d_tiles, P.ntiles, P.tile_mass, P.S,
-                                               P.stage_elems, P.nth_max, false, P.grid, P.block,
+                                               P.stage_elems, P.nth_max, P.packed, P.grid, P.block,
                                                P.smem, s);
   }
   const StepArgs<float>* a = (const StepArgs<float>*)B->d_args + (size_t)table * n;
   if (B->V == 8)
     return mm::launch_substep_batch<float, 8>(a, P.d_tiles, P.ntiles, P.tile_mass, P.S,
-                                              P.stage_elems, P.nth_max, true, P.grid, P.block,
+                                              P.stage_elems, P.nth_max, P.packed, P.grid, P.block,
                                               P.smem, s);
   return mm::launch_substep_batch<float, 4>(a, P.d_tiles, P.ntiles, P.tile_mass, P.S,
-                                            P.stage_elems, P.nth_max, true, P.grid, P.block,
+                                            P.stage_elems, P.nth_max, P.packed, P.grid, P.block,
                                             P.smem, s);
 }
 

@@ -19,14 +19,11 @@
 #endif
 
 #include "mm_internal.cuh"
+#include "mm_plan.h"
 
 using mm::DevParams;
 using mm::StepArgs;
 
-// Widest vector (values per lane) of the float32 substep kernel.
-#ifndef MM_FP32_VMAX
-#define MM_FP32_VMAX 8
-#endif
 // 1: the motor reverse kernel streams rows by bulk copies where they allow it.
 #ifndef MM_ADJ_RING
 #define MM_ADJ_RING 1
@@ -181,7 +178,7 @@ struct mm_handle {
   // substep launch configuration
   int V = 1, seg = 1, block = 128, grid_step = 1, grid_mom = 1;
   int stages = 1, chunk_rows = 1, chunks_per_cell = 1;
-  bool tma = false;
+  bool tma = false, packed = false;  // bulk copies; packed rows (mm_plan.h)
   size_t smem = 0;
   // many substeps in one launch with Mb on the chip (mm_resident.cu; grid 0: off)
   int res_grid = 0, res_NL = 0;

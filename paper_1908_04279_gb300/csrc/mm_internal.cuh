@@ -55,7 +55,7 @@ struct StepArgs {
   int nx, ny, nth, ns;
   int seg;            // lanes per s-row segment (power of two <= 32)
   int stages;         // shared-memory ring depth per warp
-  int chunk_rows;     // s-rows per ring stage (divides nth)
+  int chunk_rows;     // s-rows per ring stage (a cell's last chunk may be shorter)
   int chunks_per_cell;
   int nb_tma;         // 1: stage the psi / n_b neighbourhood by bulk copies
   long long ncells;
@@ -132,7 +132,7 @@ struct BatchTile {
   int ncell;       // units (of cpu cells) in the tile
   int tile0;       // index of the instance's first tile
   int inst_tiles;  // tiles of the instance
-  int ch, rc;      // chunks per unit, s-rows per chunk
+  int ch, rc;      // chunks per unit, s-rows per chunk (the last may be shorter)
   int cpu;         // cells per unit: 1, or 2 (two cells of one row: one chunk holds both
                    // cells' rows; a half-warp each takes psi and the close)
 };
@@ -141,19 +141,21 @@ struct BatchTile {
 // previous kernel of the stream (direct launches only).
 template <typename T>
 cudaError_t launch_substep(const StepArgs<T>& a, int grid, int block, size_t smem, bool tma,
-                           cudaStream_t s, bool overlap);
+                           bool packed, cudaStream_t s, bool overlap);
 size_t step_smem_per_warp(int S, int chunk_elems, int nth, int tsz);
 template <typename T>
-cudaError_t substep_prepare(int ns, int block, size_t smem, bool tma, int* blocks_per_sm);
+cudaError_t substep_prepare(int ns, int block, size_t smem, bool tma, bool packed,
+                            int* blocks_per_sm);
 
 // Batched-ensemble launchers (mm_batch.cu): every instance's arguments in a
 // device table, tiles in a device table, per-tile float64 sums of psi.
+// packed: rows packed (mm_plan.h; float64 only), else V nodes to a lane.
 template <typename T, int V>
 cudaError_t launch_substep_batch(const StepArgs<T>* insts, const BatchTile* tiles, int ntiles,
                                  double* tile_mass, int S, int stage_elems, int nth_max,
-                                 bool masscorr, int grid, int block, size_t smem, cudaStream_t s);
+                                 bool packed, int grid, int block, size_t smem, cudaStream_t s);
 template <typename T, int V>
-cudaError_t substep_batch_prepare(int block, size_t smem, int* blocks_per_sm);
+cudaError_t substep_batch_prepare(int block, size_t smem, bool packed, int* blocks_per_sm);
 
 // Auxiliary kernels (mm_aux.cu).
 template <typename TO, typename TI>

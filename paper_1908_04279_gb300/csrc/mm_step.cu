@@ -37,28 +37,26 @@ size_t step_smem_per_warp(int S, int chunk_elems, int nth, int tsz) {
   return warp_smem_layout(S, chunk_elems, nth, tsz).total;
 }
 
-// VW: rows eight nodes to a lane whatever ns is, moved in vectors of VW values
-// (rows_packed: float64, and float32 rows of no multiple of 8 nodes); 0: float32
-// rows of a multiple of 8 (rows_chunk). Without TMA (a chunk or a cell is no
-// multiple of 16 bytes; packed only) the warp copies each chunk to its one stage
-// itself. float64 takes 3 blocks per SM: its 168 registers hold both stages of
-// eight nodes, and 12 warps keep the float64 pipe busy.
+// VW: packed rows, eight nodes to a lane whatever ns is, moved in vectors of VW
+// values (rows_packed); 0: V nodes to a lane (rows_chunk; row_plan says which).
+// Without TMA (a chunk or a cell is no multiple of 16 bytes) the warp copies each
+// chunk to its one stage itself. float64 takes 3 blocks per SM: its 168 registers
+// hold both stages of eight nodes, and 12 warps keep the float64 pipe busy.
 template <typename T>
 constexpr int step_min_blocks() {
   return sizeof(T) == 8 ? 3 : MM_STEP_MIN_BLOCKS;
 }
 
-template <typename T, int VW, bool TMA>
+template <typename T, int VW, int V, bool TMA>
 __global__ void __launch_bounds__(128, step_min_blocks<T>()) k_substep(const StepArgs<T> a) {
   constexpr bool MASSCORR = sizeof(T) == 4, PACKED = VW > 0;
   // rows of whole 16-byte vectors are stored straight to global memory
-  constexpr bool direct = VW == 0 || VW * sizeof(T) == 16;
+  constexpr bool direct = !PACKED || VW * sizeof(T) == 16;
   griddep_wait();  // launched overlapped outside graphs (recording, replays)
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int nth = a.nth, ns = a.ns, seg = a.seg;
   const int S = a.stages, RC = a.chunk_rows, CH = a.chunks_per_cell;
   const int chunk_elems = RC * ns;
-  const uint32_t chunk_bytes = (uint32_t)(chunk_elems * sizeof(T));
   const WarpSmem L = warp_smem_layout(S, chunk_elems, nth, (int)sizeof(T));
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   unsigned char* wbase = smem_raw + (size_t)wib * L.total;
@@ -80,7 +78,7 @@ __global__ void __launch_bounds__(128, step_min_blocks<T>()) k_substep(const Ste
   const int my_cells = gw < nc ? (nc - 1 - gw) / W + 1 : 0;
   const int nchunks = my_cells * CH;
 
-  const LaneGeom lg = PACKED ? packed_lanes(lane, ns) : lane_geom(lane, seg, ns, 8);
+  const LaneGeom lg = PACKED ? packed_lanes(lane, ns) : lane_geom(lane, seg, ns, V);
 
   const DevParams* P = a.prm;
   const StepScalars<T> sc = step_scalars<T, MASSCORR>(P, a, lane);
@@ -95,9 +93,10 @@ __global__ void __launch_bounds__(128, step_min_blocks<T>()) k_substep(const Ste
   // producer cursor: next chunk to issue (cell, part, stage)
   int icell = gw, ipart = 0, istage = 0, issued = 0;
   auto issue_next = [&]() {
-    mbar_expect_tx(&bars[istage], chunk_bytes);
+    const uint32_t bytes = (uint32_t)(min(RC, nth - ipart * RC) * ns * sizeof(T));
+    mbar_expect_tx(&bars[istage], bytes);
     bulk_g2s(stages + (size_t)istage * chunk_elems,
-             a.mb_in + ((size_t)icell * nth + (size_t)ipart * RC) * ns, chunk_bytes, &bars[istage]);
+             a.mb_in + ((size_t)icell * nth + (size_t)ipart * RC) * ns, bytes, &bars[istage]);
     ++issued;
     if (++ipart == CH) { ipart = 0; icell += W; }
     if (++istage == S) istage = 0;
@@ -172,8 +171,9 @@ __global__ void __launch_bounds__(128, step_min_blocks<T>()) k_substep(const Ste
     // ---- motor rows of this chunk
     const size_t chunk_off = ((size_t)cell * nth + (size_t)part * RC) * ns;
     T* stage = stages + (size_t)s * chunk_elems;
+    const int rc = min(RC, nth - part * RC), elems = rc * ns;
     if (!TMA) {
-      for (int e = lane; e < chunk_elems; e += 32) stage[e] = a.mb_in[chunk_off + e];
+      for (int e = lane; e < elems; e += 32) stage[e] = a.mb_in[chunk_off + e];
       __syncwarp();
     } else {
       const bool ok = __all_sync(0xffffffffu, wait_never ? mbar_wait(never, 0u, wait_limit)
@@ -190,21 +190,21 @@ __global__ void __launch_bounds__(128, step_min_blocks<T>()) k_substep(const Ste
     }
     if constexpr (PACKED) {
       T* out = a.mb_out + chunk_off;
-      rows_packed<T, VW>(stage, out, RC, ns, lg, rk, ds, s_nb + part * RC);
+      rows_packed<T, VW>(stage, out, rc, ns, lg, rk, ds, s_nb + part * RC);
       if constexpr (!direct) {  // the chunk as it lies, coalesced
         __syncwarp();
         if (TMA) {
           constexpr int kv = 16 / sizeof(T);
-          for (int e = lane; e < chunk_elems / kv; e += 32)
+          for (int e = lane; e < elems / kv; e += 32)
             reinterpret_cast<float4*>(out)[e] = reinterpret_cast<const float4*>(stage)[e];
           // the rows written into the stage, before the next bulk copy into it
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         } else {
-          for (int e = lane; e < chunk_elems; e += 32) out[e] = stage[e];
+          for (int e = lane; e < elems; e += 32) out[e] = stage[e];
         }
       }
     } else {
-      rows_chunk<T, 8>(stage, a.mb_out + chunk_off, RC, ns, seg, lg, rk, ds, s_nb + part * RC);
+      rows_chunk<T, V>(stage, a.mb_out + chunk_off, rc, ns, seg, lg, rk, ds, s_nb + part * RC);
     }
     __syncwarp();
     // the stage is consumed: refill it with the chunk S ahead
@@ -315,27 +315,32 @@ __global__ void __launch_bounds__(128, step_min_blocks<T>()) k_substep(const Ste
 
 // The instance of the kernel for rows of ns nodes.
 template <typename T>
-auto step_kernel(int ns, bool tma) -> void (*)(StepArgs<T>) {
+auto step_kernel(int ns, bool tma, bool packed) -> void (*)(StepArgs<T>) {
   if constexpr (sizeof(T) == 4) {
-    if (ns % 8 == 0) return k_substep<T, 0, true>;
-    if (ns % 4 == 0) return k_substep<T, 4, true>;
+    if (!packed) return ns % 8 == 0 ? k_substep<T, 0, 8, true> : k_substep<T, 0, 4, true>;
+    if (ns % 4 == 0) return k_substep<T, 4, 8, true>;
+    if (ns % 2 == 0) return tma ? k_substep<T, 2, 8, true> : k_substep<T, 2, 8, false>;
+  } else if (ns % 2 == 0) {
+    return packed ? k_substep<T, 2, 8, true> : k_substep<T, 0, 2, true>;
+  } else if (!packed) {
+    return tma ? k_substep<T, 0, 1, true> : k_substep<T, 0, 1, false>;
   }
-  if (ns % 2 == 0) return tma ? k_substep<T, 2, true> : k_substep<T, 2, false>;
-  return tma ? k_substep<T, 1, true> : k_substep<T, 1, false>;
+  return tma ? k_substep<T, 1, 8, true> : k_substep<T, 1, 8, false>;
 }
 
 template <typename T>
 cudaError_t launch_substep(const StepArgs<T>& a, int grid, int block, size_t smem, bool tma,
-                           cudaStream_t s, bool overlap) {
-  void (*k)(StepArgs<T>) = step_kernel<T>(a.ns, tma);
+                           bool packed, cudaStream_t s, bool overlap) {
+  void (*k)(StepArgs<T>) = step_kernel<T>(a.ns, tma, packed);
   if (overlap) return launch_overlapped(k, grid, block, smem, s, a);
   k<<<grid, block, smem, s>>>(a);
   return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t substep_prepare(int ns, int block, size_t smem, bool tma, int* blocks_per_sm) {
-  void (*k)(StepArgs<T>) = step_kernel<T>(ns, tma);
+cudaError_t substep_prepare(int ns, int block, size_t smem, bool tma, bool packed,
+                            int* blocks_per_sm) {
+  void (*k)(StepArgs<T>) = step_kernel<T>(ns, tma, packed);
   const cudaError_t e = mm::raise_smem_limit(k, smem);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, block, smem);
@@ -343,8 +348,8 @@ cudaError_t substep_prepare(int ns, int block, size_t smem, bool tma, int* block
 
 #define MM_STEP_INST(T)                                                              \
   template cudaError_t launch_substep<T>(const StepArgs<T>&, int, int, size_t, bool, \
-                                         cudaStream_t, bool);                        \
-  template cudaError_t substep_prepare<T>(int, int, size_t, bool, int*);
+                                         bool, cudaStream_t, bool);                  \
+  template cudaError_t substep_prepare<T>(int, int, size_t, bool, bool, int*);
 MM_STEP_INST(float)
 MM_STEP_INST(double)
 

@@ -1,0 +1,68 @@
+"""The plan of the streaming kernels' rows (mm_plan.h, compiled for the host):
+chunks of whole passes, and by its own cost of a pass never dearer than rows of
+V nodes to a lane in equal chunks that divide the orientations, which packed
+rows replaced."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_1908_04279_gb300", "csrc")
+
+
+def cases():
+    for tsz in (4, 8):
+        for ns in range(1, 129 if tsz == 4 else 65):
+            V = (8 if ns % 8 == 0 else 4 if ns % 4 == 0 else 1) if tsz == 4 else 2 - ns % 2
+            if ns // V > 32:
+                continue
+            for nth in [*range(1, 130), 256, 509, 512, 1024]:
+                yield nth, ns, tsz, V
+
+
+@pytest.fixture(scope="module")
+def plans(tmp_path_factory):
+    cxx = shutil.which("g++")
+    if not cxx:
+        pytest.skip("g++ not available")
+    exe = str(tmp_path_factory.mktemp("plan") / "step_plan_host")
+    subprocess.check_call([cxx, "-std=c++17", "-O1", "-I" + CSRC,
+                           os.path.join(HERE, "step_plan_host.cpp"), "-o", exe])
+    text = "\n".join(" ".join(map(str, c)) for c in cases())
+    out = subprocess.run([exe], input=text, capture_output=True, text=True, check=True).stdout
+    got = [line.split() for line in out.splitlines()]
+    return {c: (int(q[0]), int(q[1]), int(q[2]), int(q[3]), float(q[4]))
+            for c, q in zip(cases(), got)}
+
+
+def lane_rpp(ns, V):
+    seg = 1
+    while seg < ns // V:
+        seg *= 2
+    return 32 // seg
+
+
+def test_chunks_are_whole_passes(plans):
+    for (nth, ns, tsz, V), (packed, rows, chunks, passes, _) in plans.items():
+        rpp = 32 // -(-ns // 8) if packed else lane_rpp(ns, V)
+        at = (nth, ns, tsz, V)
+        assert rows <= nth and (chunks - 1) * rows < nth <= chunks * rows, at
+        assert rows == nth or rows % rpp == 0, at
+        assert rows * ns * tsz <= 4096 or rows <= rpp, at
+        assert passes == (chunks - 1) * -(-rows // rpp) + -(-(nth - (chunks - 1) * rows) // rpp), at
+        # bulk copies wherever a cell is a whole number of 16-byte vectors
+        assert nth * ns * tsz % 16 or rows * ns * tsz % 16 == 0, at
+
+
+def test_no_dearer_than_equal_chunks_of_lanes(plans):
+    for (nth, ns, tsz, V), (*_, cost) in plans.items():
+        if tsz == 4 and V == 1:
+            continue  # (one node to a lane costs 3.5 times a packed one)
+        c = 1
+        while c < nth and (nth % c or nth // c * ns * tsz > 4096):
+            c += 1
+        passes = c * -(-(nth // c) // lane_rpp(ns, V))
+        before = passes * (V if tsz == 4 else 36.0 if V == 2 else 23.0)
+        assert cost <= before * (1 + 1e-12), (nth, ns, tsz, V)
