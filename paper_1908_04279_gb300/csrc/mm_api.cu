@@ -86,7 +86,7 @@ StepArgs<T> step_args(mm_handle* h, int parity) {
   a.stages = h->stages;
   a.chunk_rows = h->chunk_rows;
   a.chunks_per_cell = h->chunks_per_cell;
-  a.nb_tma = h->tma && ((size_t)h->g.ntheta * h->tsz) % 16 == 0;
+  a.nb_tma = h->form.tma && ((size_t)h->g.ntheta * h->tsz) % 16 == 0;
   a.ncells = h->ncells;
   a.inv_dx = (double)h->g.nx;
   a.inv_dy = (double)h->g.ny;
@@ -124,7 +124,7 @@ template StepArgs<double> step_args<double>(mm_handle*, int);
 // The substep kernel of h's plan on given arguments.
 template <typename T>
 cudaError_t launch_step(const mm_handle* h, const StepArgs<T>& a, cudaStream_t s, bool overlap) {
-  return mm::launch_substep<T>(a, h->grid_step, h->block, h->smem, h->tma, h->packed, s, overlap);
+  return mm::launch_substep<T>(a, h->grid_step, h->block, h->smem, h->form, s, overlap);
 }
 cudaError_t launch_plain(mm_handle* h, int parity, cudaStream_t s) {
   return h->prec == MM_FP64 ? launch_step(h, step_args<double>(h, parity), s, false)
@@ -192,14 +192,15 @@ mm_status configure(mm_handle* h) {
   while (seg < nl) seg <<= 1;
   h->seg = seg;
   const RowPlan rows = row_plan(nth, ns, h->V, (int)h->tsz, kChunkBytes);
-  h->packed = rows.packed;
   h->chunks_per_cell = rows.chunks;
   h->chunk_rows = rows.rows;
   const size_t row_bytes = (size_t)ns * h->tsz, chunk_bytes = rows.rows * row_bytes;
-  h->tma = chunk_bytes % 16 == 0 && nth * row_bytes % 16 == 0;
+  h->form.tma = chunk_bytes % 16 == 0 && nth * row_bytes % 16 == 0;
+  h->form.packed = rows.packed;
+  h->form.even = rows.rows * rows.chunks == nth;
   int S = (int)(kWarpInflightBytes / std::max<size_t>(chunk_bytes, 1));
   S = std::max(2, std::min(8, S));
-  h->stages = h->tma ? S : 1;
+  h->stages = h->form.tma ? S : 1;
   const size_t per_warp = mm::step_smem_per_warp(h->stages, h->chunk_rows * ns, nth, (int)h->tsz);
   const int wpb = (int)std::min<size_t>(kMaxWarpsPerBlock, kSmemBudget / per_warp);
   if (wpb < 1) return fail(h, MM_ERR_UNSUPPORTED, "ntheta too large for the shared-memory plan");
@@ -208,9 +209,9 @@ mm_status configure(mm_handle* h) {
   int bps = 0;
   cudaError_t e;
   if (h->prec == MM_FP64)
-    e = mm::substep_prepare<double>(ns, h->block, h->smem, h->tma, h->packed, &bps);
+    e = mm::substep_prepare<double>(ns, h->block, h->smem, h->form, &bps);
   else
-    e = mm::substep_prepare<float>(ns, h->block, h->smem, h->tma, h->packed, &bps);
+    e = mm::substep_prepare<float>(ns, h->block, h->smem, h->form, &bps);
   CK(e);
   if (bps < 1) return fail(h, MM_ERR_UNSUPPORTED, "substep kernel cannot be resident");
   long long g = (long long)bps * h->sms;
@@ -882,7 +883,7 @@ mm_status mm_debug_set(mm_handle* h, unsigned int wait_limit, unsigned int flags
 mm_status mm_get_launch_info(mm_handle* h, int* info, int n) {
   if (!h || !info || n < 1) return MM_ERR_INVALID;
   if (h->batch) return batch_launch_info(h, info, n);
-  const int v[10] = {h->grid_step, h->block, (int)h->smem, h->tma ? 1 : 0, h->stages,
+  const int v[10] = {h->grid_step, h->block, (int)h->smem, h->form.tma ? 1 : 0, h->stages,
                      h->chunk_rows, h->chunks_per_cell, h->V, h->seg, h->sms};
   for (int i = 0; i < n && i < 10; ++i) info[i] = v[i];
   return MM_OK;

@@ -93,8 +93,8 @@ __device__ __forceinline__ void pair_motor_close(T acc, T mtot, const T* s_nb, i
 }
 
 // PACKED: rows packed (float64, an even ns: whole 16-byte vectors), else V nodes
-// to a lane.
-template <typename T, int V, bool PACKED>
+// to a lane. EVEN: every unit's chunks are all alike.
+template <typename T, int V, bool PACKED, bool EVEN>
 __global__ void __launch_bounds__(128, batch_min_blocks<T, PACKED>())
     k_substep_batch(const StepArgs<T>* __restrict__ insts, const BatchTile* __restrict__ tiles,
                     int ntiles, double* tile_mass, int S, int stage_elems, int nth_max) {
@@ -128,8 +128,8 @@ __global__ void __launch_bounds__(128, batch_min_blocks<T, PACKED>())
     pns = insts[pt.inst].ns;
   };
   auto issue_next = [&]() {
-    const uint32_t bytes =
-        (uint32_t)(min(pt.rc, pnth * pt.cpu - ppart * pt.rc) * pns * sizeof(T));
+    const int rc = EVEN ? pt.rc : min(pt.rc, pnth * pt.cpu - ppart * pt.rc);
+    const uint32_t bytes = (uint32_t)(rc * pns * sizeof(T));
     mbar_expect_tx(&bars[istage], bytes);
     bulk_g2s(stages + (size_t)istage * stage_elems,
              pmb + ((size_t)(pt.cell0 + pcell * pt.cpu) * pnth + (size_t)ppart * pt.rc) * pns, bytes,
@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(128, batch_min_blocks<T, PACKED>())
     // (rows from the unit's row nth on -- the second cell of a unit of 2 --
     // bind to that cell's Mf; a chunk may hold rows of either or both)
     rk.rsplit = nth - part * ct.rc;
-    const int rc = min(ct.rc, nth * ct.cpu - part * ct.rc);  // (the last may be shorter)
+    const int rc = EVEN ? ct.rc : min(ct.rc, nth * ct.cpu - part * ct.rc);
     if constexpr (PACKED)
       rows_packed<T, 2, true>(stages + (size_t)s * stage_elems, A->mb_out + chunk_off, rc, ns, lg,
                               rk, ds, s_nb + part * ct.rc);
@@ -385,35 +385,40 @@ __global__ void __launch_bounds__(128, batch_min_blocks<T, PACKED>())
   }
 }
 
-template <typename T, int V>
-auto batch_kernel(bool packed) -> decltype(&k_substep_batch<T, V, false>) {
+template <typename T, int V, bool EVEN>
+auto batch_kernel(bool packed) -> decltype(&k_substep_batch<T, V, false, EVEN>) {
   if constexpr (sizeof(T) == 8)
-    if (packed) return k_substep_batch<T, V, true>;
-  return k_substep_batch<T, V, false>;
+    if (packed) return k_substep_batch<T, V, true, EVEN>;
+  return k_substep_batch<T, V, false, EVEN>;
+}
+template <typename T, int V>
+auto batch_kernel(const StepForm& f) {
+  return f.even ? batch_kernel<T, V, true>(f.packed) : batch_kernel<T, V, false>(f.packed);
 }
 
 template <typename T, int V>
 cudaError_t launch_substep_batch(const StepArgs<T>* insts, const BatchTile* tiles, int ntiles,
                                  double* tile_mass, int S, int stage_elems, int nth_max,
-                                 bool packed, int grid, int block, size_t smem, cudaStream_t s) {
-  batch_kernel<T, V>(packed)<<<grid, block, smem, s>>>(insts, tiles, ntiles, tile_mass, S,
-                                                       stage_elems, nth_max);
+                                 const StepForm& f, int grid, int block, size_t smem,
+                                 cudaStream_t s) {
+  batch_kernel<T, V>(f)<<<grid, block, smem, s>>>(insts, tiles, ntiles, tile_mass, S, stage_elems,
+                                                  nth_max);
   return cudaGetLastError();
 }
 
 template <typename T, int V>
-cudaError_t substep_batch_prepare(int block, size_t smem, bool packed, int* blocks_per_sm) {
-  auto k = batch_kernel<T, V>(packed);
+cudaError_t substep_batch_prepare(int block, size_t smem, const StepForm& f, int* blocks_per_sm) {
+  auto k = batch_kernel<T, V>(f);
   const cudaError_t e = mm::raise_smem_limit((const void*)k, smem);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, block, smem);
 }
 
-#define MM_BATCH_INST(T, V)                                                                    \
-  template cudaError_t launch_substep_batch<T, V>(const StepArgs<T>*, const BatchTile*, int,   \
-                                                  double*, int, int, int, bool, int, int,      \
-                                                  size_t, cudaStream_t);                       \
-  template cudaError_t substep_batch_prepare<T, V>(int, size_t, bool, int*);
+#define MM_BATCH_INST(T, V)                                                                   \
+  template cudaError_t launch_substep_batch<T, V>(const StepArgs<T>*, const BatchTile*, int,  \
+                                                  double*, int, int, int, const StepForm&,    \
+                                                  int, int, size_t, cudaStream_t);            \
+  template cudaError_t substep_batch_prepare<T, V>(int, size_t, const StepForm&, int*);
 MM_BATCH_INST(float, 8)
 MM_BATCH_INST(float, 4)
 MM_BATCH_INST(double, 2)

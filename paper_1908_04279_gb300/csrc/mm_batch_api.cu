@@ -24,7 +24,7 @@ namespace mmh {
 // Tiles and launch shape of the batched kernel over a set of members.
 struct TilePlan {
   int S = 2, stage_elems = 0, nth_max = 0, block = 128, grid = 1, ntiles = 0;
-  bool packed = false;  // form of the rows (mm_plan.h)
+  mm::StepForm form;  // (mm_plan.h)
   size_t smem = 0;
   mm::BatchTile* d_tiles = nullptr;
   double* tile_mass = nullptr;
@@ -91,10 +91,10 @@ bool member_pairs(const mm_handle* m, int V) {
   return fits && nth % (32 / seg) == 0 && m->g.nx % 2 == 0 && ((size_t)nth * m->tsz) % 16 == 0;
 }
 
-cudaError_t prepare(bool fp64, int V, int block, size_t smem, bool packed, int* bps) {
-  return fp64     ? mm::substep_batch_prepare<double, 2>(block, smem, packed, bps)
-         : V == 8 ? mm::substep_batch_prepare<float, 8>(block, smem, packed, bps)
-                  : mm::substep_batch_prepare<float, 4>(block, smem, packed, bps);
+cudaError_t prepare(bool fp64, int V, int block, size_t smem, const mm::StepForm& f, int* bps) {
+  return fp64     ? mm::substep_batch_prepare<double, 2>(block, smem, f, bps)
+         : V == 8 ? mm::substep_batch_prepare<float, 8>(block, smem, f, bps)
+                  : mm::substep_batch_prepare<float, 4>(block, smem, f, bps);
 }
 
 // The rows of a member's unit (of one cell or two) in chunks; units of two in at
@@ -113,7 +113,7 @@ mm_status make_tiles(mm_handle* h, TilePlan& P, bool rest_only, int tile_work, i
   std::vector<mm::BatchTile> tiles;
   int max_chunk_elems = 1, nth_max = 1;
   // float64: the form of the rows that costs less over all members (mm_plan.h)
-  P.packed = false;
+  P.form = mm::StepForm{true, false, true};
   if (h->prec == MM_FP64) {
     double cost[2] = {0.0, 0.0};
     for (const mm_handle* m : B->members)
@@ -122,15 +122,16 @@ mm_status make_tiles(mm_handle* h, TilePlan& P, bool rest_only, int tile_work, i
         cost[f] += (double)(m->ncells / cpu) * pass_cost(f, B->V, 8) *
                    unit_plan(m, B->V, cpu, f, chunk_bytes).passes;
       }
-    P.packed = cost[1] <= cost[0];
+    P.form.packed = cost[1] <= cost[0];
   }
   for (int i = 0; i < n; ++i) {
     const mm_handle* m = B->members[i];
     if (rest_only && B->resident[i]) continue;
     // units of 1 cell or of 2 cells; tiles of about tile_work motor values, whole units
     const int cpu = B->pairs && member_pairs(m, B->V) ? 2 : 1;
-    const RowPlan rows = unit_plan(m, B->V, cpu, P.packed, chunk_bytes);
+    const RowPlan rows = unit_plan(m, B->V, cpu, P.form.packed, chunk_bytes);
     const int rc = rows.rows, ch = rows.chunks;
+    P.form.even = P.form.even && rc * ch == cpu * m->g.ntheta;
     max_chunk_elems = std::max(max_chunk_elems, rc * m->g.ns);
     nth_max = std::max(nth_max, cpu * m->g.ntheta);  // a pair stages two neighbourhoods
     const long long nu = m->ncells / cpu;             // nx even for pairs: ncells is too
@@ -161,7 +162,7 @@ mm_status make_tiles(mm_handle* h, TilePlan& P, bool rest_only, int tile_work, i
   const int block = 32 * wpb;
   const size_t smem = (size_t)wpb * per_warp;
   int bps = 0;
-  CK(prepare(h->prec == MM_FP64, B->V, block, smem, P.packed, &bps));
+  CK(prepare(h->prec == MM_FP64, B->V, block, smem, P.form, &bps));
   if (bps < 1) return fail(h, MM_ERR_UNSUPPORTED, "batch: the substep kernel cannot be resident");
   long long grid = (long long)bps * h->sms;
   const long long need = ((long long)tiles.size() + wpb - 1) / wpb;
@@ -233,16 +234,16 @@ cudaError_t launch_batch(mm_handle* h, const TilePlan& P, int table, cudaStream_
   if (h->prec == MM_FP64) {
     const StepArgs<double>* a = (const StepArgs<double>*)B->d_args + (size_t)table * n;
     return mm::launch_substep_batch<double, 2>(a, P.d_tiles, P.ntiles, P.tile_mass, P.S,
-                                               P.stage_elems, P.nth_max, P.packed, P.grid, P.block,
+                                               P.stage_elems, P.nth_max, P.form, P.grid, P.block,
                                                P.smem, s);
   }
   const StepArgs<float>* a = (const StepArgs<float>*)B->d_args + (size_t)table * n;
   if (B->V == 8)
     return mm::launch_substep_batch<float, 8>(a, P.d_tiles, P.ntiles, P.tile_mass, P.S,
-                                              P.stage_elems, P.nth_max, P.packed, P.grid, P.block,
+                                              P.stage_elems, P.nth_max, P.form, P.grid, P.block,
                                               P.smem, s);
   return mm::launch_substep_batch<float, 4>(a, P.d_tiles, P.ntiles, P.tile_mass, P.S,
-                                            P.stage_elems, P.nth_max, P.packed, P.grid, P.block,
+                                            P.stage_elems, P.nth_max, P.form, P.grid, P.block,
                                             P.smem, s);
 }
 

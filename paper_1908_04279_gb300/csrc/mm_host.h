@@ -178,7 +178,7 @@ struct mm_handle {
   // substep launch configuration
   int V = 1, seg = 1, block = 128, grid_step = 1, grid_mom = 1;
   int stages = 1, chunk_rows = 1, chunks_per_cell = 1;
-  bool tma = false, packed = false;  // bulk copies; packed rows (mm_plan.h)
+  mm::StepForm form;  // (mm_plan.h)
   size_t smem = 0;
   // many substeps in one launch with Mb on the chip (mm_resident.cu; grid 0: off)
   int res_grid = 0, res_NL = 0;

@@ -137,25 +137,31 @@ struct BatchTile {
                    // cells' rows; a half-warp each takes psi and the close)
 };
 
+// Form of the streaming kernels: bulk copies (a batch always), packed rows (a
+// batch in float64 only), equal chunks.
+struct StepForm {
+  bool tma = false, packed = false, even = true;
+};
+
 // Kernel launchers (defined in mm_step.cu); overlap: launched overlapped with the
 // previous kernel of the stream (direct launches only).
 template <typename T>
-cudaError_t launch_substep(const StepArgs<T>& a, int grid, int block, size_t smem, bool tma,
-                           bool packed, cudaStream_t s, bool overlap);
+cudaError_t launch_substep(const StepArgs<T>& a, int grid, int block, size_t smem,
+                           const StepForm& f, cudaStream_t s, bool overlap);
 size_t step_smem_per_warp(int S, int chunk_elems, int nth, int tsz);
 template <typename T>
-cudaError_t substep_prepare(int ns, int block, size_t smem, bool tma, bool packed,
+cudaError_t substep_prepare(int ns, int block, size_t smem, const StepForm& f,
                             int* blocks_per_sm);
 
 // Batched-ensemble launchers (mm_batch.cu): every instance's arguments in a
 // device table, tiles in a device table, per-tile float64 sums of psi.
-// packed: rows packed (mm_plan.h; float64 only), else V nodes to a lane.
 template <typename T, int V>
 cudaError_t launch_substep_batch(const StepArgs<T>* insts, const BatchTile* tiles, int ntiles,
                                  double* tile_mass, int S, int stage_elems, int nth_max,
-                                 bool packed, int grid, int block, size_t smem, cudaStream_t s);
+                                 const StepForm& f, int grid, int block, size_t smem,
+                                 cudaStream_t s);
 template <typename T, int V>
-cudaError_t substep_batch_prepare(int block, size_t smem, bool packed, int* blocks_per_sm);
+cudaError_t substep_batch_prepare(int block, size_t smem, const StepForm& f, int* blocks_per_sm);
 
 // Auxiliary kernels (mm_aux.cu).
 template <typename TO, typename TI>

@@ -39,6 +39,13 @@ inline RowPlan chunk_plan(bool packed, int total, size_t row_bytes, int rpp, int
   p.chunks = (total + p.rows - 1) / p.rows;
   const int last = total - (p.chunks - 1) * p.rows;
   p.passes = (p.chunks - 1) * ((p.rows + rpp - 1) / rpp) + (last + rpp - 1) / rpp;
+  // equal chunks after all where they take no more passes
+  const int even = total / n;
+  if (even * n == total && n * ((even + rpp - 1) / rpp) <= p.passes &&
+      (total * row_bytes % 16 != 0 || even * row_bytes % 16 == 0)) {
+    p.rows = even;
+    p.chunks = n;
+  }
   return p;
 }
 

@@ -40,14 +40,16 @@ size_t step_smem_per_warp(int S, int chunk_elems, int nth, int tsz) {
 // VW: packed rows, eight nodes to a lane whatever ns is, moved in vectors of VW
 // values (rows_packed); 0: V nodes to a lane (rows_chunk; row_plan says which).
 // Without TMA (a chunk or a cell is no multiple of 16 bytes) the warp copies each
-// chunk to its one stage itself. float64 takes 3 blocks per SM: its 168 registers
+// chunk to its one stage itself. EVEN: a cell's chunks are all alike (a count of
+// rows that changes from chunk to chunk costs 3 % at 200^2 x 64 x 64 and, without
+// TMA, 15 % at 31 x 30). float64 takes 3 blocks per SM: its 168 registers
 // hold both stages of eight nodes, and 12 warps keep the float64 pipe busy.
 template <typename T>
 constexpr int step_min_blocks() {
   return sizeof(T) == 8 ? 3 : MM_STEP_MIN_BLOCKS;
 }
 
-template <typename T, int VW, int V, bool TMA>
+template <typename T, int VW, int V, bool TMA, bool EVEN>
 __global__ void __launch_bounds__(128, step_min_blocks<T>()) k_substep(const StepArgs<T> a) {
   constexpr bool MASSCORR = sizeof(T) == 4, PACKED = VW > 0;
   // rows of whole 16-byte vectors are stored straight to global memory
@@ -57,6 +59,8 @@ __global__ void __launch_bounds__(128, step_min_blocks<T>()) k_substep(const Ste
   const int nth = a.nth, ns = a.ns, seg = a.seg;
   const int S = a.stages, RC = a.chunk_rows, CH = a.chunks_per_cell;
   const int chunk_elems = RC * ns;
+  const uint32_t chunk_bytes = (uint32_t)(chunk_elems * sizeof(T));
+  const int last_rows = EVEN ? RC : nth - (CH - 1) * RC;
   const WarpSmem L = warp_smem_layout(S, chunk_elems, nth, (int)sizeof(T));
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   unsigned char* wbase = smem_raw + (size_t)wib * L.total;
@@ -93,7 +97,8 @@ __global__ void __launch_bounds__(128, step_min_blocks<T>()) k_substep(const Ste
   // producer cursor: next chunk to issue (cell, part, stage)
   int icell = gw, ipart = 0, istage = 0, issued = 0;
   auto issue_next = [&]() {
-    const uint32_t bytes = (uint32_t)(min(RC, nth - ipart * RC) * ns * sizeof(T));
+    const uint32_t bytes = EVEN || ipart + 1 < CH ? chunk_bytes
+                                                  : (uint32_t)(last_rows * ns * sizeof(T));
     mbar_expect_tx(&bars[istage], bytes);
     bulk_g2s(stages + (size_t)istage * chunk_elems,
              a.mb_in + ((size_t)icell * nth + (size_t)ipart * RC) * ns, bytes, &bars[istage]);
@@ -171,7 +176,8 @@ __global__ void __launch_bounds__(128, step_min_blocks<T>()) k_substep(const Ste
     // ---- motor rows of this chunk
     const size_t chunk_off = ((size_t)cell * nth + (size_t)part * RC) * ns;
     T* stage = stages + (size_t)s * chunk_elems;
-    const int rc = min(RC, nth - part * RC), elems = rc * ns;
+    const int rc = EVEN || part + 1 < CH ? RC : last_rows;
+    const int elems = EVEN ? chunk_elems : rc * ns;
     if (!TMA) {
       for (int e = lane; e < elems; e += 32) stage[e] = a.mb_in[chunk_off + e];
       __syncwarp();
@@ -314,42 +320,48 @@ __global__ void __launch_bounds__(128, step_min_blocks<T>()) k_substep(const Ste
 }
 
 // The instance of the kernel for rows of ns nodes.
-template <typename T>
+template <typename T, bool EVEN>
 auto step_kernel(int ns, bool tma, bool packed) -> void (*)(StepArgs<T>) {
   if constexpr (sizeof(T) == 4) {
-    if (!packed) return ns % 8 == 0 ? k_substep<T, 0, 8, true> : k_substep<T, 0, 4, true>;
-    if (ns % 4 == 0) return k_substep<T, 4, 8, true>;
-    if (ns % 2 == 0) return tma ? k_substep<T, 2, 8, true> : k_substep<T, 2, 8, false>;
+    if (!packed)
+      return ns % 8 == 0 ? k_substep<T, 0, 8, true, EVEN> : k_substep<T, 0, 4, true, EVEN>;
+    if (ns % 4 == 0) return k_substep<T, 4, 8, true, EVEN>;
+    if (ns % 2 == 0) return tma ? k_substep<T, 2, 8, true, EVEN> : k_substep<T, 2, 8, false, EVEN>;
   } else if (ns % 2 == 0) {
-    return packed ? k_substep<T, 2, 8, true> : k_substep<T, 0, 2, true>;
+    return packed ? k_substep<T, 2, 8, true, EVEN> : k_substep<T, 0, 2, true, EVEN>;
   } else if (!packed) {
-    return tma ? k_substep<T, 0, 1, true> : k_substep<T, 0, 1, false>;
+    return tma ? k_substep<T, 0, 1, true, EVEN> : k_substep<T, 0, 1, false, EVEN>;
   }
-  return tma ? k_substep<T, 1, 8, true> : k_substep<T, 1, 8, false>;
+  return tma ? k_substep<T, 1, 8, true, EVEN> : k_substep<T, 1, 8, false, EVEN>;
+}
+template <typename T>
+auto step_kernel(const StepForm& f, int ns) -> void (*)(StepArgs<T>) {
+  return f.even ? step_kernel<T, true>(ns, f.tma, f.packed)
+                : step_kernel<T, false>(ns, f.tma, f.packed);
 }
 
 template <typename T>
-cudaError_t launch_substep(const StepArgs<T>& a, int grid, int block, size_t smem, bool tma,
-                           bool packed, cudaStream_t s, bool overlap) {
-  void (*k)(StepArgs<T>) = step_kernel<T>(a.ns, tma, packed);
+cudaError_t launch_substep(const StepArgs<T>& a, int grid, int block, size_t smem,
+                           const StepForm& f, cudaStream_t s, bool overlap) {
+  void (*k)(StepArgs<T>) = step_kernel<T>(f, a.ns);
   if (overlap) return launch_overlapped(k, grid, block, smem, s, a);
   k<<<grid, block, smem, s>>>(a);
   return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t substep_prepare(int ns, int block, size_t smem, bool tma, bool packed,
+cudaError_t substep_prepare(int ns, int block, size_t smem, const StepForm& f,
                             int* blocks_per_sm) {
-  void (*k)(StepArgs<T>) = step_kernel<T>(ns, tma, packed);
+  void (*k)(StepArgs<T>) = step_kernel<T>(f, ns);
   const cudaError_t e = mm::raise_smem_limit(k, smem);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, block, smem);
 }
 
-#define MM_STEP_INST(T)                                                              \
-  template cudaError_t launch_substep<T>(const StepArgs<T>&, int, int, size_t, bool, \
-                                         bool, cudaStream_t, bool);                  \
-  template cudaError_t substep_prepare<T>(int, int, size_t, bool, bool, int*);
+#define MM_STEP_INST(T)                                                                     \
+  template cudaError_t launch_substep<T>(const StepArgs<T>&, int, int, size_t,              \
+                                         const StepForm&, cudaStream_t, bool);              \
+  template cudaError_t substep_prepare<T>(int, int, size_t, const StepForm&, int*);
 MM_STEP_INST(float)
 MM_STEP_INST(double)
 

@@ -338,9 +338,36 @@ __device__ __forceinline__ float row_sum_x2(const float2 (&M)[4], int vl, int nl
     const float2 a = __fadd2_rn(M[0], M[1]), b = __fadd2_rn(M[2], M[3]);
     return packed_sum(a.x + a.y, nl, sl) + packed_sum(b.x + b.y, nl, sl);
   }
+  if (nl == 4) {
+    // two or four lanes a row: each keeps half of the sums at every stride
+    const bool up2 = (sl & 2) != 0, up1 = (sl & 1) != 0;
+    float k[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const float give = up2 ? M[h].x : M[h].y;
+      k[h] = (up2 ? M[h].y : M[h].x) + __shfl_xor_sync(0xffffffffu, give, 2);
+    }
+    const float g0 = up1 ? k[0] : k[1], g1 = up1 ? k[2] : k[3];
+    const float m0 = (up1 ? k[1] : k[0]) + __shfl_xor_sync(0xffffffffu, g0, 1);
+    const float m1 = (up1 ? k[3] : k[2]) + __shfl_xor_sync(0xffffffffu, g1, 1);
+    float u = m0 + m1;
+    u += __shfl_xor_sync(0xffffffffu, u, 1);
+    return u + __shfl_xor_sync(0xffffffffu, u, 2);
+  }
+  if (nl == 2) {
+    const bool up = (sl & 1) != 0;
+    float k[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const float give = up ? M[h].x : M[h].y;
+      k[h] = (up ? M[h].y : M[h].x) + __shfl_xor_sync(0xffffffffu, give, 1);
+    }
+    const float u = (k[0] + k[2]) + (k[1] + k[3]);
+    return u + __shfl_xor_sync(0xffffffffu, u, 1);
+  }
   float2 s[4] = {M[0], M[1], M[2], M[3]};
 #pragma unroll
-  for (int o = 2; o > 0; o >>= 1) {  // (ns <= 32 here: four lanes at most)
+  for (int o = 2; o > 0; o >>= 1) {  // (one lane or three: ns <= 32 here)
     if (o < nl) {
 #pragma unroll
       for (int h = 0; h < 4; ++h) {

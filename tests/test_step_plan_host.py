@@ -1,5 +1,5 @@
 """The plan of the streaming kernels' rows (mm_plan.h, compiled for the host):
-chunks of whole passes, and by its own cost of a pass never dearer than rows of
+no more passes of rows than the cell has, and by its own cost of a pass never dearer than rows of
 V nodes to a lane in equal chunks that divide the orientations, which packed
 rows replaced."""
 import os
@@ -44,12 +44,12 @@ def lane_rpp(ns, V):
     return 32 // seg
 
 
-def test_chunks_are_whole_passes(plans):
+def test_chunks_cost_no_pass(plans):
     for (nth, ns, tsz, V), (packed, rows, chunks, passes, _) in plans.items():
         rpp = 32 // -(-ns // 8) if packed else lane_rpp(ns, V)
         at = (nth, ns, tsz, V)
         assert rows <= nth and (chunks - 1) * rows < nth <= chunks * rows, at
-        assert rows == nth or rows % rpp == 0, at
+        assert passes == -(-nth // rpp), at  # no pass is cut short but the last
         assert rows * ns * tsz <= 4096 or rows <= rpp, at
         assert passes == (chunks - 1) * -(-rows // rpp) + -(-(nth - (chunks - 1) * rows) // rpp), at
         # bulk copies wherever a cell is a whole number of 16-byte vectors
