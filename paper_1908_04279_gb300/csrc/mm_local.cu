@@ -45,7 +45,7 @@ constexpr int kLocalStatusBit = 4;  // status bit 2: a local step count out of r
 template <typename T>
 struct LocalArgs {
   int nth, ns, seg;
-  int rows_per_warp;  // consecutive s-rows of a cell per warp (multiple of 32 / seg)
+  int rows_per_warp;  // consecutive s-rows of a cell per warp (whole passes)
   int nbuf;           // shared-memory row buffers (2: the next cell's copy overlaps)
   int bulk;           // 1: the cell's rows arrive by one bulk copy
   long long ncells;
@@ -126,7 +126,8 @@ __host__ __device__ inline LocalSmem local_smem_layout(int nbuf, int nth, int ns
   return L;
 }
 
-template <typename T, int V>
+// PACKED: rows packed (float64), else V nodes to a lane.
+template <typename T, int V, bool PACKED>
 __global__ void __launch_bounds__(256, 2) k_motor_local(const LocalArgs<T> a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int nth = a.nth, ns = a.ns, seg = a.seg, nbuf = a.nbuf;
@@ -164,7 +165,7 @@ __global__ void __launch_bounds__(256, 2) k_motor_local(const LocalArgs<T> a) {
   }
   __syncthreads();
 
-  const LaneGeom lg = sizeof(T) == 8 ? packed_lanes(lane, ns) : lane_geom(lane, seg, ns, V);
+  const LaneGeom lg = PACKED ? packed_lanes(lane, ns) : lane_geom(lane, seg, ns, V);
   const int r0 = w * a.rows_per_warp;
   const int cnt = max(0, min(a.rows_per_warp, nth - r0));
   const T ds = (T)a.ds, dth = (T)a.dth;
@@ -208,7 +209,7 @@ __global__ void __launch_bounds__(256, 2) k_motor_local(const LocalArgs<T> a) {
       const bool last = step == n - 1;
       T* nbs = nbcol + (step & 1) * nth;
       T* dst = last ? gdst : rows;
-      if constexpr (sizeof(T) == 8) {
+      if constexpr (PACKED) {
         // eight nodes to a lane (the float64 pipe bounds this kernel too); rows of
         // odd length are updated in place and copied out at the end
         if (cnt > 0) {
@@ -394,17 +395,10 @@ __global__ void __launch_bounds__(32 * kLocalRegWarps)
 }
 
 template <typename T, int V>
-cudaError_t local_prepare(int block, size_t smem, int* bps) {
-  cudaError_t e = mm::raise_smem_limit(k_motor_local<T, V>, smem);
-  if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, k_motor_local<T, V>, block, smem);
-}
-
-template <typename T, int V>
-cudaError_t launch_motor_local(const LocalArgs<T>& a, int grid, int block, size_t smem,
-                               cudaStream_t s) {
-  k_motor_local<T, V><<<grid, block, smem, s>>>(a);
-  return cudaGetLastError();
+auto local_kernel(bool packed) -> decltype(&k_motor_local<T, V, false>) {
+  if constexpr (sizeof(T) == 8)
+    if (packed) return k_motor_local<T, V, true>;
+  return k_motor_local<T, V, false>;
 }
 
 }  // namespace mm
@@ -413,17 +407,21 @@ using namespace mmh;
 
 namespace {
 
-// Block shape of the motor kernel: rows in groups of rpp = 32 / seg (one warp
-// pass), at most 8 warps, each warp owning `passes` consecutive groups.
+// Block shape of the motor kernel: rows in groups of rpp (one warp pass), at most
+// 8 warps, each warp owning `passes` consecutive groups.
 struct LocalPlan {
   int block, rows_per_warp, nbuf, bulk, grid;
+  bool packed;  // form of the rows: what a pass costs decides (mm_plan.h)
   size_t smem;
 };
 
 template <typename T, int V>
 mm_status local_plan(mm_handle* h, LocalPlan* p) {
   const int nth = h->g.ntheta, ns = h->g.ns;
-  const int rpp = sizeof(T) == 8 ? 32 / ((ns + 7) / 8) : 32 / h->seg;
+  const int pr = packed_rpp(ns), lr = 32 / h->seg;
+  p->packed = sizeof(T) == 8 && (nth + pr - 1) / pr * pass_cost(true, V, 8) <=
+                                    (nth + lr - 1) / lr * pass_cost(false, V, 8);
+  const int rpp = p->packed ? pr : lr;
   const int groups = (nth + rpp - 1) / rpp;
   const int passes = (groups + 7) / 8;
   const int nw = (groups + passes - 1) / passes;
@@ -440,7 +438,9 @@ mm_status local_plan(mm_handle* h, LocalPlan* p) {
     return fail(h, MM_ERR_UNSUPPORTED,
                 "ntheta * ns too large: one cell's motor rows must fit in shared memory");
   int bps = 0;
-  CK((mm::local_prepare<T, V>(p->block, p->smem, &bps)));
+  auto k = mm::local_kernel<T, V>(p->packed);
+  CK(mm::raise_smem_limit(k, p->smem));
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k, p->block, p->smem));
   if (bps < 1) return fail(h, MM_ERR_UNSUPPORTED, "local-step kernel cannot be resident");
   long long g = (long long)bps * h->sms;
   if (g > h->ncells) g = h->ncells;
@@ -510,7 +510,8 @@ mm_status run_local(mm_handle* h, double Tint, const int* nin) {
       return MM_OK;
     }
   }
-  CK((mm::launch_motor_local<T, V>(a, p.grid, p.block, p.smem, h->stream)));
+  mm::local_kernel<T, V>(p.packed)<<<p.grid, p.block, p.smem, h->stream>>>(a);
+  CK(cudaGetLastError());
   return MM_OK;
 }
 
