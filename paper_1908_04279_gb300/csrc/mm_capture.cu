@@ -128,20 +128,21 @@ __device__ __forceinline__ void rc_walk(const T (&M)[kRcV], unsigned mask, T (&D
   }
 }
 
-// Alg. 2 per anchor r0 (block per anchor, grid-strided): the RK2 of Eq. 4 on
+// Alg. 2 per anchor r0 (WPA warps per anchor, grid-strided): the RK2 of Eq. 4 on
 // every configuration of B_rc(r0) (Mf(r0) frozen over both stages, binding
 // k_on Mf(r0) w), the line sums of Mb ds, C(r0) = sum over lines of
 // psi(filament cell, k) (line sum) dtheta with psi = psi_c (psi^{n+1}), the
-// scale-down where C exceeds M (the block rescales the entries and line sums it
+// scale-down where C exceeds M (the warps rescale the entries and line sums they
 // wrote) and Mf = M - C. init = 1: dt = 0 (the set-up: C, the scale-down, Mf
 // and the line sums of a loaded state).
-// A block rather than a warp takes an anchor so that the last wave is short: at
+// Four warps (a block) rather than one take an anchor so that the last wave is short: at
 // 64^2 x 32^2 the 4096 anchors are 4.5 to a block, six blocks to an SM, but were one
 // to a warp, 27 of an SM's 32 warps each 62 chunks deep. Six blocks per SM leave 80
 // registers (eight leave 64). Bound by instruction issue and the latency of the
 // tables and of psi: 222 -> 180 us at 64^2 x 32^2, r_c = 1.5 cells. Factors in place
 // of the flags' selects (packed products) and table entries loaded a chunk ahead
-// cost more in registers than they saved.
+// cost more in registers than they saved. Anchors of few chunks go to a warp each
+// (rc_warps).
 // A warp's (anchor, chunk) items stream through a ring of S shared-memory
 // stages filled by asynchronous copies S items ahead (coalesced 4/8-byte
 // copies: a chunk may start anywhere); lane l computes the chunk's entries
@@ -150,7 +151,7 @@ __device__ __forceinline__ void rc_walk(const T (&M)[kRcV], unsigned mask, T (&D
 #ifndef MM_RC_MIN_BLOCKS
 #define MM_RC_MIN_BLOCKS 6
 #endif
-template <typename T, int S>
+template <typename T, int S, int WPA>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? MM_RC_MIN_BLOCKS : 1)
     k_rc_motor(const RcArgs<T> x, const T* psi_c, int init) {
   extern __shared__ __align__(16) unsigned char rc_ring_raw[];
@@ -163,11 +164,13 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? MM_RC_MIN_BLOCKS : 1)
   const T hk = hdt * kon, fk = dt * kon;
   const T ds = (T)x.ds, dth = (T)x.dth;
   const int nx = x.nx, ny = x.ny, nth = x.nth, nch = x.nchunks;
-  const long long G = gridDim.x;
-  // this warp's items: chunks wib, wib + 4, ... of the block's anchors in turn;
-  // the cursor of the next one to copy runs S items ahead
-  long long ia = wib < nch ? blockIdx.x : x.ncells;
-  int ich = wib, istage = 0;
+  // this warp's group and its place there; anchors a0, a0 + G, ... are the group's
+  const int grp = wib / WPA, wi = wib - grp * WPA;
+  const long long a0 = blockIdx.x * (4LL / WPA) + grp, G = gridDim.x * (4LL / WPA);
+  // its items: chunks wi, wi + WPA, ... of the group's anchors in turn; the cursor
+  // of the next one to copy runs S items ahead
+  long long ia = wi < nch ? a0 : x.ncells;
+  int ich = wi, istage = 0;
   auto issue = [&]() {
     if (ia < x.ncells) {
       const int4 cd = x.chunk[ich];
@@ -178,8 +181,8 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? MM_RC_MIN_BLOCKS : 1)
         const int p = 32 * v + lane;
         if (p < cd.y) cp_async_t(st + p, src + p);
       }
-      if ((ich += 4) >= nch) {
-        ich = wib;
+      if ((ich += WPA) >= nch) {
+        ich = wi;
         ia += G;
       }
       if (++istage == S) istage = 0;
@@ -190,12 +193,12 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? MM_RC_MIN_BLOCKS : 1)
   for (int q = 0; q < S; ++q) issue();
   __shared__ T s_c[2][4];
   int stage = 0, par = 0;
-  for (long long a = blockIdx.x; a < x.ncells; a += G, par ^= 1) {
+  for (long long a = a0; a < x.ncells; a += G, par ^= 1) {
     const T mfa = x.mf[a];
     const int ay = (int)a / nx, ax = (int)a - ay * nx;
     T* La = x.ls + a;  // (line l at l ncells)
     T cacc = T(0);
-    for (int ch = wib; ch < nch; ch += 4) {
+    for (int ch = wi; ch < nch; ch += WPA) {
       const int4 cd = x.chunk[ch];
       const unsigned mask = x.cmask[ch * 32 + lane];
       T wv[kRcV];
@@ -288,20 +291,29 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? MM_RC_MIN_BLOCKS : 1)
       __syncwarp();
       issue();
     }
-    // the anchor's coarse density over the block's warps, in order
-    cacc = warp_sum_t(cacc);
-    if (lane == 0) s_c[par][wib] = cacc;
-    __syncthreads();
-    const T C = ((s_c[par][0] + s_c[par][1]) + s_c[par][2]) + s_c[par][3];
+    // the anchor's coarse density over its warps, in order
+    T C = warp_sum_t(cacc);
+    if constexpr (WPA > 1) {
+      if (lane == 0) s_c[par][wib] = C;
+      static_assert(WPA == 4, "a block's barrier");
+      __syncthreads();
+      const T* sc = s_c[par] + grp * WPA;
+      C = sc[0];
+#pragma unroll
+      for (int q = 1; q < WPA; ++q) C += sc[q];
+    } else {
+      __syncwarp();
+    }
     const T Mt = x.mtot[a];
-    if (Mt < C) {  // Alg. 2 scale-down at r0 (rare): the block rescales what it wrote
+    const int t = wi * 32 + lane;
+    if (Mt < C) {  // Alg. 2 scale-down at r0 (rare): its warps rescale what they wrote
       const T f = Mt / C;
       T* Mall = x.mb + (size_t)a * x.nconf;
-      for (int e = threadIdx.x; e < x.nconf; e += blockDim.x) Mall[e] = __ldcg(Mall + e) * f;
-      for (int l = threadIdx.x; l < x.nlines; l += blockDim.x)
+      for (int e = t; e < x.nconf; e += 32 * WPA) Mall[e] = __ldcg(Mall + e) * f;
+      for (int l = t; l < x.nlines; l += 32 * WPA)
         La[(size_t)l * x.ncells] = __ldcg(La + (size_t)l * x.ncells) * f;
     }
-    if (threadIdx.x == 0) {
+    if (t == 0) {
       const T Cc = Mt < C ? Mt : C;
       x.c[a] = Cc;
       x.mf[a] = Mt - Cc;
@@ -593,6 +605,19 @@ constexpr size_t rc_ring_bytes() {
   return (size_t)4 * kRcStages * mm::kRcChunk * sizeof(T);
 }
 
+// Warps of an anchor: a block's four where there are at least three chunks to each,
+// or fewer anchors than blocks at once; else one, so that none waits for the others
+// at every anchor (us a substep with one and with four: 8 x 8 rows, 3 chunks, 164
+// and 201; 16 x 16, 11 chunks, 101 and 108; 32 x 12, 16 chunks, 116 and 106; 32 x 32, 43
+// chunks, 87 and 74).
+int rc_warps(const mm_handle* h, int chunks) {
+  return chunks >= 12 || h->ncells <= 6LL * h->sms ? 4 : 1;
+}
+template <typename T>
+auto rc_motor(int warps) -> decltype(&mm::k_rc_motor<T, kRcStages, 4>) {
+  return warps == 4 ? mm::k_rc_motor<T, kRcStages, 4> : mm::k_rc_motor<T, kRcStages, 1>;
+}
+
 int rc_grid(mm_handle* h, long long work, int per_block) {
   long long b = (work + per_block - 1) / per_block;
   return (int)std::max<long long>(1, std::min<long long>(b, 16LL * h->sms));
@@ -610,7 +635,7 @@ cudaError_t rc_substep_t(mm_handle* h, int parity, cudaStream_t s) {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const mm::RcArgs<T> x = rc_args<T>(h);
-  mm::k_rc_motor<T, kRcStages><<<h->rc_motor_grid, 128, rc_ring_bytes<T>(), s>>>(
+  rc_motor<T>(h->rc_warps)<<<h->rc_motor_grid, 128, rc_ring_bytes<T>(), s>>>(
       x, (const T*)h->psi[parity ^ 1], 0);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   mm::k_rc_nb<T><<<rc_grid(h, h->ncells * h->g.ntheta, 256), 256, 0, s>>>(x, (T*)h->nb[parity ^ 1]);
@@ -620,7 +645,7 @@ cudaError_t rc_substep_t(mm_handle* h, int parity, cudaStream_t s) {
 template <typename T>
 cudaError_t rc_init_t(mm_handle* h) {
   const mm::RcArgs<T> x = rc_args<T>(h);
-  mm::k_rc_motor<T, kRcStages><<<h->rc_motor_grid, 128, rc_ring_bytes<T>(), h->stream>>>(
+  rc_motor<T>(h->rc_warps)<<<h->rc_motor_grid, 128, rc_ring_bytes<T>(), h->stream>>>(
       x, (const T*)h->psi[h->parity], 1);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -827,14 +852,16 @@ mm_status mm_set_capture(mm_handle* h, double rc) {
     q[5] = L[l].off;
   }
   h->rc_host_w = w;
+  h->rc_warps = rc_warps(h, h->rc_nchunks);
   int per_sm = 0;
   CK(h->prec == MM_FP64
-         ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-               &per_sm, mm::k_rc_motor<double, kRcStages>, 128, rc_ring_bytes<double>())
-         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-               &per_sm, mm::k_rc_motor<float, kRcStages>, 128, rc_ring_bytes<float>()));
+         ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rc_motor<double>(h->rc_warps),
+                                                         128, rc_ring_bytes<double>())
+         : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rc_motor<float>(h->rc_warps), 128,
+                                                         rc_ring_bytes<float>()));
+  const int apb = 4 / h->rc_warps;  // anchors of a block
   h->rc_motor_grid = (int)std::max<long long>(
-      1, std::min<long long>(h->ncells, (long long)std::max(per_sm, 1) * h->sms));
+      1, std::min<long long>((h->ncells + apb - 1) / apb, (long long)std::max(per_sm, 1) * h->sms));
   h->capture = true;
   // a new layout: the motors are discarded (Mb = 0, Mf = M); psi is kept
   if (h->have_state) return run_init_capture(h);

@@ -155,7 +155,7 @@ struct mm_handle {
   // finite capture radius (mm_set_capture): the anchor axis of Mb
   bool capture = false;
   double rc = 0.0;
-  int rc_nconf = 0, rc_nlines = 0, rc_nchunks = 0, rc_motor_grid = 1;
+  int rc_nconf = 0, rc_nlines = 0, rc_nchunks = 0, rc_motor_grid = 1, rc_warps = 4;
   void* rc_mb = nullptr;   // [cells][nconf] motor density, anchor-major (template order)
   void* rc_ls = nullptr;   // [cells][nlines] line sums of Mb ds
   void* rc_tab = nullptr;  // the template's device tables (one block)
