@@ -155,11 +155,13 @@ mm_status mm_set_dt(mm_handle* h, double dt);
  *      stage);
  *   3. n_b, the coarse density (Eq. 5) with psi at the new time, the
  *      scale-down of Alg. 2, and Mf = M - C (Eq. 6).
- * Asynchronous on the handle's stream. MM_FP32_MIXED instances of up to about
- * the size of L2 run all of a call's substeps (two or more) in one cooperative
- * launch with the motor density resident on the chip; other calls run one
- * launch per substep as a captured CUDA graph. A call on a capturing stream
- * always runs one launch per substep. */
+ * Asynchronous on the handle's stream. MM_FP32_MIXED instances run all of a
+ * call's substeps (two or more) in one cooperative launch with the motor density
+ * kept on the chip, as far as it fits: up to 250 MB of motor density, 100 to 200 MB
+ * beyond 32 orientations, and any size that the launch can hold where ns is no
+ * multiple of 4 and there are at most 32 orientations (half of these bytes for a
+ * call of two). Other calls run one launch per substep as a captured CUDA graph; a
+ * call on a capturing stream always does. */
 mm_status mm_micro_step(mm_handle* h, int n_substeps);
 
 /* Macroscale moments (Alg. 1 after the inner loop), all float64.

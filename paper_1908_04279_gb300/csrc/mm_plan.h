@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <cstddef>
+#include <cstdint>
 
 namespace mmh {
 
@@ -71,6 +72,32 @@ inline RowPlan row_plan(int total, int ns, int V, int tsz, int chunk_bytes) {
   const RowPlan q = chunk_plan(false, total, row_bytes, lane_rpp(ns, V), chunk_bytes);
   if (tsz == 4 && V != 4) return V == 8 ? q : p;
   return p.passes * pass_cost(true, V, tsz) <= q.passes * pass_cost(false, V, tsz) ? p : q;
+}
+
+// Most bytes of Mb for which one resident launch (mm_resident.cu) of n substeps is
+// taken rather than the streaming kernel. Up to 32 orientations, a lane each in the
+// psi phase, it is the faster one up to 250 MB, twice the L2, where HBM comes to
+// bound both (256^2 x 32^2 in us: 124 against 134; 256^2 x 64^2 498 against 390);
+// beyond, a lane takes several and the streaming kernel wins earlier, the sooner
+// the fuller its lanes: rows of a power of two of full lanes from 100 MB on (64
+// orientations x 16: 80 MB 0.94 of its time, 140 MB 1.13, 245 MB 1.20; x 32 1.12 at
+// 245 MB), of three quarters of one from 140 MB (x 24). Rows of no multiple of four
+// nodes leave the streaming kernel the slower one up to what the resident plan
+// holds at all (400^2 x 24 x 30, 460 MB: 244 against 331 us; beyond 32 orientations
+// they part at 200 MB: 48 x 31 1.06 at 450 MB). A call of two substeps pays for
+// loading and storing what is kept: half of the bytes (192^2 x 32^2, 151 MB, 85
+// against 79 us a substep).
+inline size_t resident_limit(int nth, int ns, int n) {
+  size_t mb = 250;
+  if (ns % 4 != 0) {
+    if (nth <= 32) return SIZE_MAX;
+    mb = 200;
+  } else if (nth > 32 && ns % 8 == 0) {
+    int seg = 1;
+    while (seg < ns / 8) seg <<= 1;
+    mb = ns / 8 == seg ? 100 : 4 * (ns / 8) >= 3 * seg ? 140 : 250;
+  }
+  return (mb << 20) / (n == 2 ? 2 : 1);
 }
 
 }  // namespace mmh

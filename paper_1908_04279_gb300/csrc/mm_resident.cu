@@ -45,7 +45,7 @@
 // `tiles` passes of its rows and reads and writes the others every substep, each
 // lane copying its own values to its own slots two passes ahead (cp.async) and
 // storing the new ones straight back; they stay in the L2 up to about twice its
-// size (resident_pays says where k_substep takes over).
+// size (resident_limit says where k_substep takes over).
 //
 // A batch's members are independent, so several go into one launch
 // (k_substep_resident_group), each over its own share of the SMs with its own
@@ -692,9 +692,8 @@ const void* resident_kernel(int NL) {
 // How an instance goes over `grid` blocks of one SM each: ceil(cells / grid) cells
 // to a block, the same number `own` to each worker, `tiles` passes of a worker's
 // rows kept in shared memory and, where that is not all of them, a ring for the
-// others, which are read and written every substep. False where it does not
-// fit, or where keeping too little of Mb on the chip gains nothing over
-// k_substep.
+// others, which are read and written every substep. False where it does not fit
+// (resident_limit says where it pays).
 struct ResidentPlan {
   int own, workers, tiles, ring;
   size_t smem;
@@ -716,18 +715,10 @@ bool resident_plan(const mm_handle* h, int grid, ResidentPlan* p) {
   return true;
 }
 
-// Whether the resident kernel is the faster one for an instance it can hold.
-// Its arithmetic runs at about 650 G motor updates per second (25 us a substep
-// at 128^2 x 32^2, where k_substep takes 35), k_substep's at HBM speed where a
-// row fills its lanes: from about 250 MB of Mb on, twice the L2, HBM bounds both
-// and the bulk-copy rings of k_substep keep more of it in flight (256^2 x 32^2,
-// 268 MB: 127 against 131 us; 160^2 x 64^2, 420 MB: 189 against 155). Where a row
-// is no multiple of 4 nodes k_substep's warps copy their chunks themselves, and
-// the resident kernel is the faster one up to the most cells it takes (2^16):
-// 200 x 150 x 24 x 30, 86 MB, 43 against 65 us; 256^2 x 24 x 30, 189 MB, 93 against
-// 137; 256^2 x 32 x 31, 260 MB, 146 against 165.
-bool resident_pays(const mm_handle* h) {
-  return h->g.ns % 4 != 0 || h->mbn * h->tsz <= (size_t)250 << 20;
+// Whether the resident kernel is the faster one for n substeps of an instance it
+// can hold.
+bool resident_pays(const mm_handle* h, int n) {
+  return h->mbn * h->tsz <= resident_limit(h->g.ntheta, h->g.ns, n);
 }
 
 // Kernel arguments of n substeps of h's live state; the exchange's tags and
@@ -801,7 +792,7 @@ mm_status resident_configure(mm_handle* h) {
   h->res_NL = ns % 8 == 0 && (nl == 2 || nl == 4 || nl == 8) ? nl : 0;
   const int grid = (int)std::min<long long>({h->sms, h->ncells, 32 * mm::kResXch});
   ResidentPlan p;
-  if (!resident_pays(h) || !resident_plan(h, grid, &p)) return MM_OK;
+  if (!resident_pays(h, 3) || !resident_plan(h, grid, &p)) return MM_OK;
   const void* f = resident_kernel(h->res_NL);
   CK(mm::raise_smem_limit(f, kResidentBudget));
   int bps = 0;
@@ -815,7 +806,8 @@ mm_status resident_configure(mm_handle* h) {
 // that pays, for a single substep, with another substep kernel in effect, or on
 // a stream being captured (the ordering event belongs to no capture).
 static bool resident_applies(mm_handle* h, int n) {
-  if (h->res_grid == 0 || n < 2 || h->anchors || h->capture || h->tangent) return false;
+  if (h->res_grid == 0 || n < 2 || h->anchors || h->capture || h->tangent || !resident_pays(h, n))
+    return false;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   return cudaStreamIsCapturing(h->stream, &cs) == cudaSuccess &&
          cs == cudaStreamCaptureStatusNone;

@@ -33,7 +33,7 @@ def plans(tmp_path_factory):
     text = "\n".join(" ".join(map(str, c)) for c in cases())
     out = subprocess.run([exe], input=text, capture_output=True, text=True, check=True).stdout
     got = [line.split() for line in out.splitlines()]
-    return {c: (int(q[0]), int(q[1]), int(q[2]), int(q[3]), float(q[4]))
+    return {c: (int(q[0]), int(q[1]), int(q[2]), int(q[3]), float(q[4]), int(q[5]), int(q[6]))
             for c, q in zip(cases(), got)}
 
 
@@ -45,7 +45,7 @@ def lane_rpp(ns, V):
 
 
 def test_chunks_cost_no_pass(plans):
-    for (nth, ns, tsz, V), (packed, rows, chunks, passes, _) in plans.items():
+    for (nth, ns, tsz, V), (packed, rows, chunks, passes, *_) in plans.items():
         rpp = 32 // -(-ns // 8) if packed else lane_rpp(ns, V)
         at = (nth, ns, tsz, V)
         assert rows <= nth and (chunks - 1) * rows < nth <= chunks * rows, at
@@ -57,7 +57,7 @@ def test_chunks_cost_no_pass(plans):
 
 
 def test_no_dearer_than_equal_chunks_of_lanes(plans):
-    for (nth, ns, tsz, V), (*_, cost) in plans.items():
+    for (nth, ns, tsz, V), (_, _, _, _, cost, *_) in plans.items():
         if tsz == 4 and V == 1:
             continue  # (one node to a lane costs 3.5 times a packed one)
         c = 1
@@ -66,3 +66,24 @@ def test_no_dearer_than_equal_chunks_of_lanes(plans):
         passes = c * -(-(nth // c) // lane_rpp(ns, V))
         before = passes * (V if tsz == 4 else 36.0 if V == 2 else 23.0)
         assert cost <= before * (1 + 1e-12), (nth, ns, tsz, V)
+
+
+# a substep of the resident kernel over one of the streaming kernel, as timed on a
+# GB300 in calls of 16, by orientations, nodes and MB of Mb
+TIMED = {(8, 64): {245: 0.62}, (16, 16): {180: 0.54}, (24, 64): {245: 0.95},
+         (32, 32): {80: 0.67, 140: 0.83, 245: 0.93}, (32, 64): {245: 0.99}, (32, 31): {450: 0.98},
+         (24, 30): {450: 0.74}, (40, 16): {80: 0.86, 140: 1.02, 245: 1.09}, (40, 20): {200: 0.99},
+         (48, 16): {80: 0.89, 140: 1.10, 245: 1.17}, (48, 32): {80: 0.74, 160: 1.02, 245: 1.10},
+         (64, 16): {60: 0.96, 140: 1.13, 245: 1.20}, (64, 32): {80: 0.86, 200: 1.13, 245: 1.12},
+         (64, 64): {80: 0.81, 160: 1.05, 245: 1.09}, (64, 8): {80: 0.92, 120: 1.06},
+         (64, 24): {120: 0.90, 245: 1.03}, (64, 40): {245: 0.84}, (48, 31): {120: 0.94, 450: 1.06},
+         (64, 31): {120: 0.90, 450: 1.09}}
+
+
+def test_resident_launch_where_it_was_timed_faster(plans):
+    by = {(nth, ns): q[5:] for (nth, ns, tsz, _), q in plans.items() if tsz == 4}
+    for (nth, ns), timed in TIMED.items():
+        for mb, ratio in timed.items():
+            assert (mb << 20 <= by[nth, ns][1]) == (ratio < 1.0), (nth, ns, mb)
+    # two substeps: half of the bytes (151 MB of 32 x 32 1.08, 67 MB of 16 x 16 0.65)
+    assert by[32, 32][0] < 151 << 20 and by[16, 16][0] > 67 << 20
