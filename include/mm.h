@@ -491,7 +491,9 @@ mm_status mm_sync(mm_handle* h);
 /* Test and tuning knobs of the substep kernel (no counterpart in the paper).
  * wait_limit: polls of an mbarrier before a device wait gives up (default
  * 4194304); flags bit 0: wait on a barrier nothing completes, so that
- * every wait runs out -- used by tests of the timeout path, never in production. */
+ * every wait runs out; flags >> 8, k > 0: the handle's k-th cooperative launch from
+ * here returns MM_ERR_CUDA on the host and is not made -- used by tests of the
+ * failure paths, never in production. */
 mm_status mm_debug_set(mm_handle* h, unsigned int wait_limit, unsigned int flags);
 
 /* Launch plan of the substep kernel, for tests and profiling: info[0..9] =

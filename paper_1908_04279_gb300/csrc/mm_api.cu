@@ -863,9 +863,10 @@ mm_status mm_sync(mm_handle* h) {
 
 mm_status mm_debug_set(mm_handle* h, unsigned int wait_limit, unsigned int flags) {
   if (!h) return MM_ERR_INVALID;
+  h->fail_launches = (int)(flags >> 8);
   if (h->batch) {
     for (mm_handle* m : batch_members(h)) {
-      const mm_status st = mm_debug_set(m, wait_limit, flags);
+      const mm_status st = mm_debug_set(m, wait_limit, flags & 0xffu);
       if (st != MM_OK) {
         h->err = m->err;
         return st;

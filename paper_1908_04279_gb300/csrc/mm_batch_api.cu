@@ -349,13 +349,23 @@ mm_status batch_micro_step(mm_handle* h, int n) {
     for (mm_handle* m : B->members) m->parity ^= (n & 1);
     return MM_OK;
   }
+  bool part = false;  // some members have advanced
   if (B->any_rest) {
     if ((st = graph_steps(h, B->rest, n)) != MM_OK) return st;
     for (size_t i = 0; i < B->members.size(); ++i)
       if (!B->resident[i]) B->members[i]->parity ^= (n & 1);
+    part = true;
   }
-  for (ResidentGroup& G : B->groups)
-    if ((st = resident_group_step(h, B->members, G, n)) != MM_OK) return st;
+  for (ResidentGroup& G : B->groups) {
+    if ((st = resident_group_step(h, B->members, G, n)) == MM_OK) {
+      part = true;
+      continue;
+    }
+    if (!part) return st;  // nothing ran: the states are as they were
+    for (mm_handle* m : B->members) m->have_state = false;
+    h->err += "; part of the batch had advanced: set every member's state again";
+    return st;
+  }
   return MM_OK;
 }
 

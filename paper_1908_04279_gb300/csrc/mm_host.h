@@ -184,6 +184,7 @@ struct mm_handle {
   int res_grid = 0, res_NL = 0;
   unsigned res_epoch = 0, res_arrivals = 0;  // tags and arrivals used so far
   size_t res_xch_bytes = 0;
+  int fail_launches = 0;  // tests: the resident launch, counted from here, that is refused (0: none)
   unsigned long long* res_xch = nullptr;  // arrival counter and the psi sums the blocks exchange
   std::map<long long, cudaGraphExec_t> graphs;
   bool use_graphs = true;

@@ -721,8 +721,8 @@ bool resident_pays(const mm_handle* h, int n) {
   return h->mbn * h->tsz <= resident_limit(h->g.ntheta, h->g.ns, n);
 }
 
-// Kernel arguments of n substeps of h's live state; the exchange's tags and
-// arrivals of those substeps are taken.
+// Kernel arguments of n substeps of h's live state. Nothing of h changes until the
+// launch has been made (resident_advance).
 mm::ResidentArgs resident_args(mm_handle* h, int grid, const ResidentPlan& p, int n) {
   mm::ResidentArgs a{};
   a.s = step_args<float>(h, h->parity);
@@ -742,9 +742,15 @@ mm::ResidentArgs resident_args(mm_handle* h, int grid, const ResidentPlan& p, in
   a.epoch = h->res_epoch;
   a.arrivals = h->res_arrivals;
   a.xch = h->res_xch;
+  return a;
+}
+// After the launch: the tags and arrivals of its substeps are used, and the state is
+// theirs. (Taken before a launch that then fails, they would have every later one
+// wait for arrivals that nothing makes.)
+void resident_advance(mm_handle* h, int grid, int n) {
   h->res_epoch += (unsigned)n;
   h->res_arrivals += (unsigned)n * (unsigned)grid;
-  return a;
+  h->parity ^= n & 1;
 }
 
 // Resident launches of one device run one after the other, on whatever
@@ -766,6 +772,8 @@ namespace {
 
 mm_status launch_ordered(mm_handle* h, const void* f, int grid, int block, size_t smem,
                          void** args) {
+  if (h->fail_launches > 0 && --h->fail_launches == 0)  // (tests: mm_debug_set)
+    return cuda_fail(h, "resident launch", cudaErrorLaunchOutOfResources);
   DeviceOrder& o = device_order();
   std::lock_guard<std::mutex> lock(o.m);
   cudaEvent_t& ev = o.last[h->device];
@@ -825,7 +833,7 @@ mm_status resident_substeps(mm_handle* h, int n, bool* done) {
   const mm_status st = launch_ordered(h, resident_kernel(h->res_NL), h->res_grid,
                                       32 * (p.workers + 1), p.smem, args);
   if (st != MM_OK) return st;
-  h->parity ^= n & 1;
+  resident_advance(h, h->res_grid, n);
   *done = true;
   return MM_OK;
 }
@@ -955,7 +963,8 @@ mm_status resident_group_step(mm_handle* h, const std::vector<mm_handle*>& membe
   const mm_status st = launch_ordered(h, (const void*)mm::k_substep_resident_group, G.grid,
                                       G.block, G.smem, args);
   if (st != MM_OK) return st;
-  for (int i : G.member) members[i]->parity ^= n & 1;
+  for (size_t k = 0; k < G.member.size(); ++k)
+    resident_advance(members[G.member[k]], G.blocks[k], n);
   return MM_OK;
 }
 
