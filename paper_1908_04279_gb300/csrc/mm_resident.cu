@@ -161,6 +161,7 @@ __device__ void exchange(const ResidentArgs& a, uint64_t* bars, const float2* s_
       __threadfence();
     }
     ok = __all_sync(0xffffffffu, ok);
+    const bool readable = ok;
     if (ok && lane == 0) mbar_arrive(&bars[1]);  // the neighbours' psi and n_b may be read
     // the sums, all of a lane's words in flight at once (a word may still be on
     // its way when its block's arrival has been counted: the tag tells)
@@ -184,7 +185,9 @@ __device__ void exchange(const ResidentArgs& a, uint64_t* bars, const float2* s_
         atomicOr(&P->status, 1);
         *s_abort = 1;
         __threadfence_block();
-        mbar_arrive(&bars[1]);  // (where the arrivals were counted, the next phase: none waits)
+        // (once a phase: a second arrival would complete the next one, and a worker that
+        // comes late would take this one, two back by then, for not yet completed)
+        if (!readable) mbar_arrive(&bars[1]);
         mbar_arrive(&bars[2]);
       }
       return;
