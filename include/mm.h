@@ -161,7 +161,11 @@ mm_status mm_set_dt(mm_handle* h, double dt);
  * beyond 32 orientations, and any size that the launch can hold where ns is no
  * multiple of 4 and there are at most 32 orientations (half of these bytes for a
  * call of two). Other calls run one launch per substep as a captured CUDA graph; a
- * call on a capturing stream always does. */
+ * call on a capturing stream always does. Cooperative launches of one device wait
+ * for each other where their blocks do not have an SM each: calls of 32 substeps and
+ * more of small instances (up to a quarter of a million motor values at 16 x 16)
+ * run side by side on several streams, larger ones one after the other (a batch,
+ * below, runs many in one launch). */
 mm_status mm_micro_step(mm_handle* h, int n_substeps);
 
 /* Macroscale moments (Alg. 1 after the inner loop), all float64.

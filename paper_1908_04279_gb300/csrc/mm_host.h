@@ -181,7 +181,7 @@ struct mm_handle {
   mm::StepForm form;  // (mm_plan.h)
   size_t smem = 0;
   // many substeps in one launch with Mb on the chip (mm_resident.cu; grid 0: off)
-  int res_grid = 0, res_NL = 0;
+  int res_grid = 0, res_small = 0, res_NL = 0;
   unsigned res_epoch = 0, res_arrivals = 0;  // tags and arrivals used so far
   size_t res_xch_bytes = 0;
   int fail_launches = 0;  // tests: the resident launch, counted from here, that is refused (0: none)

@@ -756,13 +756,24 @@ void resident_advance(mm_handle* h, int grid, int n) {
   h->parity ^= n & 1;
 }
 
-// Resident launches of one device run one after the other, on whatever
-// streams and from whatever threads they come: each fills every SM, and two of
-// them part-way resident would wait for each other's blocks. The event of the
-// last one orders the next.
+// Resident launches of one device, on whatever streams and from whatever threads
+// they come, may run together as long as their blocks have an SM each: two of them
+// part-way resident would wait for each other's blocks. The SMs are shared out as
+// kSlots equal slots; a launch takes as many as its blocks need, the least recently
+// used, and waits for the launches that had them last. (One after the other
+// throughout, 16 handles of 16^2 x 16^2 on as many streams took 63 us a substep of all
+// of them, one launch a substep 9.)
+struct Slots {
+  static constexpr int kSlots = 8;
+  std::vector<cudaEvent_t> ev;  // of launches
+  std::vector<int> uses;        // slots that hold each event
+  int last[kSlots];             // event of the slot's last launch, -1: none
+  unsigned long long used[kSlots] = {}, clock = 0;
+  Slots() { std::fill(last, last + kSlots, -1); }
+};
 struct DeviceOrder {
   std::mutex m;
-  std::map<int, cudaEvent_t> last;
+  std::map<int, Slots> dev;
 };
 DeviceOrder& device_order() {
   static DeviceOrder* d = new DeviceOrder();  // never destroyed: launches may outlive statics
@@ -779,15 +790,53 @@ mm_status launch_ordered(mm_handle* h, const void* f, int grid, int block, size_
     return cuda_fail(h, "resident launch", cudaErrorLaunchOutOfResources);
   DeviceOrder& o = device_order();
   std::lock_guard<std::mutex> lock(o.m);
-  cudaEvent_t& ev = o.last[h->device];
-  if (!ev)
+  Slots& S = o.dev[h->device];
+  const int per = std::max(1, h->sms / Slots::kSlots);
+  const int need = std::min(Slots::kSlots, (grid + per - 1) / per);
+  int order[Slots::kSlots];
+  for (int q = 0; q < Slots::kSlots; ++q) order[q] = q;
+  std::stable_sort(order, order + Slots::kSlots,
+                   [&](int a, int b) { return S.used[a] < S.used[b]; });
+  size_t e = 0;  // an event that no slot holds
+  while (e < S.ev.size() && S.uses[e] > 0) ++e;
+  if (e == S.ev.size()) {
+    cudaEvent_t ev;
     CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-  else
-    CK(cudaStreamWaitEvent(h->stream, ev, 0));
+    S.ev.push_back(ev);
+    S.uses.push_back(0);
+  }
+  for (size_t w = 0; w < S.ev.size(); ++w)
+    if (std::any_of(order, order + need, [&](int q) { return S.last[q] == (int)w; }))
+      CK(cudaStreamWaitEvent(h->stream, S.ev[w], 0));
   CK(cudaLaunchCooperativeKernel(f, dim3((unsigned)grid), dim3((unsigned)block), args, smem,
                                  h->stream));
-  CK(cudaEventRecord(ev, h->stream));
+  CK(cudaEventRecord(S.ev[e], h->stream));
+  ++S.clock;
+  for (int q = 0; q < need; ++q) {
+    const int s = order[q];
+    if (S.last[s] >= 0) --S.uses[S.last[s]];
+    S.last[s] = (int)e;
+    S.used[s] = S.clock;
+  }
+  S.uses[e] = need;
   return MM_OK;
+}
+
+// Blocks of a small instance's longer calls (32 substeps and more): the fewest that
+// leave a worker no more than a few passes, so that several instances run side by
+// side. The chain between the substeps bounds those: 32^2 x 16^2 takes 3.8 us a
+// substep on 35 blocks and on 152, 32^2 x 32^2 4.1 on 69 and 152, 24^2 x 32^2 4.1 on 39
+// and 3.7. A launch's start and end take up to 4 us more on fewer SMs (shorter
+// calls keep all of them), and beyond 32 orientations a substep 1.1 times as long.
+constexpr int kSmallCalls = 32;
+int resident_small_grid(const mm_handle* h, int most) {
+  for (int g = 1; g < most && h->g.ntheta <= 32; ++g) {
+    ResidentPlan p;
+    if (resident_plan(h, g, &p) && p.ring == 0 && p.own <= 2 && p.tiles <= 4 &&
+        p.workers * p.tiles <= 60)
+      return g;
+  }
+  return most;
 }
 
 }  // namespace
@@ -810,6 +859,7 @@ mm_status resident_configure(mm_handle* h) {
   CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, f, 32 * (p.workers + 1), p.smem));
   if (bps < 1) return MM_OK;
   h->res_grid = grid;
+  h->res_small = resident_small_grid(h, grid);
   return MM_OK;
 }
 
@@ -829,14 +879,15 @@ static bool resident_applies(mm_handle* h, int n) {
 mm_status resident_substeps(mm_handle* h, int n, bool* done) {
   *done = false;
   if (!resident_applies(h, n)) return MM_OK;
+  const int grid = n >= kSmallCalls ? h->res_small : h->res_grid;
   ResidentPlan p;
-  if (!resident_plan(h, h->res_grid, &p)) return MM_OK;
-  mm::ResidentArgs a = resident_args(h, h->res_grid, p, n);
+  if (!resident_plan(h, grid, &p)) return MM_OK;
+  mm::ResidentArgs a = resident_args(h, grid, p, n);
   void* args[1] = {&a};
-  const mm_status st = launch_ordered(h, resident_kernel(h->res_NL), h->res_grid,
-                                      32 * (p.workers + 1), p.smem, args);
+  const mm_status st = launch_ordered(h, resident_kernel(h->res_NL), grid, 32 * (p.workers + 1),
+                                      p.smem, args);
   if (st != MM_OK) return st;
-  resident_advance(h, h->res_grid, n);
+  resident_advance(h, grid, n);
   *done = true;
   return MM_OK;
 }

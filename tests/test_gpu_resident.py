@@ -167,3 +167,36 @@ def test_batch_groups(mmod):
             ref = sim.get_state()
         for k in KEYS:
             assert rel_l2(got[i][k], ref[k]) <= 1e-6, (i, k)
+
+
+@pytest.mark.parametrize("dims,handles", [((16, 16, 16, 16), 12), ((32, 32, 16, 16), 6),
+                                          ((20, 17, 24, 30), 5), ((48, 40, 8, 12), 4)])
+def test_small_instances_side_by_side(mmod, dims, handles):
+    """Handles on a stream each, their launches on the chip together, with a large one
+    that takes all of it among them, calls of many substeps and of few: every result
+    is that of the handle alone, bit for bit."""
+    import torch
+    grids = [Grid(*dims)] * handles + [Grid(96, 80, 32, 32)]
+    streams = [torch.cuda.Stream() for _ in grids]
+    got = []
+    for together in (False, True):
+        sims = []
+        for i, (g, s) in enumerate(zip(grids, streams)):
+            sim = mmod.Simulation(g, Rates(k_off=0.5 + 0.1 * i), "fp32", stream=s.cuda_stream)
+            psi, mb, u = inputs(g, 3 + i, 0.3)
+            sim.set_state(psi, mb)
+            sim.set_velocity(u)
+            sims.append(sim)
+        calls = (40, 33, 5, 64)
+        order = ([(i, n) for n in calls for i in range(len(sims))] if together
+                 else [(i, n) for i in range(len(sims)) for n in calls])
+        for i, n in order:
+            sims[i].step(n)
+            if not together:
+                sims[i].sync()
+        got.append([sim.get_state() for sim in sims])
+        for sim in sims:
+            sim.close()
+    for i, (a, b) in enumerate(zip(*got)):
+        for k in KEYS:
+            assert np.array_equal(a[k], b[k]), (i, k)
