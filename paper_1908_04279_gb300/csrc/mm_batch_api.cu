@@ -344,7 +344,7 @@ mm_status batch_micro_step(mm_handle* h, int n) {
     }
     return MM_OK;
   }
-  if (B->groups.empty() || !resident_group_applies(h, n)) {
+  if (B->groups.empty() || !resident_group_applies(h, B->members, n)) {
     if ((st = graph_steps(h, B->all, n)) != MM_OK) return st;
     for (mm_handle* m : B->members) m->parity ^= (n & 1);
     return MM_OK;

@@ -278,7 +278,7 @@ mm_status resident_group_plan(mm_handle* h, const std::vector<mm_handle*>& membe
 void resident_group_free(std::vector<ResidentGroup>* groups);
 mm_status resident_group_step(mm_handle* h, const std::vector<mm_handle*>& members,
                               ResidentGroup& G, int n);
-bool resident_group_applies(mm_handle* h, int n);
+bool resident_group_applies(mm_handle* h, const std::vector<mm_handle*>& members, int n);
 
 // Defined in mm_fluid.cu (thin-gap fluid solve).
 void fluid_free(mm_handle* h);
