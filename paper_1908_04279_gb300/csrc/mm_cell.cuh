@@ -313,20 +313,27 @@ __device__ __forceinline__ void rows_chunk(const T* src_rows, T* dst, int RC, in
 #pragma unroll
     for (int v = 0; v < V; ++v) Ms[v] = fma_t(k.c1, D[v], fma_t(k.c2, M[v], c3));
     walk_dflux<T, V>(Ms, D, lg.first, lg.last, seg);
-    T snb = T(0);
+    T part[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       M[v] = fma_t(k.e1, D[v], fma_t(k.e2, Ms[v], add_rn(M[v], e3)));
-      snb += M[v];
+      part[v] = act ? M[v] : T(0);
     }
-    if (!act) snb = T(0);
     if (act) {
       Pack<T, V> q;
 #pragma unroll
       for (int v = 0; v < V; ++v) q.v[v] = M[v];
       *reinterpret_cast<Pack<T, V>*>(dst + off) = q;
     }
-    snb = seg_sum(snb, seg);
+    T snb;
+    if constexpr (sizeof(T) == 8) {
+      snb = row_sum_lanes<V>(part, seg, lg.sl);
+    } else {
+      snb = part[0];
+#pragma unroll
+      for (int v = 1; v < V; ++v) snb += part[v];
+      snb = seg_sum(snb, seg);
+    }
     if (lg.first && row_ok) s_nb_chunk[r] = snb * ds;
   }
 }

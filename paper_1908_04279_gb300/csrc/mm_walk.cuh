@@ -381,6 +381,31 @@ __device__ __forceinline__ float row_sum_x2(const float2 (&M)[4], int vl, int nl
   return a.x + a.y;
 }
 
+// Sum of a float64 row held V nodes to a lane (2 or 1) over `seg` lanes, zero past
+// its end, valid in its first lane: the additions of packed rows (the even nodes of
+// eight one after the other, the odd ones, the two, then the eights in halving
+// strides), so that n_b has the same bits in either form.
+template <int V>
+__device__ __forceinline__ double row_sum_lanes(const double (&M)[V], int seg, int sl) {
+  constexpr int n = 8 / V;  // lanes of eight nodes
+  double s;
+  auto from = [&](double x, int o) {
+    const double y = __shfl_down_sync(0xffffffffu, x, o);
+    return sl + o < seg ? y : 0.0;
+  };
+  if constexpr (V == 2) {
+    const double x1 = from(M[0], 1), x2 = from(M[0], 2), x3 = from(M[0], 3);
+    const double y1 = from(M[1], 1), y2 = from(M[1], 2), y3 = from(M[1], 3);
+    s = (((M[0] + x1) + x2) + x3) + (((M[1] + y1) + y2) + y3);
+  } else {
+    const double x2 = from(M[0], 2), x4 = from(M[0], 4), x6 = from(M[0], 6);
+    const double e = ((M[0] + x2) + x4) + x6;
+    s = e + from(e, 1);
+  }
+  for (int o = seg >> 1; o >= n; o >>= 1) s += from(s, o);
+  return s;
+}
+
 template <typename T>
 __device__ __forceinline__ T seg_sum(T x, int seg) {
   for (int o = seg >> 1; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o, seg);

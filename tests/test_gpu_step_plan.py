@@ -91,3 +91,29 @@ def test_batch_tiles(mmod, precision, dims):
         _, st = oracle_run(g, r, 7 + i, 3)
         for k in ("psi", "mb", "mf", "c"):
             assert rel_l2(got[i][k], getattr(st, k)) <= TOL[precision], (i, k)
+
+
+def test_fp64_batch_equals_alone_in_either_form(mmod):
+    """The members of a float64 batch share one form of the rows, which need not be the
+    form of a member alone: the same bits all the same."""
+    for dims in ([(12, 9, 8, 8), (20, 16, 31, 32)], [(40, 30, 8, 8), (6, 4, 20, 28)],
+                 [(9, 7, 8, 12), (24, 20, 34, 30)]):
+        grids = [Grid(*d) for d in dims]
+        r = Rates(glide=0.3)
+        with mmod.Batch(grids, [r] * 2, "fp64") as b:
+            for i, sim in enumerate(b.members):
+                psi, mb, u = inputs(sim.grid, 7 + i)
+                sim.set_state(psi, mb)
+                sim.set_velocity(u)
+            b.step(5)
+            b.sync()
+            got = [sim.get_state() for sim in b.members]
+        for i, g in enumerate(grids):
+            psi, mb, u = inputs(g, 7 + i)
+            with mmod.Simulation(g, r, "fp64") as sim:
+                sim.set_state(psi, mb)
+                sim.set_velocity(u)
+                sim.step(5)
+                ref = sim.get_state()
+            for k in ("psi", "mb", "mf", "c"):
+                assert np.array_equal(got[i][k], ref[k]), (dims, i, k)
