@@ -663,9 +663,9 @@ def run_ours(args):
     def ensemble_run(steps):
         """ensemble64: 64 members with uneven grids (N in {32..128}, Ntheta and
         Ns in {16, 32}), k_off log-uniform in [0.05, 5], v_walk in [0.5, 2];
-        after mm_batch_autotune, a step is 500 batched substeps (the members in
-        groups, each group one resident launch; kernel_ms_per_launch is the
-        time of one substep of all members)."""
+        a step is 500 batched substeps (the members in groups, each group one
+        resident launch; kernel_ms_per_launch is the time of one substep of all
+        members)."""
         from paper_1908_04279_gb300.inputs import ensemble_members, member_inputs
         ms_ = ensemble_members()
         b = mm.Batch([m.grid for m in ms_], [m.rates for m in ms_], "fp32",
@@ -700,9 +700,12 @@ def run_ours(args):
                 "ms_per_step": ms_step, "kernel_ms_per_launch": launch,
                 "motor_cells_per_substep": cells, "algorithmic_bytes_per_launch": algo_e,
                 "achieved_gbs": algo_e / (launch * 1e-3) / 1e9,
-                "plan": {k: info[k] for k in ("grid", "block", "tiles", "V", "tile_work",
-                                              "chunk_bytes", "pair_cells")},
-                "autotune_best_ms_per_substep": best["ms_per_substep"],
+                # the tiles of single substeps and recordings: the timed steps are the
+                # groups' resident launches
+                "single_substep_plan": {k: info[k] for k in ("grid", "block", "tiles", "V",
+                                                             "tile_work", "chunk_bytes",
+                                                             "pair_cells")},
+                "single_substep_ms_autotuned": best["ms_per_substep"],
                 "autotune_candidates": len(tune)}
 
     w = WORKLOADS[name]

@@ -443,9 +443,13 @@ mm_status mm_fluid_response(mm_handle* h, double* out, int on_device);
  * together: mm_micro_step on the batch handle runs each substep as ONE launch
  * over all instances (a table of tiles, each a run of cells of one instance
  * holding about the same number of motor values), and the n_substeps of one
- * call as one captured CUDA graph; float32 instances whose motor density the
- * chip can hold go several to one cooperative launch of all n_substeps instead. No counterpart in the paper, which runs one
- * instance at a time.
+ * call as one captured CUDA graph; float32 instances that mm_micro_step would
+ * take whole in one cooperative launch go several to one such launch of all
+ * n_substeps instead (two or more; two only where the members' motor density
+ * together is at most 125 MB), unless a member records an adjoint. No
+ * counterpart in the paper, which runs one instance at a time. If a launch fails
+ * after others of the same call have been made, the members are no longer at the
+ * same substep: the error says so, and every member's state must be set again.
  *
  * mm_create_batch(n, grids, rates, prec, stream, &batch): grids[i], rates[i]
  * for instance i; every instance needs ns divisible by 4 (MM_FP32_MIXED) or 2
@@ -461,10 +465,13 @@ mm_status mm_fluid_response(mm_handle* h, double* out, int on_device);
  * every member; mm_sync on the batch checks every member.
  *
  * mm_batch_autotune(batch, substeps, results, max_results, &n_results): times
- * `substeps` batched substeps for each (tile_work, chunk_bytes) in
+ * `substeps` substeps over tiles for each (tile_work, chunk_bytes) in
  * {1024 .. 32768} x {2048, 4096, 8192} (motor values per tile, bytes per
  * s-row chunk) from the current state, restores the state, and keeps the
- * fastest; results (may be NULL) receives up to max_results timings. The
+ * fastest; results (may be NULL) receives up to max_results timings. The tiles are
+ * those of the members that no cooperative launch takes, or of every member where
+ * there are none of these or no cooperative launches; tiles of every member are
+ * launched by calls of one substep, by recordings and on capturing streams. The
  * choice is cached for the process: a later batch with the same member grids
  * and precision starts with it.
  *
@@ -472,9 +479,10 @@ mm_status mm_fluid_response(mm_handle* h, double* out, int on_device);
  * row length) two cells to a warp (cells_per_warp 2: one chunk holds both
  * cells' rows, half-warps take psi and the close) and one cell to a warp (1).
  *
- * mm_get_launch_info on a batch: grid, block, shared memory, 1, ring stages,
- * largest chunk (values), tiles, values per lane, tile_work, chunk_bytes,
- * tuned (0/1), two cells per warp where possible (0/1). */
+ * mm_get_launch_info on a batch, of the tiles that mm_batch_autotune times: grid,
+ * block, shared memory, 1, ring stages, largest chunk (values), tiles, values per
+ * lane, tile_work, chunk_bytes, tuned (0/1), two cells per warp where possible
+ * (0/1). */
 typedef struct {
   int tile_work;
   int chunk_bytes;

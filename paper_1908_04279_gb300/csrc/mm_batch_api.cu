@@ -41,6 +41,9 @@ struct BatchPlan {
   int chunk_bytes = kChunkBytes;
   int pairs = 1;              // members that can go two cells to a warp do
   TilePlan all, rest;         // every member; the members of no group (when there are both)
+  // the tiles that the longest calls launch: those of the members of no group, or,
+  // where there are none or no groups, those of every member
+  TilePlan& tuned_plan() { return !groups.empty() && any_rest ? rest : all; }
   void* d_args = nullptr;     // [2][n] StepArgs: members at their parities, and flipped
   std::vector<int> args_par;  // member parities the argument tables were built for
   int tuned = 0;
@@ -390,8 +393,8 @@ const std::vector<mm_handle*>& batch_members(mm_handle* h) { return h->batch->me
 // grid, block, shared memory, bulk copies (always), ring stages, largest
 // chunk (values), tiles, V, tile_work, chunk_bytes, tuned, two cells per warp
 mm_status batch_launch_info(mm_handle* h, int* info, int n) {
-  const BatchPlan* B = h->batch;
-  const TilePlan& P = B->all;
+  BatchPlan* B = h->batch;
+  const TilePlan& P = B->tuned_plan();
   const int v[12] = {P.grid,   P.block, (int)P.smem,  1,              P.S,      P.stage_elems,
                      P.ntiles, B->V,    B->tile_work, B->chunk_bytes, B->tuned, B->pairs};
   for (int i = 0; i < n && i < 12; ++i) info[i] = v[i];
@@ -531,9 +534,10 @@ mm_status mm_batch_autotune(mm_handle* h, int substeps, mm_batch_tune* results, 
       B->args_par.clear();
       if ((st = upload_args(h)) != MM_OK) break;
       // one warm-up substep, then the timed ones, all from the saved state
-      CK(launch_batch(h, B->all, 0, h->stream));
+      const TilePlan& P = B->tuned_plan();
+      CK(launch_batch(h, P, 0, h->stream));
       CK(cudaEventRecord(e0, h->stream));
-      for (int i = 0; i < substeps; ++i) CK(launch_batch(h, B->all, (i + 1) & 1, h->stream));
+      for (int i = 0; i < substeps; ++i) CK(launch_batch(h, P, (i + 1) & 1, h->stream));
       CK(cudaEventRecord(e1, h->stream));
       CK(cudaEventSynchronize(e1));
       float ms = 0.f;

@@ -529,7 +529,8 @@ class Simulation:
 class Batch:
     """An ensemble of independent instances advanced together: one launch per
     substep over all members, the substeps of one step() call in one CUDA
-    graph (mm_create_batch). members[i] is a Simulation view of instance i
+    graph, or in float32 several members to one launch of all substeps
+    (mm_create_batch). members[i] is a Simulation view of instance i
     for its per-instance calls (set_state, set_velocity, moments, adjoint)."""
 
     def __init__(self, grids, rates, precision: str = "fp32", stream: int | None = None):
@@ -571,8 +572,9 @@ class Batch:
         self._check(self.lib.mm_debug_set(self.h, int(wait_limit), int(flags)))
 
     def autotune(self, substeps: int = 5):
-        """Time every (tile_work, chunk_bytes, cells per warp) candidate; keep
-        the fastest. Returns the list of timings."""
+        """Time every (tile_work, chunk_bytes, cells per warp) candidate for the
+        members that step over tiles (mm_batch_autotune); keep the fastest. Returns
+        the list of timings."""
         res = (mm_batch_tune * 64)()
         n = C.c_int()
         self._check(self.lib.mm_batch_autotune(self.h, int(substeps), res, 64, C.byref(n)))

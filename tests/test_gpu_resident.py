@@ -200,3 +200,26 @@ def test_small_instances_side_by_side(mmod, dims, handles):
     for i, (a, b) in enumerate(zip(*got)):
         for k in KEYS:
             assert np.array_equal(a[k], b[k]), (i, k)
+
+
+def test_autotune_times_the_tiles_in_use(mmod):
+    """A batch with a member that goes over tiles beside one that does not: the tuned
+    plan, and the launch information, are those of the first one's tiles."""
+    grids = [Grid(64, 64, 32, 32), Grid(192, 128, 64, 48)]
+    with mmod.Batch(grids, [Rates()] * 2, "fp32") as b:
+        for i, sim in enumerate(b.members):
+            psi, mb, u = inputs(sim.grid, 7 + i, 0.3)
+            sim.set_state(psi, mb)
+            sim.set_velocity(u)
+        before = [sim.get_state() for sim in b.members]
+        res = b.autotune(substeps=1)
+        info = b.launch_info()
+        after = [sim.get_state() for sim in b.members]
+        b.step(3)
+        b.sync()
+    assert len(res) == 36
+    for x, y in zip(before, after):
+        for k in KEYS:
+            assert np.array_equal(x[k], y[k]), k
+    cells = max(1, info["tile_work"] // (64 * 48))  # of a tile
+    assert info["tiles"] == -(-192 * 128 // cells)
