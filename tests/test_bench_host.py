@@ -88,3 +88,12 @@ def test_float64_operation_split(bench):
     integer pipe and the rest on the float64 pipe."""
     assert bench.SUBSTEP_OPS == 2 * 11 + 1
     assert bench.SUBSTEP_FP64_PIPE_OPS == bench.SUBSTEP_OPS - 2 * 5
+
+
+def test_float64_operations_of_the_roofline(bench):
+    """The float64 roofline counts what runs on the float64 pipe: the scheme's
+    operations without the sign transfers, minima and maximum (10) and without the
+    two halves, both taken on bit patterns."""
+    assert bench.SUBSTEP_FP64_PIPE_OPS_LEFT == bench.SUBSTEP_OPS - 2 * 5 - 2
+    src = open(bench.__file__).read()
+    assert src.count("SUBSTEP_FP64_PIPE_OPS_LEFT") >= 3  # defined, counted, reported
