@@ -744,7 +744,6 @@ cudaError_t launch_moments(const T* psi, const T* mb, const T* mf, const T* c,
       case 4: return go(k_moments<T, 4, 4>);
       case 8: return go(k_moments<T, 4, 8>);
       case 16: return go(k_moments<T, 4, 16>);
-      case 32: return go(k_moments<T, 4, 32>);
     }
     if (vw == 4) return go(k_moments<T, 4, 0>);
   }
