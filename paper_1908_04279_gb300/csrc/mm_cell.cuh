@@ -367,9 +367,9 @@ __device__ __forceinline__ void store_packed(T* p, int nv, const T (&m)[8]) {
 // in float32 where a row is not a power of two of full lanes. Rows of whole
 // 16-byte vectors (VW values) go straight to dst; others are written back into
 // the stage, from where the caller copies the chunk coalesced. Per substep on a
-// GB300: float64 128^2 x 32^2 850 (two nodes per lane) -> 585 us, 64^2 x 32 x 31
-// 297 (one) -> 160; float32 480 x 400 x 24 x 30 1630 (one) -> 388, 512^2 x 24 x 20
-// 513 (four) -> 502.
+// GB300: float64 128^2 x 32^2 850 (two nodes per lane) -> 586 us, 64^2 x 32 x 31
+// 297 (one) -> 162; float32 480 x 400 x 24 x 30 1630 (one) -> 395, 60^2 x 48 x 36 63
+// (four) -> 49. row_plan (mm_plan.h) says where it is taken.
 template <typename T, int VW, bool SPLIT = false>
 __device__ __forceinline__ void rows_packed(T* stage, T* dst, int RC, int ns, const LaneGeom& lg,
                                             const RkConst<T>& k, T ds, T* s_nb_chunk) {

@@ -62,10 +62,11 @@ inline double pass_cost(bool packed, int V, int tsz) {
 // Packed rows or V nodes to a lane, whichever costs less for `total` rows of ns
 // nodes: packed wastes lanes on few rows (float64 8 x 8 a cell: 733 against 507 us),
 // V nodes to a lane on rows that are no power of two of lanes (float32 48 x 36: 63
-// against 47). float32 rows of a multiple of eight nodes have eight to a lane
+// against 49). float32 rows of a multiple of eight nodes have eight to a lane
 // already (packing them leaves fewer idle lanes where their lanes are no power of
 // two, but its remainders cost more: 400^2 x 24 x 24 343 against 266 us), and of no
-// multiple of four are always packed (one node to a lane: 225 against 65).
+// multiple of four are always packed (one node to a lane: 200 x 150 x 24 x 30 228
+// against 69).
 inline RowPlan row_plan(int total, int ns, int V, int tsz, int chunk_bytes) {
   const size_t row_bytes = (size_t)ns * tsz;
   const RowPlan p = chunk_plan(true, total, row_bytes, packed_rpp(ns), chunk_bytes);

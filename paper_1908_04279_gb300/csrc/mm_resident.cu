@@ -1,10 +1,10 @@
 // Many substeps in one launch with the motor density resident on the chip
-// (float32 form): the substeps of k_substep for instances up to about the size
-// of L2. Mb is kept in the shared memory of all SMs together (about 33 MB),
-// whole or in part; the row passes that do not fit are read and written every
-// substep through each worker's ring.
+// (float32 form): the substeps of k_substep for instances up to about twice the
+// size of L2 (resident_limit, mm_plan.h). Mb is kept in the shared memory of all SMs
+// together (about 33 MB), whole or in part; the row passes that do not fit are
+// read and written every substep through each worker's ring.
 //
-// One block per SM owns a run of consecutive cells for the whole call and
+// A block (one per SM; fewer of a small instance) owns a run of cells for the call and
 // keeps their s-rows in shared memory: what is kept crosses HBM once per call
 // instead of once per substep, and the launch, the ring set-up, the scalar loads and
 // the last-block sum that every k_substep launch pays are paid once. Between
@@ -33,8 +33,7 @@
 // one run: a row takes nl = ceil(ns / 8) lanes of eight nodes each and a pass
 // takes the next floor(32 / nl) rows, of one cell or of several, so that neither
 // short rows, nor odd ones, nor a row count that is no multiple of a pass
-// leaves lanes idle (the streaming kernel gives a lane one node where ns is not
-// a multiple of 4). With RAG the nodes past a row's end are kept at zero and
+// leaves lanes idle. With RAG the nodes past a row's end are kept at zero and
 // the last node's slope is dropped by a factor. Rows in shared memory are
 // lane-major: a pass is two arrays of 32 float4, lane l's eight nodes at [0][l]
 // and [1][l], four conflict-free 16-byte accesses per lane whatever ns is. Psi
@@ -56,10 +55,9 @@
 // chain rows -> close -> arrival -> neighbours' psi at the smallest. 15 workers of
 // 128 registers: 19 of 96 are within 3 %, 11 or 23 slower. Measured on a GB300,
 // us per substep against k_substep in a CUDA graph: 32^2 x 16^2 7.2 -> 4.1, 64^2 x
-// 32^2 13.4 -> 6.4, 128^2 x 16^2 23 -> 9.8, 128^2 x 32^2 35.2 -> 25.3, 256^2 x 16^2
-// 77 -> 35, 85 x 61 x 24 x 30 57 -> 8.0, 200 x 150 x 24 x 30 65 -> 43
-// (231 before k_substep's rows were packed; the 57 is from then too); the 64-member
-// ensemble 594 (tuned) -> 427.
+// 32^2 13.4 -> 6.4, 128^2 x 16^2 23 -> 9.7, 128^2 x 32^2 35.2 -> 25.4, 256^2 x 16^2
+// 77 -> 35; against one launch a call 85 x 61 x 24 x 30 20 -> 8.0, 200 x 150 x 24 x 30 69 ->
+// 45, 400^2 x 24 x 30 331 -> 243; the 64-member ensemble 594 (tuned) -> 424.
 #include <map>
 #include <mutex>
 

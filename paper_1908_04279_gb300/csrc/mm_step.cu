@@ -8,8 +8,8 @@
 //      stages filled by bulk asynchronous copies (cp.async.bulk, the Tensor
 //      Memory Accelerator) that complete on mbarriers; lane 0 keeps up to S
 //      chunks in flight ahead of the warp. A row takes ceil(ns / 8) lanes of
-//      eight consecutive s-nodes each (rows_chunk pads them to a power of two);
-//      the Superbee stencil reaches across lanes with warp shuffles; the new
+//      eight consecutive s-nodes each (rows_chunk pads them to a power of two), or
+//      lanes of four, two or one where that costs less (row_plan); the Superbee stencil reaches across lanes with warp shuffles; the new
 //      row goes straight back to global memory in place;
 //   2. n_b of every row by a shuffle reduction over s (the force and force
 //      dipole are reduced in float64 by the moments kernel instead);

@@ -326,7 +326,7 @@ __device__ __forceinline__ T packed_sum(T x, int nl, int sl) {
 // wherever a row is summed. Gradients need that: which Superbee branch nearly tied
 // differences take follows the last bits of n_b through the substeps, and
 // derivatives in k_off and v_walk, small differences of large terms, then move
-// by up to 2e-4 (41 x 37 x 52 x 14 over 60 substeps). V = 4: the two halves of a
+// by up to 2e-4 (37 x 41 x 52 x 14 over 60 substeps). V = 4: the two halves of a
 // lane as a lane each, the last stride between them. V = 1: the strides of 16
 // and 8 nodes across lanes for each node of a lane, then 4, 2 and 1 within it.
 __device__ __forceinline__ float row_sum_x2(const float2 (&M)[4], int vl, int nl, int sl) {
