@@ -234,11 +234,12 @@ __device__ __forceinline__ void rows_chunk_x2(const float* src_rows, float* dst,
                                               const RkConst<float>& k, float ds,
                                               float* s_nb_chunk) {
   constexpr int H = V / 2;
+  const int passes = (RC + lg.rpp - 1) / lg.rpp;
   const float2 c1 = make_float2(k.c1, k.c1), c2 = make_float2(k.c2, k.c2);
   const float2 e1 = make_float2(k.e1, k.e1), e2 = make_float2(k.e2, k.e2);
 #pragma unroll kStepUnroll
-  for (int r0 = 0; r0 < RC; r0 += lg.rpp) {
-    const int r = r0 + lg.rslot;  // row within the chunk
+  for (int p = 0; p < passes; ++p) {
+    const int r = p * lg.rpp + lg.rslot;  // row within the chunk
     const bool hi = SPLIT && r >= k.rsplit;
     const float c3s = hi ? k.c3b : k.c3, e3s = hi ? k.e3b : k.e3;
     const float2 c3 = make_float2(c3s, c3s), e3 = make_float2(e3s, e3s);
@@ -291,9 +292,10 @@ __device__ __forceinline__ void rows_chunk(const T* src_rows, T* dst, int RC, in
     rows_chunk_x2<V, SPLIT>(src_rows, dst, RC, ns, seg, lg, k, ds, s_nb_chunk);
     return;
   }
+  const int passes = (RC + lg.rpp - 1) / lg.rpp;
 #pragma unroll kStepUnroll
-  for (int r0 = 0; r0 < RC; r0 += lg.rpp) {
-    const int r = r0 + lg.rslot;  // row within the chunk
+  for (int p = 0; p < passes; ++p) {
+    const int r = p * lg.rpp + lg.rslot;  // row within the chunk
     const bool hi = SPLIT && r >= k.rsplit;
     const T c3 = hi ? k.c3b : k.c3, e3 = hi ? k.e3b : k.e3;
     const bool row_ok = r < RC;
@@ -374,6 +376,7 @@ template <typename T, int VW, bool SPLIT = false>
 __device__ __forceinline__ void rows_packed(T* stage, T* dst, int RC, int ns, const LaneGeom& lg,
                                             const RkConst<T>& k, T ds, T* s_nb_chunk) {
   constexpr bool direct = VW * sizeof(T) == 16;
+  const int passes = (RC + lg.rpp - 1) / lg.rpp;
   [[maybe_unused]] float2 keep[4];
   if constexpr (sizeof(T) == 4) {
 #pragma unroll
@@ -383,8 +386,8 @@ __device__ __forceinline__ void rows_packed(T* stage, T* dst, int RC, int ns, co
   }
   constexpr int kUnroll = sizeof(T) == 4 ? kStepUnroll : 1;
 #pragma unroll kUnroll
-  for (int r0 = 0; r0 < RC; r0 += lg.rpp) {
-    const int r = r0 + lg.rslot;  // row within the chunk
+  for (int p = 0; p < passes; ++p) {
+    const int r = p * lg.rpp + lg.rslot;  // row within the chunk
     const bool hi = SPLIT && r >= k.rsplit;
     const T c3 = hi ? k.c3b : k.c3, e3 = hi ? k.e3b : k.e3;
     const bool act = r < RC && lg.lane_ok;
