@@ -769,7 +769,7 @@ def run_ours(args):
     achieved = algo / (launch_ms * 1e-3) / 1e9
     # the large case's capture is taken at a quarter of its cells (256x256 x
     # 64 x 64) and scaled to a full launch by the motor cells
-    # (workloads up to about the size of L2 run a macro step in one resident launch)
+    # (workloads up to 250 MB of motor density run a macro step in one resident launch)
     kernel, o_kernel = ("k_substep" if w_ == "large512" else "k_substep_resident"
                         for w_ in (name, other))
     traffic = read_profile_traffic(kernel, name, "fp32")
